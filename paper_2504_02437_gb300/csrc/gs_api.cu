@@ -149,7 +149,7 @@ const gs_ctx::Tuned* find_tuned(const gs_ctx* c, int w, int h, int views) {
 }
 
 // Tile size and pixels per thread of a render: the autotuner's candidate while
-// it times one, else the configured values, else the tuned choice, else 16 / 1.
+// it times one, else the configured values, else the tuned choice, else 16 / 2 (8 / 1).
 void pick_layout(gs_ctx* c, int w, int h, int views, int& tile, int& ppt) {
     if (c->cfg.deterministic) {   // one warp per tile: no ordering question inside a CTA
         tile = 8;
@@ -167,7 +167,10 @@ void pick_layout(gs_ctx* c, int w, int h, int views, int& tile, int& ppt) {
     if (want == 1 || want == 2 || (want == 4 && tile == 16))
         ppt = want;
     else
-        ppt = (t && t->tile == tile) ? t->ppt : 1;
+        // 16 x 2 (with halved long tiles) is the fastest 16-px layout at every size measured: iteration
+        // with 16 x 1 / 16 x 2 of a 160x120 keyframe with 2k Gaussians 112 / 104 us, 1200x680 with 300k
+        // 551 / 502 us, 8 x 640x480 with 150k 1,148 / 1,045 us
+        ppt = (t && t->tile == tile) ? t->ppt : (tile == 16 ? 2 : 1);
 }
 
 // Set up the per-view cameras of a render and upload them with a kernel (no
@@ -423,9 +426,8 @@ int gs_create(const gs_config* cfg, int device, gs_ctx** out) {
         }
         ok = ok && dalloc(&c->offsets, V * cap) == cudaSuccess;
         ok = ok && dalloc(&c->ranges, (size_t)c->max_bins) == cudaSuccess;
-        ok = ok && dalloc(&c->work_order, (size_t)c->max_bins) == cudaSuccess;
-        ok = ok && dalloc(&c->work_order_next, (size_t)c->max_bins) == cudaSuccess;
-        ok = ok && dalloc(&c->work_order_graph, (size_t)c->max_bins) == cudaSuccess;
+        ok = ok && dalloc(&c->work_order, work_order_words(c->max_bins)) == cudaSuccess;
+        ok = ok && dalloc(&c->work_order_graph, work_order_words(c->max_bins)) == cudaSuccess;
         ok = ok && dalloc(&c->T_final, V * maxpix) == cudaSuccess;
         ok = ok && dalloc(&c->n_last, V * maxpix) == cudaSuccess;
         ok = ok && dalloc(&c->dLdC, 3 * V * maxpix) == cudaSuccess;
@@ -450,7 +452,7 @@ int gs_create(const gs_config* cfg, int device, gs_ctx** out) {
         ok = ok && cudaMallocHost((void**)&c->hflags, sizeof(uint32_t) * 16) == cudaSuccess;
         ok = ok && cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) == cudaSuccess;
         ok = ok && cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) == cudaSuccess;
-        for (int i = 0; i < 6; ++i)
+        for (int i = 0; i < 5; ++i)
             ok = ok && cudaEventCreateWithFlags(&c->side_ev[i], cudaEventDisableTiming) == cudaSuccess;
         ok = ok && cudaEventCreateWithFlags(&c->graph_done, cudaEventDisableTiming) == cudaSuccess;
         ok = ok && cudaStreamCreateWithFlags(&c->copy, cudaStreamNonBlocking) == cudaSuccess;
@@ -491,7 +493,7 @@ void gs_destroy(gs_ctx* c) {
     for (auto e : c->tpool) cudaEventDestroy(e);
     void* ptrs[] = {c->params, c->grads, c->adam_m, c->adam_v, c->dens_sum, c->dens_cnt, c->dom_cnt, c->adam_pw, c->dcam, c->rec,
                     c->tiles_touched, c->depth, c->dkey[0], c->dkey[1], c->dval[0], c->dval[1], c->offsets, c->ranges,
-                    c->work_order, c->work_order_next, c->work_order_graph, c->T_final, c->n_last, c->dLdC, c->grad2d, c->hist, c->vis_blocks, (void*)c->target_slot, c->ssim_maps, c->ssim_part, c->dcount,
+                    c->work_order, c->work_order_graph, c->T_final, c->n_last, c->dLdC, c->grad2d, c->hist, c->vis_blocks, (void*)c->target_slot, c->ssim_maps, c->ssim_part, c->dcount,
                     c->partials, c->psnr_part, c->reg_part, c->tile_part, c->fpart,
                     c->own_rgb, c->tgt_stage[0], c->tgt_stage[1]};
     for (void* p : ptrs) cudaFree(p);
@@ -500,7 +502,7 @@ void gs_destroy(gs_ctx* c) {
     if (c->hflags) cudaFreeHost(c->hflags);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
     if (c->side) cudaStreamDestroy(c->side);
-    for (int i = 0; i < 6; ++i)
+    for (int i = 0; i < 5; ++i)
         if (c->side_ev[i]) cudaEventDestroy(c->side_ev[i]);
     if (c->graph_done) cudaEventDestroy(c->graph_done);
     if (c->copy) cudaStreamDestroy(c->copy);
@@ -720,9 +722,7 @@ static int iteration_tail(gs_ctx* c, const DevConst& k, const float* target, con
         CK(launch_loss_tail(c, k, det ? c->tile_part : c->fpart, det ? c->n_bins : fgrid, loss_out, ts));
     }
     if (capture) CK(cudaMemcpyAsync(c->hflags, c->dcount, sizeof(uint32_t) * 11, cudaMemcpyDeviceToHost, ts));
-    if (c->order_ahead)   // the compositing is done with the current order: the next one goes in place
-        CK(cudaMemcpyAsync(c->work_order, c->work_order_next, sizeof(uint32_t) * (size_t)c->n_bins,
-                           cudaMemcpyDeviceToDevice, ts));
+    if (c->order_ahead) CK(launch_work_order(c, ts));   // the compositing has read its order: the next one
     {
         Phase ph(c, GS_PHASE_PROJECT_BWD, s);
         CK(reduce_pair_grads(c, s));
@@ -913,7 +913,7 @@ static int iterate_core(gs_ctx* c, const gs_camera* cams, int n_views, const flo
     c->rendered_rgb = rgb;
     const int64_t launches0 = c->launches;
     // the first replay composites in the order this direct call computed for the shape
-    CK(cudaMemcpyAsync(c->work_order_graph, c->work_order, sizeof(uint32_t) * (size_t)c->n_bins,
+    CK(cudaMemcpyAsync(c->work_order_graph, c->work_order, sizeof(uint32_t) * work_order_words(c->n_bins),
                        cudaMemcpyDeviceToDevice, s));
     c->cap_phases.clear();
     c->capturing = true;
@@ -1173,8 +1173,12 @@ int gs_debug_grad2d(gs_ctx* c, float* out) {
     const size_t n = (size_t)c->n, items = n * c->n_views;
     float* g = (float*)malloc(sizeof(float) * kGrad2dStride * items);
     if (!g) return fail(c, GS_ERR_OOM, "host buffer");
+    std::vector<float> opac(items);   // each record's opacity (the w of its first float4)
     cudaError_t e = cudaDeviceSynchronize();
     if (e == cudaSuccess) e = cudaMemcpy(g, c->grad2d, sizeof(float) * kGrad2dStride * items, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess && items)
+        e = cudaMemcpy2D(opac.data(), sizeof(float), reinterpret_cast<const float*>(c->rec) + 3,
+                         sizeof(float4) * kRecFloat4, sizeof(float), items, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) {
         free(g);
         return fail(c, GS_ERR_CUDA, "debug copy", e);
@@ -1190,7 +1194,7 @@ int gs_debug_grad2d(gs_ctx* c, float* out) {
             o[2 * n + i] = r[2] * -0.5f;
             o[3 * n + i] = -r[3];
             o[4 * n + i] = r[4] * -0.5f;
-            o[5 * n + i] = r[5];
+            o[5 * n + i] = r[5] != 0.f ? r[5] / opac[v * n + i] : 0.f;   // the records hold o dL/do
             o[6 * n + i] = r[6];
             o[7 * n + i] = r[7];
             o[8 * n + i] = r[8];

@@ -22,6 +22,12 @@ constexpr float kLn2 = 0.6931471805599453f;
 // largest pair buffer (pair indices are 32-bit)
 constexpr int64_t kMaxPairs = 0xFFFFFFF0ll;
 
+// Work list of the compositing kernels: [0] the number of items, then the items, longest first. An
+// item is a bin, or half of one (1 + half above kItemShift); a bin may take two.
+constexpr int kItemShift = 30;
+constexpr uint32_t kItemBin = (1u << kItemShift) - 1u;
+constexpr size_t work_order_words(int n_bins) { return 1 + 2 * (size_t)n_bins; }
+
 // Camera as the kernels read it (one per view, in device memory).
 struct DevCamera {
     float R[9];
@@ -104,8 +110,8 @@ struct gs_ctx {
     uint32_t* emit_item = nullptr;          // [pair capacity]
     float* pairgrad = nullptr;              // [pair capacity * 9]
     float* tile_part = nullptr;             // [max bins] photometric loss per (view, tile)
-    uint32_t* work_order = nullptr;         // [max bins] bins by decreasing pair count (while a
-                                            // replay is captured: the graph's own buffer)
+    uint32_t* work_order = nullptr;         // [work_order_words(max bins)] items by decreasing pair
+                                            // count (while a replay is captured: the graph's own)
     int max_bins = 0;
     float* T_final = nullptr;               // [max_views * H * W]
     uint32_t* n_last = nullptr;             // [max_views * H * W] entries up to the last blended
@@ -151,14 +157,13 @@ struct gs_ctx {
     // overlapping the projection and the sorts, and the loss total runs there beside the
     // projection adjoint and Adam (a fork and joins, which a captured graph keeps as branches)
     cudaStream_t side = nullptr;
-    cudaEvent_t side_ev[6] = {};            // fork, overflow flag + ranges zeroed, grad2d zeroed,
-                                            // second fork, side work done, ranges ready
+    cudaEvent_t side_ev[5] = {};            // fork, overflow flag + ranges zeroed, grad2d zeroed,
+                                            // second fork, side work done
     bool side_zeroed = false;               // this iteration's zeroing was issued on `side`
-    // a replayed iteration composites in the longest-first order the previous one computed (any
-    // order of the same bins gives the same result) and computes the next order on `side`
+    // a replayed iteration composites in the longest-first order the previous one left (any order of
+    // the same bins gives the same result) and writes the next one, on `side`, once it has composited
     bool order_ahead = false;
-    uint32_t* work_order_next = nullptr;    // [max bins]
-    uint32_t* work_order_graph = nullptr;   // [max bins] the order a replay composites in: its own
+    uint32_t* work_order_graph = nullptr;   // [work_order_words(max bins)] the order a replay composites in: its own
                                             // buffer, so that a render of another shape between
                                             // replays (which writes work_order) cannot change it
     cudaEvent_t graph_done = nullptr;       // recorded after each replay
@@ -220,6 +225,8 @@ cudaError_t emit_pairs(gs_ctx* c, uint32_t n_items, const uint32_t* n_dev, cudaS
 // exclusive scan of n u32 values (in may equal out); the total goes to *total_dev
 cudaError_t scan_u32(gs_ctx* c, const uint32_t* in, uint32_t* out, uint32_t n, uint32_t* total_dev, cudaStream_t s);
 cudaError_t compute_ranges(gs_ctx* c, cudaStream_t s);
+// the compositing kernels' work list, from the bin ranges
+cudaError_t launch_work_order(gs_ctx* c, cudaStream_t s);
 // deterministic mode: per-item fixed-order sum of the pair gradient slots into grad2d
 cudaError_t reduce_pair_grads(gs_ctx* c, cudaStream_t s);
 cudaError_t launch_raster_forward(gs_ctx* c, const DevConst& k, float* rgb, int32_t* argmax, cudaStream_t s);

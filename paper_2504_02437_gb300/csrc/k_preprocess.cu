@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(128, 6) k_preprocess_backward(
     G[7 * c + gid] = (dx - x * dot) * iq;
     G[8 * c + gid] = (dy - y * dot) * iq;
     G[9 * c + gid] = (dz - z * dot) * iq;
-    G[10 * c + gid] = dop * oa * (1.f - oa);
+    G[10 * c + gid] = dop * (1.f - oa);   // the records hold o dL/do, do/dlogit = o (1 - o)
     G[11 * c + gid] = dr;
     G[12 * c + gid] = dg;
     G[13 * c + gid] = db;

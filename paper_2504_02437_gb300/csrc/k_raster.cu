@@ -6,6 +6,13 @@
 // sorted pair list is walked in batches of records staged in shared memory
 // (gathered by Gaussian id from the 48-byte raster records).
 //
+// Two things bound a launch: the SMs' issue slots where tiles are many and alike,
+// and the longest tile's chain of dependent visits where they are few or unlike
+// (a 16 x 2 tile of a 1200x680 keyframe took one CTA 541 us while the average CTA
+// was busy for 264). Whole tiles of two pixels a thread are written for the first
+// (branches around pixels that are not hit); long tiles go as halves of one pixel
+// a thread, written for the second (visits two at a time and without branches).
+//
 // Membership is pixel-exact (|px - u| <= r and |py - v| <= r), so the image is
 // the same for every tile size: tiles only bound which Gaussians a pixel tests.
 #include <algorithm>
@@ -37,6 +44,44 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
+// Two floats in one 64-bit register and the packed IEEE operations on them (each half rounds as the
+// scalar operation does): in the adjoint a thread's pixels go in pairs, one instruction for both, and
+// a pixel that a Gaussian misses takes part with alpha 0 instead of branching around.
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 pack2(float a, float b) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ F2 pack2(float a) { return pack2(a, a); }
+__device__ __forceinline__ void unpack2(F2 x, float& a, float& b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x.v));
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// A colour or an upstream gradient that is not finite, or so large that a product of two overflows:
+// times a weight of zero it would not vanish, so a batch (or warp) with one masks its operands.
+__device__ __forceinline__ bool unsafe(float x) { return !(fabsf(x) <= 1e15f); }
 
 // A raster record staged for one tile, relative to the local origin (ox, oy),
 // the tile's corner rounded down to a multiple of 32 px:
@@ -110,11 +155,12 @@ __device__ __forceinline__ void short_axis_strip(const float4 s1, float thr, flo
     wn = fmaf(sqrtf(-thr / lam), 1.001f, 0.01f);
 }
 
-// Thread layout of a TILE x TILE tile: each thread owns PPT pixels of one
-// column, 4 rows apart; warp w owns an 8 x (4 PPT) block.
-template <int TILE, int PPT>
+// Thread layout of a work item, 1 / SPLIT of the rows of a TILE x TILE tile: each thread owns PPT
+// pixels of one column, 4 rows apart; warp w owns an 8 x (4 PPT) block.
+template <int TILE, int PPT, int SPLIT = 1>
 struct Layout {
-    static constexpr int kThreads = TILE * TILE / PPT;
+    static constexpr int kThreads = TILE * TILE / PPT / SPLIT;
+    static constexpr int kRows = TILE / SPLIT;
     static constexpr int kBlocksX = TILE / 8;
     // resident CTAs per SM the fused kernel is compiled for (its register cap): 16 x 1 (8 warps a
     // CTA) capped at 64 registers for 4 CTAs instead of 3 (8-view 640x480 window: fused kernel
@@ -122,12 +168,19 @@ struct Layout {
     // keep the compiler's own register count (an explicit bound of 1 let it take more: 16 x 2
     // rose from 80 to 96 registers, 5 CTAs per SM instead of 6, 5 % slower)
     static constexpr int kMinBlocks = (TILE == 16 && PPT == 1) ? 4 : 0;
+    // visit-list entries a thread of one pixel takes together: two in halves of long tiles, whose
+    // latency counts (1200x680 keyframe with 300k Gaussians: fused kernel 362, 355 and 345 us for 1, 2
+    // and 4; 8-view window 785 us with 2, 856 with 4), one where a launch is bound by issue slots
+    // (16 x 1: 376, 398 and 427 us)
+    static constexpr int kVisits = SPLIT == 2 ? 2 : 1;
+    // long tiles go as two items of one pixel a thread, in the same CTAs as whole tiles of two
+    static constexpr bool kHalves = TILE == 16 && PPT == 2;
     // the adjoint reuses the forward's staged batch and visit lists when the tile's whole list
     // fits one batch, and then starts without CTA barriers (each warp cuts its own list at its
     // own end): 16 x 1 window 0.645 -> 0.634 ms, 8 x 1 0.653 -> 0.636 ms; not for 16 x 2, where
     // the warps' imbalance moves to the work queue's barrier (300k-Gaussian keyframe: 0.362 ->
     // 0.383 ms)
-    static constexpr bool kReuseStaged = !(TILE == 16 && PPT == 2);
+    static constexpr bool kReuseStaged = !(TILE == 16 && PPT == 2) && SPLIT == 1;
     __device__ static void pixel(int tid, int& lx, int& ly0) {
         const int w = tid >> 5, l = tid & 31;
         lx = (w % kBlocksX) * 8 + (l & 7);
@@ -221,20 +274,21 @@ __device__ __forceinline__ Stage<B, NW>& stage() {
 }
 
 // Geometry of one work item (a tile of one view) as seen by one thread.
-template <int TILE, int PPT>
+template <int TILE, int PPT, int SPLIT = 1>
 struct TileGeom {
-    int view, txi, tyi, px, py0;
+    int view, txi, row0, px, py0;
     float ox, oy, fx;
     uint2 rg;
-    __device__ TileGeom(int bin, const uint2* __restrict__ ranges, int tiles_x, int tiles_per_view) {
+    __device__ TileGeom(int bin, int part, const uint2* __restrict__ ranges, int tiles_x, int tiles_per_view) {
         view = bin / tiles_per_view;
         const int t = bin - view * tiles_per_view;
-        tyi = t / tiles_x;
+        const int tyi = t / tiles_x;
         txi = t - tyi * tiles_x;
         int lx, ly0;
-        Layout<TILE, PPT>::pixel(threadIdx.x, lx, ly0);
+        Layout<TILE, PPT, SPLIT>::pixel(threadIdx.x, lx, ly0);
         px = txi * TILE + lx;
-        py0 = tyi * TILE + ly0;
+        row0 = tyi * TILE + part * Layout<TILE, PPT, SPLIT>::kRows;
+        py0 = row0 + ly0;
         // pixel offsets are taken from a 32-px-aligned local origin (see load_record)
         ox = (float)((txi * TILE) & ~31);
         oy = (float)((tyi * TILE) & ~31);
@@ -246,16 +300,16 @@ struct TileGeom {
 
 // Warps of the CTA whose 8 x (4 PPT) pixel block meets the box u +- hx, v +- hy and the
 // short-axis strip |n . (x - u)| <= wn.
-template <int TILE, int PPT>
-__device__ __forceinline__ uint32_t warp_mask(const TileGeom<TILE, PPT>& g, const float4 s0, const float4 s1,
+template <int TILE, int PPT, int SPLIT>
+__device__ __forceinline__ uint32_t warp_mask(const TileGeom<TILE, PPT, SPLIT>& g, const float4 s0, const float4 s1,
                                               float thr) {
     float nx, ny, wn;
     short_axis_strip(s1, thr, nx, ny, wn);
     // half-extents of a warp's pixel block projected on n, plus the rounding slack of the box test
     const float hb = 3.5f * fabsf(nx) + 0.5f * (float)(4 * PPT - 1) * fabsf(ny) + wn + 0.01f;
-    constexpr int NW = Layout<TILE, PPT>::kThreads / 32;
-    constexpr int BX = Layout<TILE, PPT>::kBlocksX;
-    const float tox = (float)(g.txi * TILE) - g.ox, toy = (float)(g.tyi * TILE) - g.oy;
+    constexpr int NW = Layout<TILE, PPT, SPLIT>::kThreads / 32;
+    constexpr int BX = Layout<TILE, PPT, SPLIT>::kBlocksX;
+    const float tox = (float)(g.txi * TILE) - g.ox, toy = (float)g.row0 - g.oy;
     // widened by 0.01 px so that rounding cannot drop a pixel the per-pixel test would keep
     const float x0 = s0.x - s0.z - 0.01f, x1 = s0.x + s0.z + 0.01f, y0 = s0.y - s0.w - 0.01f,
                 y1 = s0.y + s0.w + 0.01f;
@@ -276,12 +330,13 @@ __device__ __forceinline__ uint32_t warp_mask(const TileGeom<TILE, PPT>& g, cons
 // The return value is the length of the warp's visit list when the tile's whole
 // list was staged as one batch (it is left in shared memory for the adjoint),
 // else -1; which of the two is the same for every warp of the CTA.
-template <int TILE, int PPT, bool ARGMAX, bool DET>
-__device__ __forceinline__ int fwd_core(const TileGeom<TILE, PPT>& g, const bool (&inside)[PPT],
+template <int TILE, int PPT, int SPLIT, bool ARGMAX, bool DET>
+__device__ __forceinline__ int fwd_core(const TileGeom<TILE, PPT, SPLIT>& g, const bool (&inside)[PPT],
                                          const uint32_t* __restrict__ pval, const uint32_t* __restrict__ emit_item,
                                          const float4* __restrict__ rec, const DevConst& kc, float (&T)[PPT], float (&cr)[PPT], float (&cg)[PPT],
-                                         float (&cb)[PPT], uint32_t (&last)[PPT], uint32_t (&amax)[PPT]) {
-    constexpr int NT = Layout<TILE, PPT>::kThreads;
+                                         float (&cb)[PPT], uint32_t (&last)[PPT], uint32_t (&amax)[PPT],
+                                         bool& masked) {
+    constexpr int NT = Layout<TILE, PPT, SPLIT>::kThreads;
     constexpr int kBatch = batch_for(NT);
     Stage<kBatch, NT / 32>& st = stage<kBatch, NT / 32>();
     float4* s0 = st.s0;
@@ -305,8 +360,12 @@ __device__ __forceinline__ int fwd_core(const TileGeom<TILE, PPT>& g, const bool
     }
     const uint2 rg = g.rg;
     int staged = -1;
+    // for an adjoint that reuses the staged batch: whether its colours need masking there
+    constexpr bool kMarkWild = !DET && Layout<TILE, PPT, SPLIT>::kReuseStaged;
+    masked = false;
     for (uint32_t bs = rg.x; bs < rg.y; bs += kBatch) {
         if (__syncthreads_count(nlive > 0) == 0) break;
+        bool wild = false;
         for (int i = threadIdx.x; i < kBatch; i += NT) {
             const uint32_t j = bs + i;
             if (j < rg.y) {
@@ -314,14 +373,63 @@ __device__ __forceinline__ int fwd_core(const TileGeom<TILE, PPT>& g, const bool
                 const uint32_t item = DET ? emit_item[pv] : pv;
                 stage_record(rec, item, g.ox, g.oy, kc.alpha_min, s0[i], s1[i], s2[i]);
                 sid[i] = pv;
-                st.mask[i] = warp_mask<TILE, PPT>(g, s0[i], s1[i], s2[i].w);
+                st.mask[i] = warp_mask(g, s0[i], s1[i], s2[i].w);
+                if constexpr (kMarkWild) wild |= unsafe(s2[i].x) || unsafe(s2[i].y) || unsafe(s2[i].z);
             }
         }
-        __syncthreads();
+        if constexpr (kMarkWild)
+            masked = __syncthreads_or(wild);
+        else
+            __syncthreads();
         const int cnt = min((uint32_t)kBatch, rg.y - bs);
         const int nk = build_warp_list(st, cnt, 0u, 0xFFFFFFFFu);
         if (rg.y - rg.x <= (uint32_t)kBatch) staged = nk;
         const typename Stage<kBatch, NT / 32>::Idx* wl = st.list[threadIdx.x >> 5];
+        if constexpr (PPT == 1) {
+            // one pixel a thread: kVisits entries at a time, their loads, tests and alphas without
+            // branches, so that their latencies overlap; only T runs through them in turn (16 x 1, one
+            // entry at a time, with the adjoint in the same form: 1200x680 keyframe 416 -> 376 us,
+            // 160x120 47 -> 36 us)
+            constexpr int U = Layout<TILE, PPT, SPLIT>::kVisits;
+            bool live = nlive > 0;
+            for (int i = 0; i < nk; i += U) {
+                if (!__any_sync(0xFFFFFFFFu, live)) break;
+                int k[U];
+                float al[U];
+                bool hit[U];
+                float4 c[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    k[u] = (int)wl[i + u] & (kBatch - 1);   // past nk: any entry, not hit
+                    const float4 a = s0[k[u]], q = s1[k[u]];
+                    c[u] = s2[k[u]];
+                    const float dx = g.fx - a.x, dy = fy[0] - a.y;
+                    const float p2 = power2_dy(q.z, __fmul_rn(q.y, dx), __fmul_rn(__fmul_rn(q.x, dx), dx), dy);
+                    hit[u] = i + u < nk && fabsf(dx) <= a.z && fabsf(dy) <= a.w && p2 >= c[u].w;
+                    al[u] = fminf(kc.alpha_max, __fmul_rn(q.w, ex2_approx(p2)));
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const float Tn = __fmul_rn(T[0], 1.f - al[u]);
+                    const bool in = hit[u] && live;
+                    live = live && !(in && Tn < kc.T_min);   // a pixel stops before it falls below T_min
+                    if (in && live) {
+                        const float wgt = al[u] * T[0];
+                        cr[0] = fmaf(c[u].x, wgt, cr[0]);
+                        cg[0] = fmaf(c[u].y, wgt, cg[0]);
+                        cb[0] = fmaf(c[u].z, wgt, cb[0]);
+                        T[0] = Tn;
+                        last[0] = bs + k[u] - rg.x + 1;
+                        if (ARGMAX && wgt > wmax[0]) {
+                            wmax[0] = wgt;
+                            amax[0] = DET ? emit_item[sid[k[u]]] : sid[k[u]];
+                        }
+                    }
+                }
+            }
+            nlive = live ? 1 : 0;
+            continue;
+        }
         int knext = nk > 0 ? (int)wl[0] : 0;   // the next entry's index is loaded one visit ahead
         // unrolled by two: the next entry's record loads and membership tests interleave with
         // this entry's blending (A/B on the 300k-Gaussian keyframe, 16 x 2 layout: fused kernel
@@ -377,25 +485,69 @@ __device__ __forceinline__ int fwd_core(const TileGeom<TILE, PPT>& g, const bool
     return staged;
 }
 
+// The nine screen partials of one Gaussian from a thread's sums of g2 = dL/dp2 (without ln 2),
+// g2 dy, g2 dy^2 and minus the colour gradients over pixels that share dx: u, v, a', b', c', the
+// opacity's times the opacity (its readers divide), r, g, b.
+__device__ __forceinline__ void screen_partials(const float4 q, float dx, float g2, float g2y, float g2yy, float ncr,
+                                                float ncg, float ncb, float (&acc)[9]) {
+    acc[0] = -fmaf(2.f * q.x * dx, g2, q.y * g2y);
+    acc[1] = -fmaf(q.y * dx, g2, 2.f * q.z * g2y);
+    acc[2] = dx * dx * g2;
+    acc[3] = dx * g2y;
+    acc[4] = g2yy;
+    acc[5] = g2;
+    acc[6] = -ncr;
+    acc[7] = -ncg;
+    acc[8] = -ncb;
+}
+
+// Adds a warp's partials of one Gaussian (lanes with `any` blended it) to its record.
+template <bool DET>
+__device__ __forceinline__ void add_gradient(bool any, const float (&acc)[9], uint32_t id, int lane,
+                                             float* __restrict__ grad2d, float* __restrict__ pairgrad) {
+    const uint32_t who = __ballot_sync(0xFFFFFFFFu, any);
+    if (who == 0u) return;
+    if constexpr (DET) {
+        // deterministic mode (one warp per tile): the warp's fixed-order sum is the
+        // whole tile's contribution; it goes to the pair's own slot, no atomics
+        int idx;
+        const float v = warp_sum9(acc, lane, idx);
+        if (idx >= 0) pairgrad[(size_t)id * kPairGradStride + idx] = v;
+    } else if (__popc(who) <= kLaneAtomicMax) {
+        // few lanes blended this Gaussian: each adds its own values (no warp sum)
+        if (any) {
+            float* gp = grad2d + (size_t)id * kGrad2dStride;
+            atomicAdd(reinterpret_cast<float4*>(gp), make_float4(acc[0], acc[1], acc[2], acc[3]));
+            atomicAdd(reinterpret_cast<float4*>(gp + 4), make_float4(acc[4], acc[5], acc[6], acc[7]));
+            atomicAdd(gp + 8, acc[8]);
+        }
+    } else {
+        int idx;
+        const float v = warp_sum9(acc, lane, idx);
+        if (idx >= 0) atomicAdd(grad2d + (size_t)id * kGrad2dStride + idx, v);
+    }
+}
+
 // Adjoint of the compositing for a thread's PPT pixels: walks the tile's list
 // back to front from the block's largest last-blended entry, recovering
 // T_i = T_{i+1} / (1 - alpha_i) from the final T, and accumulates the
 // gradients w.r.t. each Gaussian's screen quantities (the first five, u, v and
-// the exp2-scaled conic a', b', c', without the factor ln 2 of d 2^p / dp) (when at most
+// the exp2-scaled conic a', b', c', without the factor ln 2 of d 2^p / dp; the opacity's times
+// the opacity) (when at most
 // kLaneAtomicMax lanes blended it, each adds its own 9 values with two float4
 // atomics and one scalar; else a warp sum, then one 9-lane atomic). Each
 // warp visits only the batch entries its compacted list holds, which stop at
 // the warp's largest last-blended entry. With staged >= 0 (the forward left the
 // tile's whole list staged, and this warp's visit list of that length) each
 // warp cuts its own list at its own end and walks it without a CTA barrier.
-template <int TILE, int PPT, bool DET>
-__device__ __forceinline__ void bwd_core(const TileGeom<TILE, PPT>& g, const uint32_t* __restrict__ pval,
+template <int TILE, int PPT, int SPLIT, bool DET>
+__device__ __forceinline__ void bwd_core(const TileGeom<TILE, PPT, SPLIT>& g, const uint32_t* __restrict__ pval,
                                          const uint32_t* __restrict__ emit_item, const float4* __restrict__ rec,
                                          const DevConst& kc, float (&T)[PPT], const uint32_t (&cnt_last)[PPT],
                                          const float (&gr)[PPT], const float (&gg)[PPT], const float (&gb)[PPT],
                                          float* __restrict__ grad2d, float* __restrict__ pairgrad, int staged,
-                                         bool fwd_masks) {
-    constexpr int NT = Layout<TILE, PPT>::kThreads;
+                                         bool fwd_masks, bool masked) {
+    constexpr int NT = Layout<TILE, PPT, SPLIT>::kThreads;
     constexpr int kBatch = batch_for(NT);
     Stage<kBatch, NT / 32>& st = stage<kBatch, NT / 32>();
     float4* s0 = st.s0;
@@ -405,13 +557,15 @@ __device__ __forceinline__ void bwd_core(const TileGeom<TILE, PPT>& g, const uin
     __shared__ uint32_t smax;
     const int lane = threadIdx.x & 31;
     const uint2 rg = g.rg;
-    float fy[PPT], ga[PPT];   // ga: upstream gradient . normalised colour behind the current Gaussian
+    float fy[PPT], ga[PPT];   // ga: minus the upstream gradient . normalised colour behind the Gaussian
     uint32_t my_end[PPT];
     uint32_t thread_end = rg.x;
+    bool wild = false;
 #pragma unroll
     for (int p = 0; p < PPT; ++p) {
         fy[p] = (float)g.py(p) - g.oy;
         ga[p] = 0.f;
+        wild |= unsafe(gr[p]) || unsafe(gg[p]) || unsafe(gb[p]);
         my_end[p] = rg.x + cnt_last[p];
         thread_end = max(thread_end, my_end[p]);
     }
@@ -426,6 +580,7 @@ __device__ __forceinline__ void bwd_core(const TileGeom<TILE, PPT>& g, const uin
         end = smax;
     }
     const uint32_t warp_end = wm;
+    const bool warp_wild = __any_sync(0xFFFFFFFFu, wild);
     for (uint32_t be = end; be > rg.x;) {
         const uint32_t bs = be - rg.x > (uint32_t)kBatch ? be - kBatch : rg.x;
         const typename Stage<kBatch, NT / 32>::Idx* wl = st.list[threadIdx.x >> 5];
@@ -443,6 +598,7 @@ __device__ __forceinline__ void bwd_core(const TileGeom<TILE, PPT>& g, const uin
             // the forward's warp masks of a one-batch tile are still staged (nothing writes them
             // in between): only the records are staged again
             const bool keep_masks = fwd_masks && rg.y - rg.x <= (uint32_t)kBatch;
+            wild = false;
             __syncthreads();
             for (int i = threadIdx.x; i < kBatch; i += NT) {
                 const uint32_t j = bs + i;
@@ -451,118 +607,203 @@ __device__ __forceinline__ void bwd_core(const TileGeom<TILE, PPT>& g, const uin
                     const uint32_t item = DET ? emit_item[pv] : pv;
                     stage_record(rec, item, g.ox, g.oy, kc.alpha_min, s0[i], s1[i], s2[i]);
                     sid[i] = pv;
-                    if (!keep_masks) st.mask[i] = warp_mask<TILE, PPT>(g, s0[i], s1[i], s2[i].w);
+                    if (!keep_masks) st.mask[i] = warp_mask(g, s0[i], s1[i], s2[i].w);
+                    wild |= unsafe(s2[i].x) || unsafe(s2[i].y) || unsafe(s2[i].z);
                 }
             }
-            __syncthreads();
+            masked = __syncthreads_or(wild);
             nk = build_warp_list(st, (int)(be - bs), bs, warp_end);
         }
-        int knext = nk > 0 ? (int)wl[nk - 1] : 0;   // as in the forward: one visit ahead
-        for (int i = nk - 1; i >= 0; --i) {
-            const int k = knext;
-            if (i > 0) knext = wl[i - 1];
-            const uint32_t pos = bs + k;
-            const float4 a = s0[k];
-            const float dx = g.fx - a.x;
-            const bool col = fabsf(dx) <= a.z && pos < thread_end;
-            float acc[9];
+        if constexpr (PPT == 1) {
+            // U entries at a time: their loads, tests and alphas first and without branches (a pixel that
+            // is not hit has alpha 0 and adds zeros), then T and g . a through them in turn, then their sums
+            constexpr int U = Layout<TILE, PPT, SPLIT>::kVisits;
+            for (int i = nk - 1; i >= 0; i -= U) {
+                int k[U];
+                float acc[U][9];
+                float4 c[U], q[U];
+                float dx[U], dy[U], oG[U], nal[U], rc[U];
+                bool hit[U];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) acc[i] = 0.f;
-            bool any = false;
-            if (col) {
-                const float4 q = s1[k];
-                const float4 c = s2[k];
-                const float qydx = __fmul_rn(q.y, dx), qxdx2 = __fmul_rn(__fmul_rn(q.x, dx), dx);
-                float p2v[PPT];
-                bool hit[PPT];
-#pragma unroll
-                for (int p = 0; p < PPT; ++p) {   // as in the forward: all pixels' tests first
-                    const float dy = fy[p] - a.y;
-                    p2v[p] = power2_dy(q.z, qydx, qxdx2, dy);
-                    hit[p] = pos < my_end[p] && fabsf(dy) <= a.w && p2v[p] >= c.w;
+                for (int u = 0; u < U; ++u) {
+                    k[u] = (int)wl[U == 1 ? i : max(i - u, 0)];
+                    const float4 a = s0[k[u]];
+                    q[u] = s1[k[u]];
+                    c[u] = s2[k[u]];
+                    dx[u] = g.fx - a.x;
+                    dy[u] = fy[0] - a.y;
+                    const float p2 = power2_dy(q[u].z, __fmul_rn(q[u].y, dx[u]),
+                                               __fmul_rn(__fmul_rn(q[u].x, dx[u]), dx[u]), dy[u]);
+                    hit[u] = (U == 1 || i - u >= 0) && bs + k[u] < my_end[0] && fabsf(dx[u]) <= a.z &&
+                             fabsf(dy[u]) <= a.w && p2 >= c[u].w;
+                    oG[u] = __fmul_rn(q[u].w, ex2_approx(p2));
+                    nal[u] = hit[u] ? -fminf(kc.alpha_max, oG[u]) : 0.f;
+                    rc[u] = rcp_approx(1.f + nal[u]);   // 1 - alpha >= 1 - alpha_max = 0.01
                 }
-                float Gv[PPT];   // all pixels' ex2 back to back (the MUFU pipe has room)
 #pragma unroll
-                for (int p = 0; p < PPT; ++p) Gv[p] = ex2_approx(p2v[p]);
-#pragma unroll
-                for (int p = 0; p < PPT; ++p) {
-                    if (!hit[p]) continue;
-                    const float dy = fy[p] - a.y;
-                    const float G = Gv[p];
-                    const float oG = __fmul_rn(q.w, G);
-                    const float alpha = fminf(kc.alpha_max, oG);
-                    any = true;
-                    const float oma = 1.f - alpha;       // >= 1 - alpha_max = 0.01
-                    T[p] = __fdividef(T[p], oma);        // transmittance in front of this Gaussian (2 ulp)
-                    const float wgt = alpha * T[p];
-                    acc[6] = fmaf(gr[p], wgt, acc[6]);
-                    acc[7] = fmaf(gg[p], wgt, acc[7]);
-                    acc[8] = fmaf(gb[p], wgt, acc[8]);
+                for (int u = 0; u < U; ++u) {
+                    float gx = gr[0], gy = gg[0], gz = gb[0];
+                    if ((masked | warp_wild) && !hit[u]) gx = gy = gz = 0.f;
+                    T[0] *= rc[u];   // transmittance in front of this Gaussian
+                    const float nw = nal[u] * T[0];
                     // dL/dalpha = T (g . c - g . a), with a the normalised colour behind this
-                    // Gaussian, a <- a + alpha (c - a); g is fixed per pixel, so only g . a is kept
-                    const float d = fmaf(gr[p], c.x, fmaf(gg[p], c.y, gb[p] * c.z)) - ga[p];
-                    const float dalpha = T[p] * d;
-                    ga[p] = fmaf(alpha, d, ga[p]);
+                    // Gaussian, a <- a + alpha (c - a); g is fixed per pixel, so only -g . a is kept
+                    const float d = fmaf(gx, c[u].x, fmaf(gy, c[u].y, gz * c[u].z)) + ga[0];
+                    ga[0] = hit[u] ? fmaf(nal[u], d, ga[0]) : ga[0];
                     // through alpha = o 2^p2, zero where the 0.99 clamp holds; the factor ln 2
                     // of d(2^p2)/dp2 is left to the readers of the screen gradients
-                    const bool open = oG <= kc.alpha_max;
-                    const float g2 = open ? dalpha * oG : 0.f;
-                    acc[0] -= g2 * (2.f * q.x * dx + q.y * dy);
-                    acc[1] -= g2 * (q.y * dx + 2.f * q.z * dy);
-                    acc[2] = fmaf(g2 * dx, dx, acc[2]);
-                    acc[3] = fmaf(g2 * dx, dy, acc[3]);
-                    acc[4] = fmaf(g2 * dy, dy, acc[4]);
-                    acc[5] = fmaf(dalpha, open ? G : 0.f, acc[5]);
+                    const float g2 = hit[u] && oG[u] <= kc.alpha_max ? T[0] * d * oG[u] : 0.f;
+                    const float g2y = g2 * dy[u];
+                    screen_partials(q[u], dx[u], g2, g2y, g2y * dy[u], nw * gx, nw * gy, nw * gz, acc[u]);
                 }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    add_gradient<DET>(hit[u], acc[u], sid[k[u]], lane, grad2d, pairgrad);
             }
-            const uint32_t who = __ballot_sync(0xFFFFFFFFu, any);
-            if (who == 0u) continue;
-            if constexpr (DET) {
-                // deterministic mode (one warp per tile): the warp's fixed-order sum is the
-                // whole tile's contribution; it goes to the pair's own slot, no atomics
-                int idx;
-                const float v = warp_sum9(acc, lane, idx);
-                if (idx >= 0) pairgrad[(size_t)sid[k] * kPairGradStride + idx] = v;
-                continue;
-            }
-            if (__popc(who) <= kLaneAtomicMax) {
-                // few lanes blended this Gaussian: each adds its own values (no warp sum)
-                if (any) {
-                    float* gp = grad2d + (size_t)sid[k] * kGrad2dStride;
-                    atomicAdd(reinterpret_cast<float4*>(gp), make_float4(acc[0], acc[1], acc[2], acc[3]));
-                    atomicAdd(reinterpret_cast<float4*>(gp + 4), make_float4(acc[4], acc[5], acc[6], acc[7]));
-                    atomicAdd(gp + 8, acc[8]);
+        } else {
+            int knext = nk > 0 ? (int)wl[nk - 1] : 0;   // as in the forward: one visit ahead
+            for (int i = nk - 1; i >= 0; --i) {
+                const int k = knext;
+                if (i > 0) knext = wl[i - 1];
+                const uint32_t pos = bs + k;
+                const float4 a = s0[k];
+                const float dx = g.fx - a.x;
+                // sums over the thread's pixels, which share dx: g2 = dL/dp2 (without ln 2), g2 dy,
+                // g2 dy^2, and minus the colour gradients; the nine screen partials follow from them
+                float g2s = 0.f, g2y = 0.f, g2yy = 0.f, ncr = 0.f, ncg = 0.f, ncb = 0.f;
+                bool any = false;
+                float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (fabsf(dx) <= a.z && pos < thread_end) {
+                    q = s1[k];
+                    const float4 c = s2[k];
+                    const float qydx = __fmul_rn(q.y, dx), qxdx2 = __fmul_rn(__fmul_rn(q.x, dx), dx);
+                    // the pixels in pairs; one that is not hit has alpha 0 and adds zeros (16 x 2 fused
+                    // kernel against a branch per pixel: 1200x680 keyframe 348 -> 343 us, 8 x 640x480
+                    // window of small splats 837 -> 792 us; the same in the forward was 4 % slower)
+                    F2 dyv[PPT / 2];
+                    float p2v[PPT];
+                    bool hit[PPT];
+#pragma unroll
+                    for (int p = 0; p + 1 < PPT; p += 2) {
+                        dyv[p / 2] = add2(pack2(fy[p], fy[p + 1]), pack2(-a.y));
+                        const F2 pw = fma2(fma2(pack2(q.z), dyv[p / 2], pack2(qydx)), dyv[p / 2], pack2(qxdx2));
+                        float dy0, dy1;
+                        unpack2(dyv[p / 2], dy0, dy1);
+                        unpack2(pw, p2v[p], p2v[p + 1]);
+                        hit[p] = pos < my_end[p] && fabsf(dy0) <= a.w && p2v[p] >= c.w;
+                        hit[p + 1] = pos < my_end[p + 1] && fabsf(dy1) <= a.w && p2v[p + 1] >= c.w;
+                        any |= hit[p] | hit[p + 1];
+                    }
+                    if (any) {
+#pragma unroll
+                        for (int p = 0; p + 1 < PPT; p += 2) {
+                            const F2 oG = mul2(pack2(q.w), pack2(ex2_approx(p2v[p]), ex2_approx(p2v[p + 1])));
+                            float oG0, oG1;
+                            unpack2(oG, oG0, oG1);
+                            const F2 nal = pack2(hit[p] ? -fminf(kc.alpha_max, oG0) : 0.f,
+                                                 hit[p + 1] ? -fminf(kc.alpha_max, oG1) : 0.f);
+                            float om0, om1;
+                            unpack2(add2(pack2(1.f), nal), om0, om1);
+                            const F2 Tp = mul2(pack2(T[p], T[p + 1]), pack2(rcp_approx(om0), rcp_approx(om1)));
+                            unpack2(Tp, T[p], T[p + 1]);
+                            float g0r = gr[p], g1r = gr[p + 1], g0g = gg[p], g1g = gg[p + 1], g0b = gb[p],
+                                  g1b = gb[p + 1];
+                            F2 cx = pack2(c.x), cy = pack2(c.y), cz = pack2(c.z);
+                            if (masked | warp_wild) {
+                                cx = pack2(hit[p] ? c.x : 0.f, hit[p + 1] ? c.x : 0.f);
+                                cy = pack2(hit[p] ? c.y : 0.f, hit[p + 1] ? c.y : 0.f);
+                                cz = pack2(hit[p] ? c.z : 0.f, hit[p + 1] ? c.z : 0.f);
+                                if (!hit[p]) g0r = g0g = g0b = 0.f;
+                                if (!hit[p + 1]) g1r = g1g = g1b = 0.f;
+                            }
+                            const F2 nw = mul2(nal, Tp);
+                            float nw0, nw1;
+                            unpack2(nw, nw0, nw1);
+                            ncr = fmaf(nw0, g0r, fmaf(nw1, g1r, ncr));
+                            ncg = fmaf(nw0, g0g, fmaf(nw1, g1g, ncg));
+                            ncb = fmaf(nw0, g0b, fmaf(nw1, g1b, ncb));
+                            // dL/dalpha and g . a as for one pixel a thread
+                            const F2 gap = pack2(ga[p], ga[p + 1]);
+                            const F2 d = add2(fma2(pack2(g0r, g1r), cx, fma2(pack2(g0g, g1g), cy,
+                                                                              mul2(pack2(g0b, g1b), cz))), gap);
+                            unpack2(fma2(nal, d, gap), ga[p], ga[p + 1]);
+                            float t0, t1;
+                            unpack2(mul2(mul2(Tp, d), oG), t0, t1);
+                            t0 = hit[p] && oG0 <= kc.alpha_max ? t0 : 0.f;
+                            t1 = hit[p + 1] && oG1 <= kc.alpha_max ? t1 : 0.f;
+                            float y0, y1, dy0, dy1;
+                            unpack2(dyv[p / 2], dy0, dy1);
+                            unpack2(mul2(pack2(t0, t1), dyv[p / 2]), y0, y1);
+                            g2s += t0 + t1;
+                            g2y += y0 + y1;
+                            g2yy = fmaf(y0, dy0, fmaf(y1, dy1, g2yy));
+                        }
+                    }
                 }
-                continue;
+                float acc[9];
+                screen_partials(q, dx, g2s, g2y, g2yy, ncr, ncg, ncb, acc);
+                add_gradient<DET>(any, acc, sid[k], lane, grad2d, pairgrad);
             }
-            int idx;
-            const float v = warp_sum9(acc, lane, idx);
-            if (idx >= 0) atomicAdd(grad2d + (size_t)sid[k] * kGrad2dStride + idx, v);
         }
         be = bs;
     }
 }
 
 // Persistent compositing kernels: a grid sized to the GPU's resident capacity
-// walks the (view, tile) work list through an atomic counter, so the load
-// stays balanced across tiles of very different cost and across the views of
-// a window. `order` (optional) lists the bins in the order to take them.
-__device__ __forceinline__ bool next_work(uint32_t* __restrict__ queue, uint32_t n_items,
-                                          const uint32_t* __restrict__ order, int& bin) {
+// walks the list of work items (tiles, or halves of tiles with long pair lists)
+// through an atomic counter, so the load stays balanced across tiles of very
+// different cost and across the views of a window. order[0] is the number of
+// items, order[1 ..] the items: a bin, with the half plus one above kItemShift.
+__device__ __forceinline__ bool next_work(uint32_t* __restrict__ queue, const uint32_t* __restrict__ order,
+                                          int& bin, int& half) {
     __shared__ uint32_t s_work;
     __syncthreads();
-    if (threadIdx.x == 0) s_work = atomicAdd(queue, 1u);
+    if (threadIdx.x == 0) {
+        const uint32_t w = atomicAdd(queue, 1u);
+        s_work = w < order[0] ? order[1 + w] : 0xFFFFFFFFu;
+    }
     __syncthreads();
     const uint32_t w = s_work;
-    if (w >= n_items) return false;
-    bin = order ? (int)order[w] : (int)w;
+    if (w == 0xFFFFFFFFu) return false;
+    bin = (int)(w & kItemBin);
+    half = (int)(w >> kItemShift) - 1;
     return true;
 }
 
-template <int TILE, int PPT>
-__device__ __forceinline__ void inside_mask(const TileGeom<TILE, PPT>& g, int width, int height, bool (&inside)[PPT]) {
+template <int TILE, int PPT, int SPLIT>
+__device__ __forceinline__ void inside_mask(const TileGeom<TILE, PPT, SPLIT>& g, int width, int height, bool (&inside)[PPT]) {
 #pragma unroll
     for (int p = 0; p < PPT; ++p) inside[p] = g.px < width && g.py(p) < height;
+}
+
+// One work item's forward pass.
+template <int TILE, int PPT, int SPLIT, bool ARGMAX, bool DET>
+__device__ __forceinline__ void fwd_item(int bin, int part, const uint2* __restrict__ ranges,
+                                         const uint32_t* __restrict__ pval, const float4* __restrict__ rec, int width,
+                                         int height, int tiles_x, int tiles_per_view, int n, const DevConst& kc,
+                                         float* __restrict__ out_rgb, float* __restrict__ out_T,
+                                         uint32_t* __restrict__ out_last, int32_t* __restrict__ out_argmax,
+                                         const uint32_t* __restrict__ emit_item) {
+    const size_t HW = (size_t)width * height;
+    const TileGeom<TILE, PPT, SPLIT> g(bin, part, ranges, tiles_x, tiles_per_view);
+    bool inside[PPT];
+    inside_mask(g, width, height, inside);
+    float T[PPT], cr[PPT], cg[PPT], cb[PPT];
+    uint32_t last[PPT], amax[PPT];
+    bool masked;
+    fwd_core<TILE, PPT, SPLIT, ARGMAX, DET>(g, inside, pval, emit_item, rec, kc, T, cr, cg, cb, last, amax, masked);
+#pragma unroll
+    for (int p = 0; p < PPT; ++p) {
+        if (!inside[p]) continue;
+        const size_t pix = (size_t)g.py(p) * width + g.px;
+        out_rgb[(size_t)g.view * 3 * HW + pix] = cr[p];
+        out_rgb[(size_t)g.view * 3 * HW + HW + pix] = cg[p];
+        out_rgb[(size_t)g.view * 3 * HW + 2 * HW + pix] = cb[p];
+        out_T[g.view * HW + pix] = T[p];
+        out_last[g.view * HW + pix] = last[p];
+        if (ARGMAX)
+            out_argmax[g.view * HW + pix] = amax[p] == 0xFFFFFFFFu ? -1 : (int32_t)(amax[p] - (uint32_t)g.view * n);
+    }
 }
 
 template <int TILE, int PPT, bool ARGMAX, bool DET>
@@ -570,31 +811,51 @@ __global__ void __launch_bounds__(Layout<TILE, PPT>::kThreads)
     k_raster_fwd(const uint2* __restrict__ ranges, const uint32_t* __restrict__ pval, const float4* __restrict__ rec,
                  int width, int height, int tiles_x, int tiles_per_view, int n, DevConst kc,
                  float* __restrict__ out_rgb, float* __restrict__ out_T, uint32_t* __restrict__ out_last,
-                 int32_t* __restrict__ out_argmax, uint32_t* __restrict__ queue, uint32_t n_items,
+                 int32_t* __restrict__ out_argmax, uint32_t* __restrict__ queue,
                  const uint32_t* __restrict__ order, const uint32_t* __restrict__ emit_item) {
-    int bin;
+    int bin, half;
+    while (next_work(queue, order, bin, half)) {
+        if constexpr (Layout<TILE, PPT>::kHalves) {
+            if (half >= 0) {
+                fwd_item<TILE, 1, 2, ARGMAX, DET>(bin, half, ranges, pval, rec, width, height, tiles_x,
+                                                  tiles_per_view, n, kc, out_rgb, out_T, out_last, out_argmax,
+                                                  emit_item);
+                continue;
+            }
+        }
+        fwd_item<TILE, PPT, 1, ARGMAX, DET>(bin, 0, ranges, pval, rec, width, height, tiles_x, tiles_per_view, n, kc,
+                                            out_rgb, out_T, out_last, out_argmax, emit_item);
+    }
+}
+
+// One work item's adjoint.
+template <int TILE, int PPT, int SPLIT, bool DET>
+__device__ __forceinline__ void bwd_item(int bin, int part, const uint2* __restrict__ ranges,
+                                         const uint32_t* __restrict__ pval, const float4* __restrict__ rec, int width,
+                                         int height, int tiles_x, int tiles_per_view, const DevConst& kc,
+                                         const float* __restrict__ T_final, const uint32_t* __restrict__ n_last,
+                                         const float* __restrict__ dLdC, float* __restrict__ grad2d,
+                                         const uint32_t* __restrict__ emit_item, float* __restrict__ pairgrad) {
     const size_t HW = (size_t)width * height;
-    while (next_work(queue, n_items, order, bin)) {
-        const TileGeom<TILE, PPT> g(bin, ranges, tiles_x, tiles_per_view);
-        bool inside[PPT];
-        inside_mask(g, width, height, inside);
-        float T[PPT], cr[PPT], cg[PPT], cb[PPT];
-        uint32_t last[PPT], amax[PPT];
-        fwd_core<TILE, PPT, ARGMAX, DET>(g, inside, pval, emit_item, rec, kc, T, cr, cg, cb, last, amax);
+    const TileGeom<TILE, PPT, SPLIT> g(bin, part, ranges, tiles_x, tiles_per_view);
+    float T[PPT], gr[PPT], gg[PPT], gb[PPT];
+    uint32_t cnt[PPT];
 #pragma unroll
-        for (int p = 0; p < PPT; ++p) {
-            if (!inside[p]) continue;
+    for (int p = 0; p < PPT; ++p) {
+        T[p] = 1.f;
+        gr[p] = gg[p] = gb[p] = 0.f;
+        cnt[p] = 0;
+        if (g.px < width && g.py(p) < height) {
             const size_t pix = (size_t)g.py(p) * width + g.px;
-            out_rgb[(size_t)g.view * 3 * HW + pix] = cr[p];
-            out_rgb[(size_t)g.view * 3 * HW + HW + pix] = cg[p];
-            out_rgb[(size_t)g.view * 3 * HW + 2 * HW + pix] = cb[p];
-            out_T[g.view * HW + pix] = T[p];
-            out_last[g.view * HW + pix] = last[p];
-            if (ARGMAX)
-                out_argmax[g.view * HW + pix] =
-                    amax[p] == 0xFFFFFFFFu ? -1 : (int32_t)(amax[p] - (uint32_t)g.view * n);
+            T[p] = T_final[g.view * HW + pix];
+            cnt[p] = n_last[g.view * HW + pix];
+            gr[p] = dLdC[(size_t)g.view * 3 * HW + pix];
+            gg[p] = dLdC[(size_t)g.view * 3 * HW + HW + pix];
+            gb[p] = dLdC[(size_t)g.view * 3 * HW + 2 * HW + pix];
         }
     }
+    bwd_core<TILE, PPT, SPLIT, DET>(g, pval, emit_item, rec, kc, T, cnt, gr, gg, gb, grad2d, pairgrad, -1, false,
+                                    false);
 }
 
 template <int TILE, int PPT, bool DET>
@@ -603,93 +864,106 @@ __global__ void __launch_bounds__(Layout<TILE, PPT>::kThreads)
                  int width, int height, int tiles_x, int tiles_per_view, DevConst kc,
                  const float* __restrict__ T_final, const uint32_t* __restrict__ n_last,
                  const float* __restrict__ dLdC, float* __restrict__ grad2d, uint32_t* __restrict__ queue,
-                 uint32_t n_items, const uint32_t* __restrict__ order, const uint32_t* __restrict__ emit_item,
+                 const uint32_t* __restrict__ order, const uint32_t* __restrict__ emit_item,
                  float* __restrict__ pairgrad) {
-    int bin;
-    const size_t HW = (size_t)width * height;
-    while (next_work(queue, n_items, order, bin)) {
-        const TileGeom<TILE, PPT> g(bin, ranges, tiles_x, tiles_per_view);
-        float T[PPT], gr[PPT], gg[PPT], gb[PPT];
-        uint32_t cnt[PPT];
-#pragma unroll
-        for (int p = 0; p < PPT; ++p) {
-            T[p] = 1.f;
-            gr[p] = gg[p] = gb[p] = 0.f;
-            cnt[p] = 0;
-            if (g.px < width && g.py(p) < height) {
-                const size_t pix = (size_t)g.py(p) * width + g.px;
-                T[p] = T_final[g.view * HW + pix];
-                cnt[p] = n_last[g.view * HW + pix];
-                gr[p] = dLdC[(size_t)g.view * 3 * HW + pix];
-                gg[p] = dLdC[(size_t)g.view * 3 * HW + HW + pix];
-                gb[p] = dLdC[(size_t)g.view * 3 * HW + 2 * HW + pix];
+    int bin, half;
+    while (next_work(queue, order, bin, half)) {
+        if constexpr (Layout<TILE, PPT>::kHalves) {
+            if (half >= 0) {
+                bwd_item<TILE, 1, 2, DET>(bin, half, ranges, pval, rec, width, height, tiles_x, tiles_per_view, kc,
+                                          T_final, n_last, dLdC, grad2d, emit_item, pairgrad);
+                continue;
             }
         }
-        bwd_core<TILE, PPT, DET>(g, pval, emit_item, rec, kc, T, cnt, gr, gg, gb, grad2d, pairgrad, -1, false);
+        bwd_item<TILE, PPT, 1, DET>(bin, 0, ranges, pval, rec, width, height, tiles_x, tiles_per_view, kc, T_final,
+                                    n_last, dLdC, grad2d, emit_item, pairgrad);
     }
 }
 
-// One mapping iteration's compositing for every (view, tile): forward (Eq. 3),
-// the L1 term of Eq. 10 and dL/dC = lambda sign(C - I) / 3HW for the tile's
-// pixels, then the adjoint, with final T, last index and dL/dC kept in
-// registers. Writes the image and one photometric partial sum per CTA.
+// One work item of a mapping iteration: forward (Eq. 3), the L1 term of Eq. 10 and
+// dL/dC = lambda sign(C - I) / 3HW for its pixels, then the adjoint, with final T, last
+// index and dL/dC kept in registers. Writes the image; returns the thread's photometric sum.
+template <int TILE, int PPT, int SPLIT, bool DET>
+__device__ __forceinline__ float fused_item(int bin, int part, const uint2* __restrict__ ranges,
+                                            const uint32_t* __restrict__ pval, const float4* __restrict__ rec,
+                                            int width, int height, int tiles_x, int tiles_per_view,
+                                            const DevConst& kc, const float* __restrict__ target, float scale,
+                                            float* __restrict__ out_rgb, float* __restrict__ grad2d,
+                                            const uint32_t* __restrict__ emit_item, float* __restrict__ pairgrad,
+                                            float* __restrict__ tile_part) {
+    const size_t HW = (size_t)width * height;
+    const TileGeom<TILE, PPT, SPLIT> g(bin, part, ranges, tiles_x, tiles_per_view);
+    bool inside[PPT];
+    inside_mask(g, width, height, inside);
+    float T[PPT], cr[PPT], cg[PPT], cb[PPT], gr[PPT], gg[PPT], gb[PPT];
+    uint32_t last[PPT], amax[PPT];
+    bool masked;   // the last staged batch (of a one-batch tile: the one the adjoint may reuse)
+    const int staged = fwd_core<TILE, PPT, SPLIT, false, DET>(g, inside, pval, emit_item, rec, kc, T, cr, cg, cb, last,
+                                                              amax, masked);
+    float tl = 0.f;   // this thread's photometric sum over the item
+#pragma unroll
+    for (int p = 0; p < PPT; ++p) {
+        gr[p] = gg[p] = gb[p] = 0.f;
+        if (!inside[p]) {
+            last[p] = 0;
+            continue;
+        }
+        const size_t pix = (size_t)g.py(p) * width + g.px;
+        const size_t o = (size_t)g.view * 3 * HW + pix;
+        out_rgb[o] = cr[p];
+        out_rgb[o + HW] = cg[p];
+        out_rgb[o + 2 * HW] = cb[p];
+        const float r0 = cr[p] - target[o], r1 = cg[p] - target[o + HW], r2 = cb[p] - target[o + 2 * HW];
+        tl += (fabsf(r0) + fabsf(r1)) + fabsf(r2);
+        gr[p] = scale * (float)((r0 > 0.f) - (r0 < 0.f));
+        gg[p] = scale * (float)((r1 > 0.f) - (r1 < 0.f));
+        gb[p] = scale * (float)((r2 > 0.f) - (r2 < 0.f));
+    }
+    if constexpr (DET) {
+        // deterministic mode: each tile's sum on its own (fixed tree), whichever CTA took it
+        __shared__ float tred[32];
+        float ts = tl;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ts += __shfl_xor_sync(0xFFFFFFFFu, ts, o);
+        if ((threadIdx.x & 31) == 0) tred[threadIdx.x >> 5] = ts;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            float t = 0.f;
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += tred[w];
+            tile_part[bin] = t * scale;
+        }
+        __syncthreads();
+    }
+    bwd_core<TILE, PPT, SPLIT, DET>(g, pval, emit_item, rec, kc, T, last, gr, gg, gb, grad2d, pairgrad,
+                                    (DET || !Layout<TILE, PPT, SPLIT>::kReuseStaged) ? -1 : staged, true, masked);
+    return tl;
+}
+
+// One mapping iteration's compositing for every (view, tile). Writes the image and one
+// photometric partial sum per CTA.
 template <int TILE, int PPT, bool DET>
 __global__ void __launch_bounds__(Layout<TILE, PPT>::kThreads, Layout<TILE, PPT>::kMinBlocks)
     k_raster_fused(const uint2* __restrict__ ranges, const uint32_t* __restrict__ pval,
                    const float4* __restrict__ rec, int width, int height, int tiles_x, int tiles_per_view,
                    DevConst kc, const float* __restrict__ target, const float* const* __restrict__ target_slot,
                    float scale, float* __restrict__ out_rgb, float* __restrict__ grad2d, float* __restrict__ partials,
-                   uint32_t* __restrict__ queue, uint32_t n_items, const uint32_t* __restrict__ order,
+                   uint32_t* __restrict__ queue, const uint32_t* __restrict__ order,
                    const uint32_t* __restrict__ emit_item, float* __restrict__ pairgrad,
                    float* __restrict__ tile_part) {
     if (target_slot != nullptr) target = *target_slot;   // a replayed graph's per-call target
-    int bin;
-    const size_t HW = (size_t)width * height;
+    int bin, half;
     float loss = 0.f;
-    while (next_work(queue, n_items, order, bin)) {
-        const TileGeom<TILE, PPT> g(bin, ranges, tiles_x, tiles_per_view);
-        bool inside[PPT];
-        inside_mask(g, width, height, inside);
-        float T[PPT], cr[PPT], cg[PPT], cb[PPT], gr[PPT], gg[PPT], gb[PPT];
-        uint32_t last[PPT], amax[PPT];
-        const int staged =
-            fwd_core<TILE, PPT, false, DET>(g, inside, pval, emit_item, rec, kc, T, cr, cg, cb, last, amax);
-        float tl = 0.f;   // this thread's photometric sum over the tile
-#pragma unroll
-        for (int p = 0; p < PPT; ++p) {
-            gr[p] = gg[p] = gb[p] = 0.f;
-            if (!inside[p]) {
-                last[p] = 0;
+    while (next_work(queue, order, bin, half)) {
+        if constexpr (Layout<TILE, PPT>::kHalves) {
+            if (half >= 0) {
+                loss += fused_item<TILE, 1, 2, DET>(bin, half, ranges, pval, rec, width, height, tiles_x,
+                                                    tiles_per_view, kc, target, scale, out_rgb, grad2d, emit_item,
+                                                    pairgrad, tile_part);
                 continue;
             }
-            const size_t pix = (size_t)g.py(p) * width + g.px;
-            const size_t o = (size_t)g.view * 3 * HW + pix;
-            out_rgb[o] = cr[p];
-            out_rgb[o + HW] = cg[p];
-            out_rgb[o + 2 * HW] = cb[p];
-            const float r0 = cr[p] - target[o], r1 = cg[p] - target[o + HW], r2 = cb[p] - target[o + 2 * HW];
-            tl += (fabsf(r0) + fabsf(r1)) + fabsf(r2);
-            gr[p] = scale * (float)((r0 > 0.f) - (r0 < 0.f));
-            gg[p] = scale * (float)((r1 > 0.f) - (r1 < 0.f));
-            gb[p] = scale * (float)((r2 > 0.f) - (r2 < 0.f));
         }
-        loss += tl;
-        if constexpr (DET) {
-            // deterministic mode: each tile's sum on its own (fixed tree), whichever CTA took it
-            __shared__ float tred[32];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) tl += __shfl_xor_sync(0xFFFFFFFFu, tl, o);
-            if ((threadIdx.x & 31) == 0) tred[threadIdx.x >> 5] = tl;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                float t = 0.f;
-                for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += tred[w];
-                tile_part[bin] = t * scale;
-            }
-            __syncthreads();
-        }
-        bwd_core<TILE, PPT, DET>(g, pval, emit_item, rec, kc, T, last, gr, gg, gb, grad2d, pairgrad,
-                                 (DET || !Layout<TILE, PPT>::kReuseStaged) ? -1 : staged, true);
+        loss += fused_item<TILE, PPT, 1, DET>(bin, 0, ranges, pval, rec, width, height, tiles_x, tiles_per_view, kc,
+                                              target, scale, out_rgb, grad2d, emit_item, pairgrad, tile_part);
     }
     // per-CTA photometric partial (already scaled)
     __shared__ float red[32];
@@ -778,48 +1052,50 @@ static int resident_grid(K kernel, int threads, int num_sms) {
 
 template <int TILE, int PPT, bool DET>
 static void fwd_launch(gs_ctx* c, const DevConst& k, float* rgb, int32_t* argmax, cudaStream_t s, int tpv) {
-    constexpr int NT = Layout<TILE, PPT>::kThreads;
+    constexpr int NT = Layout<TILE, PPT>::kThreads, kParts = Layout<TILE, PPT>::kHalves ? 2 : 1;
     if (argmax) {
         const int grid =
-            std::min(resident_grid<0 + 4 * DET, TILE, PPT>(k_raster_fwd<TILE, PPT, true, DET>, NT, c->num_sms), c->n_bins);
+            std::min(resident_grid<0 + 4 * DET, TILE, PPT>(k_raster_fwd<TILE, PPT, true, DET>, NT, c->num_sms),
+                     kParts * c->n_bins);
         k_raster_fwd<TILE, PPT, true, DET><<<grid, NT, 0, s>>>(c->ranges, c->pval[c->pair_buf], c->rec, c->width, c->height,
                                                           c->hcam[0].tiles_x, tpv, c->n, k, rgb, c->T_final,
-                                                          c->n_last, argmax, c->dcount + 6, (uint32_t)c->n_bins,
-                                                          c->work_order, c->emit_item);
+                                                          c->n_last, argmax, c->dcount + 6, c->work_order,
+                                                          c->emit_item);
     } else {
         const int grid =
             std::min(resident_grid<1 + 4 * DET, TILE, PPT>(k_raster_fwd<TILE, PPT, false, DET>, NT, c->num_sms),
-                     c->n_bins);
+                     kParts * c->n_bins);
         k_raster_fwd<TILE, PPT, false, DET><<<grid, NT, 0, s>>>(c->ranges, c->pval[c->pair_buf], c->rec, c->width,
                                                            c->height, c->hcam[0].tiles_x, tpv, c->n, k, rgb,
                                                            c->T_final, c->n_last, nullptr, c->dcount + 6,
-                                                           (uint32_t)c->n_bins, c->work_order, c->emit_item);
+                                                           c->work_order, c->emit_item);
     }
 }
 
 template <int TILE, int PPT, bool DET>
 static void bwd_launch(gs_ctx* c, const DevConst& k, const float* dLdC, cudaStream_t s, int tpv) {
-    constexpr int NT = Layout<TILE, PPT>::kThreads;
+    constexpr int NT = Layout<TILE, PPT>::kThreads, kParts = Layout<TILE, PPT>::kHalves ? 2 : 1;
     const int grid =
-        std::min(resident_grid<2 + 4 * DET, TILE, PPT>(k_raster_bwd<TILE, PPT, DET>, NT, c->num_sms), c->n_bins);
+        std::min(resident_grid<2 + 4 * DET, TILE, PPT>(k_raster_bwd<TILE, PPT, DET>, NT, c->num_sms), kParts * c->n_bins);
     k_raster_bwd<TILE, PPT, DET><<<grid, NT, 0, s>>>(c->ranges, c->pval[c->pair_buf], c->rec, c->width, c->height,
                                                 c->hcam[0].tiles_x, tpv, k, c->T_final, c->n_last, dLdC, c->grad2d,
-                                                c->dcount + 7, (uint32_t)c->n_bins, c->work_order, c->emit_item,
+                                                c->dcount + 7, c->work_order, c->emit_item,
                                                 c->pairgrad);
 }
 
 template <int TILE, int PPT, bool DET>
 static void fused_launch(gs_ctx* c, const DevConst& k, const float* target, const float* const* target_slot,
                          float* rgb, cudaStream_t s, int tpv, float* partials, int max_grid, int* grid_out) {
-    constexpr int NT = Layout<TILE, PPT>::kThreads;
+    constexpr int NT = Layout<TILE, PPT>::kThreads, kParts = Layout<TILE, PPT>::kHalves ? 2 : 1;
     const int grid = std::min(
-        std::min(resident_grid<3 + 4 * DET, TILE, PPT>(k_raster_fused<TILE, PPT, DET>, NT, c->num_sms), c->n_bins),
+        std::min(resident_grid<3 + 4 * DET, TILE, PPT>(k_raster_fused<TILE, PPT, DET>, NT, c->num_sms),
+                 kParts * c->n_bins),
         max_grid);
     const float scale = k.lambda_color / (float)(3 * (size_t)c->width * c->height);
     k_raster_fused<TILE, PPT, DET><<<grid, NT, 0, s>>>(c->ranges, c->pval[c->pair_buf], c->rec, c->width, c->height,
                                                   c->hcam[0].tiles_x, tpv, k, target, target_slot, scale, rgb,
                                                   c->grad2d, partials,
-                                                  c->dcount + 6, (uint32_t)c->n_bins, c->work_order, c->emit_item,
+                                                  c->dcount + 6, c->work_order, c->emit_item,
                                                   c->pairgrad, c->tile_part);
     *grid_out = grid;
 }

@@ -399,19 +399,28 @@ __device__ __forceinline__ uint32_t order_slot(uint2 r) {
     return 1023u - key;
 }
 
-// Longest-first order of the bins for the persistent compositing kernels
+// Longest-first list of work items for the persistent compositing kernels
 // (list scheduling, largest job first): their work queue hands out the tiles
 // with the most pairs first, so a launch does not end on a long tile taken
-// late. One CTA, a counting sort by bucket; bins of one bucket come in any
-// order (the compositing result does not depend on which CTA takes a tile).
+// late. With `halves` a bin of more than split_min pairs and more than
+// 1 / split_share of all pairs becomes two items, its upper and lower half:
+// one CTA walking such a list would outlast the launch's average (see
+// launch_work_order). One CTA, a counting sort by bucket; items of one bucket
+// come in any order (the compositing result does not depend on which CTA takes
+// an item, nor on whether a tile is halved).
 __global__ void __launch_bounds__(1024) k_work_order(const uint2* __restrict__ ranges, uint32_t n_bins,
-                                                      uint32_t* __restrict__ order) {
+                                                      uint32_t* __restrict__ order, int halves, uint32_t split_min,
+                                                      uint32_t split_share, const uint32_t* __restrict__ n_pairs) {
     __shared__ uint32_t cnt[1024];
     __shared__ uint32_t wsum[32];
     const int t = threadIdx.x, lane = t & 31;
+    const uint32_t longest = halves ? max(split_min, *n_pairs / split_share) : 0xFFFFFFFFu;
     cnt[t] = 0;
     __syncthreads();
-    for (uint32_t b = t; b < n_bins; b += 1024) atomicAdd(&cnt[order_slot(ranges[b])], 1u);
+    for (uint32_t b = t; b < n_bins; b += 1024) {
+        const uint2 r = ranges[b];
+        atomicAdd(&cnt[order_slot(r)], r.y - r.x > longest ? 2u : 1u);
+    }
     __syncthreads();
     const uint32_t v = cnt[t];
     uint32_t x = v;   // inclusive scan within the warp
@@ -434,8 +443,18 @@ __global__ void __launch_bounds__(1024) k_work_order(const uint2* __restrict__ r
     }
     __syncthreads();
     cnt[t] = x - v + wsum[t >> 5];
+    if (t == 1023) order[0] = x + wsum[31];
     __syncthreads();
-    for (uint32_t b = t; b < n_bins; b += 1024) order[atomicAdd(&cnt[order_slot(ranges[b])], 1u)] = b;
+    for (uint32_t b = t; b < n_bins; b += 1024) {
+        const uint2 r = ranges[b];
+        if (r.y - r.x > longest) {
+            const uint32_t p = atomicAdd(&cnt[order_slot(r)], 2u);
+            order[1 + p] = b | (1u << kItemShift);
+            order[2 + p] = b | (2u << kItemShift);
+        } else {
+            order[1 + atomicAdd(&cnt[order_slot(r)], 1u)] = b;
+        }
+    }
 }
 
 }  // namespace
@@ -526,16 +545,24 @@ cudaError_t compute_ranges(gs_ctx* c, cudaStream_t s) {
     ++c->launches;
     k_ranges<<<c->num_sms * 8, 256, 0, s>>>(c->pkey[c->pair_buf], c->dcount, (uint64_t)c->pair_cap,
                                             (uint32_t)c->n_bins, c->ranges);
+    return c->order_ahead ? cudaGetLastError() : launch_work_order(c, s);
+}
+
+cudaError_t launch_work_order(gs_ctx* c, cudaStream_t s) {
     ++c->launches;
-    if (c->order_ahead) {
-        // the next iteration's order, beside this one's compositing (which uses the order the
-        // previous iteration left); iteration_tail copies it into place after the compositing
-        cudaEventRecord(c->side_ev[5], s);
-        cudaStreamWaitEvent(c->side, c->side_ev[5], 0);
-        k_work_order<<<1, 1024, 0, c->side>>>(c->ranges, (uint32_t)c->n_bins, c->work_order_next);
-    } else {
-        k_work_order<<<1, 1024, 0, s>>>(c->ranges, (uint32_t)c->n_bins, c->work_order);
-    }
+    // The 16 x 2 layout runs 6 CTAs an SM. With no more halves than that in all, every tile is
+    // halved: a CTA's chain of dependent visits is the launch's time, and one pixel a thread instead
+    // of two shortens it (160x120 with 2k Gaussians: fused kernel 57 -> 29 us). Otherwise a bin is
+    // halved that holds more than half an average CTA's pairs (all pairs over 12 CTAs an SM); lower,
+    // the halves' second staging of the list costs more than the balance gives (fused kernel at 9, 12
+    // and 18 an SM: 1200x680 keyframe with 300k 372, 341, 320 us and 527 without halves; one with
+    // lists of similar length 337, 343, 354 us; 8 x 640x480 window 782, 785, 797 us). Bins of 128
+    // pairs or less take a CTA no longer than the launch's other latencies.
+    const int halves = c->tile == 16 && c->ppt == 2 && !c->cfg.deterministic;
+    const bool all = 2ll * c->n_bins <= 6ll * c->num_sms;
+    const uint32_t split_min = all ? 0u : 128u, split_share = all ? 0xFFFFFFFFu : 12u * (uint32_t)c->num_sms;
+    k_work_order<<<1, 1024, 0, s>>>(c->ranges, (uint32_t)c->n_bins, c->work_order, halves, split_min, split_share,
+                                    c->dcount);
     return cudaGetLastError();
 }
 
