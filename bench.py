@@ -833,7 +833,7 @@ def mlp_step_measure(steps: int, warmup: int, device: int = 0) -> dict:
     return {"metric": MLP_METRIC, "value": 1000.0 / ms, "unit": "steps/s", "steps": steps, "ms_per_step": ms,
             "forward_96_rows_ms": ms_fwd96,
             "roofline": {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
-                         "traffic": None, "kernel": "whole training step (k_gemm_tc launches + elementwise)",
+                         "traffic": None, "kernel": "whole training step (k_mlp_net, k_mlp_reduce, k_mlp_adam)",
                          "peak_source": f"MEASURED_PEAKS.json bf16_tflops ({src})"}}
 
 

@@ -5,10 +5,8 @@
 // a Gaussian inserted at a VO point from the keyframe's 5x5 patch around the
 // point, its depth and its camera-frame position.
 //
-// Every matrix product is one strided GEMM C (+)= A B on tcgen05.mma (bf16
-// operands in shared memory, f32 accumulators in TMEM): forward X W^T, input
-// gradients dZ W and weight gradients dZ^T X (split over the batch with f32
-// atomics). Upstream
+// A CTA takes 64 rows through the whole network (and, in training, back through it) in one launch,
+// on tcgen05.mma with bf16 operands in shared memory and f32 accumulators in TMEM. Upstream
 // gradients dZ enter as bf16 hi + lo pairs (two products), so the backward
 // keeps ~16 mantissa bits where one bf16 rounding would keep 8.
 #include <cuda_bf16.h>
@@ -28,22 +26,6 @@ constexpr int kOffW1 = 0, kOffB1 = kOffW1 + kHid * kIn, kOffW2 = kOffB1 + kHid, 
 
 typedef __nv_bfloat16 bf16;
 
-// ---- the strided GEMM C (+)= A B, A(m, k) = A[m sam + k sak], B(k, n) = B[k sbk + n sbn] (bf16),
-// on the 5th-generation tensor cores (tcgen05, TMEM accumulators) ----
-//
-// One CTA of 4 warps computes a 128 x NT tile of C. Its K range is walked in
-// chunks of 64: all threads gather the A (128 x 64) and B (NT x 64) chunks
-// from their strided global layout into shared memory in the canonical
-// K-major, non-swizzled UMMA layout (8 x 16-byte core matrices; the core at
-// row group g and K group j sits at g * 1024 + j * 128 bytes, so the leading
-// (K) byte offset is 128 and the stride (row-group) byte offset 1024), then one
-// elected thread issues four tcgen05.mma (M = 128, N = NT, K = 16, BF16 in,
-// FP32 accumulate in TMEM) and commits them to an mbarrier that all threads
-// wait on before the chunk is restaged. The epilogue reads the accumulator
-// with tcgen05.ld (warp w owns TMEM lanes 32w..32w+31, i.e. tile rows) and
-// stores, accumulates or atomically adds it into C. Every wait is bounded: a
-// wait that gives up sets *err, and the CTA still frees its TMEM.
-constexpr int kTcM = 128, kTcKC = 64;
 constexpr uint32_t kTcWaitLimit = 1u << 24;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -73,63 +55,143 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     return false;
 }
 
-// Gather one 64-wide K chunk of a (rows x K) operand X(r, k) = X[r * s_r + k * s_k] into the
-// canonical layout; zero outside rows < R_valid and k < k_end.
-__device__ __forceinline__ void tc_stage(uint8_t* dst, int rows, const bf16* __restrict__ X, long s_r, long s_k,
-                                         int r0, int R_valid, int k0, int k_end) {
-    const bool kvec = s_k == 1 && (s_r % 8) == 0 && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
-    if (kvec) {
-        // one 16-byte core-matrix row (8 consecutive k) per step
-        for (int e = threadIdx.x; e < rows * (kTcKC / 8); e += 128) {
-            const int r = e / (kTcKC / 8), j = e - r * (kTcKC / 8);
-            const int gr = r0 + r, gk = k0 + 8 * j;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (gr < R_valid) {
-                if (gk + 8 <= k_end) {
-                    v = *reinterpret_cast<const uint4*>(X + (long)gr * s_r + gk);
-                } else {
-                    bf16 t[8];
+__device__ __forceinline__ float gelu_f(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
+
+__device__ __forceinline__ float gelu_grad_f(float x) {
+    return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
+}
+
+// v = hi + lo with hi = bf16(v), lo = bf16(v - hi): a bf16 pair carrying ~16 mantissa bits
+__device__ __forceinline__ void split_bf16(float v, bf16& hi, bf16& lo) {
+    hi = __float2bfloat16_rn(v);
+    lo = __float2bfloat16_rn(v - __bfloat162float(hi));
+}
+
+// ---- operands in shared memory ----
+//
+// Canonical K-major, non-swizzled UMMA layout of a (rows x K) bf16 operand: 8 x 16-byte core
+// matrices, the core of row group g and K group j at (g K / 8 + j) * 128 bytes: the leading (K)
+// byte offset is 128, the stride (row-group) byte offset 16 K.
+template <int K>
+__host__ __device__ __forceinline__ constexpr uint32_t core_off(int row, int k) {
+    return (uint32_t)((row >> 3) * (K * 16) + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2);
+}
+
+constexpr int kNetThreads = 256;     // 8 warps: 4 over the 128 TMEM lanes, twice over the rows of a pass
+
+// The bf16 weights as the kernels copy them into shared memory, already in that layout (byte
+// offsets): W1, W2, W3, then the transposes the input gradients need.
+constexpr uint32_t kImgW1 = 0, kImgW2 = kImgW1 + kHid * kIn * 2, kImgW3 = kImgW2 + kHid * kHid * 2,
+                   kImgW2T = kImgW3 + kOutPad * kHid * 2, kImgW3T = kImgW2T + kHid * kHid * 2,
+                   kImgBytes = kImgW3T + kHid * kOutPad * 2, kImgForward = kImgW2T;
+
+// Shared memory (byte offsets). The product with W3 takes 128 operand rows of which 16 exist: it
+// reads 28 KB past W3, whatever lies there, into accumulator lanes nobody reads. H1 and H2 (rows x
+// hidden) are dead once Z2 and Y are formed; dZ2 (rows x hidden, hi and lo) takes their place, and
+// then dZ1^T.
+constexpr uint32_t kSmW = 0;                                   // the weight image
+template <bool TRAIN, int ROWS>
+struct Smem {
+    static constexpr uint32_t X = TRAIN ? kImgBytes : kImgForward;                // [row][in]
+    static constexpr uint32_t H1 = X + ROWS * kIn * 2;                           // [row][hid]
+    static constexpr uint32_t H2 = H1 + ROWS * kHid * 2;                         // [row][hid]
+    static constexpr uint32_t Bias = H2 + ROWS * kHid * 2;                       // b1, b2, b3 (f32)
+    static constexpr uint32_t ForwardEnd = Bias + (2 * kHid + kOutPad) * 4;
+    // training only
+    static constexpr uint32_t XT = (ForwardEnd + 127) / 128 * 128;                // [in][row]
+    static constexpr uint32_t H1T = XT + kIn * ROWS * 2;                         // [hid][row]
+    static constexpr uint32_t H2T = H1T + kHid * ROWS * 2;                       // [hid][row]
+    static constexpr uint32_t DY = H2T + kHid * ROWS * 2;                        // [row][out], hi then lo
+    static constexpr uint32_t DYT = DY + 2 * ROWS * kOutPad * 2;                 // [out][row], hi then lo
+    static constexpr uint32_t DZT = DYT + 2 * ROWS * kOutPad * 2;                // [hid][row], hi then lo
+    static constexpr uint32_t Target = DZT + 2 * kHid * ROWS * 2;                // [row][16] f32
+    static constexpr uint32_t DZ = H1;                                            // [row][hid], hi then lo
+    static constexpr uint32_t Past3 = kImgW3 + 128 * kHid * 2;                    // read by the product with W3
+    static constexpr uint32_t Bytes = TRAIN ? Target + ROWS * kOutPad * 4 : (ForwardEnd > Past3 ? ForwardEnd : Past3);
+};
+static_assert(Smem<true, 64>::Bytes <= 227 * 1024, "shared memory of the training kernel");
+static_assert(Smem<true, 32>::Past3 <= Smem<true, 32>::Bytes, "the product with W3 reads within shared memory");
+
+// TMEM columns (f32 accumulators): Z1, Z2, Y and an input gradient, hidden (output) x rows; the
+// weight gradients dW2, dW1 and dW3^T, summed over the CTA's passes.
+constexpr uint32_t kTmZ1 = 0, kTmZ2 = 64, kTmY = 128, kTmDH = 192, kTmW2 = 256, kTmW1 = 384, kTmW3T = 464;
+
+// D (128 x N, TMEM) (+)= A (128 x K) B (N x K)^T; one thread issues it.
+template <int K, int N>
+__device__ __forceinline__ void umma(uint32_t d, uint32_t a, uint32_t b, bool accumulate) {
+    constexpr uint32_t idesc = umma_idesc_bf16(128, N);
 #pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        t[q] = gk + q < k_end ? X[(long)gr * s_r + gk + q] : __float2bfloat16_rn(0.f);
-                    v = *reinterpret_cast<const uint4*>(t);
-                }
-            }
-            *reinterpret_cast<uint4*>(dst + (r >> 3) * 1024 + j * 128 + (r & 7) * 16) = v;
-        }
-    } else {
-        // element by element, consecutive threads along the unit-stride dimension
-        const bool r_fast = s_r == 1;
-        for (int e = threadIdx.x; e < rows * kTcKC; e += 128) {
-            int r, k;
-            if (r_fast) {
-                k = e / rows;
-                r = e - k * rows;
-            } else {
-                r = e / kTcKC;
-                k = e - r * kTcKC;
-            }
-            const int gr = r0 + r, gk = k0 + k;
-            const bf16 v = (gr < R_valid && gk < k_end) ? X[(long)gr * s_r + (long)gk * s_k] : __float2bfloat16_rn(0.f);
-            *reinterpret_cast<bf16*>(dst + (r >> 3) * 1024 + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2) = v;
-        }
+    for (int kk = 0; kk < K / 16; ++kk) {
+        const uint64_t ad = umma_desc(a + kk * 256, 128, K * 16);
+        const uint64_t bd = umma_desc(b + kk * 256, 128, K * 16);
+        const uint32_t acc = (accumulate || kk > 0) ? 1u : 0u;
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
+            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+            "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+            : "memory");
     }
 }
 
-template <int NT>
-__global__ void __launch_bounds__(128) k_gemm_tc(const bf16* __restrict__ A, long sam, long sak,
-                                                 const bf16* __restrict__ B, long sbk, long sbn,
-                                                 float* __restrict__ C, int ldc, int M, int N, int K, int k_split,
-                                                 int mode, uint32_t* __restrict__ err) {
-    static_assert(NT % 16 == 0 && NT >= 16 && NT <= 128, "UMMA N for M = 128");
-    constexpr uint32_t kCols = NT <= 32 ? 32u : (NT <= 64 ? 64u : 128u);
-    __shared__ __align__(1024) uint8_t sa[kTcM * kTcKC * 2];
-    __shared__ __align__(1024) uint8_t sb[NT * kTcKC * 2];
-    __shared__ __align__(8) uint64_t mbar;
+// 16 consecutive accumulator columns of the thread's TMEM lane (the load is not waited for)
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, float* f) {
+    uint32_t v[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(addr)
+        : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) f[i] = __uint_as_float(v[i]);
+}
+template <int N>
+__device__ __forceinline__ void tmem_ld(uint32_t addr, float (&f)[N]) {
+#pragma unroll
+    for (int i = 0; i < N; i += 16) tmem_ld16(addr + i, f + i);
+}
+
+// N values of one operand row, columns r0 .. r0 + N - 1, as bf16 into [row][ROWS]
+template <int ROWS, int N>
+__device__ __forceinline__ void store_row(uint8_t* dst, int row, int r0, const bf16 (&h)[N]) {
+#pragma unroll
+    for (int g = 0; g < N; g += 8)
+        *reinterpret_cast<uint4*>(dst + core_off<ROWS>(row, r0 + g)) = *reinterpret_cast<const uint4*>(h + g);
+}
+// the same values as one column (hidden unit j) of [row][kHid]
+template <int N>
+__device__ __forceinline__ void store_col(uint8_t* dst, int r0, int j, const bf16 (&h)[N]) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) *reinterpret_cast<bf16*>(dst + core_off<kHid>(r0 + i, j)) = h[i];
+}
+
+// The network over passes of ROWS rows, and in training its adjoint: forward, MSE over the 11
+// outputs, dY = 2 (Y - T) / (n 11), and the gradient of every parameter, as this CTA's partial sums
+// part[blockIdx.x][kParams], with its loss in loss_part.
+//
+// Every product has the 128 hidden units as its M dimension and rows (or units) as N, so a small
+// batch spreads over SMs and no accumulator lane is padding; a thread owns one hidden unit and 32
+// rows. What bounds it is latency: eight products, each a few hundred tensor cycles, and between
+// them a read of TMEM, an erf (and, back, an exp) a value and a rewrite of the operands. One launch
+// takes the place of 20 (elementwise kernels and strided GEMMs that gathered their operands element by
+// element): gradients of 4,096 rows 400 -> 20 us, a prediction of 96 rows 58 -> 6 us.
+template <bool TRAIN, int ROWS>
+__global__ void __launch_bounds__(kNetThreads, 1)
+    k_mlp_net(const float* __restrict__ feat, const float* __restrict__ tgt, int n, const uint8_t* __restrict__ img,
+              const float* __restrict__ par, float* __restrict__ out, float* __restrict__ part,
+              float* __restrict__ loss_part, uint32_t* __restrict__ err) {
+    typedef Smem<TRAIN, ROWS> S;
+    constexpr int N = ROWS / 2;                  // rows of a thread
+    extern __shared__ __align__(1024) uint8_t sm[];
+    __shared__ __align__(8) uint64_t bars[2];
     __shared__ uint32_t tmem_slot;
+    __shared__ float red[2][kHid];
+    constexpr uint32_t kCols = TRAIN ? 512u : 256u;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.y * kTcM, n0 = blockIdx.x * NT;
-    const int kb = blockIdx.z * k_split, ke = min(K, kb + k_split);
+    const int j = (warp & 3) * 32 + lane;        // hidden unit (output of the last layer)
+    const int r0 = (warp >> 2) * N;              // first of the thread's rows of the pass
+    const uint32_t base = smem_u32(sm), wbar = smem_u32(&bars[0]), bar = smem_u32(&bars[1]);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
                      "r"(kCols)
@@ -137,77 +199,236 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const bf16* __restrict__ A, lon
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (threadIdx.x == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar)) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(wbar) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        constexpr uint32_t bytes = TRAIN ? kImgBytes : kImgForward;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(wbar), "r"(bytes) : "memory");
+        asm volatile(
+            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(base + kSmW),
+            "l"(img), "r"(bytes), "r"(wbar)
+            : "memory");
     }
+    float* bias = reinterpret_cast<float*>(sm + S::Bias);
+    for (int i = threadIdx.x; i < 2 * kHid + kOutPad; i += kNetThreads)
+        bias[i] = par[i < kHid ? kOffB1 + i : (i < 2 * kHid ? kOffB2 + i - kHid : kOffB3 + i - 2 * kHid)];
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
-    const uint32_t bar = smem_u32(&mbar);
-    const uint32_t a_base = smem_u32(sa), b_base = smem_u32(sb);
-    constexpr uint32_t idesc = umma_idesc_bf16(kTcM, NT);
-    bool ok = true, issued = false;
+    const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    const float b1 = bias[j], b2 = bias[kHid + j];
     uint32_t parity = 0;
-    for (int k0 = kb; k0 < ke && ok; k0 += kTcKC) {
-        tc_stage(sa, kTcM, A, sam, sak, m0, M, k0, ke);
-        tc_stage(sb, NT, B, sbn, sbk, n0, N, k0, ke);
+    bool ok = true;
+    // the operands written so far become visible to the tensor cores, one thread issues, all wait
+    auto products = [&](auto issue) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
         if (threadIdx.x == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#pragma unroll
-            for (int kk = 0; kk < kTcKC / 16; ++kk) {
-                const uint64_t ad = umma_desc(a_base + kk * 256, 128, 1024);
-                const uint64_t bd = umma_desc(b_base + kk * 256, 128, 1024);
-                const uint32_t acc = (issued || kk > 0) ? 1u : 0u;
-                asm volatile(
-                    "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
-                    " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-                    "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-                    : "memory");
-            }
+            issue();
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                          : "memory");
         }
-        issued = true;
-        ok = mbar_wait(bar, parity);
+        ok = __syncthreads_and(mbar_wait(bar, parity));
         parity ^= 1u;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        __syncthreads();
-    }
-    if (ok) {
-        const int m = m0 + warp * 32 + lane;
+        return ok;
+    };
+    float db1 = 0.f, db2 = 0.f, db3 = 0.f, loss = 0.f;
+    const float scale = 2.f / ((float)n * (float)kOut);
+    bool first = true;
+    const bool feat_vec = (reinterpret_cast<uintptr_t>(feat) & 15) == 0;
+    const int passes = (n + ROWS - 1) / ROWS;
+    for (int pass = blockIdx.x; pass < passes && ok; pass += gridDim.x) {
+        const int row0 = pass * ROWS;
+        for (int e = threadIdx.x; e < ROWS * (kIn / 8); e += kNetThreads) {
+            const int g = e / ROWS, r = e - g * ROWS;
+            __align__(16) bf16 h[8];
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+            if (row0 + r < n) {
+                const float* src = feat + (size_t)(row0 + r) * kIn + 8 * g;
+                if (feat_vec) {
+                    a = *reinterpret_cast<const float4*>(src);
+                    b = *reinterpret_cast<const float4*>(src + 4);
+                } else {
+                    a = make_float4(src[0], src[1], src[2], src[3]);
+                    b = make_float4(src[4], src[5], src[6], src[7]);
+                }
+            }
+            const float x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
-        for (int c0 = 0; c0 < NT; c0 += 16) {
-            uint32_t v[16];
-            const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                : "r"(taddr)
-                : "memory");
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (m < M) {
+            for (int q = 0; q < 8; ++q) h[q] = __float2bfloat16_rn(x[q]);
+            *reinterpret_cast<uint4*>(sm + S::X + core_off<kIn>(r, 8 * g)) = *reinterpret_cast<const uint4*>(h);
+            if constexpr (TRAIN) {
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int n = n0 + c0 + j;
-                    if (n >= N) continue;
-                    const float val = issued ? __uint_as_float(v[j]) : 0.f;
-                    float* dst = C + (long)m * ldc + n;
-                    if (mode == 1) {
-                        if (issued) atomicAdd(dst, val);
-                    } else if (mode == 2) {
-                        *dst += val;
-                    } else {
-                        *dst = val;
+                for (int q = 0; q < 8; ++q)
+                    *reinterpret_cast<bf16*>(sm + S::XT + core_off<ROWS>(8 * g + q, r)) = h[q];
+            }
+        }
+        if constexpr (TRAIN) {
+            float* st = reinterpret_cast<float*>(sm + S::Target);
+            for (int e = threadIdx.x; e < ROWS * kOutPad; e += kNetThreads)
+                st[e] = row0 + e / kOutPad < n ? tgt[(size_t)row0 * kOutPad + e] : 0.f;
+        }
+        if (first && !__syncthreads_and(mbar_wait(wbar, 0))) {   // the weights have arrived
+            ok = false;
+            break;
+        }
+        float z[N];
+        __align__(16) bf16 h[N];
+        if (!products([&] { umma<kIn, ROWS>(tmem + kTmZ1, base + kSmW + kImgW1, base + S::X, false); })) break;
+        tmem_ld(tlane + kTmZ1 + r0, z);
+#pragma unroll
+        for (int i = 0; i < N; ++i) h[i] = __float2bfloat16_rn(gelu_f(z[i] + b1));
+        store_col(sm + S::H1, r0, j, h);
+        if constexpr (TRAIN) store_row<ROWS>(sm + S::H1T, j, r0, h);
+        if (!products([&] { umma<kHid, ROWS>(tmem + kTmZ2, base + kSmW + kImgW2, base + S::H1, false); })) break;
+        tmem_ld(tlane + kTmZ2 + r0, z);
+#pragma unroll
+        for (int i = 0; i < N; ++i) h[i] = __float2bfloat16_rn(gelu_f(z[i] + b2));
+        store_col(sm + S::H2, r0, j, h);
+        if constexpr (TRAIN) store_row<ROWS>(sm + S::H2T, j, r0, h);
+        if (!products([&] { umma<kHid, ROWS>(tmem + kTmY, base + kSmW + kImgW3, base + S::H2, false); })) break;
+        if ((warp & 3) == 0) {   // outputs: lanes 0 .. 15
+            tmem_ld(tlane + kTmY + r0, z);
+            if (lane < kOutPad) {
+                const float b3 = bias[2 * kHid + lane];
+                if constexpr (!TRAIN) {
+                    for (int i = 0; i < N; ++i)
+                        if (row0 + r0 + i < n) out[(size_t)(row0 + r0 + i) * kOutPad + lane] = z[i] + b3;
+                } else {
+                    const float* st = reinterpret_cast<const float*>(sm + S::Target);
+#pragma unroll
+                    for (int i = 0; i < N; ++i) {
+                        const int r = r0 + i;
+                        float g = 0.f;
+                        if (lane < kOut && row0 + r < n) {
+                            const float d = z[i] + b3 - st[r * kOutPad + lane];
+                            loss += d * d;
+                            g = scale * d;
+                            db3 += g;
+                        }
+                        bf16 hi, lo;
+                        split_bf16(g, hi, lo);
+                        *reinterpret_cast<bf16*>(sm + S::DY + core_off<kOutPad>(r, lane)) = hi;
+                        *reinterpret_cast<bf16*>(sm + S::DY + ROWS * kOutPad * 2 + core_off<kOutPad>(r, lane)) = lo;
+                        *reinterpret_cast<bf16*>(sm + S::DYT + core_off<ROWS>(lane, r)) = hi;
+                        *reinterpret_cast<bf16*>(sm + S::DYT + ROWS * kOutPad * 2 + core_off<ROWS>(lane, r)) = lo;
                     }
                 }
             }
         }
-    } else if (threadIdx.x == 0) {
-        atomicOr(err, 1u);
+        if constexpr (TRAIN) {
+            constexpr uint32_t dyl = ROWS * kOutPad * 2, dzl = ROWS * kHid * 2;
+            // dH2 = dY W3 and dW3 = dY^T H2, both transposed
+            if (!products([&] {
+                    umma<kOutPad, ROWS>(tmem + kTmDH, base + kSmW + kImgW3T, base + S::DY, false);
+                    umma<kOutPad, ROWS>(tmem + kTmDH, base + kSmW + kImgW3T, base + S::DY + dyl, true);
+                    umma<ROWS, kOutPad>(tmem + kTmW3T, base + S::H2T, base + S::DYT, !first);
+                    umma<ROWS, kOutPad>(tmem + kTmW3T, base + S::H2T, base + S::DYT + dyl, true);
+                }))
+                break;
+            __align__(16) bf16 l[N];
+            float dh[N];
+            tmem_ld(tlane + kTmDH + r0, dh);
+            tmem_ld(tlane + kTmZ2 + r0, z);
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const float v = dh[i] * gelu_grad_f(z[i] + b2);
+                db2 += v;
+                split_bf16(v, h[i], l[i]);
+            }
+            store_row<ROWS>(sm + S::DZT, j, r0, h);
+            store_row<ROWS>(sm + S::DZT + dzl, j, r0, l);
+            store_col(sm + S::DZ, r0, j, h);
+            store_col(sm + S::DZ + dzl, r0, j, l);
+            // dH1^T = W2^T dZ2^T and dW2 = dZ2^T H1
+            if (!products([&] {
+                    umma<kHid, ROWS>(tmem + kTmDH, base + kSmW + kImgW2T, base + S::DZ, false);
+                    umma<kHid, ROWS>(tmem + kTmDH, base + kSmW + kImgW2T, base + S::DZ + dzl, true);
+                    umma<ROWS, kHid>(tmem + kTmW2, base + S::DZT, base + S::H1T, !first);
+                    umma<ROWS, kHid>(tmem + kTmW2, base + S::DZT + dzl, base + S::H1T, true);
+                }))
+                break;
+            tmem_ld(tlane + kTmDH + r0, dh);
+            tmem_ld(tlane + kTmZ1 + r0, z);
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const float v = dh[i] * gelu_grad_f(z[i] + b1);
+                db1 += v;
+                split_bf16(v, h[i], l[i]);
+            }
+            store_row<ROWS>(sm + S::DZ, j, r0, h);
+            store_row<ROWS>(sm + S::DZ + dzl, j, r0, l);
+            // dW1 = dZ1^T X
+            if (!products([&] {
+                    umma<ROWS, kIn>(tmem + kTmW1, base + S::DZ, base + S::XT, !first);
+                    umma<ROWS, kIn>(tmem + kTmW1, base + S::DZ + dzl, base + S::XT, true);
+                }))
+                break;
+        } else {
+            __syncthreads();
+        }
+        first = false;
+    }
+    if (!ok) {
+        if (threadIdx.x == 0) *err = 1u;   // pinned host memory: the next call reports it
+    } else if constexpr (TRAIN) {
+        float* P = part + (size_t)blockIdx.x * kParams;
+        const int half = warp >> 2;
+        float f[32];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int i0 = half * 64 + c * 32;
+            tmem_ld(tlane + kTmW2 + i0, f);
+#pragma unroll
+            for (int i = 0; i < 32; i += 4)
+                *reinterpret_cast<float4*>(P + kOffW2 + j * kHid + i0 + i) = make_float4(f[i], f[i + 1], f[i + 2], f[i + 3]);
+        }
+        {   // dW1: 80 columns, 48 and 32 of them a half
+            tmem_ld(tlane + kTmW1 + half * 48, f);
+#pragma unroll
+            for (int i = 0; i < 32; i += 4)
+                *reinterpret_cast<float4*>(P + kOffW1 + j * kIn + half * 48 + i) =
+                    make_float4(f[i], f[i + 1], f[i + 2], f[i + 3]);
+            float e[16];
+            tmem_ld(tlane + (half == 0 ? kTmW1 + 32 : kTmW3T), e);
+            if (half == 0) {
+#pragma unroll
+                for (int i = 0; i < 16; i += 4)
+                    *reinterpret_cast<float4*>(P + kOffW1 + j * kIn + 32 + i) =
+                        make_float4(e[i], e[i + 1], e[i + 2], e[i + 3]);
+            } else {
+                // the padding rows of the output layer are not trained
+#pragma unroll
+                for (int o = 0; o < kOutPad; ++o) P[kOffW3 + o * kHid + j] = o < kOut ? e[o] : 0.f;
+            }
+        }
+        // the two row halves' bias gradients and losses
+        if (half == 1) {
+            red[0][j] = db1;
+            red[1][j] = db2;
+        }
+        __syncthreads();
+        if (half == 0) {
+            P[kOffB1 + j] = db1 + red[0][j];
+            P[kOffB2 + j] = db2 + red[1][j];
+        }
+        __syncthreads();
+        if (warp == 4 && lane < kOutPad) {
+            red[0][lane] = db3;
+            red[1][lane] = loss;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            float t = lane < kOutPad ? loss + red[1][lane] : 0.f;
+            if (lane < kOutPad) P[kOffB3 + lane] = db3 + red[0][lane];
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+            if (lane == 0) loss_part[blockIdx.x] = t / ((float)n * (float)kOut);
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -217,122 +438,90 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const bf16* __restrict__ A, lon
     }
 }
 
-__device__ __forceinline__ float gelu_f(float x) { return 0.5f * x * (1.f + erff(x * 0.70710678118654752f)); }
-
-__device__ __forceinline__ float gelu_grad_f(float x) {
-    return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * 0.39894228040143268f * expf(-0.5f * x * x);
-}
-
-__global__ void k_to_bf16(const float* __restrict__ x, bf16* __restrict__ y, long n) {
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-        y[i] = __float2bfloat16_rn(x[i]);
-}
-
-// z <- z + b (kept as the pre-activation), h <- bf16(GELU(z + b)); rows of width `w`
-__global__ void k_bias_gelu(float* __restrict__ z, const float* __restrict__ b, bf16* __restrict__ h, long n, int w) {
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const float v = z[i] + b[i % w];
-        z[i] = v;
-        h[i] = __float2bfloat16_rn(gelu_f(v));
-    }
-}
-
-__global__ void k_bias(float* __restrict__ y, const float* __restrict__ b, long n, int w) {
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-        y[i] += b[i % w];
-}
-
-// v = hi + lo with hi = bf16(v), lo = bf16(v - hi): a bf16 pair carrying ~16 mantissa bits
-__device__ __forceinline__ void split_bf16(float v, bf16& hi, bf16& lo) {
-    hi = __float2bfloat16_rn(v);
-    lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-}
-
-// dZ = dH * GELU'(z) as a bf16 hi/lo pair for the next products; the bias gradient sums dZ
-// (f32) per column.
-__global__ void k_gelu_back(const float* __restrict__ dh, const float* __restrict__ z, bf16* __restrict__ dz,
-                            bf16* __restrict__ dz_lo, float* __restrict__ db, int rows) {
-    __shared__ float colsum[kHid];
-    for (int c = threadIdx.x; c < kHid; c += blockDim.x) colsum[c] = 0.f;
-    __syncthreads();
-    const long n = (long)rows * kHid;
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const float v = dh[i] * gelu_grad_f(z[i]);
-        split_bf16(v, dz[i], dz_lo[i]);
-        atomicAdd(&colsum[i % kHid], v);
-    }
-    __syncthreads();
-    for (int c = threadIdx.x; c < kHid; c += blockDim.x) atomicAdd(&db[c], colsum[c]);
-}
-
-// MSE over the 11 outputs: dY = 2 (Y - T) / (n 11) (bf16 hi/lo pair, padding columns 0), bias
-// gradient of the output layer, and per-block partial loss sums.
-__global__ void k_mse(const float* __restrict__ y, const float* __restrict__ tgt, int rows, bf16* __restrict__ dy,
-                      bf16* __restrict__ dy_lo, float* __restrict__ db3, float* __restrict__ partials) {
-    __shared__ float colsum[kOutPad];
-    __shared__ float red[8];
-    for (int c = threadIdx.x; c < kOutPad; c += blockDim.x) colsum[c] = 0.f;
-    __syncthreads();
-    const float s = 2.f / ((float)rows * (float)kOut);
-    float loss = 0.f;
-    const long n = (long)rows * kOutPad;
-    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const int c = (int)(i % kOutPad);
-        float g = 0.f;
-        if (c < kOut) {
-            const float r = y[i] - tgt[i];
-            loss += r * r;
-            g = s * r;
-            atomicAdd(&colsum[c], g);
+// The CTAs' partial gradients and losses, added in a fixed order (so a step repeats bit for bit):
+// 32 groups of four parameters a CTA, eight threads a group. Bound by its one read of the partials
+// (113 KB a CTA of k_mlp_net, from L2).
+__global__ void __launch_bounds__(256) k_mlp_reduce(const float* __restrict__ part, const float* __restrict__ loss_part,
+                                                    int n_part, float* __restrict__ g, float* __restrict__ loss) {
+    __shared__ float4 sh[8][32];
+    const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + c;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i < kParams / 4) {
+#pragma unroll 4
+        for (int p = w; p < n_part; p += 8) {
+            const float4 v = reinterpret_cast<const float4*>(part + (size_t)p * kParams)[i];
+            a.x += v.x;
+            a.y += v.y;
+            a.z += v.z;
+            a.w += v.w;
         }
-        split_bf16(g, dy[i], dy_lo[i]);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xFFFFFFFFu, loss, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = loss;
+    sh[w][c] = a;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float tsum = 0.f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tsum += red[w];
-        partials[blockIdx.x] = tsum / ((float)rows * (float)kOut);
+    if (w == 0 && i < kParams / 4) {
+#pragma unroll
+        for (int q = 1; q < 8; ++q) {
+            const float4 v = sh[q][c];
+            a.x += v.x;
+            a.y += v.y;
+            a.z += v.z;
+            a.w += v.w;
+        }
+        reinterpret_cast<float4*>(g)[i] = a;
     }
-    for (int c = threadIdx.x; c < kOutPad; c += blockDim.x) atomicAdd(&db3[c], colsum[c]);
+    if (loss != nullptr && blockIdx.x == 0 && w == 1) {
+        double t = 0.0;
+        for (int p = c; p < n_part; p += 32) t += loss_part[p];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+        if (c == 0) *loss = (float)t;
+    }
 }
 
-__global__ void k_sum_partials(const float* __restrict__ p, int n, float* __restrict__ out) {
-    double a = 0.0;
-    for (int i = threadIdx.x; i < n; i += 32) a += p[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xFFFFFFFFu, a, o);
-    if (threadIdx.x == 0) *out = (float)a;
+// A parameter's place(s) in the bf16 weight image (biases have none)
+__device__ __forceinline__ void store_weight(uint8_t* img, int i, float v) {
+    const bf16 h = __float2bfloat16_rn(v);
+    auto put = [&](uint32_t off) { *reinterpret_cast<bf16*>(img + off) = h; };
+    if (i < kOffB1) {
+        put(kImgW1 + core_off<kIn>(i / kIn, i % kIn));
+    } else if (i >= kOffW2 && i < kOffB2) {
+        const int r = (i - kOffW2) / kHid, k = (i - kOffW2) % kHid;
+        put(kImgW2 + core_off<kHid>(r, k));
+        put(kImgW2T + core_off<kHid>(k, r));
+    } else if (i >= kOffW3 && i < kOffB3) {
+        const int r = (i - kOffW3) / kHid, k = (i - kOffW3) % kHid;
+        put(kImgW3 + core_off<kHid>(r, k));
+        put(kImgW3T + core_off<kOutPad>(k, r));
+    }
 }
 
 __global__ void k_mlp_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                            float* __restrict__ v, int n, float lr, float b1, float b2, float eps, float bc1,
-                           float bc2) {
+                           float bc2, uint8_t* __restrict__ img) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi, vi = b2 * v[i] + (1.f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    p[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+    const float w = p[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+    p[i] = w;
+    store_weight(img, i, w);
 }
 
-__global__ void k_weights_bf16(const float* __restrict__ p, bf16* __restrict__ w) {
-    // W1, W2, W3 of the flat layout, contiguous in the bf16 copy
+__global__ void k_weight_image(const float* __restrict__ p, uint8_t* __restrict__ img) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int n1 = kHid * kIn, n2 = kHid * kHid, n3 = kOutPad * kHid;
-    if (i < n1) w[i] = __float2bfloat16_rn(p[kOffW1 + i]);
-    else if (i < n1 + n2) w[i] = __float2bfloat16_rn(p[kOffW2 + i - n1]);
-    else if (i < n1 + n2 + n3) w[i] = __float2bfloat16_rn(p[kOffW3 + i - n1 - n2]);
+    if (i < kParams) store_weight(img, i, p[i]);
 }
 
 // MLP input of each point: 5x5 RGB patch around its nearest pixel (clamped to the
 // image; row-major, RGB interleaved), depth, camera-frame position, 0.
-__global__ void k_features(DevCamera cam, const float* __restrict__ image, const float* __restrict__ pts, int n,
-                           float* __restrict__ f) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp a point: lanes load the patch side by side (a thread that walked the 75 values alone took
+// 12 us for 96 points; 4 us).
+__global__ void __launch_bounds__(128) k_features(DevCamera cam, const float* __restrict__ image,
+                                                  const float* __restrict__ pts, int n, float* __restrict__ f) {
+    const int i = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (i >= n) return;
     const float x = pts[3 * i], y = pts[3 * i + 1], z = pts[3 * i + 2];
     const float tx = cam.R[0] * x + cam.R[1] * y + cam.R[2] * z + cam.t[0];
@@ -344,20 +533,18 @@ __global__ void k_features(DevCamera cam, const float* __restrict__ image, const
     const int py = (int)fminf(fmaxf(floorf(v + 0.5f), 0.f), (float)(cam.height - 1));
     const size_t HW = (size_t)cam.width * cam.height;
     float* o = f + (size_t)i * kIn;
-    int k = 0;
-    for (int dy = -2; dy <= 2; ++dy)
-        for (int dx = -2; dx <= 2; ++dx) {
+#pragma unroll
+    for (int k = lane; k < kIn; k += 32) {
+        float val;
+        if (k < 75) {
+            const int q = k / 3, ch = k - 3 * q, dy = q / 5 - 2, dx = q - 5 * (q / 5) - 2;
             const int xx = min(max(px + dx, 0), cam.width - 1), yy = min(max(py + dy, 0), cam.height - 1);
-            const size_t pix = (size_t)yy * cam.width + xx;
-            o[k++] = image[pix];
-            o[k++] = image[HW + pix];
-            o[k++] = image[2 * HW + pix];
+            val = image[(size_t)ch * HW + (size_t)yy * cam.width + xx];
+        } else {
+            val = k == 76 ? tx : (k == 77 ? ty : (k == 79 ? 0.f : tz));
         }
-    o[75] = tz;
-    o[76] = tx;
-    o[77] = ty;
-    o[78] = tz;
-    o[79] = 0.f;
+        o[k] = val;
+    }
 }
 
 // Gaussian parameters [14][cap] columns base.. of the kept points from the MLP
@@ -412,103 +599,81 @@ using namespace gs;
 
 struct gs_mlp {
     int device = 0;
+    int num_sms = 1;
     float* p = nullptr;      // f32 master parameters [kParams]
     float* g = nullptr;      // gradient
     float* m = nullptr;
     float* v = nullptr;
-    bf16* wb = nullptr;      // bf16 W1 | W2 | W3
+    uint8_t* img = nullptr;  // bf16 weights in the kernels' shared-memory layout [kImgBytes]
     int t = 0;
     int rows_cap = 0;
-    bf16* xb = nullptr;      // [rows][80]
-    float* z1 = nullptr;     // [rows][128] pre-activations
-    bf16* h1 = nullptr;
-    float* z2 = nullptr;
-    bf16* h2 = nullptr;
-    float* y = nullptr;      // [rows][16]
-    bf16* dy = nullptr;
-    bf16* dy_lo = nullptr;
-    float* dh = nullptr;     // [rows][128] f32 input gradient of a hidden layer
-    bf16* dz = nullptr;      // [rows][128] pre-activation gradient, bf16 hi part
-    bf16* dz_lo = nullptr;   // ... and lo part
-    float* part = nullptr;   // loss partials
-    uint32_t* err = nullptr;   // device flag: a tensor-core wait gave up
-    uint32_t* herr = nullptr;  // pinned copy of it, refreshed after each forward / backward
+    float* y = nullptr;      // [rows][16] predictions for an insertion
+    int part_cap = 0;
+    float* part = nullptr;        // [CTAs][kParams] partial gradients
+    float* loss_part = nullptr;   // [CTAs]
+    uint32_t* herr = nullptr;  // pinned flag that a kernel sets when a wait of its gave up
 };
 
 namespace {
 
-constexpr int kEwBlocks = 256, kEwThreads = 256;
-
-void mlp_free_rows(gs_mlp* M) {
-    void* ps[] = {M->xb, M->z1, M->h1, M->z2, M->h2, M->y, M->dy, M->dy_lo, M->dh, M->dz, M->dz_lo};
-    for (void* q : ps) cudaFree(q);
-    M->xb = nullptr;
-    M->z1 = M->z2 = M->y = M->dh = nullptr;
-    M->h1 = M->h2 = M->dy = M->dy_lo = M->dz = M->dz_lo = nullptr;
-    M->rows_cap = 0;
-}
-
 int mlp_rows(gs_mlp* M, int rows) {
     if (rows <= M->rows_cap) return GS_OK;
-    mlp_free_rows(M);
+    cudaFree(M->y);
+    M->y = nullptr;
+    M->rows_cap = 0;
     const size_t r = (size_t)std::max(rows, 1024);
-    bool ok = cudaMalloc(&M->xb, sizeof(bf16) * r * kIn) == cudaSuccess;
-    ok = ok && cudaMalloc(&M->z1, sizeof(float) * r * kHid) == cudaSuccess;
-    ok = ok && cudaMalloc(&M->h1, sizeof(bf16) * r * kHid) == cudaSuccess;
-    ok = ok && cudaMalloc(&M->z2, sizeof(float) * r * kHid) == cudaSuccess;
-    ok = ok && cudaMalloc(&M->h2, sizeof(bf16) * r * kHid) == cudaSuccess;
-    ok = ok && cudaMalloc(&M->y, sizeof(float) * r * kOutPad) == cudaSuccess;
-    ok = ok && cudaMalloc(&M->dy, sizeof(bf16) * r * kOutPad) == cudaSuccess;
-    ok = ok && cudaMalloc(&M->dh, sizeof(float) * r * kHid) == cudaSuccess;
-    ok = ok && cudaMalloc(&M->dz, sizeof(bf16) * r * kHid) == cudaSuccess;
-    ok = ok && cudaMalloc(&M->dy_lo, sizeof(bf16) * r * kOutPad) == cudaSuccess;
-    ok = ok && cudaMalloc(&M->dz_lo, sizeof(bf16) * r * kHid) == cudaSuccess;
-    if (!ok) {
-        mlp_free_rows(M);
+    if (cudaMalloc(&M->y, sizeof(float) * r * kOutPad) != cudaSuccess) {
+        M->y = nullptr;
+        cudaGetLastError();
         return GS_ERR_OOM;
     }
     M->rows_cap = (int)r;
     return GS_OK;
 }
 
-// C (+)= A B on the tcgen05 tensor cores; split-K (f32 atomics) when `split`.
-void gemm(const bf16* A, long sam, long sak, const bf16* B, long sbk, long sbn, float* C, int ldc, int M, int N,
-          int K, bool split, cudaStream_t s, uint32_t* err, bool accumulate = false) {
-    // these products are small (a few MFLOP): spread them over more CTAs, narrower N tiles
-    // for the row-parallel products and K splits of 256 rows for the weight gradients
-    int splits = 1, kps = K;
-    if (split) {
-        splits = std::max(1, std::min(256, K / 256));
-        kps = ((K + splits - 1) / splits + kTcKC - 1) / kTcKC * kTcKC;
-        splits = (K + kps - 1) / kps;
+int mlp_parts(gs_mlp* M, int ctas) {
+    if (ctas <= M->part_cap) return GS_OK;
+    cudaFree(M->part);
+    cudaFree(M->loss_part);
+    M->part = M->loss_part = nullptr;
+    M->part_cap = 0;
+    if (cudaMalloc(&M->part, sizeof(float) * (size_t)ctas * kParams) != cudaSuccess ||
+        cudaMalloc(&M->loss_part, sizeof(float) * (size_t)ctas) != cudaSuccess) {
+        cudaFree(M->part);
+        M->part = M->loss_part = nullptr;
+        cudaGetLastError();
+        return GS_ERR_OOM;
     }
-    const int mode = split ? 1 : (accumulate ? 2 : 0);
-    int nt = N <= 16 ? 16 : (N <= 32 ? 32 : (N <= 64 ? 64 : 128));
-    const int m_tiles = (M + kTcM - 1) / kTcM;
-    while (nt > 32 && m_tiles * ((N + nt - 1) / nt) * splits < 128) nt /= 2;
-    dim3 grid((N + nt - 1) / nt, (M + kTcM - 1) / kTcM, splits);
-    if (nt == 16)
-        k_gemm_tc<16><<<grid, 128, 0, s>>>(A, sam, sak, B, sbk, sbn, C, ldc, M, N, K, kps, mode, err);
-    else if (nt == 32)
-        k_gemm_tc<32><<<grid, 128, 0, s>>>(A, sam, sak, B, sbk, sbn, C, ldc, M, N, K, kps, mode, err);
-    else if (nt == 64)
-        k_gemm_tc<64><<<grid, 128, 0, s>>>(A, sam, sak, B, sbk, sbn, C, ldc, M, N, K, kps, mode, err);
-    else
-        k_gemm_tc<128><<<grid, 128, 0, s>>>(A, sam, sak, B, sbk, sbn, C, ldc, M, N, K, kps, mode, err);
+    M->part_cap = ctas;
+    return GS_OK;
 }
 
-// forward of `rows` feature rows (f32 [rows][80]) into M->y [rows][16]
-cudaError_t mlp_forward_rows(gs_mlp* M, const float* feat, int rows, cudaStream_t s) {
-    const bf16* W1 = M->wb;
-    const bf16* W2 = W1 + kHid * kIn;
-    const bf16* W3 = W2 + kHid * kHid;
-    k_to_bf16<<<kEwBlocks, kEwThreads, 0, s>>>(feat, M->xb, (long)rows * kIn);
-    gemm(M->xb, kIn, 1, W1, 1, kIn, M->z1, kHid, rows, kHid, kIn, false, s, M->err);
-    k_bias_gelu<<<kEwBlocks, kEwThreads, 0, s>>>(M->z1, M->p + kOffB1, M->h1, (long)rows * kHid, kHid);
-    gemm(M->h1, kHid, 1, W2, 1, kHid, M->z2, kHid, rows, kHid, kHid, false, s, M->err);
-    k_bias_gelu<<<kEwBlocks, kEwThreads, 0, s>>>(M->z2, M->p + kOffB2, M->h2, (long)rows * kHid, kHid);
-    gemm(M->h2, kHid, 1, W3, 1, kHid, M->y, kOutPad, rows, kOutPad, kHid, false, s, M->err);
-    k_bias<<<kEwBlocks, kEwThreads, 0, s>>>(M->y, M->p + kOffB3, (long)rows * kOutPad, kOutPad);
+// Passes of 32 rows while the GPU has an SM for each, else of 64 (fewer, each with twice the work
+// between the same products: gradients of 4,096 rows with the reduction 20 us in 128 CTAs of 32 rows,
+// 28 in 64 of 64; 96 rows forward 6.2 and 8.2 us); as many CTAs as share the passes evenly.
+int net_rows(const gs_mlp* M, int rows) { return (rows + 31) / 32 <= M->num_sms ? 32 : 64; }
+int net_ctas(const gs_mlp* M, int rows) {
+    const int per = net_rows(M, rows), passes = (rows + per - 1) / per;
+    const int rounds = (passes + M->num_sms - 1) / M->num_sms;
+    return (passes + rounds - 1) / rounds;
+}
+
+template <bool TRAIN, int ROWS>
+void net_launch(gs_mlp* M, const float* feat, const float* tgt, int n, float* out, cudaStream_t s) {
+    k_mlp_net<TRAIN, ROWS><<<net_ctas(M, n), kNetThreads, Smem<TRAIN, ROWS>::Bytes, s>>>(
+        feat, tgt, n, M->img, M->p, out, M->part, M->loss_part, M->herr);
+}
+
+template <bool TRAIN, int ROWS>
+bool net_smem() {
+    return cudaFuncSetAttribute(k_mlp_net<TRAIN, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                Smem<TRAIN, ROWS>::Bytes) == cudaSuccess;
+}
+
+// predictions out [rows][16] of feature rows (f32 [rows][80])
+cudaError_t mlp_forward_rows(gs_mlp* M, const float* feat, int rows, float* out, cudaStream_t s) {
+    if (net_rows(M, rows) == 32) net_launch<false, 32>(M, feat, nullptr, rows, out, s);
+    else net_launch<false, 64>(M, feat, nullptr, rows, out, s);
     return cudaGetLastError();
 }
 
@@ -538,14 +703,19 @@ int gs_mlp_create(int device, uint64_t seed, gs_mlp** out) {
     ok = ok && cudaMalloc(&M->g, sizeof(float) * kParams) == cudaSuccess;
     ok = ok && cudaMalloc(&M->m, sizeof(float) * kParams) == cudaSuccess;
     ok = ok && cudaMalloc(&M->v, sizeof(float) * kParams) == cudaSuccess;
-    ok = ok && cudaMalloc(&M->wb, sizeof(bf16) * (kHid * kIn + kHid * kHid + kOutPad * kHid)) == cudaSuccess;
-    ok = ok && cudaMalloc(&M->part, sizeof(float) * (kEwBlocks + 1)) == cudaSuccess;
-    ok = ok && cudaMalloc(&M->err, sizeof(uint32_t)) == cudaSuccess && cudaMemset(M->err, 0, sizeof(uint32_t)) == cudaSuccess;
+    ok = ok && cudaMalloc(&M->img, kImgBytes) == cudaSuccess;
     ok = ok && cudaMallocHost((void**)&M->herr, sizeof(uint32_t)) == cudaSuccess;
     if (ok) *M->herr = 0u;
     if (!ok) {
         gs_mlp_destroy(M);
         return GS_ERR_OOM;
+    }
+    if (cudaDeviceGetAttribute(&M->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || M->num_sms < 1)
+        M->num_sms = 1;
+    if (!net_smem<false, 32>() || !net_smem<false, 64>() || !net_smem<true, 32>() || !net_smem<true, 64>()) {
+        cudaGetLastError();
+        gs_mlp_destroy(M);
+        return GS_ERR_CUDA;
     }
     // uniform(-1/sqrt(fan_in), 1/sqrt(fan_in)) weights from SplitMix64, zero biases; output rows >= 11 zero
     float* h = (float*)calloc(kParams, sizeof(float));
@@ -576,8 +746,7 @@ int gs_mlp_create(int device, uint64_t seed, gs_mlp** out) {
 void gs_mlp_destroy(gs_mlp* M) {
     if (!M) return;
     cudaSetDevice(M->device);
-    mlp_free_rows(M);
-    void* ps[] = {M->p, M->g, M->m, M->v, M->wb, M->part, M->err};
+    void* ps[] = {M->p, M->g, M->m, M->v, M->img, M->y, M->part, M->loss_part};
     for (void* q : ps) cudaFree(q);
     if (M->herr) cudaFreeHost(M->herr);
     delete M;
@@ -593,7 +762,7 @@ int gs_mlp_set_params(gs_mlp* M, const float* flat_dev, void* stream) {
     cudaMemsetAsync(M->v, 0, sizeof(float) * kParams, s);
     cudaMemsetAsync(M->g, 0, sizeof(float) * kParams, s);
     M->t = 0;
-    k_weights_bf16<<<(kHid * kIn + kHid * kHid + kOutPad * kHid + 255) / 256, 256, 0, s>>>(M->p, M->wb);
+    k_weight_image<<<(kParams + 255) / 256, 256, 0, s>>>(M->p, M->img);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
@@ -628,53 +797,26 @@ int gs_mlp_features(const gs_camera* cam, const float* image_dev, const float* p
     d.cy = cam->cy;
     d.width = cam->width;
     d.height = cam->height;
-    k_features<<<(n + 127) / 128, 128, 0, (cudaStream_t)stream>>>(d, image_dev, points_dev, n, feat_dev);
+    k_features<<<(n + 3) / 4, 128, 0, (cudaStream_t)stream>>>(d, image_dev, points_dev, n, feat_dev);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
 int gs_mlp_forward(gs_mlp* M, const float* feat_dev, int n, float* out_dev, void* stream) {
     if (!M || n < 0 || (n > 0 && (!feat_dev || !out_dev))) return GS_ERR_ARG;
     if (n == 0) return GS_OK;
-    cudaStream_t s = (cudaStream_t)stream;
-    if (*M->herr != 0u) return GS_ERR_TIMEOUT;   // a tensor-core wait of an earlier call gave up
-    if (mlp_rows(M, n) != GS_OK) return GS_ERR_OOM;
-    if (mlp_forward_rows(M, feat_dev, n, s) != cudaSuccess) return GS_ERR_CUDA;
-    if (cudaMemcpyAsync(out_dev, M->y, sizeof(float) * (size_t)n * kOutPad, cudaMemcpyDeviceToDevice, s) !=
-        cudaSuccess)
-        return GS_ERR_CUDA;
-    return cudaMemcpyAsync(M->herr, M->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) == cudaSuccess
-               ? GS_OK
-               : GS_ERR_CUDA;
+    if (*(volatile uint32_t*)M->herr != 0u) return GS_ERR_TIMEOUT;   // a wait of an earlier call gave up
+    return mlp_forward_rows(M, feat_dev, n, out_dev, (cudaStream_t)stream) == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
 int gs_mlp_backward(gs_mlp* M, const float* feat_dev, const float* target_dev, int n, float* loss_dev, void* stream) {
     if (!M || n <= 0 || !feat_dev || !target_dev) return GS_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    if (*M->herr != 0u) return GS_ERR_TIMEOUT;   // a tensor-core wait of an earlier call gave up
-    if (mlp_rows(M, n) != GS_OK) return GS_ERR_OOM;
-    if (mlp_forward_rows(M, feat_dev, n, s) != cudaSuccess) return GS_ERR_CUDA;
-    const bf16* W2 = M->wb + kHid * kIn;
-    const bf16* W3 = W2 + kHid * kHid;
-    cudaMemsetAsync(M->g, 0, sizeof(float) * kParams, s);
-    k_mse<<<kEwBlocks, kEwThreads, 0, s>>>(M->y, target_dev, n, M->dy, M->dy_lo, M->g + kOffB3, M->part);
-    if (loss_dev) k_sum_partials<<<1, 32, 0, s>>>(M->part, kEwBlocks, loss_dev);
-    // Upstream gradients enter the tensor cores as bf16 hi + lo pairs: two products each.
-    // output layer: dW3 = dY^T H2, dH2 = dY W3
-    for (const bf16* d : {M->dy, M->dy_lo}) gemm(d, 1, kOutPad, M->h2, kHid, 1, M->g + kOffW3, kHid, kOutPad, kHid, n, true, s, M->err);
-    gemm(M->dy, kOutPad, 1, W3, kHid, 1, M->dh, kHid, n, kHid, kOutPad, false, s, M->err);
-    gemm(M->dy_lo, kOutPad, 1, W3, kHid, 1, M->dh, kHid, n, kHid, kOutPad, false, s, M->err, true);
-    k_gelu_back<<<kEwBlocks, kEwThreads, 0, s>>>(M->dh, M->z2, M->dz, M->dz_lo, M->g + kOffB2, n);
-    // second layer: dW2 = dZ2^T H1, dH1 = dZ2 W2
-    for (const bf16* d : {M->dz, M->dz_lo}) gemm(d, 1, kHid, M->h1, kHid, 1, M->g + kOffW2, kHid, kHid, kHid, n, true, s, M->err);
-    gemm(M->dz, kHid, 1, W2, kHid, 1, M->dh, kHid, n, kHid, kHid, false, s, M->err);
-    gemm(M->dz_lo, kHid, 1, W2, kHid, 1, M->dh, kHid, n, kHid, kHid, false, s, M->err, true);
-    k_gelu_back<<<kEwBlocks, kEwThreads, 0, s>>>(M->dh, M->z1, M->dz, M->dz_lo, M->g + kOffB1, n);
-    // first layer: dW1 = dZ1^T X
-    for (const bf16* d : {M->dz, M->dz_lo}) gemm(d, 1, kHid, M->xb, kIn, 1, M->g + kOffW1, kIn, kHid, kIn, n, true, s, M->err);
-    // the padding rows of the output layer are not trained
-    cudaMemsetAsync(M->g + kOffW3 + kOut * kHid, 0, sizeof(float) * (kOutPad - kOut) * kHid, s);
-    cudaMemsetAsync(M->g + kOffB3 + kOut, 0, sizeof(float) * (kOutPad - kOut), s);
-    cudaMemcpyAsync(M->herr, M->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+    if (*(volatile uint32_t*)M->herr != 0u) return GS_ERR_TIMEOUT;   // a wait of an earlier call gave up
+    const int ctas = net_ctas(M, n);
+    if (mlp_parts(M, ctas) != GS_OK) return GS_ERR_OOM;
+    if (net_rows(M, n) == 32) net_launch<true, 32>(M, feat_dev, target_dev, n, nullptr, s);
+    else net_launch<true, 64>(M, feat_dev, target_dev, n, nullptr, s);
+    k_mlp_reduce<<<(kParams / 4 + 31) / 32, 256, 0, s>>>(M->part, M->loss_part, ctas, M->g, loss_dev);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
@@ -684,8 +826,8 @@ int gs_mlp_step(gs_mlp* M, float lr, void* stream) {
     M->t += 1;
     const double b1 = 0.9, b2 = 0.999;
     k_mlp_adam<<<(kParams + 255) / 256, 256, 0, s>>>(M->p, M->g, M->m, M->v, kParams, lr, (float)b1, (float)b2, 1e-8f,
-                                                     (float)(1.0 - std::pow(b1, M->t)), (float)(1.0 - std::pow(b2, M->t)));
-    k_weights_bf16<<<(kHid * kIn + kHid * kHid + kOutPad * kHid + 255) / 256, 256, 0, s>>>(M->p, M->wb);
+                                                     (float)(1.0 - std::pow(b1, M->t)), (float)(1.0 - std::pow(b2, M->t)),
+                                                     M->img);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
@@ -701,8 +843,8 @@ cudaError_t mlp_initialise(gs_mlp* M, const DevCamera& cam, const float* image, 
                            float* feat_tmp, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
     if (mlp_rows(M, n) != GS_OK) return cudaErrorMemoryAllocation;
-    k_features<<<(n + 127) / 128, 128, 0, s>>>(cam, image, pts, n, feat_tmp);
-    cudaError_t e = mlp_forward_rows(M, feat_tmp, n, s);
+    k_features<<<(n + 3) / 4, 128, 0, s>>>(cam, image, pts, n, feat_tmp);
+    cudaError_t e = mlp_forward_rows(M, feat_tmp, n, M->y, s);
     if (e != cudaSuccess) return e;
     k_apply_mlp<<<(n + 127) / 128, 128, 0, s>>>(M->y, pts, n, stage);
     return cudaGetLastError();
