@@ -299,10 +299,8 @@ int front_half(gs_ctx* c, const DevConst& k, cudaStream_t s) {
     Phase ph(c, GS_PHASE_PROJECT, s);
     CK(launch_preprocess(c, c->n_views, k, s));
     // the visible items, compacted in item order, sorted by depth (dcount[8] of them)
-    int buf = 0;
     const uint32_t hint = c->visible_hint ? std::min(c->visible_hint + c->visible_hint / 4 + 256, items) : items;
-    CK(radix_sort_pairs(c, c->dkey, c->dval, c->dcount + 8, items, hint, 32, &buf, s));
-    CK(scan_tiles(c, items, c->dcount + 8, s));
+    CK(sort_depth(c, items, hint, s));
     return GS_OK;
 }
 
@@ -400,6 +398,8 @@ int gs_create(const gs_config* cfg, int device, gs_ctx** out) {
         if (e != cudaSuccess) { code = fail(c, GS_ERR_CUDA, "cudaSetDevice", e); break; }
         cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
         if (c->num_sms <= 0) c->num_sms = 1;
+        e = sort_kernels_init();
+        if (e != cudaSuccess) { code = fail(c, GS_ERR_CUDA, "kernel attributes", e); break; }
         c->sort_blocks = c->num_sms * 4;
         c->n_partials = 2 * c->num_sms * 2;
         const size_t cap = (size_t)c->cap, V = (size_t)cfg->max_views;
@@ -432,9 +432,11 @@ int gs_create(const gs_config* cfg, int device, gs_ctx** out) {
         ok = ok && dalloc(&c->n_last, V * maxpix) == cudaSuccess;
         ok = ok && dalloc(&c->dLdC, 3 * V * maxpix) == cudaSuccess;
         ok = ok && dalloc(&c->grad2d, kGrad2dStride * V * cap) == cudaSuccess;
-        ok = ok && dalloc(&c->hist, (size_t)256 * c->sort_blocks + 256) == cudaSuccess;
+        ok = ok && dalloc(&c->hist, sort_hist_words(c->sort_blocks)) == cudaSuccess;
         ok = ok && dalloc(&c->dcount, 16) == cudaSuccess;
         ok = ok && dalloc(&c->vis_blocks, V * ((cap + 255) / 256) + 1) == cudaSuccess;
+        ok = ok && dalloc(&c->vis_range, V * ((cap + 255) / 256) + 1) == cudaSuccess;
+        ok = ok && dalloc(&c->tile_blocks, (V * cap + 255) / 256 + 1) == cudaSuccess;
         ok = ok && dalloc(&c->target_slot, 1) == cudaSuccess;
         if (cfg->lambda_photo > 0.f) {
             ok = ok && dalloc(&c->ssim_maps, (size_t)3 * 3 * V * maxpix) == cudaSuccess;
@@ -493,7 +495,7 @@ void gs_destroy(gs_ctx* c) {
     for (auto e : c->tpool) cudaEventDestroy(e);
     void* ptrs[] = {c->params, c->grads, c->adam_m, c->adam_v, c->dens_sum, c->dens_cnt, c->dom_cnt, c->adam_pw, c->dcam, c->rec,
                     c->tiles_touched, c->depth, c->dkey[0], c->dkey[1], c->dval[0], c->dval[1], c->offsets, c->ranges,
-                    c->work_order, c->work_order_graph, c->T_final, c->n_last, c->dLdC, c->grad2d, c->hist, c->vis_blocks, (void*)c->target_slot, c->ssim_maps, c->ssim_part, c->dcount,
+                    c->work_order, c->work_order_graph, c->T_final, c->n_last, c->dLdC, c->grad2d, c->hist, c->vis_blocks, c->vis_range, c->tile_blocks, (void*)c->target_slot, c->ssim_maps, c->ssim_part, c->dcount,
                     c->partials, c->psnr_part, c->reg_part, c->tile_part, c->fpart,
                     c->own_rgb, c->tgt_stage[0], c->tgt_stage[1]};
     for (void* p : ptrs) cudaFree(p);

@@ -98,7 +98,7 @@ struct gs_ctx {
     float* depth = nullptr;                 // [max_views * cap] float32 view depth
     uint32_t* dkey[2] = {nullptr, nullptr}; // depth-sort keys   [max_views * cap]
     uint32_t* dval[2] = {nullptr, nullptr}; // depth-sort values [max_views * cap]
-    uint32_t* offsets = nullptr;            // exclusive scan of tiles touched in depth order
+    uint32_t* offsets = nullptr;            // deterministic mode: exclusive scan of tiles touched in depth order
     int64_t pair_cap = 0;
     uint32_t* pkey[2] = {nullptr, nullptr}; // bin of each pair
     uint32_t* pval[2] = {nullptr, nullptr}; // (view * cap + id) of each pair
@@ -131,8 +131,11 @@ struct gs_ctx {
                                             // ticket, [3] UINT32_MAX, [4] Adam steps, [5] totals,
                                             // [6], [7] work queues, [8] visible (view, Gaussian) items,
                                             // [10] a non-finite loss or gradient was seen (sticky until
-                                            // a call reports it)
-    uint32_t* vis_blocks = nullptr;         // visible items per preprocess CTA, then their offsets
+                                            // a call reports it), [11], [12] smallest and largest visible
+                                            // depth key
+    uint32_t* vis_blocks = nullptr;         // visible items per preprocess CTA
+    uint2* vis_range = nullptr;             // smallest and largest visible depth key per preprocess CTA
+    uint32_t* tile_blocks = nullptr;        // tiles touched per 256 items of the depth order
     uint32_t visible_hint = 0;              // host copy of dcount[8] from the last synchronising render
     uint32_t* hcount = nullptr;             // pinned host mirror
     float* partials = nullptr;              // reduction partials
@@ -220,7 +223,11 @@ cudaError_t launch_preprocess_backward(gs_ctx* c, const DevConst& k, bool add_re
 // The count is min(*n_dev, n_max); n_hint (host estimate) only sizes the grid.
 cudaError_t radix_sort_pairs(gs_ctx* c, uint32_t** keys, uint32_t** vals, const uint32_t* n_dev, uint32_t n_max,
                              uint32_t n_hint, int bits, int* out_buf, cudaStream_t s);
-cudaError_t scan_tiles(gs_ctx* c, uint32_t n_max, const uint32_t* n_dev, cudaStream_t s);
+// Depth order of the visible items of the projection: dval[0], with tile_blocks and the pair total.
+cudaError_t sort_depth(gs_ctx* c, uint32_t n_max, uint32_t n_hint, cudaStream_t s);
+bool depth_sort_small(const gs_ctx* c);    // the map is small enough for the one-CTA depth sort
+cudaError_t sort_kernels_init();           // once per context, on its device
+size_t sort_hist_words(int sort_blocks);
 cudaError_t emit_pairs(gs_ctx* c, uint32_t n_items, const uint32_t* n_dev, cudaStream_t s);
 // exclusive scan of n u32 values (in may equal out); the total goes to *total_dev
 cudaError_t scan_u32(gs_ctx* c, const uint32_t* in, uint32_t* out, uint32_t n, uint32_t* total_dev, cudaStream_t s);

@@ -159,8 +159,8 @@ __device__ __forceinline__ void project_one(const float p[kParamRows], const Sha
 __device__ __forceinline__ bool preprocess_one(const float* __restrict__ P, int n, int cap, int gid, int view,
                                                const DevCamera* __restrict__ cams, const DevConst& kc, int tile,
                                                float4* __restrict__ rec, uint32_t* __restrict__ tiles,
-                                               uint32_t* __restrict__ dkey, uint32_t* __restrict__ dval,
-                                               float* __restrict__ depth, float& planar) {
+                                               uint32_t* __restrict__ dkey, float* __restrict__ depth, float& planar,
+                                               uint32_t& key) {
     const DevCamera& cam = cams[view];
     size_t item = (size_t)view * n + gid;
     float p[kParamRows];
@@ -208,14 +208,15 @@ __device__ __forceinline__ bool preprocess_one(const float* __restrict__ P, int 
     rec[item * 3 + 2] = make_float4(p[11], p[12], p[13], vf);
     tiles[item] = ntiles;
     depth[item] = tz32;
-    dkey[item] = valid ? __float_as_uint(tz32) : 0xFFFFFFFFu;
-    dval[item] = (uint32_t)item;
+    key = valid ? __float_as_uint(tz32) : 0xFFFFFFFFu;
+    dkey[item] = key;
     return valid;
 }
 
 // One thread per (view, Gaussian) item; each CTA also writes how many of its 256
 // consecutive items are visible (block_vis[view * gridDim.x + blockIdx.x]), the
-// first step of the order-keeping compaction ahead of the depth sort, and the
+// first step of the order-keeping compaction ahead of the depth sort, with the
+// range of their keys, and the
 // CTAs of view 0 the sum of their Gaussians' planar terms times reg_scale
 // (reg_part[blockIdx.x]; the loss adds these partials in index order).
 // Six CTAs of 256 threads per SM (at most 40 registers): 48 resident warps for a latency-bound
@@ -223,17 +224,29 @@ __device__ __forceinline__ bool preprocess_one(const float* __restrict__ P, int 
 __global__ void __launch_bounds__(256, 6) k_preprocess(const float* __restrict__ P, int n, int cap,
                                                     const DevCamera* __restrict__ cams, DevConst kc, int tile,
                                                     float4* __restrict__ rec, uint32_t* __restrict__ tiles,
-                                                    uint32_t* __restrict__ dkey, uint32_t* __restrict__ dval,
+                                                    uint32_t* __restrict__ dkey,
                                                     float* __restrict__ depth, uint32_t* __restrict__ block_vis,
+                                                    uint2* __restrict__ block_range,
                                                     float reg_scale, float* __restrict__ reg_part) {
     __shared__ float wsum[8];
+    __shared__ uint2 wrange[8];
     const int gid = blockIdx.x * blockDim.x + threadIdx.x;
     const int view = blockIdx.y;
     bool vis = false;
     float planar = 0.f;
-    if (gid < n) vis = preprocess_one(P, n, cap, gid, view, cams, kc, tile, rec, tiles, dkey, dval, depth, planar);
+    uint32_t key = 0xFFFFFFFFu;
+    if (gid < n) vis = preprocess_one(P, n, cap, gid, view, cams, kc, tile, rec, tiles, dkey, depth, planar, key);
+    {
+        const uint32_t lo = __reduce_min_sync(0xFFFFFFFFu, key), hi = __reduce_max_sync(0xFFFFFFFFu, vis ? key : 0u);
+        if ((threadIdx.x & 31) == 0) wrange[threadIdx.x >> 5] = make_uint2(lo, hi);
+    }
     const int cnt = __syncthreads_count(vis);
-    if (threadIdx.x == 0) block_vis[(size_t)view * gridDim.x + blockIdx.x] = (uint32_t)cnt;
+    if (threadIdx.x == 0) {
+        uint2 r = wrange[0];
+        for (int w = 1; w < 8; ++w) r = make_uint2(umin(r.x, wrange[w].x), umax(r.y, wrange[w].y));
+        block_vis[(size_t)view * gridDim.x + blockIdx.x] = (uint32_t)cnt;
+        block_range[(size_t)view * gridDim.x + blockIdx.x] = r;
+    }
     if (view == 0) {   // uniform over the CTA
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) planar += __shfl_xor_sync(0xFFFFFFFFu, planar, o);
@@ -251,13 +264,14 @@ __global__ void __launch_bounds__(256, 6) k_preprocess(const float* __restrict__
 // ascending ids through the stable sort. CTA B takes the items of projection CTAs 4B .. 4B + 3
 // (linear index view * gx + x): it first adds the visible counts of the projection CTAs before
 // them (a few thousand values at most, read straight from block_vis: no separate scan launch),
-// then writes each one's visible keys and items in turn; the last CTA writes the total.
+// then writes each one's visible keys and items in turn; the last CTA writes the total and the
+// range of the keys, and zeroes the pair total.
 constexpr int kCompactSub = 4;
-__global__ void __launch_bounds__(256) k_compact_visible(const uint32_t* __restrict__ kin,
-                                                         const uint32_t* __restrict__ vin, int n, int gx,
+__global__ void __launch_bounds__(256) k_compact_visible(const uint32_t* __restrict__ kin, int n, int gx,
                                                          int nblocks, const uint32_t* __restrict__ block_vis,
+                                                         const uint2* __restrict__ block_range,
                                                          uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
-                                                         uint32_t* __restrict__ total_out) {
+                                                         uint32_t* __restrict__ counts) {
     __shared__ uint32_t wsum[8];
     __shared__ uint32_t s_off;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -297,11 +311,31 @@ __global__ void __launch_bounds__(256) k_compact_visible(const uint32_t* __restr
         if (vis) {
             const uint32_t pos = off + pre + __popc(bal & lt);
             kout[pos] = key;
-            vout[pos] = vin[item];
+            vout[pos] = (uint32_t)item;
         }
         off += cnt;
     }
-    if (total_out != nullptr && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *total_out = off;
+    if (blockIdx.x == gridDim.x - 1) {
+        uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+        for (int b = threadIdx.x; b < nblocks; b += 256) {
+            const uint2 r = block_range[b];
+            lo = umin(lo, r.x);
+            hi = umax(hi, r.y);
+        }
+        lo = __reduce_min_sync(0xFFFFFFFFu, lo);
+        hi = __reduce_max_sync(0xFFFFFFFFu, hi);
+        __shared__ uint2 wrange[8];
+        if (lane == 0) wrange[w] = make_uint2(lo, hi);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            uint2 r = wrange[0];
+            for (int k = 1; k < 8; ++k) r = make_uint2(umin(r.x, wrange[k].x), umax(r.y, wrange[k].y));
+            counts[0] = 0u;
+            counts[8] = off;
+            counts[11] = r.x;
+            counts[12] = r.y;
+        }
+    }
 }
 
 // Six CTAs of 128 threads per SM (at most 85 registers): the kernel is latency-bound on its
@@ -467,18 +501,22 @@ __global__ void __launch_bounds__(128, 6) k_preprocess_backward(
 
 }  // namespace
 
-// Projection of every (view, Gaussian) item, then the visible items compacted in
-// item order into dkey[0] / dval[0] (their number in dcount[8]).
+// Projection of every (view, Gaussian) item; above the size that one CTA sorts, then the visible items
+// compacted in item order into dkey[1] / dval[1] (their number in dcount[8], their keys' range in
+// dcount[11], dcount[12]).
 cudaError_t launch_preprocess(gs_ctx* c, int n_views, const DevConst& k, cudaStream_t s) {
     if (c->n == 0) return cudaSuccess;
     dim3 grid((c->n + 255) / 256, n_views);
     const uint32_t nblocks = grid.x * grid.y;
-    c->launches += 2;
+    ++c->launches;
     k_preprocess<<<grid, 256, 0, s>>>(c->params, c->n, c->cap, c->dcam, k, c->tile, c->rec, c->tiles_touched,
-                                       c->dkey[1], c->dval[1], c->depth, c->vis_blocks,
+                                       c->dkey[0], c->depth, c->vis_blocks, c->vis_range,
                                        k.lambda_reg / (float)c->n, c->reg_part);
-    k_compact_visible<<<(nblocks + kCompactSub - 1) / kCompactSub, 256, 0, s>>>(
-        c->dkey[1], c->dval[1], c->n, (int)grid.x, (int)nblocks, c->vis_blocks, c->dkey[0], c->dval[0], c->dcount + 8);
+    if (!depth_sort_small(c)) {
+        ++c->launches;
+        k_compact_visible<<<(nblocks + kCompactSub - 1) / kCompactSub, 256, 0, s>>>(
+            c->dkey[0], c->n, (int)grid.x, (int)nblocks, c->vis_blocks, c->vis_range, c->dkey[1], c->dval[1], c->dcount);
+    }
     return cudaGetLastError();
 }
 

@@ -2,17 +2,24 @@
 //
 // The order the compositing needs is lexicographic in (view, tile, depth,
 // Gaussian id). It is built in two stable steps instead of one 64-bit sort:
-//   1. a stable LSD radix sort of the V*N depth keys (32 bits, 4 passes of 8),
-//      whose stability keeps equal depths in id order;
+//   1. a stable LSD radix sort of the visible items' depth keys, three passes
+//      over the bits their range needs (nine bits a pass for depths up to 2^16
+//      times the nearest, at most eleven), whose stability keeps equal depths
+//      in id order; maps of at most kSmallItems (view, Gaussian) items do it in
+//      one CTA;
 //   2. pairs are emitted in that depth order (one per tile a Gaussian's pixel
 //      box touches), then stably radix-sorted by bin = view * tiles + tile
-//      (ceil(log2 bins) bits, 2 passes for up to 65536 bins).
+//      (2 passes for up to 65536 bins).
 // The second sort moves 8-byte pairs over P elements only twice instead of six
 // times for a 64-bit key, and the depth sort touches N elements, not P.
 //
 // Every pass is reduce-then-scan over a fixed grid of G blocks, each owning a
-// contiguous slice of the input; element counts are read from device memory so
-// the same launches can sit in a CUDA graph.
+// contiguous slice of the input: one launch counts digits per block, the next
+// adds the counts it needs itself (of many blocks, a launch between them does)
+// and scatters. Element counts (and the depth
+// keys' range) are read from device memory so the same launches can sit in a
+// CUDA graph. These launches move a few MB at most; what they cost is the
+// launches and their dependent latencies.
 #include <algorithm>
 
 #include "gs_internal.cuh"
@@ -39,19 +46,47 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
     return m;
 }
 
-// Histogram of one digit over each block's slice: hist[d * G + b]. Each warp
-// counts into its own shared sub-histogram (shared-memory atomics); every
-// thread has four keys in flight per round.
+// The digit of one pass: the low `bits` bits of key - base in `passes` passes of equal width, with
+// bits given, or base and bits from the keys' {min, max} on the device.
+struct DigitSpec {
+    const uint32_t* range;
+    int bits, pass, passes;
+};
+struct Digit {
+    uint32_t base, mask;
+    int shift, nbits;
+    __device__ __forceinline__ Digit(const DigitSpec& s) {
+        base = 0;
+        int bits = s.bits;
+        if (s.range != nullptr) {
+            base = s.range[0];
+            bits = 32 - __clz(s.range[1] - base);
+        }
+        const int w = (bits + s.passes - 1) / s.passes;
+        shift = s.pass * w;
+        nbits = max(min(w, bits - shift), 0);
+        if (nbits == 0) shift = 0;
+        mask = (1u << nbits) - 1u;
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t key) const { return ((key - base) >> shift) & mask; }
+};
+
+// Histogram of one digit over each block's slice: hist[b << nbits | d]. Up to eight shared
+// sub-histograms, one a warp (shared-memory atomics); every thread has four keys in flight.
+template <int MAXBITS>
 __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t* __restrict__ keys,
                                                              const uint32_t* __restrict__ n_dev, uint32_t n_max,
-                                                             int shift, int nbits, uint32_t* __restrict__ hist) {
-    __shared__ uint32_t h[kSortWarps][256];
-    const int G = gridDim.x, b = blockIdx.x, w = threadIdx.x >> 5;
-    const uint32_t mask = (1u << nbits) - 1u;
-    for (int d = threadIdx.x; d < kSortWarps * 256; d += kSortThreads) (&h[0][0])[d] = 0;
-    __syncthreads();
+                                                             DigitSpec spec, uint32_t* __restrict__ hist) {
+    constexpr int kWords = kSortWarps << (MAXBITS <= 8 ? MAXBITS : 9);
+    __shared__ uint32_t h[kWords];
+    const int G = gridDim.x, b = blockIdx.x;
     uint32_t n = umin(*n_dev, n_max), begin, end;
     slice_of(n, G, b, begin, end);
+    const Digit dig(spec);
+    const int nsub = min(kSortWarps, kWords >> dig.nbits);
+    for (int d = threadIdx.x; d < nsub << dig.nbits; d += kSortThreads) h[d] = 0;
+    __syncthreads();
+    uint32_t* hw = h + (((threadIdx.x >> 5) & (nsub - 1)) << dig.nbits);
     for (uint32_t base = begin + threadIdx.x; base < end; base += 4 * kSortThreads) {
         uint32_t k[4];
 #pragma unroll
@@ -61,76 +96,85 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t* __r
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            if (base + u * kSortThreads < end) atomicAdd(&h[w][(k[u] >> shift) & mask], 1u);
+            if (base + u * kSortThreads < end) atomicAdd(&hw[dig(k[u])], 1u);
     }
     __syncthreads();
-    for (int d = threadIdx.x; d <= (int)mask; d += kSortThreads) {
+    for (int d = threadIdx.x; d <= (int)dig.mask; d += kSortThreads) {
         uint32_t t = 0;
-#pragma unroll
-        for (int ww = 0; ww < kSortWarps; ++ww) t += h[ww][d];
-        hist[(size_t)d * G + b] = t;
+        for (int q = 0; q < nsub; ++q) t += h[(q << dig.nbits) + d];
+        hist[((size_t)b << dig.nbits) + d] = t;
     }
 }
 
-// Exclusive scan of each digit's row of block counts (one CTA per digit):
-// hist[d * G + b] <- sum of hist[d * G + b'] for b' < b; dtot[d] <- row total.
-__global__ void __launch_bounds__(256) k_digit_scan(uint32_t* __restrict__ hist, int G, uint32_t* __restrict__ dtot) {
-    __shared__ uint32_t ws[8];
-    __shared__ uint32_t carry;
-    const int d = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
-    uint32_t* row = hist + (size_t)d * G;
-    if (t == 0) carry = 0;
+// Of more than kScanGrid blocks: the rows' exclusive scan over the blocks, in place, and each digit's
+// total. A CTA takes eight digits, 32 threads each.
+constexpr int kScanGrid = 128;
+__global__ void __launch_bounds__(256) k_digit_scan(uint32_t* __restrict__ hist, int G, DigitSpec spec,
+                                                    uint32_t* __restrict__ dtot) {
+    __shared__ uint32_t part[32][8];
+    const Digit dig(spec);
+    const int c = threadIdx.x & 7, g = threadIdx.x >> 3;
+    const int d = blockIdx.x * 8 + c, ndig = 1 << dig.nbits;
+    if (blockIdx.x * 8 >= ndig) return;   // the whole CTA (the grid is for the widest digit)
+    const int chunk = (G + 31) / 32, r0 = g * chunk, r1 = min(G, r0 + chunk);
+    uint32_t* col = hist + d;
+    uint32_t sum = 0;
+    if (d < ndig) {
+#pragma unroll 8
+        for (int r = r0; r < r1; ++r) sum += col[(size_t)r << dig.nbits];
+    }
+    part[g][c] = sum;
     __syncthreads();
-    for (int base = 0; base < G; base += 256) {
-        const int i = base + t;
-        const uint32_t c = i < G ? row[i] : 0u;
-        uint32_t x = c;
+    uint32_t run = 0, all = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) ws[w] = x;
-        __syncthreads();
-        uint32_t pre = 0, tot = 0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            uint32_t v = ws[k];
-            pre += (k < w) ? v : 0u;
-            tot += v;
-        }
-        const uint32_t before = carry;
-        if (i < G) row[i] = before + pre + x - c;
-        __syncthreads();
-        if (t == 0) carry = before + tot;
-        __syncthreads();
+    for (int q = 0; q < 32; ++q) {
+        const uint32_t v = part[q][c];
+        run += q < g ? v : 0u;
+        all += v;
     }
-    if (t == 0) dtot[d] = carry;
+    if (d < ndig) {
+#pragma unroll 8
+        for (int r = r0; r < r1; ++r) {
+            const uint32_t v = col[(size_t)r << dig.nbits];
+            col[(size_t)r << dig.nbits] = run;
+            run += v;
+        }
+        if (g == 0) dtot[d] = all;
+    }
 }
 
-// Stable scatter of one digit pass. Each block walks its slice in rounds of
-// kRound elements; warp w of a round owns a contiguous run of 32*kSortItems
-// elements, ranked within the warp by __match_any_sync, across warps by a
-// per-digit prefix over the warps' counts, and across blocks by the scanned
-// histogram. The ranked round is first regrouped by digit in shared memory,
+// Stable scatter of one digit pass. Up to kScanGrid blocks the block first adds the digit counts of
+// the blocks before its own, and of all blocks, straight from the histogram rows (16-byte loads, rows
+// in parallel: less than a separate scan launch takes; at 608 blocks and 128 digits it took 25 us more
+// than the scan), else it finds them in its row and in dtot. Then it
+// walks its slice in rounds of kRound elements; warp w of a round owns a contiguous run of
+// 32*kSortItems elements, ranked within the warp by __match_any_sync, across warps by a
+// per-digit prefix over the warps' counts, and across blocks by those sums.
+// The ranked round is first regrouped by digit in shared memory,
 // then written out by consecutive threads, so each digit's run of the round
 // leaves in coalesced stores instead of one scattered store per element.
-// Five CTAs per SM (at most 51 registers; A/B on the 300k-Gaussian keyframe: iteration
-// 0.5494 -> 0.5467 ms).
-__global__ void __launch_bounds__(kSortThreads, 5) k_radix_scatter(
+template <int MAXBITS>
+struct ScatterSmem {
+    static constexpr int D = 1 << MAXBITS;
+    uint32_t run[D];      // global position of the block's next element of each digit
+    uint32_t lstart[D];   // start of each digit's group in the staged round
+    uint16_t wcnt[kSortWarps][D];
+    uint32_t skey[kRound], sval[kRound];
+    uint32_t wsum[kSortWarps];
+};
+template <int MAXBITS>
+__global__ void __launch_bounds__(kSortThreads, MAXBITS <= 8 ? 5 : 3) k_radix_scatter(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
-    uint32_t* __restrict__ vout, const uint32_t* __restrict__ n_dev, uint32_t n_max, int shift, int nbits,
+    uint32_t* __restrict__ vout, const uint32_t* __restrict__ n_dev, uint32_t n_max, DigitSpec spec,
     const uint32_t* __restrict__ hist, const uint32_t* __restrict__ dtot) {
-    __shared__ uint32_t run[256];      // global position of the block's next element of each digit
-    __shared__ uint32_t lstart[256];   // start of each digit's group in the staged round
-    __shared__ uint32_t wsum[kSortWarps];
-    __shared__ uint32_t wcnt[kSortWarps][256];
-    __shared__ uint32_t skey[kRound], sval[kRound];
-    const int G = gridDim.x, b = blockIdx.x;
-    const uint32_t mask = (1u << nbits) - 1u;
-    const int ndig = 1 << nbits;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    // exclusive scan of one value per thread (thread d holds digit d) over the block
+    extern __shared__ __align__(16) uint8_t scatter_smem[];
+    ScatterSmem<MAXBITS>& sm = *reinterpret_cast<ScatterSmem<MAXBITS>*>(scatter_smem);
+    constexpr int E = (1 << MAXBITS) / kSortThreads < 1 ? 1 : (1 << MAXBITS) / kSortThreads;   // digits a thread
+    const int G = gridDim.x, b = blockIdx.x, t = threadIdx.x;
+    const Digit dig(spec);
+    const int ndig = 1 << dig.nbits;
+    const int lane = t & 31, w = t >> 5;
+    // exclusive scan of one value per thread over the block
     auto block_scan = [&](uint32_t c) -> uint32_t {
         uint32_t x = c;
 #pragma unroll
@@ -138,23 +182,84 @@ __global__ void __launch_bounds__(kSortThreads, 5) k_radix_scatter(
             const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
             if (lane >= o) x += y;
         }
-        if (lane == 31) wsum[w] = x;
+        if (lane == 31) sm.wsum[w] = x;
         __syncthreads();
         uint32_t pre = 0;
-        for (int k = 0; k < w; ++k) pre += wsum[k];
+        for (int k = 0; k < w; ++k) pre += sm.wsum[k];
         __syncthreads();
         return pre + x - c;
     };
-    {
-        const int d = threadIdx.x;
-        const uint32_t start = block_scan(d < ndig ? dtot[d] : 0u);
-        if (d < ndig) run[d] = start + hist[(size_t)d * G + b];
+    // run: counts before this block; lstart: totals
+    for (int d = t; d < ndig; d += kSortThreads) {
+        sm.run[d] = dtot != nullptr ? hist[((size_t)b << dig.nbits) + d] : 0u;
+        sm.lstart[d] = dtot != nullptr ? dtot[d] : 0u;
     }
+    __syncthreads();
+    if (dtot != nullptr) {
+    } else if (dig.nbits >= 2) {
+        const int cols = ndig / 4, groups = max(1, kSortThreads / cols);
+        for (int c = t % min(cols, kSortThreads); c < cols; c += kSortThreads) {
+            uint4 bef = make_uint4(0, 0, 0, 0), tot = bef;
+            const uint4* row = reinterpret_cast<const uint4*>(hist) + c;
+            for (int r0 = t / min(cols, kSortThreads); r0 < G; r0 += 8 * groups) {
+                uint4 v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int r = r0 + u * groups;
+                    v[u] = r < G ? row[(size_t)r * cols] : make_uint4(0, 0, 0, 0);
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const bool before = r0 + u * groups < b;
+                    tot.x += v[u].x;
+                    tot.y += v[u].y;
+                    tot.z += v[u].z;
+                    tot.w += v[u].w;
+                    bef.x += before ? v[u].x : 0u;
+                    bef.y += before ? v[u].y : 0u;
+                    bef.z += before ? v[u].z : 0u;
+                    bef.w += before ? v[u].w : 0u;
+                }
+            }
+            const uint32_t vb[4] = {bef.x, bef.y, bef.z, bef.w}, vt[4] = {tot.x, tot.y, tot.z, tot.w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                atomicAdd(&sm.run[4 * c + q], vb[q]);
+                atomicAdd(&sm.lstart[4 * c + q], vt[q]);
+            }
+        }
+    } else {
+        for (int r = t; r < G; r += kSortThreads)
+            for (int d = 0; d < ndig; ++d) {
+                const uint32_t v = hist[(size_t)r * ndig + d];
+                atomicAdd(&sm.lstart[d], v);
+                if (r < b) atomicAdd(&sm.run[d], v);
+            }
+    }
+    __syncthreads();
+    {   // thread t holds digits t * per .. : exclusive scan of the totals
+        const int per = max(1, ndig / kSortThreads);
+        uint32_t v[E], sum = 0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int d = t * per + e;
+            v[e] = e < per && d < ndig ? sm.lstart[d] : 0u;
+            sum += v[e];
+        }
+        uint32_t start = block_scan(sum);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int d = t * per + e;
+            if (e < per && d < ndig) sm.run[d] += start;
+            start += v[e];
+        }
+    }
+    __syncthreads();
     uint32_t n = umin(*n_dev, n_max), begin, end;
     slice_of(n, G, b, begin, end);
     const uint32_t lt = lanemask_lt();
     for (uint32_t rbase = begin; rbase < end; rbase += kRound) {
-        for (int d = lane; d < ndig; d += 32) wcnt[w][d] = 0;
+        for (int d = lane; d < ndig; d += 32) sm.wcnt[w][d] = 0;
         __syncwarp();
         uint32_t key[kSortItems], val[kSortItems], rank[kSortItems];
         const uint32_t wbase = rbase + (uint32_t)w * 32u * kSortItems;
@@ -164,68 +269,288 @@ __global__ void __launch_bounds__(kSortThreads, 5) k_radix_scatter(
             bool ok = i < end;
             key[it] = ok ? kin[i] : 0u;
             val[it] = ok ? vin[i] : 0u;
-            uint32_t d = ok ? (key[it] >> shift) & mask : 0xFFFFFFFFu;
+        }
+#pragma unroll
+        for (int it = 0; it < kSortItems; ++it) {
+            const bool ok = wbase + it * 32 + lane < end;
+            uint32_t d = ok ? dig(key[it]) : 0xFFFFFFFFu;
             uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
             uint32_t r = 0;
-            if (ok) r = wcnt[w][d] + __popc(peers & lt);
+            if (ok) r = sm.wcnt[w][d] + __popc(peers & lt);
             rank[it] = r;
             __syncwarp();
-            if (ok && (__ffs(peers) - 1) == lane) wcnt[w][d] += __popc(peers);
+            if (ok && (__ffs(peers) - 1) == lane) sm.wcnt[w][d] += (uint16_t)__popc(peers);
             __syncwarp();
         }
         __syncthreads();
         // per digit: prefix over the warps, the round's count, and its group start in the round
-        uint32_t tot = 0;
+        uint32_t tot[E];
         {
-            const int d = threadIdx.x;
-            if (d < ndig) {
+            const int per = max(1, ndig / kSortThreads);
+            uint32_t sum = 0;
 #pragma unroll
-                for (int ww = 0; ww < kSortWarps; ++ww) {
-                    const uint32_t c = wcnt[ww][d];
-                    wcnt[ww][d] = tot;
-                    tot += c;
+            for (int e = 0; e < E; ++e) {
+                const int d = t * per + e;
+                tot[e] = 0;
+                if (e < per && d < ndig) {
+#pragma unroll
+                    for (int ww = 0; ww < kSortWarps; ++ww) {
+                        const uint32_t c = sm.wcnt[ww][d];
+                        sm.wcnt[ww][d] = (uint16_t)tot[e];
+                        tot[e] += c;
+                    }
                 }
+                sum += tot[e];
             }
-            const uint32_t ls = block_scan(tot);   // synchronises the block
-            if (d < ndig) lstart[d] = ls;
+            uint32_t ls = block_scan(sum);   // synchronises the block
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const int d = t * per + e;
+                if (e < per && d < ndig) sm.lstart[d] = ls;
+                ls += tot[e];
+            }
         }
         __syncthreads();
 #pragma unroll
         for (int it = 0; it < kSortItems; ++it) {
             const uint32_t i = wbase + it * 32 + lane;
             if (i < end) {
-                const uint32_t d = (key[it] >> shift) & mask;
-                const uint32_t lp = lstart[d] + wcnt[w][d] + rank[it];
-                skey[lp] = key[it];
-                sval[lp] = val[it];
+                const uint32_t d = dig(key[it]);
+                const uint32_t lp = sm.lstart[d] + sm.wcnt[w][d] + rank[it];
+                sm.skey[lp] = key[it];
+                sm.sval[lp] = val[it];
             }
         }
         __syncthreads();
         const uint32_t cnt = umin((uint32_t)kRound, end - rbase);
-        for (uint32_t j = threadIdx.x; j < cnt; j += kSortThreads) {
-            const uint32_t k2 = skey[j], d = (k2 >> shift) & mask;
-            const uint32_t pos = run[d] + (j - lstart[d]);
+        for (uint32_t j = t; j < cnt; j += kSortThreads) {
+            const uint32_t k2 = sm.skey[j], d = dig(k2);
+            const uint32_t pos = sm.run[d] + (j - sm.lstart[d]);
             kout[pos] = k2;
-            vout[pos] = sval[j];
+            vout[pos] = sm.sval[j];
         }
         __syncthreads();
-        if (threadIdx.x < ndig) run[threadIdx.x] += tot;
+        {
+            const int per = max(1, ndig / kSortThreads);
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const int d = t * per + e;
+                if (e < per && d < ndig) sm.run[d] += tot[e];
+            }
+        }
         __syncthreads();
     }
 }
 
-// ---- scan of the tiles touched, in depth order ----
+template <int MAXBITS>
+cudaError_t launch_radix_pass(int G, const uint32_t* kin, const uint32_t* vin, uint32_t* kout, uint32_t* vout,
+                              const uint32_t* n_dev, uint32_t n_max, const DigitSpec& spec, uint32_t* hist,
+                              uint32_t* dtot, cudaStream_t s) {
+    k_radix_hist<MAXBITS><<<G, kSortThreads, 0, s>>>(kin, n_dev, n_max, spec, hist);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    if (G > kScanGrid) {
+        k_digit_scan<<<(1 << MAXBITS) / 8, 256, 0, s>>>(hist, G, spec, dtot);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    } else {
+        dtot = nullptr;
+    }
+    k_radix_scatter<MAXBITS><<<G, kSortThreads, sizeof(ScatterSmem<MAXBITS>), s>>>(kin, vin, kout, vout, n_dev, n_max,
+                                                                                  spec, hist, dtot);
+    return cudaGetLastError();
+}
 
-__global__ void __launch_bounds__(256) k_tile_block_sums(const uint32_t* __restrict__ order,
-                                                         const uint32_t* __restrict__ tiles, uint32_t n,
-                                                         const uint32_t* __restrict__ n_dev,
-                                                         uint32_t* __restrict__ bsum) {
+// ---- small maps: the visible items compacted and depth-sorted in one CTA ----
+//
+// Raw keys and items 0 .. n - 1 in, the order and the tile counts' sums per 256 ordered items out
+// (with the visible count and the pair total). In place of eight launches (compaction, three passes
+// of two, tile sums) of about 3 us each.
+constexpr int kSmallThreads = 1024, kSmallPer = 8, kSmallItems = kSmallThreads * kSmallPer, kSmallBits = 7;
+struct SmallSmem {
+    uint32_t key[kSmallItems], val[kSmallItems];
+    uint16_t wcnt[32][1 << kSmallBits];
+    uint32_t start[1 << kSmallBits];
+    uint32_t wsum[32], kmin, kmax, total;
+};
+__global__ void __launch_bounds__(kSmallThreads, 1) k_small_depth(const uint32_t* __restrict__ kin, uint32_t n,
+                                                                 const uint32_t* __restrict__ tiles,
+                                                                 uint32_t* __restrict__ order,
+                                                                 uint32_t* __restrict__ tile_blocks,
+                                                                 uint32_t* __restrict__ counts) {
+    extern __shared__ __align__(16) uint8_t scatter_smem[];
+    SmallSmem& sm = *reinterpret_cast<SmallSmem*>(scatter_smem);
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const uint32_t lt = lanemask_lt();
+    if (t == 0) {
+        sm.kmin = 0xFFFFFFFFu;
+        sm.kmax = 0u;
+    }
+    // exclusive scan over the block of one value a warp's lane 0 (returned to the warp), and the total
+    auto warps_scan = [&](uint32_t c, uint32_t& total) -> uint32_t {
+        if (lane == 0) sm.wsum[w] = c;
+        __syncthreads();
+        const uint32_t v = sm.wsum[lane];
+        uint32_t x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += y;
+        }
+        total = __shfl_sync(0xFFFFFFFFu, x, 31);
+        const uint32_t e = __shfl_sync(0xFFFFFFFFu, x - v, w);
+        __syncthreads();
+        return e;
+    };
+    uint32_t key[kSmallPer], val[kSmallPer], rank[kSmallPer];
+    uint32_t m;
+    {
+        const int per = (int)((n + kSmallThreads - 1) / kSmallThreads);
+        uint32_t bal[kSmallPer], cnt = 0, lo = 0xFFFFFFFFu, hi = 0u;
+#pragma unroll
+        for (int it = 0; it < kSmallPer; ++it) {
+            const uint32_t i = (uint32_t)(w * per + it) * 32u + lane;
+            const bool in = it < per && i < n;
+            key[it] = in ? kin[i] : 0xFFFFFFFFu;
+            const bool vis = key[it] != 0xFFFFFFFFu;
+            bal[it] = __ballot_sync(0xFFFFFFFFu, vis);
+            cnt += __popc(bal[it]);
+            lo = umin(lo, key[it]);
+            if (vis) hi = umax(hi, key[it]);
+        }
+        lo = __reduce_min_sync(0xFFFFFFFFu, lo);
+        hi = __reduce_max_sync(0xFFFFFFFFu, hi);
+        uint32_t pos = warps_scan(cnt, m);
+        if (lane == 0) {
+            atomicMin(&sm.kmin, lo);
+            atomicMax(&sm.kmax, hi);
+        }
+#pragma unroll
+        for (int it = 0; it < kSmallPer; ++it) {
+            if (bal[it] >> lane & 1u) {
+                const uint32_t p = pos + __popc(bal[it] & lt);
+                sm.key[p] = key[it];
+                sm.val[p] = (uint32_t)(w * per + it) * 32u + lane;
+            }
+            pos += __popc(bal[it]);
+        }
+    }
+    __syncthreads();
+    const uint32_t base = sm.kmin;
+    const int bits = m ? 32 - __clz(sm.kmax - base) : 0;
+    const int passes = (bits + kSmallBits - 1) / kSmallBits, width = passes ? (bits + passes - 1) / passes : 0;
+    const int ndig = 1 << width;
+    const uint32_t mask = (uint32_t)ndig - 1u;
+    const int per = (int)((m + kSmallThreads - 1) / kSmallThreads);
+    for (int pass = 0; pass < passes; ++pass) {
+        const int shift = pass * width;
+        for (int d = lane; d < ndig; d += 32) sm.wcnt[w][d] = 0;
+        __syncwarp();
+#pragma unroll
+        for (int it = 0; it < kSmallPer; ++it) {
+            if (it >= per) break;
+            const uint32_t i = (uint32_t)(w * per + it) * 32u + lane;
+            const bool ok = i < m;
+            key[it] = ok ? sm.key[i] : 0u;
+            val[it] = ok ? sm.val[i] : 0u;
+            const uint32_t d = ok ? ((key[it] - base) >> shift) & mask : 0xFFFFFFFFu;
+            const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
+            rank[it] = ok ? sm.wcnt[w][d] + __popc(peers & lt) : 0u;
+            __syncwarp();
+            if (ok && (__ffs(peers) - 1) == lane) sm.wcnt[w][d] += (uint16_t)__popc(peers);
+            __syncwarp();
+        }
+        __syncthreads();
+        uint32_t tot = 0;
+        if (t < ndig) {
+#pragma unroll 8
+            for (int ww = 0; ww < 32; ++ww) {
+                const uint32_t c = sm.wcnt[ww][t];
+                sm.wcnt[ww][t] = (uint16_t)tot;
+                tot += c;
+            }
+        }
+        uint32_t x = tot;   // digits 32 w + lane: inclusive scan in the warp, then over the warps
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+            if (lane >= o) x += y;
+        }
+        uint32_t all;
+        const uint32_t pre = warps_scan(__shfl_sync(0xFFFFFFFFu, x, 31), all);
+        if (t < ndig) sm.start[t] = pre + x - tot;
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < kSmallPer; ++it) {
+            if (it >= per) break;
+            const uint32_t i = (uint32_t)(w * per + it) * 32u + lane;
+            if (i < m) {
+                const uint32_t d = ((key[it] - base) >> shift) & mask;
+                const uint32_t p = sm.start[d] + sm.wcnt[w][d] + rank[it];
+                sm.key[p] = key[it];
+                sm.val[p] = val[it];
+            }
+        }
+        __syncthreads();
+    }
+    if (t == 0) sm.total = 0;
+    __syncthreads();
+    // tile counts per 256 ordered items (eight warps of 32 a block): sums for the emission
+    for (uint32_t i0 = 0; i0 < m; i0 += kSmallThreads) {
+        const uint32_t i = i0 + t;
+        uint32_t c = 0;
+        if (i < m) {
+            const uint32_t item = sm.val[i];
+            order[i] = item;
+            c = tiles[item];
+        }
+        c = __reduce_add_sync(0xFFFFFFFFu, c);
+        if (lane == 0) sm.wsum[w] = c;
+        __syncthreads();
+        if (t < 4 && i0 + 256u * t < m) {
+            uint32_t b = 0;
+            for (int q = 0; q < 8; ++q) b += sm.wsum[8 * t + q];
+            tile_blocks[i0 / 256 + t] = b;
+            atomicAdd(&sm.total, b);
+        }
+        __syncthreads();
+    }
+    if (t == 0) {
+        counts[0] = sm.total;
+        counts[8] = m;
+    }
+}
+
+// Tiles touched by each 256 items of the depth order (the emission's CTAs), and their total.
+__global__ void __launch_bounds__(256) k_item_tiles(const uint32_t* __restrict__ order,
+                                                    const uint32_t* __restrict__ tiles, uint32_t n_items,
+                                                    const uint32_t* __restrict__ n_dev,
+                                                    uint32_t* __restrict__ tile_blocks, uint32_t* __restrict__ total) {
     __shared__ uint32_t ws[8];
-    if (n_dev != nullptr) n = umin(n, *n_dev);
+    const uint32_t nv = umin(n_items, *n_dev);
+    for (uint32_t b = blockIdx.x; b * 256u < nv; b += gridDim.x) {
+        const uint32_t k = b * 256u + threadIdx.x;
+        const uint32_t c = __reduce_add_sync(0xFFFFFFFFu, k < nv ? tiles[order[k]] : 0u);
+        if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = c;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            uint32_t t = 0;
+            for (int q = 0; q < 8; ++q) t += ws[q];
+            tile_blocks[b] = t;
+            atomicAdd(total, t);   // (zeroed by the compaction)
+        }
+        __syncthreads();
+    }
+}
+
+// ---- exclusive scan of u32 values (map management) ----
+
+__global__ void __launch_bounds__(256) k_block_sums(const uint32_t* __restrict__ in, uint32_t n,
+                                                    uint32_t* __restrict__ bsum) {
+    __shared__ uint32_t ws[8];
     uint32_t begin, end;
     slice_of(n, gridDim.x, blockIdx.x, begin, end);
     uint32_t s = 0;
-    for (uint32_t i = begin + threadIdx.x; i < end; i += 256) s += tiles[order ? order[i] : i];
+    for (uint32_t i = begin + threadIdx.x; i < end; i += 256) s += in[i];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
     if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
@@ -237,17 +562,14 @@ __global__ void __launch_bounds__(256) k_tile_block_sums(const uint32_t* __restr
     }
 }
 
-// Exclusive scan of the slices of k_tile_block_sums: block b first adds the block sums of the
+// Exclusive scan of the slices of k_block_sums: block b first adds the block sums of the
 // slices before its own (a few hundred values, read straight from bsum: no separate scan
 // launch), then scans its slice; the last block writes the total.
-__global__ void __launch_bounds__(256) k_tile_scan(const uint32_t* __restrict__ order,
-                                                   const uint32_t* __restrict__ tiles, uint32_t n,
-                                                   const uint32_t* __restrict__ n_dev,
-                                                   const uint32_t* __restrict__ bsum, uint32_t* __restrict__ off,
-                                                   uint32_t* __restrict__ total_out) {
+__global__ void __launch_bounds__(256) k_scan(const uint32_t* __restrict__ in, uint32_t n,
+                                              const uint32_t* __restrict__ bsum, uint32_t* __restrict__ off,
+                                              uint32_t* __restrict__ total_out) {
     __shared__ uint32_t ws[8];
     __shared__ uint32_t carry;
-    if (n_dev != nullptr) n = umin(n, *n_dev);
     uint32_t begin, end;
     slice_of(n, gridDim.x, blockIdx.x, begin, end);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -267,7 +589,7 @@ __global__ void __launch_bounds__(256) k_tile_scan(const uint32_t* __restrict__ 
     }
     for (uint32_t base = begin; base < end; base += 256) {
         uint32_t i = base + threadIdx.x;
-        uint32_t c = i < end ? tiles[order ? order[i] : i] : 0u;
+        uint32_t c = i < end ? in[i] : 0u;
         uint32_t x = c;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -291,8 +613,9 @@ __global__ void __launch_bounds__(256) k_tile_scan(const uint32_t* __restrict__ 
     if (total_out != nullptr && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *total_out = carry;
 }
 
-// Pair emission: item k of the depth order owns pairs off[k] .. off[k] + tiles
-// - 1, one per tile of its pixel box in row-major order (bin, item). Each warp
+// Pair emission: item k of the depth order owns pairs o .. o + tiles - 1, with o
+// the tiles of the items before it (the CTA adds the block sums before its own
+// and scans its 256 items), one per tile of its pixel box in row-major order (bin, item). Each warp
 // takes 32 consecutive items, scans their tile counts, and writes the warp's
 // pairs (a contiguous run of the output) 32 at a time: lane j writes pair t =
 // t0 + j of the run, owned by the last lane whose exclusive count is <= t, so
@@ -300,25 +623,48 @@ __global__ void __launch_bounds__(256) k_tile_scan(const uint32_t* __restrict__ 
 // warp. An item whose pairs would pass pair_cap is skipped and sets *overflow.
 // In the deterministic mode (emit_item != NULL) a pair's value is its emission
 // index e instead of its item, emit_item[e] holds the item, and the pair's
-// gradient slot pairgrad[9 e ..] is cleared.
+// gradient slot pairgrad[9 e ..] is cleared; off[k] = o for its reduction.
 __global__ void __launch_bounds__(256) k_emit(const uint32_t* __restrict__ order, const uint32_t* __restrict__ tiles,
-                                              const uint32_t* __restrict__ off, const float4* __restrict__ rec,
+                                              const uint32_t* __restrict__ tile_blocks, uint32_t* __restrict__ off,
+                                              const float4* __restrict__ rec,
                                               const DevCamera* __restrict__ cams, int n, int tile, uint32_t n_items,
                                               const uint32_t* __restrict__ n_dev, uint64_t pair_cap,
                                               uint32_t* __restrict__ pkey, uint32_t* __restrict__ pval,
                                               uint32_t* __restrict__ overflow, uint32_t* __restrict__ emit_item,
                                               float* __restrict__ pairgrad) {
+    __shared__ uint32_t sbef[8], stot[8];
     const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t nv = umin(n_items, *n_dev);
-    if (k - (uint32_t)lane >= nv) return;   // the whole warp is past the visible items
+    if (blockIdx.x * blockDim.x >= nv) return;   // the whole CTA is past the visible items
     uint32_t item = 0, cnt = 0, o = 0, bin0 = 0, tiles_x = 0;
     int tx0 = 0, ty0 = 0, wt = 1;
     if (k < nv) {
         item = order[k];
         cnt = tiles[item];
+    }
+    {
+        uint32_t bef = 0;
+        for (uint32_t b = threadIdx.x; b < blockIdx.x; b += 256) bef += tile_blocks[b];
+        bef = __reduce_add_sync(0xFFFFFFFFu, bef);
+        uint32_t x = cnt;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, d);
+            if (lane >= d) x += y;
+        }
+        if (lane == 31) {
+            sbef[w] = bef;
+            stot[w] = x;
+        }
+        __syncthreads();
+        o = x - cnt;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) o += sbef[q] + (q < w ? stot[q] : 0u);
+    }
+    if (k < nv) {
+        if (emit_item != nullptr) off[k] = o;
         if (cnt != 0) {
-            o = off[k];
             if ((uint64_t)o + cnt > pair_cap) {
                 atomicMax(overflow, 1u);
                 cnt = 0;
@@ -459,47 +805,77 @@ __global__ void __launch_bounds__(1024) k_work_order(const uint2* __restrict__ r
 
 }  // namespace
 
-cudaError_t radix_sort_pairs(gs_ctx* c, uint32_t** keys, uint32_t** vals, const uint32_t* n_dev, uint32_t n_max,
-                             uint32_t n_hint, int bits, int* out_buf, cudaStream_t s) {
-    int cur = 0;
-    // about 2048 elements (one scatter round) per block, each block owning one contiguous slice
-    const int G = (int)std::max<uint32_t>(1u, std::min<uint32_t>((uint32_t)c->sort_blocks, (n_hint + 2047u) / 2048u));
-    for (int shift = 0; shift < bits; shift += 8) {
-        int nb = bits - shift < 8 ? bits - shift : 8;
-        c->launches += 3;
-        uint32_t* dtot = c->hist + (size_t)256 * c->sort_blocks;
-        k_radix_hist<<<G, kSortThreads, 0, s>>>(keys[cur], n_dev, n_max, shift, nb, c->hist);
-        k_digit_scan<<<1 << nb, 256, 0, s>>>(c->hist, G, dtot);
-        k_radix_scatter<<<G, kSortThreads, 0, s>>>(keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], n_dev, n_max,
-                                                   shift, nb, c->hist, dtot);
+cudaError_t sort_kernels_init() {
+    cudaError_t e = cudaFuncSetAttribute(k_radix_scatter<11>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(ScatterSmem<11>));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_small_depth, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem));
+    return e;
+}
+
+size_t sort_hist_words(int sort_blocks) { return ((size_t)sort_blocks << 11) + (1u << 11); }
+static uint32_t* sort_totals(const gs_ctx* c) { return c->hist + ((size_t)c->sort_blocks << 11); }
+
+// about 2048 elements (one scatter round) per block, each block owning one contiguous slice
+static int sort_grid(const gs_ctx* c, uint32_t n_hint) {
+    return (int)std::max<uint32_t>(1u, std::min<uint32_t>((uint32_t)c->sort_blocks, (n_hint + 2047u) / 2048u));
+}
+
+bool depth_sort_small(const gs_ctx* c) { return (uint64_t)c->n_views * (uint64_t)c->n <= (uint64_t)kSmallItems; }
+
+// Raw keys in dkey[0] (and, above kSmallItems, the compacted ones in dkey[1] / dval[1]): the visible
+// items in depth order to dval[0], their tile sums to tile_blocks and dcount[0].
+cudaError_t sort_depth(gs_ctx* c, uint32_t n_max, uint32_t n_hint, cudaStream_t s) {
+    if (depth_sort_small(c)) {
+        ++c->launches;
+        k_small_depth<<<1, kSmallThreads, sizeof(SmallSmem), s>>>(c->dkey[0], n_max, c->tiles_touched, c->dval[0],
+                                                                 c->tile_blocks, c->dcount);
+        return cudaGetLastError();
+    }
+    const int G = sort_grid(c, n_hint);
+    int cur = 1;
+    for (int pass = 0; pass < 3; ++pass) {
+        c->launches += G > kScanGrid ? 3 : 2;
+        const cudaError_t e =
+            launch_radix_pass<11>(G, c->dkey[cur], c->dval[cur], c->dkey[cur ^ 1], c->dval[cur ^ 1], c->dcount + 8, n_max,
+                                  DigitSpec{c->dcount + 11, 0, pass, 3}, c->hist, sort_totals(c), s);
+        if (e != cudaSuccess) return e;
         cur ^= 1;
     }
-    *out_buf = cur;
+    ++c->launches;
+    const int blocks = (int)std::max<uint32_t>(1u, std::min<uint32_t>((n_max + 255u) / 256u, (n_hint + 255u) / 256u));
+    k_item_tiles<<<blocks, 256, 0, s>>>(c->dval[0], c->tiles_touched, n_max, c->dcount + 8, c->tile_blocks, c->dcount);
     return cudaGetLastError();
 }
 
-cudaError_t scan_tiles(gs_ctx* c, uint32_t n_max, const uint32_t* n_dev, cudaStream_t s) {
-    // the depth-sorted order is in dval[0] after the even number (4) of depth passes
-    const int G = c->sort_blocks;
-    c->launches += 2;
-    k_tile_block_sums<<<G, 256, 0, s>>>(c->dval[0], c->tiles_touched, n_max, n_dev, c->hist);
-    k_tile_scan<<<G, 256, 0, s>>>(c->dval[0], c->tiles_touched, n_max, n_dev, c->hist, c->offsets, c->dcount);
-    return cudaGetLastError();
+cudaError_t radix_sort_pairs(gs_ctx* c, uint32_t** keys, uint32_t** vals, const uint32_t* n_dev, uint32_t n_max,
+                             uint32_t n_hint, int bits, int* out_buf, cudaStream_t s) {
+    int cur = 0;
+    const int G = sort_grid(c, n_hint), passes = (bits + 7) / 8;
+    for (int pass = 0; pass < passes; ++pass) {
+        c->launches += G > kScanGrid ? 3 : 2;
+        const cudaError_t e = launch_radix_pass<8>(G, keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], n_dev, n_max,
+                                                   DigitSpec{nullptr, bits, pass, passes}, c->hist, sort_totals(c), s);
+        if (e != cudaSuccess) return e;
+        cur ^= 1;
+    }
+    *out_buf = cur;
+    return cudaSuccess;
 }
 
 cudaError_t scan_u32(gs_ctx* c, const uint32_t* in, uint32_t* out, uint32_t n, uint32_t* total_dev,
                      cudaStream_t s) {
     const int G = c->sort_blocks;
     c->launches += 2;
-    k_tile_block_sums<<<G, 256, 0, s>>>(nullptr, in, n, nullptr, c->hist);
-    k_tile_scan<<<G, 256, 0, s>>>(nullptr, in, n, nullptr, c->hist, out, total_dev);
+    k_block_sums<<<G, 256, 0, s>>>(in, n, c->hist);
+    k_scan<<<G, 256, 0, s>>>(in, n, c->hist, out, total_dev);
     return cudaGetLastError();
 }
 
 cudaError_t emit_pairs(gs_ctx* c, uint32_t n_items, const uint32_t* n_dev, cudaStream_t s) {
     if (n_items == 0) return cudaSuccess;
     ++c->launches;
-    k_emit<<<(n_items + 255) / 256, 256, 0, s>>>(c->dval[0], c->tiles_touched, c->offsets, c->rec, c->dcam, c->n,
+    k_emit<<<(n_items + 255) / 256, 256, 0, s>>>(c->dval[0], c->tiles_touched, c->tile_blocks, c->offsets, c->rec, c->dcam, c->n,
                                                  c->tile, n_items, n_dev, (uint64_t)c->pair_cap, c->pkey[0],
                                                  c->pval[0], c->dcount + 1, c->emit_item, c->pairgrad);
     return cudaGetLastError();
@@ -641,14 +1017,9 @@ extern "C" int gs_sort_pairs_static(const uint32_t* keys_in, const uint32_t* val
         const bool to_out = ((passes - i) & 1) == 1;
         uint32_t* dk = to_out ? keys_out : tmp_k;
         uint32_t* dv = to_out ? vals_out : tmp_v;
-        const int shift = 8 * i;
-        const int nb = bits - shift < 8 ? bits - shift : 8;
-        k_radix_hist<<<G, kSortThreads, 0, s>>>(src_k, sentinel, un, shift, nb, hist);
-        if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
-        k_digit_scan<<<1 << nb, 256, 0, s>>>(hist, G, dtot);
-        if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
-        k_radix_scatter<<<G, kSortThreads, 0, s>>>(src_k, src_v, dk, dv, sentinel, un, shift, nb, hist, dtot);
-        if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
+        if (launch_radix_pass<8>(G, src_k, src_v, dk, dv, sentinel, un, DigitSpec{nullptr, bits, i, passes}, hist, dtot, s) !=
+            cudaSuccess)
+            return GS_ERR_CUDA;
         src_k = dk;
         src_v = dv;
     }
