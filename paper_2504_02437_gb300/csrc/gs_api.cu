@@ -497,7 +497,7 @@ void gs_destroy(gs_ctx* c) {
                     c->tiles_touched, c->depth, c->dkey[0], c->dkey[1], c->dval[0], c->dval[1], c->offsets, c->ranges,
                     c->work_order, c->work_order_graph, c->T_final, c->n_last, c->dLdC, c->grad2d, c->hist, c->vis_blocks, c->vis_range, c->tile_blocks, (void*)c->target_slot, c->ssim_maps, c->ssim_part, c->dcount,
                     c->partials, c->psnr_part, c->reg_part, c->tile_part, c->fpart,
-                    c->own_rgb, c->tgt_stage[0], c->tgt_stage[1]};
+                    c->own_rgb, c->tgt_stage[0], c->tgt_stage[1], c->scratch, c->spare[0], c->spare[1], c->spare[2]};
     for (void* p : ptrs) cudaFree(p);
     free_pairs(c);
     if (c->hcount) cudaFreeHost(c->hcount);
@@ -1211,20 +1211,33 @@ int gs_debug_grad2d(gs_ctx* c, float* out) {
 
 namespace {
 
-struct Temp {
-    void* p[8] = {nullptr};
-    int k = 0;
+// The context's scratch memory, handed out in 256-byte aligned pieces: add() every piece, then
+// reserve() (which may move the memory), then take() them in the same order.
+struct Scratch {
+    gs_ctx* c;
+    size_t need = 0, used = 0;
+    explicit Scratch(gs_ctx* c_) : c(c_) {}
+    static size_t round(size_t b) { return (b + 255) & ~(size_t)255; }
     template <typename T>
-    bool get(T** out, size_t count) {
-        if (cudaMalloc((void**)out, sizeof(T) * (count ? count : 1)) != cudaSuccess) {
-            *out = nullptr;
+    void add(size_t count) { need += round(sizeof(T) * count); }
+    bool reserve() {
+        if (need <= c->scratch_bytes) return true;
+        cudaFree(c->scratch);   // (no call of this context is using it: each synchronises at its end)
+        c->scratch = nullptr;
+        c->scratch_bytes = 0;
+        if (cudaMalloc((void**)&c->scratch, need) != cudaSuccess) {
+            c->scratch = nullptr;
+            cudaGetLastError();
             return false;
         }
-        p[k++] = *out;
+        c->scratch_bytes = need;
         return true;
     }
-    ~Temp() {
-        for (int i = 0; i < k; ++i) cudaFree(p[i]);
+    template <typename T>
+    T* take(size_t count) {
+        T* p = reinterpret_cast<T*>(c->scratch + used);
+        used += round(sizeof(T) * count);
+        return p;
     }
 };
 
@@ -1245,12 +1258,16 @@ int gs_init_map(gs_ctx* c, const float* pts, const float* rgb, int n, void* stre
     if (n == 0) return GS_OK;
     cudaStream_t s = (cudaStream_t)stream;
     CK(cudaSetDevice(c->device));
-    Temp t;
-    float *ref = nullptr, *stage = nullptr;
-    if (!t.get(&ref, 3 * (size_t)n) || !t.get(&stage, kParamRows * (size_t)n))
-        return fail(c, GS_ERR_OOM, "temporary buffers");
+    Scratch t(c);
+    t.add<float>(3 * (size_t)n);
+    t.add<float>(kParamRows * (size_t)n);
+    t.add<float>(knn_scratch(c, n, n));
+    if (!t.reserve()) return fail(c, GS_ERR_OOM, "temporary buffers");
+    float* ref = t.take<float>(3 * (size_t)n);
+    float* stage = t.take<float>(kParamRows * (size_t)n);
+    float* part = t.take<float>(knn_scratch(c, n, n));
     CK(launch_points_planar(pts, n, ref, s));
-    CK(launch_init_points(c, pts, rgb, n, ref, n, n, 1, stage, n, s));
+    CK(launch_init_points(c, pts, rgb, n, ref, n, n, 1, part, stage, n, s));
     CK(cudaMemcpy2DAsync(c->params + c->n, sizeof(float) * c->cap, stage, sizeof(float) * n, sizeof(float) * n,
                          kParamRows, cudaMemcpyDeviceToDevice, s));
     for (float* a : {c->adam_m, c->adam_v})
@@ -1262,11 +1279,6 @@ int gs_init_map(gs_ctx* c, const float* pts, const float* rgb, int n, void* stre
     c->n += n;
     invalidate_render(c);
     return GS_OK;
-}
-
-__global__ void k_mask_u8(const uint32_t* __restrict__ keep, int n, uint8_t* __restrict__ out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = keep[i] ? 1 : 0;
 }
 
 int gs_set_initializer(gs_ctx* c, gs_mlp* mlp) {
@@ -1284,13 +1296,21 @@ int gs_insert(gs_ctx* c, const gs_camera* cam, const float* image, const float* 
     if ((int64_t)c->n + n > c->cap) return fail(c, GS_ERR_CAPACITY, "insertion could exceed the capacity");
     cudaStream_t s = (cudaStream_t)stream;
     CK(cudaSetDevice(c->device));
-    Temp t;
-    float *img = nullptr, *stage = nullptr, *feat = nullptr;
-    uint32_t *keep = nullptr, *pos = nullptr;
-    const size_t HW = (size_t)cam->width * cam->height;
-    if (!t.get(&img, 3 * HW) || !t.get(&stage, kParamRows * (size_t)n) || !t.get(&keep, (size_t)n) ||
-        !t.get(&pos, (size_t)n) || !t.get(&feat, 80 * (size_t)n))
-        return fail(c, GS_ERR_OOM, "temporary buffers");
+    const size_t HW = (size_t)cam->width * cam->height, np = (size_t)n;
+    if (!camera_ok(*cam, c->cfg)) return fail(c, GS_ERR_ARG, "invalid camera");
+    const size_t n_part = knn_scratch(c, n, c->n), n_feat = c->init_mlp ? 80 * np : 0;
+    Scratch t(c);
+    t.add<float>(3 * HW);
+    t.add<float>(kParamRows * np);
+    t.add<uint32_t>(np);
+    t.add<float>(n_part);
+    t.add<float>(n_feat);
+    if (!t.reserve()) return fail(c, GS_ERR_OOM, "temporary buffers");
+    float* img = t.take<float>(3 * HW);
+    float* stage = t.take<float>(kParamRows * np);
+    uint32_t* keep = t.take<uint32_t>(np);
+    float* part = t.take<float>(n_part);
+    float* feat = t.take<float>(n_feat);
     if (c->cfg.insert_tau > 0.f) {
         // distance rule: no render, only the camera (pixel colours of the plain initialisation)
         CamBatch b;
@@ -1300,15 +1320,9 @@ int gs_insert(gs_ctx* c, const gs_camera* cam, const float* image, const float* 
         const int code = gs_render(c, cam, 1, img, nullptr, nullptr, stream);
         if (code != GS_OK) return code;
     }
-    CK(launch_insert_test(c, c->hcam[0], pts, n, image, keep, stage, s));
+    CK(launch_insert_test(c, c->hcam[0], pts, n, image, part, keep, stage, s));
     if (c->init_mlp) CK(mlp_initialise(c->init_mlp, c->hcam[0], image, pts, n, stage, feat, s));
-    if (inserted_dev) {
-        k_mask_u8<<<(n + 255) / 256, 256, 0, s>>>(keep, n, inserted_dev);
-        CK(cudaGetLastError());
-    }
-    CK(scan_u32(c, keep, pos, (uint32_t)n, c->dcount + 5, s));
-    CK(launch_append(c, stage, n, keep, pos, s));
-    CK(cudaMemcpyAsync(c->hcount + 5, c->dcount + 5, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    CK(launch_append(c, stage, n, keep, inserted_dev, c->hcount + 5, s));
     CK(cudaStreamSynchronize(s));
     *n_ins = (int)c->hcount[5];
     c->n += *n_ins;
@@ -1322,11 +1336,14 @@ int gs_count_dominant(gs_ctx* c, const gs_camera* cams, int n_views, void* strea
     if (c->n == 0) return GS_OK;
     cudaStream_t s = (cudaStream_t)stream;
     CK(cudaSetDevice(c->device));
+    if (!camera_ok(cams[0], c->cfg)) return fail(c, GS_ERR_ARG, "invalid camera");
     const size_t pix = (size_t)n_views * cams[0].width * cams[0].height;
-    Temp t;
-    float* img = nullptr;
-    int32_t* am = nullptr;
-    if (!t.get(&img, 3 * pix) || !t.get(&am, pix)) return fail(c, GS_ERR_OOM, "temporary buffers");
+    Scratch t(c);
+    t.add<float>(3 * pix);
+    t.add<int32_t>(pix);
+    if (!t.reserve()) return fail(c, GS_ERR_OOM, "temporary buffers");
+    float* img = t.take<float>(3 * pix);
+    int32_t* am = t.take<int32_t>(pix);
     const int code = gs_render(c, cams, n_views, img, nullptr, am, stream);
     if (code != GS_OK) return code;
     CK(launch_count_dominant(c, am, pix, s));
@@ -1340,9 +1357,12 @@ int gs_densify(gs_ctx* c, const float* normals, int* n_split_out, void* stream) 
     if (c->n == 0) return GS_OK;
     cudaStream_t s = (cudaStream_t)stream;
     CK(cudaSetDevice(c->device));
-    Temp t;
-    uint32_t *flags = nullptr, *pos = nullptr;
-    if (!t.get(&flags, (size_t)c->n) || !t.get(&pos, (size_t)c->n)) return fail(c, GS_ERR_OOM, "temporary buffers");
+    Scratch t(c);
+    t.add<uint32_t>((size_t)c->n);
+    t.add<uint32_t>((size_t)c->n);
+    if (!t.reserve()) return fail(c, GS_ERR_OOM, "temporary buffers");
+    uint32_t* flags = t.take<uint32_t>((size_t)c->n);
+    uint32_t* pos = t.take<uint32_t>((size_t)c->n);
     CK(launch_split_flags(c, flags, s));
     CK(scan_u32(c, flags, pos, (uint32_t)c->n, c->dcount + 5, s));
     CK(cudaMemcpyAsync(c->hcount + 5, c->dcount + 5, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
@@ -1350,32 +1370,16 @@ int gs_densify(gs_ctx* c, const float* normals, int* n_split_out, void* stream) 
     const uint32_t n_split = c->hcount[5];
     if ((int64_t)c->n + n_split > c->cap) return fail(c, GS_ERR_CAPACITY, "splitting would exceed the capacity");
     if (n_split > 0) {
-        float *P2 = nullptr, *M2 = nullptr, *V2 = nullptr;
-        const size_t sz = kParamRows * (size_t)c->cap;
-        if (dalloc(&P2, sz) != cudaSuccess) return fail(c, GS_ERR_OOM, "split buffers");
-        if (dalloc(&M2, sz) != cudaSuccess) {
-            cudaFree(P2);
-            return fail(c, GS_ERR_OOM, "split buffers");
-        }
-        if (dalloc(&V2, sz) != cudaSuccess) {
-            cudaFree(P2);
-            cudaFree(M2);
-            return fail(c, GS_ERR_OOM, "split buffers");
-        }
-        cudaError_t e = launch_split_scatter(c, flags, pos, n_split, normals, P2, M2, V2, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) {
-            cudaFree(P2);
-            cudaFree(M2);
-            cudaFree(V2);
-            return fail(c, GS_ERR_CUDA, "split", e);
-        }
-        cudaFree(c->params);
-        cudaFree(c->adam_m);
-        cudaFree(c->adam_v);
-        c->params = P2;
-        c->adam_m = M2;
-        c->adam_v = V2;
+        // into the other set of buffers, which this call's first split allocates
+        for (float*& q : c->spare)
+            if (q == nullptr && dalloc(&q, kParamRows * (size_t)c->cap) != cudaSuccess) {
+                q = nullptr;
+                return fail(c, GS_ERR_OOM, "split buffers", cudaErrorMemoryAllocation);
+            }
+        CK(launch_split_scatter(c, flags, pos, n_split, normals, c->spare[0], c->spare[1], c->spare[2], s));
+        std::swap(c->params, c->spare[0]);
+        std::swap(c->adam_m, c->spare[1]);
+        std::swap(c->adam_v, c->spare[2]);
         c->n += (int)n_split;
     }
     CK(cudaMemsetAsync(c->dens_sum, 0, sizeof(float) * c->cap, s));

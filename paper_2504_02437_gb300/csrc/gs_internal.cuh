@@ -212,6 +212,11 @@ struct gs_ctx {
     std::vector<Tuned> tuned;
     int force_tile = 0, force_ppt = 0;      // set while the autotuner times a candidate
     gs_mlp* init_mlp = nullptr;             // learned initialiser of gs_insert (NULL = plain)
+    // what the map-management calls need while they run (each ends with a synchronisation): kept from
+    // call to call, grown when a call needs more, freed with the context
+    uint8_t* scratch = nullptr;
+    size_t scratch_bytes = 0;
+    float* spare[3] = {};                   // [14][cap] the other parameter and moment buffers of a split
 };
 
 namespace gs {
@@ -303,13 +308,15 @@ cudaError_t launch_copy_T(gs_ctx* c, float* T_out, cudaStream_t s);
 cudaError_t mlp_initialise(gs_mlp* M, const DevCamera& cam, const float* image, const float* pts, int n, float* stage,
                            float* feat_tmp, cudaStream_t s);
 // map management (k_map.cu)
+size_t knn_scratch(const gs_ctx* c, int n, int n_ref);   // floats of `part` for n queries of n_ref references
 cudaError_t launch_init_points(gs_ctx* c, const float* pts, const float* rgb, int n, const float* ref, int ref_stride,
-                               int n_ref, int ref_is_self, float* out_params, int out_stride, cudaStream_t s);
+                               int n_ref, int ref_is_self, float* part, float* out_params, int out_stride,
+                               cudaStream_t s);
 cudaError_t launch_points_planar(const float* pts, int n, float* out, cudaStream_t s);
 cudaError_t launch_insert_test(gs_ctx* c, const DevCamera& cam, const float* pts, int n, const float* image,
-                               uint32_t* keep, float* stage, cudaStream_t s);
-cudaError_t launch_append(gs_ctx* c, const float* stage, int n_stage, const uint32_t* keep, const uint32_t* pos,
-                          cudaStream_t s);
+                               float* part, uint32_t* keep, float* stage, cudaStream_t s);
+cudaError_t launch_append(gs_ctx* c, const float* stage, int n_stage, const uint32_t* keep, uint8_t* mask,
+                          uint32_t* count_host, cudaStream_t s);
 cudaError_t launch_count_dominant(gs_ctx* c, const int32_t* argmax, size_t n_pix, cudaStream_t s);
 cudaError_t launch_split_flags(gs_ctx* c, uint32_t* flags, cudaStream_t s);
 cudaError_t launch_split_scatter(gs_ctx* c, const uint32_t* flags, const uint32_t* pos, uint32_t n_split,

@@ -8,95 +8,128 @@
 namespace gs {
 namespace {
 
-// 3 smallest squared distances from q to the reference points (one CTA per query).
-// ref is planar [3][ref_stride]; skip index `self` (or -1). Returns the RMS of
-// those distances (0.01 if there is no reference point) to every thread, and
-// the smallest squared distance (+inf if none) in *dmin2 of thread 0.
-__device__ float knn3_rms(const float* __restrict__ ref, int ref_stride, int n_ref, float qx, float qy, float qz,
-                          int self, float* dmin2) {
-    __shared__ float best[256 * 3];
+// ---- the 3 nearest reference points of each query ----
+//
+// Brute force over all pairs, split over chunks of the reference points so that a keyframe's
+// hundred queries fill the GPU: a warp takes kKnnQueries queries through one chunk, its lanes the
+// references side by side (a load serves all its queries), and leaves the chunk's 3 smallest squared
+// distances; the kernels that use them merge the chunks, a warp a query. Bound by some eight
+// instructions a pair: 96 queries of 150,000 points 310 us with one CTA walking all references for
+// each query, and one thread merging 768 candidates; 18 us and 6 for the merge.
+constexpr int kKnnQueries = 4, kKnnWarps = 8;
+
+struct Best3 {
     float b0 = INFINITY, b1 = INFINITY, b2 = INFINITY;
-    for (int j = threadIdx.x; j < n_ref; j += blockDim.x) {
-        if (j == self) continue;
-        float dx = ref[j] - qx, dy = ref[ref_stride + j] - qy, dz = ref[2 * ref_stride + j] - qz;
-        float d = dx * dx + dy * dy + dz * dz;
-        if (d < b2) {
-            if (d < b1) {
-                b2 = b1;
-                if (d < b0) {
-                    b1 = b0;
-                    b0 = d;
-                } else {
-                    b1 = d;
-                }
-            } else {
-                b2 = d;
+    // (without branches: each lane's insertion would be its own; a distance that is not a number counts
+    // as infinite)
+    __device__ __forceinline__ void add(float d) {
+        d = d < INFINITY ? d : INFINITY;
+        const float t = fmaxf(b0, d), t1 = fmaxf(b1, t);
+        b0 = fminf(b0, d);
+        b1 = fminf(b1, t);
+        b2 = fminf(b2, t1);
+    }
+    // the warp's 3 smallest, to every lane (squared distances: the order of the bits is theirs)
+    __device__ __forceinline__ void merge_warp() {
+        float r[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t m = __reduce_min_sync(0xFFFFFFFFu, __float_as_uint(b0));
+            const uint32_t who = __ballot_sync(0xFFFFFFFFu, __float_as_uint(b0) == m);
+            r[k] = __uint_as_float(m);
+            if ((threadIdx.x & 31) == __ffs(who) - 1) {
+                b0 = b1;
+                b1 = b2;
+                b2 = INFINITY;
             }
         }
+        b0 = r[0];
+        b1 = r[1];
+        b2 = r[2];
     }
-    best[threadIdx.x * 3 + 0] = b0;
-    best[threadIdx.x * 3 + 1] = b1;
-    best[threadIdx.x * 3 + 2] = b2;
-    __syncthreads();
-    __shared__ float rms;
-    if (threadIdx.x == 0) {
-        float c0 = INFINITY, c1 = INFINITY, c2 = INFINITY;
-        for (int k = 0; k < (int)blockDim.x * 3; ++k) {
-            float d = best[k];
-            if (d < c2) {
-                if (d < c1) {
-                    c2 = c1;
-                    if (d < c0) {
-                        c1 = c0;
-                        c0 = d;
-                    } else {
-                        c1 = d;
-                    }
-                } else {
-                    c2 = d;
-                }
-            }
+    // root mean square of the distances there are (0.01 if there is no reference point)
+    __device__ __forceinline__ float rms() const {
+        const int cnt = (b0 < INFINITY) + (b1 < INFINITY) + (b2 < INFINITY);
+        const float s = (cnt > 0 ? b0 : 0.f) + (cnt > 1 ? b1 : 0.f) + (cnt > 2 ? b2 : 0.f);
+        return cnt > 0 ? sqrtf(s / (float)cnt) : 0.01f;
+    }
+};
+
+// Queries q [n][3]; references planar [3][ref_stride], query i's own excluded when ref_is_self.
+// part[chunk][query][3].
+__global__ void __launch_bounds__(32 * kKnnWarps) k_knn_chunks(const float* __restrict__ q, int n,
+                                                              const float* __restrict__ ref, int ref_stride, int n_ref,
+                                                              int chunk, int ref_is_self, float* __restrict__ part) {
+    const int lane = threadIdx.x & 31, q0 = (blockIdx.x * kKnnWarps + (threadIdx.x >> 5)) * kKnnQueries;
+    if (q0 >= n) return;
+    float x[kKnnQueries], y[kKnnQueries], z[kKnnQueries];
+    Best3 best[kKnnQueries];
+#pragma unroll
+    for (int k = 0; k < kKnnQueries; ++k) {
+        const size_t i = (size_t)min(q0 + k, n - 1);
+        x[k] = q[3 * i];
+        y[k] = q[3 * i + 1];
+        z[k] = q[3 * i + 2];
+    }
+    const int j0 = blockIdx.y * chunk, j1 = min(n_ref, j0 + chunk);
+#pragma unroll 4
+    for (int j = j0 + lane; j < j1; j += 32) {
+        const float rx = ref[j], ry = ref[(size_t)ref_stride + j], rz = ref[2 * (size_t)ref_stride + j];
+#pragma unroll
+        for (int k = 0; k < kKnnQueries; ++k) {
+            const float dx = rx - x[k], dy = ry - y[k], dz = rz - z[k];
+            const float d = dx * dx + dy * dy + dz * dz;
+            best[k].add(ref_is_self && j == q0 + k ? INFINITY : d);
         }
-        *dmin2 = c0;
-        int cnt = (c0 < INFINITY) + (c1 < INFINITY) + (c2 < INFINITY);
-        float s = (cnt > 0 ? c0 : 0.f) + (cnt > 1 ? c1 : 0.f) + (cnt > 2 ? c2 : 0.f);
-        rms = cnt > 0 ? sqrtf(s / (float)cnt) : 0.01f;
     }
-    __syncthreads();
-    return rms;
+#pragma unroll
+    for (int k = 0; k < kKnnQueries; ++k) {
+        best[k].merge_warp();
+        if (q0 + k < n && lane < 3)
+            part[((size_t)blockIdx.y * n + q0 + k) * 3 + lane] = lane == 0 ? best[k].b0 : (lane == 1 ? best[k].b1 : best[k].b2);
+    }
 }
 
-// Plain initialisation of one new Gaussian per block.
+// the chunks' candidates of query i, merged by its warp
+__device__ __forceinline__ Best3 knn_of(const float* __restrict__ part, int chunks, int n, int i) {
+    Best3 b;
+    for (int k = threadIdx.x & 31; k < 3 * chunks; k += 32) b.add(part[((size_t)(k / 3) * n + i) * 3 + k % 3]);
+    b.merge_warp();
+    return b;
+}
+
+// Plain initialisation, one new Gaussian per warp.
 __global__ void __launch_bounds__(256) k_init_points(const float* __restrict__ pts, const float* __restrict__ rgb,
-                                                     const float* __restrict__ ref, int ref_stride, int n_ref,
-                                                     int ref_is_self, float* __restrict__ out, int out_stride) {
-    int i = blockIdx.x;
-    float x = pts[3 * i], y = pts[3 * i + 1], z = pts[3 * i + 2];
-    float dmin2;
-    float rms = knn3_rms(ref, ref_stride, n_ref, x, y, z, ref_is_self ? i : -1, &dmin2);
-    if (threadIdx.x == 0) {
+                                                     const float* __restrict__ part, int chunks, int n,
+                                                     float* __restrict__ out, int out_stride) {
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i >= n) return;
+    const float rms = knn_of(part, chunks, n, i).rms();
+    if ((threadIdx.x & 31) == 0) {
+        float x = pts[3 * (size_t)i], y = pts[3 * (size_t)i + 1], z = pts[3 * (size_t)i + 2];
         float ls = fminf(fmaxf(logf(fmaxf(rms, 1e-30f)), -7.f), -1.f);
-        const float v[kParamRows] = {x, y, z, ls, ls, ls, 1.f, 0.f, 0.f, 0.f, 0.f, rgb[3 * i], rgb[3 * i + 1],
-                                     rgb[3 * i + 2]};
+        const float v[kParamRows] = {x, y, z, ls, ls, ls, 1.f, 0.f, 0.f, 0.f, 0.f, rgb[3 * (size_t)i],
+                                     rgb[3 * (size_t)i + 1], rgb[3 * (size_t)i + 2]};
         for (int r = 0; r < kParamRows; ++r) out[(size_t)r * out_stride + i] = v[r];
     }
 }
 
-// Insertion test of point i. Opacity gate (tau2 = 0): keep[i] = 0 iff the point
+// Insertion test of point i (a warp). Opacity gate (tau2 = 0): keep[i] = 0 iff the point
 // projects, in front of the camera, to a pixel whose rendered opacity 1 - T
 // exceeds the threshold. Distance rule (tau2 = tau^2 > 0, Eq. 7 as its text
 // states it): keep[i] = 1 iff the nearest existing mean is farther than tau
 // (T is not read). Also stages the plain initial parameters [14][n].
 __global__ void __launch_bounds__(256) k_insert_test(DevCamera cam, float near_z, float thresh, float tau2,
                                                      const float* __restrict__ pts, const float* __restrict__ T,
-                                                     const float* __restrict__ image, const float* __restrict__ ref,
-                                                     int ref_stride, int n_ref, uint32_t* __restrict__ keep,
+                                                     const float* __restrict__ image, const float* __restrict__ part,
+                                                     int chunks, uint32_t* __restrict__ keep,
                                                      float* __restrict__ stage, int n) {
-    int i = blockIdx.x;
-    float x = pts[3 * i], y = pts[3 * i + 1], z = pts[3 * i + 2];
-    float dmin2 = INFINITY;
-    float rms = knn3_rms(ref, ref_stride, n_ref, x, y, z, -1, &dmin2);
-    if (threadIdx.x != 0) return;
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i >= n) return;
+    const Best3 best = knn_of(part, chunks, n, i);
+    if ((threadIdx.x & 31) != 0) return;
+    const float rms = best.rms(), dmin2 = best.b0;
+    float x = pts[3 * (size_t)i], y = pts[3 * (size_t)i + 1], z = pts[3 * (size_t)i + 2];
     float tx = cam.R[0] * x + cam.R[1] * y + cam.R[2] * z + cam.t[0];
     float ty = cam.R[3] * x + cam.R[4] * y + cam.R[5] * z + cam.t[1];
     float tz = cam.R[6] * x + cam.R[7] * y + cam.R[8] * z + cam.t[2];
@@ -115,22 +148,47 @@ __global__ void __launch_bounds__(256) k_insert_test(DevCamera cam, float near_z
     for (int r = 0; r < kParamRows; ++r) stage[(size_t)r * n + i] = vals[r];
 }
 
-__global__ void __launch_bounds__(256) k_append(const float* __restrict__ stage, int n_stage,
-                                                const uint32_t* __restrict__ keep, const uint32_t* __restrict__ pos,
-                                                float* __restrict__ P, float* __restrict__ M, float* __restrict__ V,
-                                                float* __restrict__ dsum, float* __restrict__ dcnt,
-                                                uint32_t* __restrict__ dom, int base, int cap) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_stage || !keep[i]) return;
-    int d = base + (int)pos[i];
-    for (int r = 0; r < kParamRows; ++r) {
-        P[(size_t)r * cap + d] = stage[(size_t)r * n_stage + i];
-        M[(size_t)r * cap + d] = 0.f;
-        V[(size_t)r * cap + d] = 0.f;
+// Appends the kept points in order to the map's n Gaussians (parameters, zero moments and statistics),
+// in one CTA that scans them as it goes; writes 1 or 0 per point to mask (optional) and their number
+// to *count (pinned host memory).
+__global__ void __launch_bounds__(1024) k_append(const float* __restrict__ stage, int n_stage,
+                                                 const uint32_t* __restrict__ keep, float* __restrict__ P,
+                                                 float* __restrict__ M, float* __restrict__ V,
+                                                 float* __restrict__ dsum, float* __restrict__ dcnt,
+                                                 uint32_t* __restrict__ dom, int base, int cap,
+                                                 uint8_t* __restrict__ mask, uint32_t* __restrict__ count) {
+    __shared__ uint32_t wsum[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t before = 0;
+    for (int i0 = 0; i0 < n_stage; i0 += 1024) {
+        const int i = i0 + threadIdx.x;
+        const bool k = i < n_stage && keep[i] != 0u;
+        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, k);
+        if (lane == 0) wsum[w] = __popc(bal);
+        __syncthreads();
+        uint32_t pre = 0, all = 0;
+#pragma unroll
+        for (int q = 0; q < 32; ++q) {
+            pre += q < w ? wsum[q] : 0u;
+            all += wsum[q];
+        }
+        __syncthreads();
+        if (mask != nullptr && i < n_stage) mask[i] = k ? 1 : 0;
+        if (k) {
+            const int d = base + (int)(before + pre + __popc(bal & ((1u << lane) - 1u)));
+#pragma unroll
+            for (int r = 0; r < kParamRows; ++r) {
+                P[(size_t)r * cap + d] = stage[(size_t)r * n_stage + i];
+                M[(size_t)r * cap + d] = 0.f;
+                V[(size_t)r * cap + d] = 0.f;
+            }
+            dsum[d] = 0.f;
+            dcnt[d] = 0.f;
+            dom[d] = 0u;
+        }
+        before += all;
     }
-    dsum[d] = 0.f;
-    dcnt[d] = 0.f;
-    dom[d] = 0u;
+    if (threadIdx.x == 0) *count = before;
 }
 
 // Split mask: the gradient criterion, or (sigma > 0) more than sigma dominated
@@ -220,11 +278,36 @@ __global__ void __launch_bounds__(256) k_split_scatter(const float* __restrict__
 
 }  // namespace
 
-cudaError_t launch_init_points(gs_ctx* c, const float* pts, const float* rgb, int n, const float* ref, int ref_stride,
-                               int n_ref, int ref_is_self, float* out_params, int out_stride, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
+// Chunks of the references: 256 of them or more, fewer chunks once the queries alone fill the GPU
+// (four CTAs an SM in all; the merge reads three candidates a chunk).
+static int knn_chunks(const gs_ctx* c, int n, int n_ref) {
+    const int per_cta = kKnnQueries * kKnnWarps, groups = (n + per_cta - 1) / per_cta;
+    const int want = (4 * c->num_sms + groups - 1) / groups;
+    return std::max(1, std::min(want, (n_ref + 255) / 256));
+}
+
+size_t knn_scratch(const gs_ctx* c, int n, int n_ref) { return 3 * (size_t)n * knn_chunks(c, n, n_ref); }
+
+static cudaError_t knn(gs_ctx* c, const float* q, int n, const float* ref, int ref_stride, int n_ref, int ref_is_self,
+                       float* part, int* chunks_out, cudaStream_t s) {
+    const int per_cta = kKnnQueries * kKnnWarps, chunks = knn_chunks(c, n, n_ref);
+    const int chunk = ((n_ref + chunks - 1) / chunks + 31) & ~31;
+    *chunks_out = chunks;
     ++c->launches;
-    k_init_points<<<n, 256, 0, s>>>(pts, rgb, ref, ref_stride, n_ref, ref_is_self, out_params, out_stride);
+    k_knn_chunks<<<dim3((n + per_cta - 1) / per_cta, chunks), 32 * kKnnWarps, 0, s>>>(q, n, ref, ref_stride, n_ref,
+                                                                                       chunk, ref_is_self, part);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_init_points(gs_ctx* c, const float* pts, const float* rgb, int n, const float* ref, int ref_stride,
+                               int n_ref, int ref_is_self, float* part, float* out_params, int out_stride,
+                               cudaStream_t s) {
+    if (n == 0) return cudaSuccess;
+    int chunks = 0;
+    const cudaError_t e = knn(c, pts, n, ref, ref_stride, n_ref, ref_is_self, part, &chunks, s);
+    if (e != cudaSuccess) return e;
+    ++c->launches;
+    k_init_points<<<(n + 7) / 8, 256, 0, s>>>(pts, rgb, part, chunks, n, out_params, out_stride);
     return cudaGetLastError();
 }
 
@@ -245,21 +328,24 @@ cudaError_t launch_points_planar(const float* pts, int n, float* out, cudaStream
 }
 
 cudaError_t launch_insert_test(gs_ctx* c, const DevCamera& cam, const float* pts, int n, const float* image,
-                               uint32_t* keep, float* stage, cudaStream_t s) {
+                               float* part, uint32_t* keep, float* stage, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
+    int chunks = 0;
+    const cudaError_t e = knn(c, pts, n, c->params, c->cap, c->n, 0, part, &chunks, s);
+    if (e != cudaSuccess) return e;
     ++c->launches;
     const float tau2 = c->cfg.insert_tau > 0.f ? c->cfg.insert_tau * c->cfg.insert_tau : 0.f;
-    k_insert_test<<<n, 256, 0, s>>>(cam, c->cfg.near_z, c->cfg.insert_opacity, tau2, pts, c->T_final, image,
-                                    c->params, c->cap, c->n, keep, stage, n);
+    k_insert_test<<<(n + 7) / 8, 256, 0, s>>>(cam, c->cfg.near_z, c->cfg.insert_opacity, tau2, pts, c->T_final, image,
+                                              part, chunks, keep, stage, n);
     return cudaGetLastError();
 }
 
-cudaError_t launch_append(gs_ctx* c, const float* stage, int n_stage, const uint32_t* keep, const uint32_t* pos,
-                          cudaStream_t s) {
+cudaError_t launch_append(gs_ctx* c, const float* stage, int n_stage, const uint32_t* keep, uint8_t* mask,
+                          uint32_t* count_host, cudaStream_t s) {
     if (n_stage == 0) return cudaSuccess;
     ++c->launches;
-    k_append<<<(n_stage + 255) / 256, 256, 0, s>>>(stage, n_stage, keep, pos, c->params, c->adam_m, c->adam_v,
-                                                   c->dens_sum, c->dens_cnt, c->dom_cnt, c->n, c->cap);
+    k_append<<<1, 1024, 0, s>>>(stage, n_stage, keep, c->params, c->adam_m, c->adam_v, c->dens_sum, c->dens_cnt,
+                                c->dom_cnt, c->n, c->cap, mask, count_host);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,72 @@
+"""The 3 nearest points behind the plain initialisation, at the edges of its chunks and query groups,
+against float64: log-scale = ln of the RMS distance (2e-6, the float32 distance's rounding), and the
+appending of more points than its CTA takes in one round."""
+import numpy as np
+import pytest
+import torch
+
+from synth import frustum_scene
+
+from gpu_helpers import cuda, new_map
+
+pytestmark = pytest.mark.gpu
+
+
+def log_scale(pts, ref, own):
+    d2 = ((pts[:, None, :].astype(np.float64) - ref[None].astype(np.float64)) ** 2).sum(-1)
+    d2 = np.where(np.isfinite(d2), d2, np.inf)
+    if own:
+        np.fill_diagonal(d2, np.inf)
+    d2 = np.sort(d2, axis=1)[:, :3]
+    cnt = np.isfinite(d2).sum(1)
+    s = np.where(np.isfinite(d2), d2, 0.0).sum(1)
+    rms = np.where(cnt > 0, np.sqrt(s / np.maximum(cnt, 1)), 0.01)
+    return np.clip(np.log(np.maximum(rms, 1e-30)), -7.0, -1.0)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 33, 257, 1500])
+def test_init_map_scales(n):
+    pts = np.random.default_rng(n).uniform(-0.05, 0.05, (n, 3)).astype(np.float32)
+    if n > 4:
+        pts[3] = pts[1]                      # a distance of zero
+    gm = new_map(n)
+    gm.init_map(cuda(pts), cuda(np.zeros((n, 3))))
+    got = gm.params().cpu().numpy()
+    np.testing.assert_allclose(got[3], log_scale(pts, pts, True), atol=2e-6, rtol=0)
+    np.testing.assert_array_equal(got[0:3], pts.T)
+
+
+@pytest.mark.parametrize("n_ref,n", [(0, 3), (1, 1), (2, 5), (31, 4), (257, 33), (1025, 100), (70_000, 7), (300, 2500)])
+def test_insert_scales_and_order(n_ref, n):
+    rng = np.random.default_rng(n_ref + n)
+    p, cam = frustum_scene(n=max(n_ref, 1), seed=4)
+    p = p[:, :n_ref]
+    p[10] = -20.0                            # faint: every point is inserted, by the opacity gate
+    if n_ref > 30:
+        p[0, 5] = np.nan                     # a mean that is no point's neighbour
+    pts = np.stack([rng.uniform(-1, 1, n), rng.uniform(-1, 1, n), rng.uniform(1, 5, n)], 1).astype(np.float32)
+    pts[::7, 2] *= -1.0                      # behind the camera: kept by the gate
+    gm = new_map(n_ref + n)
+    gm.set_params(cuda(p))
+    count, mask = gm.insert(cam, torch.zeros(3, 120, 160, device="cuda"), cuda(pts), return_mask=True)
+    assert count == n and bool(mask.all()) and gm.n == n_ref + n
+    got = gm.params().cpu().numpy()[:, n_ref:]
+    np.testing.assert_array_equal(got[0:3], pts.T)
+    np.testing.assert_allclose(got[3], log_scale(pts, p[0:3].T, False), atol=2e-6, rtol=0)
+
+
+def test_a_second_split_uses_the_buffers_of_the_first():
+    """Splits swap the parameters between two sets of buffers: three in a row from one map equal the
+    same splits of fresh maps."""
+    rng = np.random.default_rng(3)
+    p, cam = frustum_scene(n=500, seed=2)
+    gm = new_map(4000, clarity_sigma=3.0)
+    gm.set_params(cuda(p))
+    for k in range(3):
+        fresh = new_map(4000, clarity_sigma=3.0)
+        fresh.set_params(gm.params())
+        nz = cuda(rng.normal(size=(gm.n, 2, 3)))
+        for m in (gm, fresh):
+            m.count_dominant(cam)
+        assert gm.densify(nz) == fresh.densify(nz) > 0
+        assert torch.equal(gm.params(), fresh.params())
