@@ -173,6 +173,7 @@ struct Layout {
     // and 4; 8-view window 785 us with 2, 856 with 4), one where a launch is bound by issue slots
     // (16 x 1: 376, 398 and 427 us)
     static constexpr int kVisits = SPLIT == 2 ? 2 : 1;
+    static constexpr int kVisitsDet = 4;   // (fused kernel 220, 204 and 197 us for 1, 2 and 4: three 321x243 views)
     // long tiles go as two items of one pixel a thread, in the same CTAs as whole tiles of two
     static constexpr bool kHalves = TILE == 16 && PPT == 2;
     // the adjoint reuses the forward's staged batch and visit lists when the tile's whole list
@@ -385,49 +386,63 @@ __device__ __forceinline__ int fwd_core(const TileGeom<TILE, PPT, SPLIT>& g, con
         const int nk = build_warp_list(st, cnt, 0u, 0xFFFFFFFFu);
         if (rg.y - rg.x <= (uint32_t)kBatch) staged = nk;
         const typename Stage<kBatch, NT / 32>::Idx* wl = st.list[threadIdx.x >> 5];
-        if constexpr (PPT == 1) {
-            // one pixel a thread: kVisits entries at a time, their loads, tests and alphas without
-            // branches, so that their latencies overlap; only T runs through them in turn (16 x 1, one
-            // entry at a time, with the adjoint in the same form: 1200x680 keyframe 416 -> 376 us,
-            // 160x120 47 -> 36 us)
-            constexpr int U = Layout<TILE, PPT, SPLIT>::kVisits;
-            bool live = nlive > 0;
+        if constexpr (PPT == 1 || DET) {
+            // U entries at a time, their loads, tests and alphas without branches, so that their
+            // latencies overlap; only T runs through them in turn (16 x 1, one entry at a time, with
+            // the adjoint in the same form: 1200x680 keyframe 416 -> 376 us, 160x120 47 -> 36 us; in
+            // the deterministic mode, whose one warp a tile takes as long as its list, four at a time)
+            constexpr int U = DET ? Layout<TILE, PPT, SPLIT>::kVisitsDet : Layout<TILE, PPT, SPLIT>::kVisits;
+            bool live[PPT];
+#pragma unroll
+            for (int p = 0; p < PPT; ++p) live[p] = fy[p] != kGone;
             for (int i = 0; i < nk; i += U) {
-                if (!__any_sync(0xFFFFFFFFu, live)) break;
+                if (!__any_sync(0xFFFFFFFFu, nlive > 0)) break;
                 int k[U];
-                float al[U];
-                bool hit[U];
+                float al[U][PPT];
+                bool hit[U][PPT];
                 float4 c[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     k[u] = (int)wl[i + u] & (kBatch - 1);   // past nk: any entry, not hit
                     const float4 a = s0[k[u]], q = s1[k[u]];
                     c[u] = s2[k[u]];
-                    const float dx = g.fx - a.x, dy = fy[0] - a.y;
-                    const float p2 = power2_dy(q.z, __fmul_rn(q.y, dx), __fmul_rn(__fmul_rn(q.x, dx), dx), dy);
-                    hit[u] = i + u < nk && fabsf(dx) <= a.z && fabsf(dy) <= a.w && p2 >= c[u].w;
-                    al[u] = fminf(kc.alpha_max, __fmul_rn(q.w, ex2_approx(p2)));
+                    const float dx = g.fx - a.x;
+                    const float qydx = __fmul_rn(q.y, dx), qxdx2 = __fmul_rn(__fmul_rn(q.x, dx), dx);
+                    const bool col = i + u < nk && fabsf(dx) <= a.z;
+#pragma unroll
+                    for (int p = 0; p < PPT; ++p) {
+                        const float dy = fy[p] - a.y;
+                        const float p2 = power2_dy(q.z, qydx, qxdx2, dy);
+                        hit[u][p] = col && fabsf(dy) <= a.w && p2 >= c[u].w;
+                        al[u][p] = fminf(kc.alpha_max, __fmul_rn(q.w, ex2_approx(p2)));
+                    }
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const float Tn = __fmul_rn(T[0], 1.f - al[u]);
-                    const bool in = hit[u] && live;
-                    live = live && !(in && Tn < kc.T_min);   // a pixel stops before it falls below T_min
-                    if (in && live) {
-                        const float wgt = al[u] * T[0];
-                        cr[0] = fmaf(c[u].x, wgt, cr[0]);
-                        cg[0] = fmaf(c[u].y, wgt, cg[0]);
-                        cb[0] = fmaf(c[u].z, wgt, cb[0]);
-                        T[0] = Tn;
-                        last[0] = bs + k[u] - rg.x + 1;
-                        if (ARGMAX && wgt > wmax[0]) {
-                            wmax[0] = wgt;
-                            amax[0] = DET ? emit_item[sid[k[u]]] : sid[k[u]];
+#pragma unroll
+                    for (int p = 0; p < PPT; ++p) {
+                        const float Tn = __fmul_rn(T[p], 1.f - al[u][p]);
+                        const bool in = hit[u][p] && live[p];
+                        const bool stop = in && Tn < kc.T_min;   // a pixel stops before it falls below T_min
+                        live[p] = live[p] && !stop;
+                        nlive -= stop ? 1 : 0;
+                        if (in && live[p]) {
+                            const float wgt = al[u][p] * T[p];
+                            cr[p] = fmaf(c[u].x, wgt, cr[p]);
+                            cg[p] = fmaf(c[u].y, wgt, cg[p]);
+                            cb[p] = fmaf(c[u].z, wgt, cb[p]);
+                            T[p] = Tn;
+                            last[p] = bs + k[u] - rg.x + 1;
+                            if (ARGMAX && wgt > wmax[p]) {
+                                wmax[p] = wgt;
+                                amax[p] = DET ? emit_item[sid[k[u]]] : sid[k[u]];
+                            }
                         }
                     }
                 }
             }
-            nlive = live ? 1 : 0;
+#pragma unroll
+            for (int p = 0; p < PPT; ++p) fy[p] = live[p] ? fy[p] : kGone;
             continue;
         }
         int knext = nk > 0 ? (int)wl[0] : 0;   // the next entry's index is loaded one visit ahead
@@ -614,16 +629,17 @@ __device__ __forceinline__ void bwd_core(const TileGeom<TILE, PPT, SPLIT>& g, co
             masked = __syncthreads_or(wild);
             nk = build_warp_list(st, (int)(be - bs), bs, warp_end);
         }
-        if constexpr (PPT == 1) {
+        if constexpr (PPT == 1 || DET) {
             // U entries at a time: their loads, tests and alphas first and without branches (a pixel that
             // is not hit has alpha 0 and adds zeros), then T and g . a through them in turn, then their sums
-            constexpr int U = Layout<TILE, PPT, SPLIT>::kVisits;
+            constexpr int U = DET ? Layout<TILE, PPT, SPLIT>::kVisitsDet : Layout<TILE, PPT, SPLIT>::kVisits;
             for (int i = nk - 1; i >= 0; i -= U) {
                 int k[U];
+                bool any[U];
                 float acc[U][9];
                 float4 c[U], q[U];
-                float dx[U], dy[U], oG[U], nal[U], rc[U];
-                bool hit[U];
+                float dx[U], dy[U][PPT], oG[U][PPT], nal[U][PPT], rc[U][PPT];
+                bool hit[U][PPT];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     k[u] = (int)wl[U == 1 ? i : max(i - u, 0)];
@@ -631,34 +647,49 @@ __device__ __forceinline__ void bwd_core(const TileGeom<TILE, PPT, SPLIT>& g, co
                     q[u] = s1[k[u]];
                     c[u] = s2[k[u]];
                     dx[u] = g.fx - a.x;
-                    dy[u] = fy[0] - a.y;
-                    const float p2 = power2_dy(q[u].z, __fmul_rn(q[u].y, dx[u]),
-                                               __fmul_rn(__fmul_rn(q[u].x, dx[u]), dx[u]), dy[u]);
-                    hit[u] = (U == 1 || i - u >= 0) && bs + k[u] < my_end[0] && fabsf(dx[u]) <= a.z &&
-                             fabsf(dy[u]) <= a.w && p2 >= c[u].w;
-                    oG[u] = __fmul_rn(q[u].w, ex2_approx(p2));
-                    nal[u] = hit[u] ? -fminf(kc.alpha_max, oG[u]) : 0.f;
-                    rc[u] = rcp_approx(1.f + nal[u]);   // 1 - alpha >= 1 - alpha_max = 0.01
+                    const float qydx = __fmul_rn(q[u].y, dx[u]), qxdx2 = __fmul_rn(__fmul_rn(q[u].x, dx[u]), dx[u]);
+                    const bool col = (U == 1 || i - u >= 0) && fabsf(dx[u]) <= a.z;
+                    any[u] = false;
+#pragma unroll
+                    for (int p = 0; p < PPT; ++p) {
+                        dy[u][p] = fy[p] - a.y;
+                        const float p2 = power2_dy(q[u].z, qydx, qxdx2, dy[u][p]);
+                        hit[u][p] = col && bs + k[u] < my_end[p] && fabsf(dy[u][p]) <= a.w && p2 >= c[u].w;
+                        any[u] |= hit[u][p];
+                        oG[u][p] = __fmul_rn(q[u].w, ex2_approx(p2));
+                        nal[u][p] = hit[u][p] ? -fminf(kc.alpha_max, oG[u][p]) : 0.f;
+                        rc[u][p] = rcp_approx(1.f + nal[u][p]);   // 1 - alpha >= 1 - alpha_max = 0.01
+                    }
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    float gx = gr[0], gy = gg[0], gz = gb[0];
-                    if ((masked | warp_wild) && !hit[u]) gx = gy = gz = 0.f;
-                    T[0] *= rc[u];   // transmittance in front of this Gaussian
-                    const float nw = nal[u] * T[0];
-                    // dL/dalpha = T (g . c - g . a), with a the normalised colour behind this
-                    // Gaussian, a <- a + alpha (c - a); g is fixed per pixel, so only -g . a is kept
-                    const float d = fmaf(gx, c[u].x, fmaf(gy, c[u].y, gz * c[u].z)) + ga[0];
-                    ga[0] = hit[u] ? fmaf(nal[u], d, ga[0]) : ga[0];
-                    // through alpha = o 2^p2, zero where the 0.99 clamp holds; the factor ln 2
-                    // of d(2^p2)/dp2 is left to the readers of the screen gradients
-                    const float g2 = hit[u] && oG[u] <= kc.alpha_max ? T[0] * d * oG[u] : 0.f;
-                    const float g2y = g2 * dy[u];
-                    screen_partials(q[u], dx[u], g2, g2y, g2y * dy[u], nw * gx, nw * gy, nw * gz, acc[u]);
+                    float g2s = 0.f, g2y = 0.f, g2yy = 0.f, ncr = 0.f, ncg = 0.f, ncb = 0.f;
+#pragma unroll
+                    for (int p = 0; p < PPT; ++p) {
+                        float gx = gr[p], gy = gg[p], gz = gb[p];
+                        if ((masked | warp_wild) && !hit[u][p]) gx = gy = gz = 0.f;
+                        T[p] *= rc[u][p];   // transmittance in front of this Gaussian
+                        const float nw = nal[u][p] * T[p];
+                        // dL/dalpha = T (g . c - g . a), with a the normalised colour behind this
+                        // Gaussian, a <- a + alpha (c - a); g is fixed per pixel, so only -g . a is kept
+                        const float d = fmaf(gx, c[u].x, fmaf(gy, c[u].y, gz * c[u].z)) + ga[p];
+                        ga[p] = hit[u][p] ? fmaf(nal[u][p], d, ga[p]) : ga[p];
+                        // through alpha = o 2^p2, zero where the 0.99 clamp holds; the factor ln 2
+                        // of d(2^p2)/dp2 is left to the readers of the screen gradients
+                        const float g2 = hit[u][p] && oG[u][p] <= kc.alpha_max ? T[p] * d * oG[u][p] : 0.f;
+                        const float y = g2 * dy[u][p];
+                        g2s += g2;
+                        g2y += y;
+                        g2yy = fmaf(y, dy[u][p], g2yy);
+                        ncr = fmaf(nw, gx, ncr);
+                        ncg = fmaf(nw, gy, ncg);
+                        ncb = fmaf(nw, gz, ncb);
+                    }
+                    screen_partials(q[u], dx[u], g2s, g2y, g2yy, ncr, ncg, ncb, acc[u]);
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u)
-                    add_gradient<DET>(hit[u], acc[u], sid[k[u]], lane, grad2d, pairgrad);
+                    add_gradient<DET>(any[u], acc[u], sid[k[u]], lane, grad2d, pairgrad);
             }
         } else {
             int knext = nk > 0 ? (int)wl[nk - 1] : 0;   // as in the forward: one visit ahead

@@ -716,10 +716,20 @@ __global__ void __launch_bounds__(256) k_emit(const uint32_t* __restrict__ order
             if (emit_item != nullptr) {
                 pval[pos] = pos;
                 emit_item[pos] = s_item;
-#pragma unroll
-                for (int q = 0; q < kPairGradStride; ++q) pairgrad[(size_t)pos * kPairGradStride + q] = 0.f;
             } else {
                 pval[pos] = s_item;
+            }
+        }
+        if (emit_item != nullptr) {
+            // the slots of the 32 pairs lie side by side (unless an item of the warp was skipped):
+            // cleared by consecutive lanes
+            const uint32_t pos = s_o + t - s_excl, first = __shfl_sync(0xFFFFFFFFu, pos, 0);
+            const bool run = __all_sync(0xFFFFFFFFu, t >= total || pos == first + (uint32_t)lane);
+            const uint32_t n = min(32u, total - t0) * kPairGradStride;
+            if (run) {
+                for (uint32_t q = lane; q < n; q += 32) pairgrad[(size_t)first * kPairGradStride + q] = 0.f;
+            } else if (t < total) {
+                for (int q = 0; q < kPairGradStride; ++q) pairgrad[(size_t)pos * kPairGradStride + q] = 0.f;
             }
         }
     }
@@ -882,34 +892,46 @@ cudaError_t emit_pairs(gs_ctx* c, uint32_t n_items, const uint32_t* n_dev, cudaS
 }
 
 // Deterministic mode: item k of the depth order owns the pair slots off[k] ..
-// off[k] + tiles - 1 (its emission indices); their screen gradients are added in
-// that order into the item's grad2d record.
+// off[k] + tiles - 1 (its emission indices); a warp adds their screen gradients,
+// lane l those l, l + 32, .. and then a fixed tree over the lanes, into the
+// item's grad2d record. (One thread an item: a Gaussian over a thousand tiles
+// was the launch's time, 65 us for 20k Gaussians in three 321x243 views; 12 us.)
 __global__ void __launch_bounds__(256) k_pairgrad_reduce(const uint32_t* __restrict__ order,
                                                          const uint32_t* __restrict__ tiles,
                                                          const uint32_t* __restrict__ off, uint32_t n_items,
                                                          const uint32_t* __restrict__ n_dev, uint64_t pair_cap,
                                                          const float* __restrict__ pairgrad,
                                                          float* __restrict__ grad2d) {
-    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n_items || k >= *n_dev) return;
-    const uint32_t item = order[k], cnt = tiles[item];
-    const uint64_t o = off[k];
-    float s[kPairGradStride];
+    const int lane = threadIdx.x & 31;
+    const uint32_t nv = umin(n_items, *n_dev);
+    for (uint32_t k = blockIdx.x * 8 + (threadIdx.x >> 5); k < nv; k += gridDim.x * 8) {
+        const uint32_t item = order[k], cnt = tiles[item];
+        const uint64_t o = off[k];
+        float s[kPairGradStride];
 #pragma unroll
-    for (int q = 0; q < kPairGradStride; ++q) s[q] = 0.f;
-    if (cnt != 0 && o + cnt <= pair_cap)
-        for (uint64_t e = o; e < o + cnt; ++e)
+        for (int q = 0; q < kPairGradStride; ++q) s[q] = 0.f;
+        if (o + cnt <= pair_cap)
+            for (uint64_t e = o + lane; e < o + cnt; e += 32)
 #pragma unroll
-            for (int q = 0; q < kPairGradStride; ++q) s[q] += pairgrad[e * kPairGradStride + q];
+                for (int q = 0; q < kPairGradStride; ++q) s[q] += pairgrad[e * kPairGradStride + q];
+        float v = 0.f;
 #pragma unroll
-    for (int q = 0; q < kPairGradStride; ++q) grad2d[(size_t)item * kGrad2dStride + q] = s[q];
+        for (int q = 0; q < kPairGradStride; ++q) {
+            float t = s[q];
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, d);
+            if (lane == q) v = t;
+        }
+        if (lane < kPairGradStride) grad2d[(size_t)item * kGrad2dStride + lane] = v;
+    }
 }
 
 cudaError_t reduce_pair_grads(gs_ctx* c, cudaStream_t s) {
     const uint32_t items = (uint32_t)c->n_views * (uint32_t)c->n;
     if (c->pairgrad == nullptr || items == 0) return cudaSuccess;
     ++c->launches;
-    k_pairgrad_reduce<<<(items + 255) / 256, 256, 0, s>>>(c->dval[0], c->tiles_touched, c->offsets, items,
+    const int grid = (int)std::min<uint32_t>((items + 7) / 8, (uint32_t)c->num_sms * 8);
+    k_pairgrad_reduce<<<grid, 256, 0, s>>>(c->dval[0], c->tiles_touched, c->offsets, items,
                                                           c->dcount + 8, (uint64_t)c->pair_cap, c->pairgrad,
                                                           c->grad2d);
     return cudaGetLastError();
