@@ -457,6 +457,7 @@ int gs_create(const gs_config* cfg, int device, gs_ctx** out) {
         for (int i = 0; i < 5; ++i)
             ok = ok && cudaEventCreateWithFlags(&c->side_ev[i], cudaEventDisableTiming) == cudaSuccess;
         ok = ok && cudaEventCreateWithFlags(&c->graph_done, cudaEventDisableTiming) == cudaSuccess;
+        ok = ok && cudaEventCreateWithFlags(&c->count_ready, cudaEventDisableTiming) == cudaSuccess;
         ok = ok && cudaStreamCreateWithFlags(&c->copy, cudaStreamNonBlocking) == cudaSuccess;
         for (int i = 0; i < 2; ++i)
             for (cudaEvent_t* ev : {&c->h2d_start[i], &c->h2d_ready[i], &c->h2d_free[i]})
@@ -507,6 +508,7 @@ void gs_destroy(gs_ctx* c) {
     for (int i = 0; i < 5; ++i)
         if (c->side_ev[i]) cudaEventDestroy(c->side_ev[i]);
     if (c->graph_done) cudaEventDestroy(c->graph_done);
+    if (c->count_ready) cudaEventDestroy(c->count_ready);
     if (c->copy) cudaStreamDestroy(c->copy);
     for (int i = 0; i < 2; ++i)
         for (cudaEvent_t ev : {c->h2d_start[i], c->h2d_ready[i], c->h2d_free[i]})
@@ -530,19 +532,7 @@ int gs_set_params(gs_ctx* c, const float* params_dev, int n, void* stream) {
     if (n > c->cap) return fail(c, GS_ERR_CAPACITY, "more Gaussians than the configured capacity");
     cudaStream_t s = (cudaStream_t)stream;
     CK(cudaSetDevice(c->device));
-    if (n > 0)
-        CK(cudaMemcpy2DAsync(c->params, sizeof(float) * c->cap, params_dev, sizeof(float) * n, sizeof(float) * n,
-                             kParamRows, cudaMemcpyDeviceToDevice, s));
-    CK(cudaMemsetAsync(c->adam_m, 0, sizeof(float) * kParamRows * c->cap, s));
-    CK(cudaMemsetAsync(c->adam_v, 0, sizeof(float) * kParamRows * c->cap, s));
-    CK(cudaMemsetAsync(c->dens_sum, 0, sizeof(float) * c->cap, s));
-    CK(cudaMemsetAsync(c->dens_cnt, 0, sizeof(float) * c->cap, s));
-    CK(cudaMemsetAsync(c->dom_cnt, 0, sizeof(uint32_t) * c->cap, s));
-    CK(cudaMemsetAsync(c->dcount + 4, 0, sizeof(uint32_t), s));
-    {
-        static const double pw1[2] = {1.0, 1.0};
-        CK(cudaMemcpyAsync(c->adam_pw, pw1, sizeof(pw1), cudaMemcpyHostToDevice, s));
-    }
+    CK(launch_set_params(c, params_dev, n, s));
     c->n = n;
     c->adam_t = 0;
     c->n_views = 0;
@@ -596,9 +586,20 @@ int gs_render(gs_ctx* c, const gs_camera* cams, int n_views, float* rgb, float* 
         c->n_views = 0;   // no image to take a loss of
         return code;
     }
-    // size the pair buffers: read P back (the one synchronisation of a render)
+    // Read P back (the one wait of a render) while the rest already runs in the pair buffers as they
+    // are, its grids sized by the last render's count; an overflow leaves every bin empty, and the
+    // rest is run again in larger buffers. (A wait before the rest left the GPU idle for the host's
+    // wake-up and launches, some 25 us.)
     CK(cudaMemcpyAsync(c->hcount, c->dcount, sizeof(uint32_t) * 11, cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
+    CK(cudaEventRecord(c->count_ready, s));
+    const uint32_t items = (uint32_t)c->n_views * (uint32_t)c->n;
+    c->pairs_hint = c->pairs_hint ? std::max(c->pairs_hint, items) : items * 4u;   // (sizes grids only)
+    code = back_half(c, k, rgb, argmax, s);
+    CK(cudaEventSynchronize(c->count_ready));
+    if (code != GS_OK) {
+        c->n_views = 0;
+        return code;
+    }
     if ((code = check_nonfinite(c, c->hcount[10], s)) != GS_OK) {
         c->n_views = 0;
         return code;
@@ -608,6 +609,7 @@ int gs_render(gs_ctx* c, const gs_camera* cams, int n_views, float* rgb, float* 
     c->pairs_hint = (uint32_t)std::min<int64_t>(P, 0xFFFFFFFFll);
     if (P > c->pair_cap) {
         drop_graph(c);
+        CK(cudaStreamSynchronize(s));
         if (alloc_pairs(c, std::min<int64_t>(P + P / 2 + 1024, kMaxPairs)) != cudaSuccess) {
             c->n_views = 0;
             return fail(c, GS_ERR_OOM, "growing the pair buffers failed");
@@ -616,10 +618,10 @@ int gs_render(gs_ctx* c, const gs_camera* cams, int n_views, float* rgb, float* 
             c->n_views = 0;
             return fail(c, GS_ERR_CAPACITY, "pair count exceeds 2^32");
         }
-    }
-    if ((code = back_half(c, k, rgb, argmax, s)) != GS_OK) {
-        c->n_views = 0;
-        return code;
+        if ((code = back_half(c, k, rgb, argmax, s)) != GS_OK) {
+            c->n_views = 0;
+            return code;
+        }
     }
     CK(launch_copy_T(c, T, s));
     return GS_OK;
@@ -1380,11 +1382,12 @@ int gs_densify(gs_ctx* c, const float* normals, int* n_split_out, void* stream) 
         std::swap(c->params, c->spare[0]);
         std::swap(c->adam_m, c->spare[1]);
         std::swap(c->adam_v, c->spare[2]);
-        c->n += (int)n_split;
+        c->n += (int)n_split;   // (the scatter cleared the statistics)
+    } else {
+        CK(cudaMemsetAsync(c->dens_sum, 0, sizeof(float) * c->cap, s));
+        CK(cudaMemsetAsync(c->dens_cnt, 0, sizeof(float) * c->cap, s));
+        CK(cudaMemsetAsync(c->dom_cnt, 0, sizeof(uint32_t) * c->cap, s));
     }
-    CK(cudaMemsetAsync(c->dens_sum, 0, sizeof(float) * c->cap, s));
-    CK(cudaMemsetAsync(c->dens_cnt, 0, sizeof(float) * c->cap, s));
-    CK(cudaMemsetAsync(c->dom_cnt, 0, sizeof(uint32_t) * c->cap, s));
     CK(cudaStreamSynchronize(s));
     *n_split_out = (int)n_split;
     invalidate_render(c);

@@ -170,6 +170,7 @@ struct gs_ctx {
                                             // buffer, so that a render of another shape between
                                             // replays (which writes work_order) cannot change it
     cudaEvent_t graph_done = nullptr;       // recorded after each replay
+    cudaEvent_t count_ready = nullptr;      // a render's counts have reached hcount
     bool graph_pending = false;             // a replay's flags have not been checked yet
     uint32_t* hflags = nullptr;             // pinned [16]: dcount[0..10] as the last replay left them
     cudaGraphNode_t cam_node = nullptr;     // kernel node that uploads the cameras
@@ -254,6 +255,8 @@ cudaError_t launch_loss_tail(gs_ctx* c, const DevConst& k, const float* photo_pa
 cudaError_t launch_loss(gs_ctx* c, const DevConst& k, const float* rgb, const float* target, float* loss_out,
                         cudaStream_t s);
 cudaError_t launch_adam(gs_ctx* c, cudaStream_t s);
+// n Gaussians from params [14][n]; moments, step count, powers of beta and statistics reset
+cudaError_t launch_set_params(gs_ctx* c, const float* params, int n, cudaStream_t s);
 // 10 log10(1 / MSE) of img against ref (n floats each) into out[0] (device)
 cudaError_t launch_psnr(gs_ctx* c, const float* img, const float* ref, size_t n, float* out, cudaStream_t s);
 int psnr_scratch_doubles();

@@ -231,16 +231,20 @@ __device__ float normal_at(uint64_t seed, uint64_t counter) {
 }
 
 // Survivors move to pos_s = i - (split parents before i); children of the
-// k-th split parent go to n_surv + 2k and n_surv + 2k + 1.
+// k-th split parent go to n_surv + 2k and n_surv + 2k + 1. The statistics restart.
 __global__ void __launch_bounds__(256) k_split_scatter(const float* __restrict__ P, const float* __restrict__ M,
                                                        const float* __restrict__ V, int n, int cap,
                                                        const uint32_t* __restrict__ flags,
                                                        const uint32_t* __restrict__ pos, uint32_t n_split,
                                                        const float* __restrict__ normals, uint64_t seed,
                                                        float log_factor, float* __restrict__ P2,
-                                                       float* __restrict__ M2, float* __restrict__ V2) {
+                                                       float* __restrict__ M2, float* __restrict__ V2,
+                                                       float* __restrict__ dsum, float* __restrict__ dcnt,
+                                                       uint32_t* __restrict__ dom) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
+    dsum[i] = dcnt[i] = 0.f;   // (beyond n they are zero)
+    dom[i] = 0u;
     uint32_t before = pos[i];
     float p[kParamRows];
     for (int r = 0; r < kParamRows; ++r) p[r] = P[(size_t)r * cap + i];
@@ -371,7 +375,7 @@ cudaError_t launch_split_scatter(gs_ctx* c, const uint32_t* flags, const uint32_
     ++c->launches;
     k_split_scatter<<<(c->n + 255) / 256, 256, 0, s>>>(c->params, c->adam_m, c->adam_v, c->n, c->cap, flags, pos,
                                                        n_split, normals, c->cfg.seed, logf(c->cfg.split_factor), P2,
-                                                       M2, V2);
+                                                       M2, V2, c->dens_sum, c->dens_cnt, c->dom_cnt);
     return cudaGetLastError();
 }
 

@@ -735,12 +735,15 @@ __global__ void __launch_bounds__(256) k_emit(const uint32_t* __restrict__ order
     }
 }
 
+// The sorted pairs' (start, end) per bin. After an overflow of the pair buffer the sorted values hold
+// slots that no item wrote: every bin stays empty then, and nothing is composited.
 __global__ void __launch_bounds__(256) k_ranges(const uint32_t* __restrict__ pkey, const uint32_t* __restrict__ P_dev,
-                                                uint64_t pair_cap, uint32_t n_bins, uint2* __restrict__ ranges) {
+                                                uint64_t pair_cap, uint32_t n_bins, const uint32_t* __restrict__ overflow,
+                                                uint2* __restrict__ ranges) {
+    if (*overflow != 0u) return;
     uint32_t P = (uint32_t)(*P_dev < pair_cap ? *P_dev : pair_cap);
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < P; i += gridDim.x * blockDim.x) {
         uint32_t b = pkey[i];
-        if (b >= n_bins) continue;   // only possible after a pair-buffer overflow
         if (i == 0 || pkey[i - 1] != b) ranges[b].x = i;
         if (i == P - 1 || pkey[i + 1] != b) ranges[b].y = i + 1;
     }
@@ -763,10 +766,11 @@ __device__ __forceinline__ uint32_t order_slot(uint2 r) {
 // one CTA walking such a list would outlast the launch's average (see
 // launch_work_order). One CTA, a counting sort by bucket; items of one bucket
 // come in any order (the compositing result does not depend on which CTA takes
-// an item, nor on whether a tile is halved).
+// an item, nor on whether a tile is halved). A non-zero *cancel leaves the list empty.
 __global__ void __launch_bounds__(1024) k_work_order(const uint2* __restrict__ ranges, uint32_t n_bins,
                                                       uint32_t* __restrict__ order, int halves, uint32_t split_min,
-                                                      uint32_t split_share, const uint32_t* __restrict__ n_pairs) {
+                                                      uint32_t split_share, const uint32_t* __restrict__ n_pairs,
+                                                      const uint32_t* __restrict__ cancel) {
     __shared__ uint32_t cnt[1024];
     __shared__ uint32_t wsum[32];
     const int t = threadIdx.x, lane = t & 31;
@@ -799,7 +803,7 @@ __global__ void __launch_bounds__(1024) k_work_order(const uint2* __restrict__ r
     }
     __syncthreads();
     cnt[t] = x - v + wsum[t >> 5];
-    if (t == 1023) order[0] = x + wsum[31];
+    if (t == 1023) order[0] = cancel != nullptr && *cancel != 0u ? 0u : x + wsum[31];
     __syncthreads();
     for (uint32_t b = t; b < n_bins; b += 1024) {
         const uint2 r = ranges[b];
@@ -942,7 +946,7 @@ cudaError_t compute_ranges(gs_ctx* c, cudaStream_t s) {
     if (!c->side_zeroed) cudaMemsetAsync(c->ranges, 0, sizeof(uint2) * (size_t)c->n_bins, s);
     ++c->launches;
     k_ranges<<<c->num_sms * 8, 256, 0, s>>>(c->pkey[c->pair_buf], c->dcount, (uint64_t)c->pair_cap,
-                                            (uint32_t)c->n_bins, c->ranges);
+                                            (uint32_t)c->n_bins, c->dcount + 1, c->ranges);
     return c->order_ahead ? cudaGetLastError() : launch_work_order(c, s);
 }
 
@@ -959,8 +963,9 @@ cudaError_t launch_work_order(gs_ctx* c, cudaStream_t s) {
     const int halves = c->tile == 16 && c->ppt == 2 && !c->cfg.deterministic;
     const bool all = 2ll * c->n_bins <= 6ll * c->num_sms;
     const uint32_t split_min = all ? 0u : 128u, split_share = all ? 0xFFFFFFFFu : 12u * (uint32_t)c->num_sms;
+    // a render with an unreported non-finite value is not made (a replay's order is for the next one)
     k_work_order<<<1, 1024, 0, s>>>(c->ranges, (uint32_t)c->n_bins, c->work_order, halves, split_min, split_share,
-                                    c->dcount);
+                                    c->dcount, c->order_ahead ? nullptr : c->dcount + 10);
     return cudaGetLastError();
 }
 

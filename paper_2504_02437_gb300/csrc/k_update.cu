@@ -132,6 +132,39 @@ __global__ void __launch_bounds__(256) k_adam(float* __restrict__ P, const float
     if (threadIdx.x == 0) adam_bias_end(st, pw, sbc, spw, gridDim.x);
 }
 
+// The map replaced by n Gaussians in[14][n]: parameters copied, moments and statistics zeroed over the
+// capacity, the Adam state reset, in one launch (one copy, six fills and an upload before). Row 14 of
+// the grid's y is the statistics.
+__global__ void __launch_bounds__(256) k_set_params(const float* __restrict__ in, int n, int cap, float* __restrict__ P,
+                                                    float* __restrict__ M, float* __restrict__ V,
+                                                    float* __restrict__ dsum, float* __restrict__ dcnt,
+                                                    uint32_t* __restrict__ dom, uint32_t* __restrict__ adam_steps,
+                                                    double* __restrict__ pw) {
+    const int row = blockIdx.y;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (row == kParamRows) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            *adam_steps = 0u;
+            pw[0] = pw[1] = 1.0;
+        }
+        for (int j = 4 * (blockIdx.x * 256 + threadIdx.x); j < cap; j += 4 * 256 * gridDim.x) {
+            *reinterpret_cast<float4*>(dsum + j) = zero;
+            *reinterpret_cast<float4*>(dcnt + j) = zero;
+            *reinterpret_cast<uint4*>(dom + j) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        return;
+    }
+    for (int j = 4 * (blockIdx.x * 256 + threadIdx.x); j < cap; j += 4 * 256 * gridDim.x) {
+        const size_t k = (size_t)row * cap + j, i = (size_t)row * n + j;
+        *reinterpret_cast<float4*>(M + k) = zero;
+        *reinterpret_cast<float4*>(V + k) = zero;
+        if (j + 3 < n)
+            *reinterpret_cast<float4*>(P + k) = make_float4(in[i], in[i + 1], in[i + 2], in[i + 3]);
+        else
+            for (int e = 0; j + e < n; ++e) P[k + e] = in[i + e];
+    }
+}
+
 // PSNR of an image against a reference: per-CTA float64 partial sums of the
 // squared differences (fixed grid, fixed order), then one CTA adds the partials
 // in index order and writes 10 log10(1 / max(MSE, 1e-12)).
@@ -226,6 +259,15 @@ cudaError_t launch_adam(gs_ctx* c, cudaStream_t s) {
     const size_t groups = (size_t)kParamRows * ((c->n + 3) / 4);
     const int grid = (int)std::min<size_t>((groups + 255) / 256, (size_t)c->num_sms * 8);
     k_adam<<<grid, 256, 0, s>>>(c->params, c->grads, c->adam_m, c->adam_v, c->n, c->cap, a, c->dcount, c->adam_pw);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_set_params(gs_ctx* c, const float* params, int n, cudaStream_t s) {
+    ++c->launches;
+    const int per_row = std::max(1, std::min((c->cap / 4 + 255) / 256, c->num_sms));   // (cap is a multiple of 4)
+    k_set_params<<<dim3(per_row, kParamRows + 1), 256, 0, s>>>(params, n, c->cap, c->params, c->adam_m, c->adam_v,
+                                                               c->dens_sum, c->dens_cnt, c->dom_cnt, c->dcount + 4,
+                                                               c->adam_pw);
     return cudaGetLastError();
 }
 
