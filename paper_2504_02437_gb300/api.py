@@ -16,16 +16,22 @@ import torch
 from . import _native as N
 
 
-def _stream() -> C.c_void_p:
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+# Small calls are bound by what the host does around them (a step of the learned initialiser runs 30 us
+# on the GPU), so addresses go to the library as plain integers, the stream is taken without building a
+# Stream object, and a camera's rotation is written in one piece.
 
 
-def _ptr(t: Optional[torch.Tensor]) -> Optional[C.c_void_p]:
+def _stream() -> int:
+    """The current stream of the current device."""
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
+def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     if t is None:
         return None
     if not t.is_cuda or not t.is_contiguous():
         raise ValueError("expected a contiguous CUDA tensor")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _hptr(t: Optional[torch.Tensor]) -> Optional[C.c_void_p]:
@@ -53,21 +59,23 @@ def _f32(t: Optional[torch.Tensor], shape: tuple, name: str, host: bool = False)
 def to_gs_camera(cam) -> N.gs_camera:
     """Any object with width, height, fx, fy, cx, cy, R (3x3 world->camera) and t."""
     g = N.gs_camera()
+    _fill_camera(g, cam)
+    return g
+
+
+def _fill_camera(g: N.gs_camera, cam) -> None:
     g.width, g.height = int(cam.width), int(cam.height)
     g.fx, g.fy, g.cx, g.cy = float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy)
-    R = np.asarray(cam.R, dtype=np.float64).reshape(9)
-    t = np.asarray(cam.t, dtype=np.float64).reshape(3)
-    for i in range(9):
-        g.R[i] = float(R[i])
-    for i in range(3):
-        g.t[i] = float(t[i])
-    return g
+    g.R[:] = np.asarray(cam.R, dtype=np.float64).reshape(9).tolist()
+    g.t[:] = np.asarray(cam.t, dtype=np.float64).reshape(3).tolist()
 
 
 def _cams(cams) -> tuple:
     if not isinstance(cams, (list, tuple)):
         cams = [cams]
-    arr = (N.gs_camera * len(cams))(*[to_gs_camera(c) for c in cams])
+    arr = (N.gs_camera * len(cams))()
+    for g, c in zip(arr, cams):
+        _fill_camera(g, c)
     return arr, len(cams), int(cams[0].height), int(cams[0].width)
 
 
@@ -91,6 +99,7 @@ class GaussianMap:
                  device: int = 0, **config):
         self.lib = N.load()
         self.device = device
+        self._dev = torch.device("cuda", device)
         self.cfg = default_config(capacity=capacity, max_views=max_views, max_width=max_width,
                                   max_height=max_height, **config)
         ctx = C.c_void_p()
@@ -134,24 +143,24 @@ class GaussianMap:
         return self.lib.gs_pixels_per_thread(self.ctx)
 
     def set_params(self, params: torch.Tensor):
-        p = params.detach().to(device=f"cuda:{self.device}", dtype=torch.float32).contiguous()
+        p = params.detach().to(device=self._dev, dtype=torch.float32).contiguous()
         if p.dim() != 2 or p.shape[0] != 14:
             raise ValueError("params must be [14, n]")
         self._check(self.lib.gs_set_params(self.ctx, _ptr(p), p.shape[1], _stream()))
 
     def params(self) -> torch.Tensor:
-        out = torch.empty(14, self.n, device=f"cuda:{self.device}", dtype=torch.float32)
+        out = torch.empty(14, self.n, device=self._dev, dtype=torch.float32)
         self._check(self.lib.gs_get_params(self.ctx, _ptr(out), _stream()))
         return out
 
     def grads(self) -> torch.Tensor:
-        out = torch.empty(14, self.n, device=f"cuda:{self.device}", dtype=torch.float32)
+        out = torch.empty(14, self.n, device=self._dev, dtype=torch.float32)
         self._check(self.lib.gs_get_grads(self.ctx, _ptr(out), _stream()))
         return out
 
     def set_grads(self, grads: torch.Tensor):
         """The gradient the next step() applies ([14, n]), e.g. of a loss computed outside."""
-        g = grads.detach().to(device=f"cuda:{self.device}", dtype=torch.float32).contiguous()
+        g = grads.detach().to(device=self._dev, dtype=torch.float32).contiguous()
         if tuple(g.shape) != (14, self.n):
             raise ValueError("grads must be [14, n]")
         self._check(self.lib.gs_set_grads(self.ctx, _ptr(g), _stream()))
@@ -165,7 +174,7 @@ class GaussianMap:
     # ---- the mapping step
     def render(self, cams, want_T: bool = False, want_argmax: bool = False):
         arr, V, H, W = _cams(cams)
-        dev = f"cuda:{self.device}"
+        dev = self._dev
         rgb = torch.empty(V, 3, H, W, device=dev, dtype=torch.float32)
         T = torch.empty(V, H, W, device=dev, dtype=torch.float32) if want_T else None
         am = torch.empty(V, H, W, device=dev, dtype=torch.int32) if want_argmax else None
@@ -181,7 +190,7 @@ class GaussianMap:
 
     def loss(self, target: torch.Tensor) -> torch.Tensor:
         tg = target.to(torch.float32).contiguous()
-        out = torch.empty(3, device=f"cuda:{self.device}", dtype=torch.float32)
+        out = torch.empty(3, device=self._dev, dtype=torch.float32)
         self._check(self.lib.gs_loss(self.ctx, _ptr(tg), _ptr(out), _stream()))
         return out
 
@@ -196,7 +205,7 @@ class GaussianMap:
                 rgb_out: Optional[torch.Tensor] = None) -> torch.Tensor:
         arr, V, H, W = _cams(cams)
         if loss_out is None:
-            loss_out = torch.empty(3, device=f"cuda:{self.device}", dtype=torch.float32)
+            loss_out = torch.empty(3, device=self._dev, dtype=torch.float32)
         target = _f32(target, (V, 3, H, W), "target")
         _f32(loss_out, (3,), "loss_out")
         _f32(rgb_out, (V, 3, H, W), "rgb_out")
@@ -258,7 +267,7 @@ class GaussianMap:
     def mlp_targets(self, first: int, count: int) -> torch.Tensor:
         """Learned-initialiser training targets [count, 16] of Gaussians first .. first + count - 1
         (log-scale, unit quaternion with w >= 0, opacity logit, colour, zeros)."""
-        out = torch.empty(count, 16, device=f"cuda:{self.device}", dtype=torch.float32)
+        out = torch.empty(count, 16, device=self._dev, dtype=torch.float32)
         self._check(self.lib.gs_mlp_targets(self.ctx, int(first), int(count), _ptr(out), _stream()))
         return out
 
@@ -268,7 +277,7 @@ class GaussianMap:
         a = _f32(img, tuple(img.shape), "img")
         b = _f32(ref, tuple(img.shape), "ref")
         if out is None:
-            out = torch.empty((), device=f"cuda:{self.device}", dtype=torch.float32)
+            out = torch.empty((), device=self._dev, dtype=torch.float32)
         self._check(self.lib.gs_psnr(self.ctx, _ptr(a), _ptr(b), a.numel(), _ptr(out), _stream()))
         return out
 
@@ -344,6 +353,7 @@ class MLP:
     def __init__(self, seed: int = 0, device: int = 0):
         self.lib = N.load()
         self.device = device
+        self._device = torch.device("cuda", device)
         h = C.c_void_p()
         with torch.cuda.device(device):
             N.check(self.lib.gs_mlp_create(device, seed, C.byref(h)))
@@ -362,7 +372,7 @@ class MLP:
             pass
 
     def _dev(self):
-        return f"cuda:{self.device}"
+        return self._device
 
     def set_params(self, flat: torch.Tensor):
         f = flat.to(device=self._dev(), dtype=torch.float32).contiguous()
