@@ -400,7 +400,7 @@ int gs_create(const gs_config* cfg, int device, gs_ctx** out) {
         if (c->num_sms <= 0) c->num_sms = 1;
         e = sort_kernels_init();
         if (e != cudaSuccess) { code = fail(c, GS_ERR_CUDA, "kernel attributes", e); break; }
-        c->sort_blocks = c->num_sms * 4;
+        c->sort_blocks = std::min(c->num_sms * 4, sort_max_blocks());
         c->n_partials = 2 * c->num_sms * 2;
         const size_t cap = (size_t)c->cap, V = (size_t)cfg->max_views;
         const size_t maxpix = (size_t)cfg->max_width * cfg->max_height;

@@ -234,6 +234,7 @@ cudaError_t sort_depth(gs_ctx* c, uint32_t n_max, uint32_t n_hint, cudaStream_t 
 bool depth_sort_small(const gs_ctx* c);    // the map is small enough for the one-CTA depth sort
 cudaError_t sort_kernels_init();           // once per context, on its device
 size_t sort_hist_words(int sort_blocks);
+int sort_max_blocks();
 cudaError_t emit_pairs(gs_ctx* c, uint32_t n_items, const uint32_t* n_dev, cudaStream_t s);
 // exclusive scan of n u32 values (in may equal out); the total goes to *total_dev
 cudaError_t scan_u32(gs_ctx* c, const uint32_t* in, uint32_t* out, uint32_t n, uint32_t* total_dev, cudaStream_t s);

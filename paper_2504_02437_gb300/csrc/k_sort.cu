@@ -106,9 +106,10 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint32_t* __r
     }
 }
 
-// Of more than kScanGrid blocks: the rows' exclusive scan over the blocks, in place, and each digit's
-// total. A CTA takes eight digits, 32 threads each.
-constexpr int kScanGrid = 128;
+// Of more than kScanGrid blocks (at most kMaxGrid): the rows' exclusive scan over the blocks, in place,
+// and each digit's total. A CTA takes eight digits, 32 threads each; a thread's rows are loaded
+// together and stay in registers.
+constexpr int kScanGrid = 128, kScanRows = 20, kMaxGrid = 32 * kScanRows;
 __global__ void __launch_bounds__(256) k_digit_scan(uint32_t* __restrict__ hist, int G, DigitSpec spec,
                                                     uint32_t* __restrict__ dtot) {
     __shared__ uint32_t part[32][8];
@@ -116,31 +117,28 @@ __global__ void __launch_bounds__(256) k_digit_scan(uint32_t* __restrict__ hist,
     const int c = threadIdx.x & 7, g = threadIdx.x >> 3;
     const int d = blockIdx.x * 8 + c, ndig = 1 << dig.nbits;
     if (blockIdx.x * 8 >= ndig) return;   // the whole CTA (the grid is for the widest digit)
-    const int chunk = (G + 31) / 32, r0 = g * chunk, r1 = min(G, r0 + chunk);
-    uint32_t* col = hist + d;
-    uint32_t sum = 0;
-    if (d < ndig) {
-#pragma unroll 8
-        for (int r = r0; r < r1; ++r) sum += col[(size_t)r << dig.nbits];
-    }
+    const int chunk = (G + 31) / 32, r0 = g * chunk, rows = d < ndig ? min(chunk, G - r0) : 0;
+    uint32_t* col = hist + ((size_t)r0 << dig.nbits) + d;
+    uint32_t v[kScanRows], sum = 0;
+#pragma unroll
+    for (int r = 0; r < kScanRows; ++r) v[r] = r < rows ? col[(size_t)r << dig.nbits] : 0u;
+#pragma unroll
+    for (int r = 0; r < kScanRows; ++r) sum += v[r];
     part[g][c] = sum;
     __syncthreads();
     uint32_t run = 0, all = 0;
 #pragma unroll
     for (int q = 0; q < 32; ++q) {
-        const uint32_t v = part[q][c];
-        run += q < g ? v : 0u;
-        all += v;
+        const uint32_t x = part[q][c];
+        run += q < g ? x : 0u;
+        all += x;
     }
-    if (d < ndig) {
-#pragma unroll 8
-        for (int r = r0; r < r1; ++r) {
-            const uint32_t v = col[(size_t)r << dig.nbits];
-            col[(size_t)r << dig.nbits] = run;
-            run += v;
-        }
-        if (g == 0) dtot[d] = all;
+#pragma unroll
+    for (int r = 0; r < kScanRows; ++r) {
+        if (r < rows) col[(size_t)r << dig.nbits] = run;
+        run += v[r];
     }
+    if (g == 0 && d < ndig) dtot[d] = all;
 }
 
 // Stable scatter of one digit pass. Up to kScanGrid blocks the block first adds the digit counts of
@@ -201,15 +199,16 @@ __global__ void __launch_bounds__(kSortThreads, MAXBITS <= 8 ? 5 : 3) k_radix_sc
         for (int c = t % min(cols, kSortThreads); c < cols; c += kSortThreads) {
             uint4 bef = make_uint4(0, 0, 0, 0), tot = bef;
             const uint4* row = reinterpret_cast<const uint4*>(hist) + c;
-            for (int r0 = t / min(cols, kSortThreads); r0 < G; r0 += 8 * groups) {
-                uint4 v[8];
+            constexpr int R = MAXBITS <= 8 ? 8 : 16;   // rows in flight
+            for (int r0 = t / min(cols, kSortThreads); r0 < G; r0 += R * groups) {
+                uint4 v[R];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
+                for (int u = 0; u < R; ++u) {
                     const int r = r0 + u * groups;
                     v[u] = r < G ? row[(size_t)r * cols] : make_uint4(0, 0, 0, 0);
                 }
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
+                for (int u = 0; u < R; ++u) {
                     const bool before = r0 + u * groups < b;
                     tot.x += v[u].x;
                     tot.y += v[u].y;
@@ -827,6 +826,7 @@ cudaError_t sort_kernels_init() {
     return e;
 }
 
+int sort_max_blocks() { return kMaxGrid; }
 size_t sort_hist_words(int sort_blocks) { return ((size_t)sort_blocks << 11) + (1u << 11); }
 static uint32_t* sort_totals(const gs_ctx* c) { return c->hist + ((size_t)c->sort_blocks << 11); }
 
@@ -983,6 +983,7 @@ namespace {
 
 constexpr uint32_t kStaticSortMaxPairs = 1u << 20;                       // largest n accepted
 constexpr int kStaticSortMaxBlocks = (int)((kStaticSortMaxPairs + 4095u) / 4096u);
+static_assert(kStaticSortMaxBlocks <= kMaxGrid, "blocks that the digit scan takes");
 constexpr size_t kStaticSortWords = 64                                  // [0] count sentinel
                                     + 2 * (size_t)kStaticSortMaxPairs    // ping-pong keys and values
                                     + 256 * (size_t)kStaticSortMaxBlocks + 256;   // histograms, digit totals
