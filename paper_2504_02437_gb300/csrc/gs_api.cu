@@ -1301,28 +1301,39 @@ int gs_insert(gs_ctx* c, const gs_camera* cam, const float* image, const float* 
     const size_t HW = (size_t)cam->width * cam->height, np = (size_t)n;
     if (!camera_ok(*cam, c->cfg)) return fail(c, GS_ERR_ARG, "invalid camera");
     const size_t n_part = knn_scratch(c, n, c->n), n_feat = c->init_mlp ? 80 * np : 0;
+    const size_t bins = ((size_t)cam->width + 7) / 8 * (((size_t)cam->height + 7) / 8);   // of the smallest tiles
     Scratch t(c);
     t.add<float>(3 * HW);
     t.add<float>(kParamRows * np);
     t.add<uint32_t>(np);
     t.add<float>(n_part);
     t.add<float>(n_feat);
+    t.add<int>(np);
+    t.add<uint32_t>(2 * bins);
     if (!t.reserve()) return fail(c, GS_ERR_OOM, "temporary buffers");
     float* img = t.take<float>(3 * HW);
     float* stage = t.take<float>(kParamRows * np);
     uint32_t* keep = t.take<uint32_t>(np);
     float* part = t.take<float>(n_part);
     float* feat = t.take<float>(n_feat);
+    PointItems points{pts, n, nullptr, nullptr};
+    points.pixel = t.take<int>(np);
+    points.flags = t.take<uint32_t>(2 * bins);
+    const bool gate = !(c->cfg.insert_tau > 0.f) && c->n > 0;
     if (c->cfg.insert_tau > 0.f) {
         // distance rule: no render, only the camera (pixel colours of the plain initialisation)
         CamBatch b;
         const int code = prepare_views(c, cam, 1, b);
         if (code != GS_OK) return code;
     } else {
+        c->points = gate ? &points : nullptr;
         const int code = gs_render(c, cam, 1, img, nullptr, nullptr, stream);
+        c->points = nullptr;
         if (code != GS_OK) return code;
     }
-    CK(launch_insert_test(c, c->hcam[0], pts, n, image, part, keep, stage, s));
+    c->n_views = 0;   // no whole image to take a loss of
+    if (!gate) CK(launch_point_items(c, points, false, s));
+    CK(launch_insert_test(c, points, image, part, keep, stage, s));
     if (c->init_mlp) CK(mlp_initialise(c->init_mlp, c->hcam[0], image, pts, n, stage, feat, s));
     CK(launch_append(c, stage, n, keep, inserted_dev, c->hcount + 5, s));
     CK(cudaStreamSynchronize(s));

@@ -28,6 +28,14 @@ constexpr int kItemShift = 30;
 constexpr uint32_t kItemBin = (1u << kItemShift) - 1u;
 constexpr size_t work_order_words(int n_bins) { return 1 + 2 * (size_t)n_bins; }
 
+// The points of an insertion: an opacity gate's render composites the tiles that hold one.
+struct PointItems {
+    const float* pts;    // [n][3]
+    int n;
+    int* pixel;          // [n] pixel each projects to, -1 for none
+    uint32_t* flags;     // [2 bins] scratch
+};
+
 // Camera as the kernels read it (one per view, in device memory).
 struct DevCamera {
     float R[9];
@@ -166,6 +174,7 @@ struct gs_ctx {
     // a replayed iteration composites in the longest-first order the previous one left (any order of
     // the same bins gives the same result) and writes the next one, on `side`, once it has composited
     bool order_ahead = false;
+    const gs::PointItems* points = nullptr; // set while an insertion renders
     uint32_t* work_order_graph = nullptr;   // [work_order_words(max bins)] the order a replay composites in: its own
                                             // buffer, so that a render of another shape between
                                             // replays (which writes work_order) cannot change it
@@ -241,6 +250,8 @@ cudaError_t scan_u32(gs_ctx* c, const uint32_t* in, uint32_t* out, uint32_t n, u
 cudaError_t compute_ranges(gs_ctx* c, cudaStream_t s);
 // the compositing kernels' work list, from the bin ranges
 cudaError_t launch_work_order(gs_ctx* c, cudaStream_t s);
+// work items may be half tiles (16 x 2 layout)
+inline bool half_tiles(const gs_ctx* c) { return c->tile == 16 && c->ppt == 2 && !c->cfg.deterministic; }
 // deterministic mode: per-item fixed-order sum of the pair gradient slots into grad2d
 cudaError_t reduce_pair_grads(gs_ctx* c, cudaStream_t s);
 cudaError_t launch_raster_forward(gs_ctx* c, const DevConst& k, float* rgb, int32_t* argmax, cudaStream_t s);
@@ -317,8 +328,10 @@ cudaError_t launch_init_points(gs_ctx* c, const float* pts, const float* rgb, in
                                int n_ref, int ref_is_self, float* part, float* out_params, int out_stride,
                                cudaStream_t s);
 cudaError_t launch_points_planar(const float* pts, int n, float* out, cudaStream_t s);
-cudaError_t launch_insert_test(gs_ctx* c, const DevCamera& cam, const float* pts, int n, const float* image,
-                               float* part, uint32_t* keep, float* stage, cudaStream_t s);
+// the points' pixels in the prepared view, and (list) the work list of the tiles that hold one
+cudaError_t launch_point_items(gs_ctx* c, const PointItems& p, bool list, cudaStream_t s);
+cudaError_t launch_insert_test(gs_ctx* c, const PointItems& p, const float* image, float* part, uint32_t* keep,
+                               float* stage, cudaStream_t s);
 cudaError_t launch_append(gs_ctx* c, const float* stage, int n_stage, const uint32_t* keep, uint8_t* mask,
                           uint32_t* count_host, cudaStream_t s);
 cudaError_t launch_count_dominant(gs_ctx* c, const int32_t* argmax, size_t n_pix, cudaStream_t s);

@@ -114,13 +114,47 @@ __global__ void __launch_bounds__(256) k_init_points(const float* __restrict__ p
     }
 }
 
+// The pixel each point projects to, in front of the camera (-1: none), and with `order` the work list of
+// the tiles (or, with `halves`, half tiles) that hold one of them: an insertion's opacity gate reads the
+// transmittance at those pixels alone, so nothing else is composited. flags: two zeroed words a bin. A
+// non-zero *cancel leaves the list empty. One CTA.
+__global__ void __launch_bounds__(1024) k_point_items(DevCamera cam, float near_z, const float* __restrict__ pts, int n,
+                                                      int tile, int halves, int* __restrict__ pixel,
+                                                      uint32_t* __restrict__ flags, uint32_t* __restrict__ order,
+                                                      const uint32_t* __restrict__ cancel) {
+    __shared__ uint32_t count;
+    if (threadIdx.x == 0) count = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += 1024) {
+        const float x = pts[3 * (size_t)i], y = pts[3 * (size_t)i + 1], z = pts[3 * (size_t)i + 2];
+        const float tx = cam.R[0] * x + cam.R[1] * y + cam.R[2] * z + cam.t[0];
+        const float ty = cam.R[3] * x + cam.R[4] * y + cam.R[5] * z + cam.t[1];
+        const float tz = cam.R[6] * x + cam.R[7] * y + cam.R[8] * z + cam.t[2];
+        const bool front = tz > near_z;
+        const float zz = front ? tz : 1.f;
+        const float u = cam.fx * tx / zz + cam.cx, v = cam.fy * ty / zz + cam.cy;
+        const float pxf = floorf(u + 0.5f), pyf = floorf(v + 0.5f);
+        const bool inside = front && pxf >= 0.f && pxf < (float)cam.width && pyf >= 0.f && pyf < (float)cam.height;
+        const int px = inside ? (int)pxf : 0, py = inside ? (int)pyf : 0;
+        pixel[i] = inside ? py * cam.width + px : -1;
+        if (order != nullptr && inside) {
+            const uint32_t bin = (uint32_t)((py / tile) * cam.tiles_x + px / tile);
+            const uint32_t half = halves ? (uint32_t)(py % tile) / (uint32_t)(tile / 2) : 0u;
+            if (atomicExch(flags + 2 * (size_t)bin + half, 1u) == 0u)
+                order[1 + atomicAdd(&count, 1u)] = halves ? bin | ((1u + half) << kItemShift) : bin;
+        }
+    }
+    __syncthreads();
+    if (order != nullptr && threadIdx.x == 0) order[0] = *cancel != 0u ? 0u : count;
+}
+
 // Insertion test of point i (a warp). Opacity gate (tau2 = 0): keep[i] = 0 iff the point
 // projects, in front of the camera, to a pixel whose rendered opacity 1 - T
 // exceeds the threshold. Distance rule (tau2 = tau^2 > 0, Eq. 7 as its text
 // states it): keep[i] = 1 iff the nearest existing mean is farther than tau
 // (T is not read). Also stages the plain initial parameters [14][n].
-__global__ void __launch_bounds__(256) k_insert_test(DevCamera cam, float near_z, float thresh, float tau2,
-                                                     const float* __restrict__ pts, const float* __restrict__ T,
+__global__ void __launch_bounds__(256) k_insert_test(size_t HW, float thresh, float tau2, const float* __restrict__ pts,
+                                                     const int* __restrict__ pixel, const float* __restrict__ T,
                                                      const float* __restrict__ image, const float* __restrict__ part,
                                                      int chunks, uint32_t* __restrict__ keep,
                                                      float* __restrict__ stage, int n) {
@@ -129,21 +163,13 @@ __global__ void __launch_bounds__(256) k_insert_test(DevCamera cam, float near_z
     const Best3 best = knn_of(part, chunks, n, i);
     if ((threadIdx.x & 31) != 0) return;
     const float rms = best.rms(), dmin2 = best.b0;
-    float x = pts[3 * (size_t)i], y = pts[3 * (size_t)i + 1], z = pts[3 * (size_t)i + 2];
-    float tx = cam.R[0] * x + cam.R[1] * y + cam.R[2] * z + cam.t[0];
-    float ty = cam.R[3] * x + cam.R[4] * y + cam.R[5] * z + cam.t[1];
-    float tz = cam.R[6] * x + cam.R[7] * y + cam.R[8] * z + cam.t[2];
-    bool front = tz > near_z;
-    float zz = front ? tz : 1.f;
-    float u = cam.fx * tx / zz + cam.cx, v = cam.fy * ty / zz + cam.cy;
-    float pxf = floorf(u + 0.5f), pyf = floorf(v + 0.5f);
-    bool inside = front && pxf >= 0.f && pxf < (float)cam.width && pyf >= 0.f && pyf < (float)cam.height;
-    int px = inside ? (int)pxf : 0, py = inside ? (int)pyf : 0;
-    size_t HW = (size_t)cam.width * cam.height, pix = (size_t)py * cam.width + px;
+    const bool inside = pixel[i] >= 0;
+    const size_t pix = inside ? (size_t)pixel[i] : 0;
     bool skip = tau2 > 0.f ? !(dmin2 > tau2) : (inside && (1.f - T[pix]) > thresh);
     keep[i] = skip ? 0u : 1u;
     float ls = fminf(fmaxf(logf(fmaxf(rms, 1e-30f)), -7.f), -1.f);
-    const float vals[kParamRows] = {x, y, z, ls, ls, ls, 1.f, 0.f, 0.f, 0.f, 0.f,
+    const float vals[kParamRows] = {pts[3 * (size_t)i], pts[3 * (size_t)i + 1], pts[3 * (size_t)i + 2],
+                                    ls, ls, ls, 1.f, 0.f, 0.f, 0.f, 0.f,
                                     image[pix], image[HW + pix], image[2 * HW + pix]};
     for (int r = 0; r < kParamRows; ++r) stage[(size_t)r * n + i] = vals[r];
 }
@@ -331,16 +357,27 @@ cudaError_t launch_points_planar(const float* pts, int n, float* out, cudaStream
     return cudaGetLastError();
 }
 
-cudaError_t launch_insert_test(gs_ctx* c, const DevCamera& cam, const float* pts, int n, const float* image,
-                               float* part, uint32_t* keep, float* stage, cudaStream_t s) {
-    if (n == 0) return cudaSuccess;
+cudaError_t launch_point_items(gs_ctx* c, const PointItems& p, bool list, cudaStream_t s) {
+    if (list) {
+        const cudaError_t e = cudaMemsetAsync(p.flags, 0, sizeof(uint32_t) * 2 * (size_t)c->n_bins, s);
+        if (e != cudaSuccess) return e;
+    }
+    ++c->launches;
+    k_point_items<<<1, 1024, 0, s>>>(c->hcam[0], c->cfg.near_z, p.pts, p.n, c->tile, half_tiles(c) ? 1 : 0, p.pixel,
+                                     p.flags, list ? c->work_order : nullptr, c->dcount + 10);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_insert_test(gs_ctx* c, const PointItems& p, const float* image, float* part, uint32_t* keep,
+                               float* stage, cudaStream_t s) {
+    if (p.n == 0) return cudaSuccess;
     int chunks = 0;
-    const cudaError_t e = knn(c, pts, n, c->params, c->cap, c->n, 0, part, &chunks, s);
+    const cudaError_t e = knn(c, p.pts, p.n, c->params, c->cap, c->n, 0, part, &chunks, s);
     if (e != cudaSuccess) return e;
     ++c->launches;
     const float tau2 = c->cfg.insert_tau > 0.f ? c->cfg.insert_tau * c->cfg.insert_tau : 0.f;
-    k_insert_test<<<(n + 7) / 8, 256, 0, s>>>(cam, c->cfg.near_z, c->cfg.insert_opacity, tau2, pts, c->T_final, image,
-                                              part, chunks, keep, stage, n);
+    k_insert_test<<<(p.n + 7) / 8, 256, 0, s>>>((size_t)c->width * c->height, c->cfg.insert_opacity, tau2, p.pts, p.pixel,
+                                                c->T_final, image, part, chunks, keep, stage, p.n);
     return cudaGetLastError();
 }
 

@@ -947,6 +947,7 @@ cudaError_t compute_ranges(gs_ctx* c, cudaStream_t s) {
     ++c->launches;
     k_ranges<<<c->num_sms * 8, 256, 0, s>>>(c->pkey[c->pair_buf], c->dcount, (uint64_t)c->pair_cap,
                                             (uint32_t)c->n_bins, c->dcount + 1, c->ranges);
+    if (c->points != nullptr) return launch_point_items(c, *c->points, true, s);
     return c->order_ahead ? cudaGetLastError() : launch_work_order(c, s);
 }
 
@@ -960,7 +961,7 @@ cudaError_t launch_work_order(gs_ctx* c, cudaStream_t s) {
     // and 18 an SM: 1200x680 keyframe with 300k 372, 341, 320 us and 527 without halves; one with
     // lists of similar length 337, 343, 354 us; 8 x 640x480 window 782, 785, 797 us). Bins of 128
     // pairs or less take a CTA no longer than the launch's other latencies.
-    const int halves = c->tile == 16 && c->ppt == 2 && !c->cfg.deterministic;
+    const int halves = half_tiles(c) ? 1 : 0;
     const bool all = 2ll * c->n_bins <= 6ll * c->num_sms;
     const uint32_t split_min = all ? 0u : 128u, split_share = all ? 0xFFFFFFFFu : 12u * (uint32_t)c->num_sms;
     // a render with an unreported non-finite value is not made (a replay's order is for the next one)

@@ -70,3 +70,32 @@ def test_a_second_split_uses_the_buffers_of_the_first():
             m.count_dominant(cam)
         assert gm.densify(nz) == fresh.densify(nz) > 0
         assert torch.equal(gm.params(), fresh.params())
+
+
+@pytest.mark.parametrize("size", [(160, 120), (490, 277)])
+@pytest.mark.parametrize("cfg", [dict(), dict(tile_size=16, pixels_per_thread=1), dict(tile_size=16, pixels_per_thread=4),
+                                 dict(tile_size=8, pixels_per_thread=1), dict(deterministic=1), dict(pair_capacity=64)])
+def test_gate_is_that_of_the_whole_render(size, cfg):
+    """The opacity gate composites only the tiles that hold a point: its decisions are those of the
+    transmittance of a whole render, away from pixel borders and the threshold."""
+    w, h = size
+    p, cam = frustum_scene(n=3000, width=w, height=h, fx=150, fy=150, cx=w / 2, cy=h / 2, seed=3, opacity_mean=2.0)
+    n = 700
+    rng = np.random.default_rng(5)
+    z = rng.uniform(0.5, 4, n)
+    px, py = rng.integers(-5, w + 5, n), rng.integers(-5, h + 5, n)
+    pts = np.stack([(px + 0.1 - w / 2) * z / 150, (py - 0.1 - h / 2) * z / 150, z], 1).astype(np.float32)
+    gm = new_map(3000 + n, W=w, H=h, **cfg)
+    gm.set_params(cuda(p))
+    T = gm.render(cam, want_T=True)[1][0].cpu().numpy()
+    inside = (px >= 0) & (px < w) & (py >= 0) & (py < h)
+    opac = np.where(inside, 1.0 - T[np.clip(py, 0, h - 1), np.clip(px, 0, w - 1)], 0.0)
+    thresh = 0.9
+    gm2 = new_map(3000 + n, W=w, H=h, insert_opacity=thresh, **cfg)
+    gm2.set_params(cuda(p))
+    count, mask = gm2.insert(cam, torch.zeros(3, h, w, device="cuda"), cuda(pts), return_mask=True)
+    sure = np.abs(opac - thresh) > 1e-6
+    want = ~(inside & (opac > thresh))
+    assert 20 < (~want).sum() and want.sum() > 20
+    np.testing.assert_array_equal(mask.cpu().numpy()[sure], want[sure])
+    assert count == int(mask.sum())
