@@ -34,11 +34,15 @@ struct CamBatch {
     DevCamera cam[GS_MAX_VIEWS];
     int n;
     const float* target;   // the iteration's target image (read through the context's target slot)
+    uint32_t fresh;        // other cameras than the last iteration's
 };
 
-__global__ void k_set_cams(CamBatch b, DevCamera* dst, const float** target_slot) {
+__global__ void k_set_cams(CamBatch b, DevCamera* dst, const float** target_slot, uint32_t* fresh) {
     int i = threadIdx.x;
-    if (i == 0 && target_slot != nullptr) *target_slot = b.target;
+    if (i == 0) {
+        *target_slot = b.target;
+        *fresh = b.fresh;
+    }
     if (i < b.n) dst[i] = b.cam[i];
 }
 
@@ -205,7 +209,7 @@ int setup_views(gs_ctx* c, const gs_camera* cams, int n_views, cudaStream_t s) {
     int code = prepare_views(c, cams, n_views, b);
     if (code != GS_OK) return code;
     ++c->launches;
-    k_set_cams<<<1, 32, 0, s>>>(b, c->dcam, c->target_slot);
+    k_set_cams<<<1, 32, 0, s>>>(b, c->dcam, c->target_slot, c->dcount + 13);
     CK(cudaGetLastError());
     return GS_OK;
 }
@@ -850,8 +854,11 @@ static int iterate_core(gs_ctx* c, const gs_camera* cams, int n_views, const flo
         // replay: new cameras go in as the upload kernel's parameters
         DevCamera* dst = c->dcam;
         const float** slot = c->target_slot;
+        uint32_t* fresh = c->dcount + 13;
         b.target = target;   // the graph reads the target through the slot: any buffer per call
-        void* args[3] = {&b, &dst, &slot};
+        b.fresh = memcmp(c->graph_cam, b.cam, sizeof(DevCamera) * n_views) != 0 ? 1u : 0u;
+        memcpy(c->graph_cam, b.cam, sizeof(DevCamera) * n_views);
+        void* args[4] = {&b, &dst, &slot, &fresh};
         cudaKernelNodeParams kp = {};
         kp.func = (void*)k_set_cams;
         kp.gridDim = dim3(1);
@@ -892,7 +899,7 @@ static int iterate_core(gs_ctx* c, const gs_camera* cams, int n_views, const flo
     c->loss_ready = c->backward_ready = false;
     b.target = target;
     ++c->launches;
-    k_set_cams<<<1, 32, 0, s>>>(b, c->dcam, c->target_slot);
+    k_set_cams<<<1, 32, 0, s>>>(b, c->dcam, c->target_slot, c->dcount + 13);
     CK(cudaGetLastError());
     auto direct = [&]() -> int {
         int cd;
@@ -930,7 +937,7 @@ static int iterate_core(gs_ctx* c, const gs_camera* cams, int n_views, const flo
     int cc = GS_OK;
     {
         ++c->launches;
-        k_set_cams<<<1, 32, 0, cs>>>(b, c->dcam, c->target_slot);
+        k_set_cams<<<1, 32, 0, cs>>>(b, c->dcam, c->target_slot, c->dcount + 13);
         cc = side_begin(c, cs);
         // the direct call above left this shape's work order in work_order_graph for the first
         // replay; every replay reads that buffer and writes the next order into it
@@ -985,6 +992,7 @@ static int iterate_core(gs_ctx* c, const gs_camera* cams, int n_views, const flo
         return fail(c, GS_ERR_CUDA, "instantiating the mapping iteration graph failed", e);
     }
     c->graph_src = g;
+    memcpy(c->graph_cam, b.cam, sizeof(DevCamera) * n_views);
     c->graph_views = n_views;
     c->graph_w = cams[0].width;
     c->graph_h = cams[0].height;

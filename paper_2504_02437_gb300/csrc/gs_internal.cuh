@@ -140,7 +140,8 @@ struct gs_ctx {
                                             // [6], [7] work queues, [8] visible (view, Gaussian) items,
                                             // [10] a non-finite loss or gradient was seen (sticky until
                                             // a call reports it), [11], [12] smallest and largest visible
-                                            // depth key
+                                            // depth key, [13] the replay's cameras are not those of
+                                            // the one before, [14] ticket of its bin ranges
     uint32_t* vis_blocks = nullptr;         // visible items per preprocess CTA
     uint2* vis_range = nullptr;             // smallest and largest visible depth key per preprocess CTA
     uint32_t* tile_blocks = nullptr;        // tiles touched per 256 items of the depth order
@@ -171,8 +172,9 @@ struct gs_ctx {
     cudaEvent_t side_ev[5] = {};            // fork, overflow flag + ranges zeroed, grad2d zeroed,
                                             // second fork, side work done
     bool side_zeroed = false;               // this iteration's zeroing was issued on `side`
-    // a replayed iteration composites in the longest-first order the previous one left (any order of
-    // the same bins gives the same result) and writes the next one, on `side`, once it has composited
+    // a replayed iteration of the same cameras composites in the longest-first order the previous one
+    // left (any order of the same bins gives the same result); each writes the next one, on `side`,
+    // once it has composited, and one of other cameras its own before
     bool order_ahead = false;
     const gs::PointItems* points = nullptr; // set while an insertion renders
     uint32_t* work_order_graph = nullptr;   // [work_order_words(max bins)] the order a replay composites in: its own
@@ -183,6 +185,7 @@ struct gs_ctx {
     bool graph_pending = false;             // a replay's flags have not been checked yet
     uint32_t* hflags = nullptr;             // pinned [16]: dcount[0..10] as the last replay left them
     cudaGraphNode_t cam_node = nullptr;     // kernel node that uploads the cameras
+    gs::DevCamera graph_cam[GS_MAX_VIEWS];  // the cameras of the last iteration of the graph's shape
     int64_t graph_kernels = 0;              // kernels per replay
     bool capturing = false;
     struct CapPhase {

@@ -734,20 +734,6 @@ __global__ void __launch_bounds__(256) k_emit(const uint32_t* __restrict__ order
     }
 }
 
-// The sorted pairs' (start, end) per bin. After an overflow of the pair buffer the sorted values hold
-// slots that no item wrote: every bin stays empty then, and nothing is composited.
-__global__ void __launch_bounds__(256) k_ranges(const uint32_t* __restrict__ pkey, const uint32_t* __restrict__ P_dev,
-                                                uint64_t pair_cap, uint32_t n_bins, const uint32_t* __restrict__ overflow,
-                                                uint2* __restrict__ ranges) {
-    if (*overflow != 0u) return;
-    uint32_t P = (uint32_t)(*P_dev < pair_cap ? *P_dev : pair_cap);
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < P; i += gridDim.x * blockDim.x) {
-        uint32_t b = pkey[i];
-        if (i == 0 || pkey[i - 1] != b) ranges[b].x = i;
-        if (i == P - 1 || pkey[i + 1] != b) ranges[b].y = i + 1;
-    }
-}
-
 // Bucket of a bin in the longest-first work order: 1023 - key, where the key
 // grows with the bin's pair count (steps of 2 pairs below 1,024 pairs, of 16
 // up to 9,200, one bucket above).
@@ -763,49 +749,66 @@ __device__ __forceinline__ uint32_t order_slot(uint2 r) {
 // late. With `halves` a bin of more than split_min pairs and more than
 // 1 / split_share of all pairs becomes two items, its upper and lower half:
 // one CTA walking such a list would outlast the launch's average (see
-// launch_work_order). One CTA, a counting sort by bucket; items of one bucket
-// come in any order (the compositing result does not depend on which CTA takes
-// an item, nor on whether a tile is halved). A non-zero *cancel leaves the list empty.
-__global__ void __launch_bounds__(1024) k_work_order(const uint2* __restrict__ ranges, uint32_t n_bins,
-                                                      uint32_t* __restrict__ order, int halves, uint32_t split_min,
-                                                      uint32_t split_share, const uint32_t* __restrict__ n_pairs,
-                                                      const uint32_t* __restrict__ cancel) {
+// order_spec). One CTA of NT threads, a counting sort by bucket; items of one
+// bucket come in any order (the compositing result does not depend on which CTA
+// takes an item, nor on whether a tile is halved). A non-zero *cancel leaves
+// the list empty.
+struct OrderSpec {
+    uint32_t n_bins;
+    int halves;
+    uint32_t split_min, split_share;
+    const uint32_t* n_pairs;
+    const uint32_t* cancel;
+};
+template <int NT>
+__device__ __forceinline__ void build_work_order(const uint2* ranges, const OrderSpec& o, uint32_t* __restrict__ order) {
+    constexpr int E = 1024 / NT;   // buckets a thread
     __shared__ uint32_t cnt[1024];
     __shared__ uint32_t wsum[32];
     const int t = threadIdx.x, lane = t & 31;
-    const uint32_t longest = halves ? max(split_min, *n_pairs / split_share) : 0xFFFFFFFFu;
-    cnt[t] = 0;
+    const uint32_t longest = o.halves ? max(o.split_min, *o.n_pairs / o.split_share) : 0xFFFFFFFFu;
+    for (int e = 0; e < E; ++e) cnt[t * E + e] = 0;
     __syncthreads();
-    for (uint32_t b = t; b < n_bins; b += 1024) {
-        const uint2 r = ranges[b];
+    for (uint32_t b = t; b < o.n_bins; b += NT) {
+        const uint2 r = __ldcg(ranges + b);   // (of this launch: past L1)
         atomicAdd(&cnt[order_slot(r)], r.y - r.x > longest ? 2u : 1u);
     }
     __syncthreads();
-    const uint32_t v = cnt[t];
-    uint32_t x = v;   // inclusive scan within the warp
+    uint32_t v[E], sum = 0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-        if (lane >= o) x += y;
+    for (int e = 0; e < E; ++e) {
+        v[e] = cnt[t * E + e];
+        sum += v[e];
+    }
+    uint32_t x = sum;   // inclusive scan within the warp, then over the warps
+#pragma unroll
+    for (int q = 1; q < 32; q <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, q);
+        if (lane >= q) x += y;
     }
     if (lane == 31) wsum[t >> 5] = x;
     __syncthreads();
     if (t < 32) {
-        const uint32_t w = wsum[t];
+        const uint32_t w = t < NT / 32 ? wsum[t] : 0u;
         uint32_t z = w;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, z, o);
-            if (lane >= o) z += y;
+        for (int q = 1; q < 32; q <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, z, q);
+            if (lane >= q) z += y;
         }
         wsum[t] = z - w;
     }
     __syncthreads();
-    cnt[t] = x - v + wsum[t >> 5];
-    if (t == 1023) order[0] = cancel != nullptr && *cancel != 0u ? 0u : x + wsum[31];
+    uint32_t start = x - sum + wsum[t >> 5];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        cnt[t * E + e] = start;
+        start += v[e];
+    }
+    if (t == NT - 1) order[0] = o.cancel != nullptr && *o.cancel != 0u ? 0u : start;
     __syncthreads();
-    for (uint32_t b = t; b < n_bins; b += 1024) {
-        const uint2 r = ranges[b];
+    for (uint32_t b = t; b < o.n_bins; b += NT) {
+        const uint2 r = __ldcg(ranges + b);   // (of this launch: past L1)
         if (r.y - r.x > longest) {
             const uint32_t p = atomicAdd(&cnt[order_slot(r)], 2u);
             order[1 + p] = b | (1u << kItemShift);
@@ -814,6 +817,40 @@ __global__ void __launch_bounds__(1024) k_work_order(const uint2* __restrict__ r
             order[1 + atomicAdd(&cnt[order_slot(r)], 1u)] = b;
         }
     }
+}
+__global__ void __launch_bounds__(1024) k_work_order(const uint2* __restrict__ ranges, OrderSpec spec,
+                                                      uint32_t* __restrict__ order) {
+    build_work_order<1024>(ranges, spec, order);
+}
+
+// The sorted pairs' (start, end) per bin. After an overflow of the pair buffer the sorted values hold
+// slots that no item wrote: every bin stays empty then, and nothing is composited. Where *fresh is set
+// (a replayed iteration whose cameras are not those of the one before, which left the work list for
+// them), the last CTA to finish writes the list of these ranges. Single views of a window in turn, with
+// the list of the view before: 522 us an iteration; with their own: 318.
+__global__ void __launch_bounds__(256) k_ranges(const uint32_t* __restrict__ pkey, const uint32_t* __restrict__ P_dev,
+                                                uint64_t pair_cap, uint32_t n_bins, const uint32_t* __restrict__ overflow,
+                                                uint2* __restrict__ ranges, const uint32_t* __restrict__ fresh,
+                                                uint32_t* __restrict__ ticket, OrderSpec spec,
+                                                uint32_t* __restrict__ order) {
+    if (*overflow == 0u) {
+        const uint32_t P = (uint32_t)(*P_dev < pair_cap ? *P_dev : pair_cap);
+        for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < P; i += gridDim.x * blockDim.x) {
+            const uint32_t b = pkey[i];
+            if (i == 0 || pkey[i - 1] != b) ranges[b].x = i;
+            if (i == P - 1 || pkey[i + 1] != b) ranges[b].y = i + 1;
+        }
+    }
+    if (fresh == nullptr || *fresh == 0u) return;
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (threadIdx.x == 0) *ticket = 0u;
+    build_work_order<256>(ranges, spec, order);
 }
 
 }  // namespace
@@ -941,18 +978,7 @@ cudaError_t reduce_pair_grads(gs_ctx* c, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t compute_ranges(gs_ctx* c, cudaStream_t s) {
-    // (a mapping iteration zeroes the ranges on its side stream)
-    if (!c->side_zeroed) cudaMemsetAsync(c->ranges, 0, sizeof(uint2) * (size_t)c->n_bins, s);
-    ++c->launches;
-    k_ranges<<<c->num_sms * 8, 256, 0, s>>>(c->pkey[c->pair_buf], c->dcount, (uint64_t)c->pair_cap,
-                                            (uint32_t)c->n_bins, c->dcount + 1, c->ranges);
-    if (c->points != nullptr) return launch_point_items(c, *c->points, true, s);
-    return c->order_ahead ? cudaGetLastError() : launch_work_order(c, s);
-}
-
-cudaError_t launch_work_order(gs_ctx* c, cudaStream_t s) {
-    ++c->launches;
+static OrderSpec order_spec(const gs_ctx* c) {
     // The 16 x 2 layout runs 6 CTAs an SM. With no more halves than that in all, every tile is
     // halved: a CTA's chain of dependent visits is the launch's time, and one pixel a thread instead
     // of two shortens it (160x120 with 2k Gaussians: fused kernel 57 -> 29 us). Otherwise a bin is
@@ -961,12 +987,33 @@ cudaError_t launch_work_order(gs_ctx* c, cudaStream_t s) {
     // and 18 an SM: 1200x680 keyframe with 300k 372, 341, 320 us and 527 without halves; one with
     // lists of similar length 337, 343, 354 us; 8 x 640x480 window 782, 785, 797 us). Bins of 128
     // pairs or less take a CTA no longer than the launch's other latencies.
-    const int halves = half_tiles(c) ? 1 : 0;
+    OrderSpec o;
+    o.n_bins = (uint32_t)c->n_bins;
+    o.halves = half_tiles(c) ? 1 : 0;
     const bool all = 2ll * c->n_bins <= 6ll * c->num_sms;
-    const uint32_t split_min = all ? 0u : 128u, split_share = all ? 0xFFFFFFFFu : 12u * (uint32_t)c->num_sms;
+    o.split_min = all ? 0u : 128u;
+    o.split_share = all ? 0xFFFFFFFFu : 12u * (uint32_t)c->num_sms;
+    o.n_pairs = c->dcount;
     // a render with an unreported non-finite value is not made (a replay's order is for the next one)
-    k_work_order<<<1, 1024, 0, s>>>(c->ranges, (uint32_t)c->n_bins, c->work_order, halves, split_min, split_share,
-                                    c->dcount, c->order_ahead ? nullptr : c->dcount + 10);
+    o.cancel = c->order_ahead ? nullptr : c->dcount + 10;
+    return o;
+}
+
+cudaError_t compute_ranges(gs_ctx* c, cudaStream_t s) {
+    // (a mapping iteration zeroes the ranges on its side stream)
+    if (!c->side_zeroed) cudaMemsetAsync(c->ranges, 0, sizeof(uint2) * (size_t)c->n_bins, s);
+    ++c->launches;
+    k_ranges<<<c->num_sms * 8, 256, 0, s>>>(c->pkey[c->pair_buf], c->dcount, (uint64_t)c->pair_cap,
+                                            (uint32_t)c->n_bins, c->dcount + 1, c->ranges,
+                                            c->order_ahead ? c->dcount + 13 : nullptr, c->dcount + 14, order_spec(c),
+                                            c->work_order);
+    if (c->points != nullptr) return launch_point_items(c, *c->points, true, s);
+    return c->order_ahead ? cudaGetLastError() : launch_work_order(c, s);
+}
+
+cudaError_t launch_work_order(gs_ctx* c, cudaStream_t s) {
+    ++c->launches;
+    k_work_order<<<1, 1024, 0, s>>>(c->ranges, order_spec(c), c->work_order);
     return cudaGetLastError();
 }
 

@@ -7,7 +7,7 @@ import torch
 
 from synth import frustum_scene, random_target
 
-from gpu_helpers import GRAD_FLOOR_DEEP, cuda, new_map
+from gpu_helpers import GRAD_FLOOR_DEEP, cuda, new_map, rotated_cam
 from test_gpu_fused import _longest_list, check_iteration, iterate_once, oracle_ref
 
 pytestmark = pytest.mark.gpu
@@ -93,3 +93,22 @@ def test_nonfinite_colour_stays_with_its_pixels(cfg):
     finite = torch.isfinite(grads[1]).all(dim=0)
     assert not finite[0] and finite.sum() > n // 4
     torch.testing.assert_close(grads[1][:, finite], grads[0][:, finite], rtol=1e-3, atol=1e-3)
+
+
+@pytest.mark.parametrize("cfg", [dict(tile_size=16, pixels_per_thread=2), dict(tile_size=16, pixels_per_thread=1),
+                                 dict(deterministic=1)])
+def test_replays_that_change_their_cameras(cfg):
+    """A replayed iteration takes the work list the one before left, or, for other cameras, one of its own:
+    each image is that of a render of the same view."""
+    p, cam, tg = mixed_scene()
+    cams = [cam, rotated_cam(cam, [0.05, -0.04, 0.0], [0.1, 0.0, 0.1]), rotated_cam(cam, [-0.06, 0.05, 0.02], [0.0, 0.1, 0.0])]
+    still = dict(lr=(0.0,) * 5, **cfg)
+    gm, ref = new_map(p.shape[1], W=W, H=H, **still), new_map(p.shape[1], W=W, H=H, **still)
+    for m in (gm, ref):
+        m.set_params(cuda(p))
+    want = [ref.render(c) for c in cams]
+    rgb = torch.empty(1, 3, H, W, device="cuda")
+    for v in [0, 0, 0, 1, 2, 2, 1, 0, 1, 1]:
+        rgb.fill_(-1.0)
+        gm.iterate(cams[v], cuda(tg), rgb_out=rgb)
+        assert torch.equal(rgb, want[v]), v
