@@ -55,6 +55,22 @@ def test_insert_scales_and_order(n_ref, n):
     np.testing.assert_allclose(got[3], log_scale(pts, p[0:3].T, False), atol=2e-6, rtol=0)
 
 
+@pytest.mark.parametrize("n", [4096, 4097, 9001])
+def test_append_in_order(n):
+    """Around the number of points from which the appending takes them in several CTAs: part of them
+    behind opaque Gaussians, the others appended in order."""
+    rng = np.random.default_rng(n)
+    p, cam = frustum_scene(n=60, seed=4)
+    p[10] = 6.0
+    pts = np.stack([rng.uniform(-1, 1, n), rng.uniform(-1, 1, n), rng.uniform(1, 5, n)], 1).astype(np.float32)
+    gm = new_map(60 + n)
+    gm.set_params(cuda(p))
+    count, mask = gm.insert(cam, torch.zeros(3, 120, 160, device="cuda"), cuda(pts), return_mask=True)
+    mask = mask.cpu().numpy()
+    assert 0 < count == mask.sum() < n and gm.n == 60 + count
+    np.testing.assert_array_equal(gm.params().cpu().numpy()[0:3, 60:], pts[mask].T)
+
+
 def test_a_second_split_uses_the_buffers_of_the_first():
     """Splits swap the parameters between two sets of buffers: three in a row from one map equal the
     same splits of fresh maps."""
