@@ -1,5 +1,6 @@
 """The (view, tile, depth, id) order of the pairs at the sizes where the sort changes its way: the
-one-CTA depth sort's last size and the first beyond it, more blocks than a scatter adds up itself,
+one-CTA depth sort's last size and the first beyond it, more blocks than a scatter or the emission
+adds up itself,
 several views, depths over a 32-bit range of keys, all depths equal, and nothing visible."""
 import numpy as np
 import pytest
@@ -52,3 +53,13 @@ def test_nothing_visible(n):
     gm.set_params(cuda(p))
     assert float(gm.render(cam).abs().max()) == 0.0
     assert check_order(gm, [cam], n) == 0
+
+
+@pytest.mark.parametrize("n", [16384 * 256, 16384 * 256 + 1, 17000 * 256 + 17])
+def test_many_blocks(n):
+    """Around the number of item blocks from which the emission reads a scan of their tile sums."""
+    p, cam = frustum_scene(n=n, width=160, height=120, fx=150, fy=150, cx=80, cy=60, seed=3, logscale_mean=-6.0)
+    gm = new_map(n, pair_capacity=8 * n)
+    gm.set_params(cuda(p.astype(np.float32)))
+    gm.render(cam)
+    assert check_order(gm, [cam], n) > n // 2
