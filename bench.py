@@ -47,7 +47,7 @@ FP32_LANES_PER_SM = 128
 # workload, with the kernel source's sha256 and layout at capture time (the figure is reported
 # only while both still match): profiles/raster_fused_replica_1200x680_300k.md (the keyframe)
 # and profiles/raster_fused_window_8x640x480_150k.md (the window)
-_RASTER_SHA = "1c013d1d402342df508bbe907f9eafb38030a04a0ffafa3a8a942ded627609ca"
+_RASTER_SHA = "a5c0d9ad2652bb4b8f7593c859b6f2b835936252c4dcc11c4f7af85283f444fd"
 NCU_TRAFFIC = {"raster_fused": {"bytes": 35.97e6, "source": "paper_2504_02437_gb300/csrc/k_raster.cu",
                                 "sha256": _RASTER_SHA, "tile": 16, "ppt": 2},
                "raster_fused_window": {"bytes": 103.19e6, "source": "paper_2504_02437_gb300/csrc/k_raster.cu",

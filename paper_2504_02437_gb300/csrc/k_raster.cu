@@ -1081,30 +1081,21 @@ static int resident_grid(K kernel, int threads, int num_sms) {
     return cached;
 }
 
-// CTAs of a launch over n_bins tiles: as many as are resident, but not so many that fewer than about
-// three tiles come to one (two CTAs an SM or more): the queue then has little left to balance, and the
-// CTAs with the long tiles, whose end is the launch's, share their SM's issue slots with more others
-// than they need to. Iterations with all resident CTAs / by this rule: two 333x251 views of 30k
-// Gaussians 214 / 175 us, one 640x480 view of 60k 217 / 200, three deterministic 321x243 views of 20k
-// 278 / 253; with more tiles it changes nothing, and fewer CTAs lose (8 x 640x480 at 6, 5 and 4 an SM:
-// fused kernel 788, 860 and 980 us).
-static int work_grid(int resident, int parts, const gs_ctx* c) {
-    return std::min(std::min(resident, parts * c->n_bins), std::max(2 * c->num_sms, c->n_bins / 3));
-}
-
 template <int TILE, int PPT, bool DET>
 static void fwd_launch(gs_ctx* c, const DevConst& k, float* rgb, int32_t* argmax, cudaStream_t s, int tpv) {
     constexpr int NT = Layout<TILE, PPT>::kThreads, kParts = Layout<TILE, PPT>::kHalves ? 2 : 1;
     if (argmax) {
         const int grid =
-            work_grid(resident_grid<0 + 4 * DET, TILE, PPT>(k_raster_fwd<TILE, PPT, true, DET>, NT, c->num_sms), kParts, c);
+            std::min(resident_grid<0 + 4 * DET, TILE, PPT>(k_raster_fwd<TILE, PPT, true, DET>, NT, c->num_sms),
+                     kParts * c->n_bins);
         k_raster_fwd<TILE, PPT, true, DET><<<grid, NT, 0, s>>>(c->ranges, c->pval[c->pair_buf], c->rec, c->width, c->height,
                                                           c->hcam[0].tiles_x, tpv, c->n, k, rgb, c->T_final,
                                                           c->n_last, argmax, c->dcount + 6, c->work_order,
                                                           c->emit_item);
     } else {
         const int grid =
-            work_grid(resident_grid<1 + 4 * DET, TILE, PPT>(k_raster_fwd<TILE, PPT, false, DET>, NT, c->num_sms), kParts, c);
+            std::min(resident_grid<1 + 4 * DET, TILE, PPT>(k_raster_fwd<TILE, PPT, false, DET>, NT, c->num_sms),
+                     kParts * c->n_bins);
         k_raster_fwd<TILE, PPT, false, DET><<<grid, NT, 0, s>>>(c->ranges, c->pval[c->pair_buf], c->rec, c->width,
                                                            c->height, c->hcam[0].tiles_x, tpv, c->n, k, rgb,
                                                            c->T_final, c->n_last, nullptr, c->dcount + 6,
@@ -1116,7 +1107,7 @@ template <int TILE, int PPT, bool DET>
 static void bwd_launch(gs_ctx* c, const DevConst& k, const float* dLdC, cudaStream_t s, int tpv) {
     constexpr int NT = Layout<TILE, PPT>::kThreads, kParts = Layout<TILE, PPT>::kHalves ? 2 : 1;
     const int grid =
-        work_grid(resident_grid<2 + 4 * DET, TILE, PPT>(k_raster_bwd<TILE, PPT, DET>, NT, c->num_sms), kParts, c);
+        std::min(resident_grid<2 + 4 * DET, TILE, PPT>(k_raster_bwd<TILE, PPT, DET>, NT, c->num_sms), kParts * c->n_bins);
     k_raster_bwd<TILE, PPT, DET><<<grid, NT, 0, s>>>(c->ranges, c->pval[c->pair_buf], c->rec, c->width, c->height,
                                                 c->hcam[0].tiles_x, tpv, k, c->T_final, c->n_last, dLdC, c->grad2d,
                                                 c->dcount + 7, c->work_order, c->emit_item,
@@ -1128,7 +1119,8 @@ static void fused_launch(gs_ctx* c, const DevConst& k, const float* target, cons
                          float* rgb, cudaStream_t s, int tpv, float* partials, int max_grid, int* grid_out) {
     constexpr int NT = Layout<TILE, PPT>::kThreads, kParts = Layout<TILE, PPT>::kHalves ? 2 : 1;
     const int grid = std::min(
-        work_grid(resident_grid<3 + 4 * DET, TILE, PPT>(k_raster_fused<TILE, PPT, DET>, NT, c->num_sms), kParts, c),
+        std::min(resident_grid<3 + 4 * DET, TILE, PPT>(k_raster_fused<TILE, PPT, DET>, NT, c->num_sms),
+                 kParts * c->n_bins),
         max_grid);
     const float scale = k.lambda_color / (float)(3 * (size_t)c->width * c->height);
     k_raster_fused<TILE, PPT, DET><<<grid, NT, 0, s>>>(c->ranges, c->pval[c->pair_buf], c->rec, c->width, c->height,
