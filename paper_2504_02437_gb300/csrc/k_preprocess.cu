@@ -9,13 +9,9 @@
 namespace gs {
 namespace {
 
-// View-independent shape of one Gaussian (Eq. 1): scales, normalised
-// quaternion, its rotation and Sigma = R S S^T R^T.
+// View-independent shape of one Gaussian (Eq. 1): scales and Sigma = R S S^T R^T.
 struct Shape {
     float s[3];
-    float qn[4];
-    float qnorm;
-    float R[9];            // row-major
     float S[6];            // Sigma (xx, xy, xz, yy, yz, zz)
 };
 
@@ -95,24 +91,31 @@ __device__ __forceinline__ void load_params(const float* __restrict__ P, int cap
     for (int r = 0; r < kParamRows; ++r) p[r] = __ldg(P + (size_t)r * cap + i);
 }
 
+// The normalised quaternion (w, x, y, z) and its rotation (row-major); returns the norm.
+__device__ __forceinline__ float rotation_of(const float p[kParamRows], float q[4], float R[9]) {
+    float qq = p[6] * p[6] + p[7] * p[7] + p[8] * p[8] + p[9] * p[9];
+    const float qnorm = sqrtf(qq);
+    float inv = 1.0f / qnorm;
+    float w = p[6] * inv, x = p[7] * inv, y = p[8] * inv, z = p[9] * inv;
+    q[0] = w; q[1] = x; q[2] = y; q[3] = z;
+    R[0] = 1.f - 2.f * (y * y + z * z); R[1] = 2.f * (x * y - w * z);       R[2] = 2.f * (x * z + w * y);
+    R[3] = 2.f * (x * y + w * z);       R[4] = 1.f - 2.f * (x * x + z * z); R[5] = 2.f * (y * z - w * x);
+    R[6] = 2.f * (x * z - w * y);       R[7] = 2.f * (y * z + w * x);       R[8] = 1.f - 2.f * (x * x + y * y);
+    return qnorm;
+}
+
 // Eq. 1 in float32.
 __device__ __forceinline__ void shape_of(const float p[kParamRows], Shape& g) {
     g.s[0] = expf(p[3]);
     g.s[1] = expf(p[4]);
     g.s[2] = expf(p[5]);
-    float qq = p[6] * p[6] + p[7] * p[7] + p[8] * p[8] + p[9] * p[9];
-    g.qnorm = sqrtf(qq);
-    float inv = 1.0f / g.qnorm;
-    float w = p[6] * inv, x = p[7] * inv, y = p[8] * inv, z = p[9] * inv;
-    g.qn[0] = w; g.qn[1] = x; g.qn[2] = y; g.qn[3] = z;
-    g.R[0] = 1.f - 2.f * (y * y + z * z); g.R[1] = 2.f * (x * y - w * z);       g.R[2] = 2.f * (x * z + w * y);
-    g.R[3] = 2.f * (x * y + w * z);       g.R[4] = 1.f - 2.f * (x * x + z * z); g.R[5] = 2.f * (y * z - w * x);
-    g.R[6] = 2.f * (x * z - w * y);       g.R[7] = 2.f * (y * z + w * x);       g.R[8] = 1.f - 2.f * (x * x + y * y);
+    float q[4], R[9];
+    rotation_of(p, q, R);
     float M[9];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int k = 0; k < 3; ++k) M[i * 3 + k] = g.R[i * 3 + k] * g.s[k];
+        for (int k = 0; k < 3; ++k) M[i * 3 + k] = R[i * 3 + k] * g.s[k];
     g.S[0] = M[0] * M[0] + M[1] * M[1] + M[2] * M[2];
     g.S[1] = M[0] * M[3] + M[1] * M[4] + M[2] * M[5];
     g.S[2] = M[0] * M[6] + M[1] * M[7] + M[2] * M[8];
@@ -338,10 +341,38 @@ __global__ void __launch_bounds__(256) k_compact_visible(const uint32_t* __restr
     }
 }
 
-// Six CTAs of 128 threads per SM (at most 85 registers): the kernel is latency-bound on its
-// per-thread chain, and 24 resident warps instead of 20 beat the few spilled registers
-// (A/B on the 300k-Gaussian keyframe: iteration 0.550 -> 0.545 ms; eight CTAs 0.548 ms).
-__global__ void __launch_bounds__(128, 6) k_preprocess_backward(
+// a b + c d with one rounding of nearly the exact sum: the two rounded products' errors come from
+// fused multiply-adds (Kahan's difference of products; its error is at most 1.5 ulp of the result:
+// Jeannerod, Louvet and Muller, Math. Comp. 82, 2013).
+__device__ __forceinline__ float dot2(float a, float b, float c, float d) {
+    const float p = __fmul_rn(c, d);
+    return __fadd_rn(__fmaf_rn(a, b, p), __fmaf_rn(c, d, -p));
+}
+
+// Adjoint of the projection, one thread a Gaussian, all its views. The conic
+// Q = (P S^2 P^T + dilation I)^-1, P = J W R the projected unit axes and S the scales, is taken back in
+// the Gaussian's own axes: with x_k = Q p_k, X = (x_0 x_1 x_2) and the symmetric matrix Gc of the
+// conic's gradient (g_a, g_c and half of g_b off the diagonal),
+//   K_jk = -2 x_j^T Gc x_k          (twice dL/dSigma in body axes),
+//   dL/dlog s_k = K_kk s_k^2,       torque about axis 0 = K_12 (s_1^2 - s_2^2), the others cyclically,
+//   dL/dJ = -2 Q Gc X S^2 (W R)^T.
+// For an elongated projection the determinant A C - B B of its covariance, the adjoint -Q Gc Q in
+// terms of A, B, C, and the products with Sigma after it cancel almost fully in float32: errors of
+// 1e-7 grew with the ratio of the axes' variances, and one such Gaussian near the camera could carry
+// most of the error of the whole gradient. Here the determinant and the x_k come from the minors n of
+// P as sums that do not cancel so:
+//   det = d (d + A0 + C0) + s_1^2 s_2^2 n_0^2 + s_0^2 s_2^2 n_1^2 + s_0^2 s_1^2 n_2^2   (d the dilation),
+//   det X = d P + (Q1 x n, -Q0 x n), Q0 and Q1 the rows of P S^2,
+// and the two contractions that cancel by their nature (Gc x_k, x_j . Gc x_k) are dot2's. Error over
+// the gradient's norm of 110 random room scenes in the deterministic mode: median 1.35e-6 -> 0.94e-6
+// (what the forward's float32 covariance leaves), 2.8e-5 -> 6e-7 in the worst conditioned one, never
+// above what it was; of thin Gaussians near the camera 1e-3 -> below 4e-5.
+//
+// Bound by its chain of dependent instructions: an item's gradients are loaded before the shape is
+// formed, the statistics are added in L2 instead of read, and four CTAs an SM leave it the registers
+// it wants (300k-Gaussian keyframe 22.7 -> 20.7 us, 8-view window of 150k 39.7 -> 37.3; five CTAs 20.7
+// and 42.0, six 23.1 and 47.5 with their spills).
+__global__ void __launch_bounds__(128, 4) k_preprocess_backward(
     const float* __restrict__ P, int n, int cap, int n_views, const DevCamera* __restrict__ cams, DevConst kc,
     const float* __restrict__ grad2d, const uint32_t* __restrict__ tiles, float* __restrict__ G,
     float* __restrict__ dens_sum, float* __restrict__ dens_cnt, int add_reg, float reg_scale) {
@@ -350,19 +381,37 @@ __global__ void __launch_bounds__(128, 6) k_preprocess_backward(
     float p[kParamRows];
     load_params(P, cap, gid, p);
     float dmu[3] = {0.f, 0.f, 0.f};
-    float dS[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // symmetric (G + G^T) of dL/dSigma
+    float K[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // K_00, K_11, K_22, K_12, K_02, K_01
     float dop = 0.f, dr = 0.f, dg = 0.f, db = 0.f;
     float gsum = 0.f, gcnt = 0.f;
-    Shape g;
-    shape_of(p, g);
-    Proj o;
+    // the screen gradients of the view at hand, where the Gaussian has tiles in it
+    float4 g0 = make_float4(0.f, 0.f, 0.f, 0.f), g1 = g0;
+    float g8 = 0.f;
+    bool seen = false;
+    auto load_view = [&](int view) {
+        const size_t item = (size_t)view * n + gid;
+        seen = tiles[item] != 0;
+        if (seen) {
+            g0 = *reinterpret_cast<const float4*>(grad2d + item * kGrad2dStride);
+            g1 = *reinterpret_cast<const float4*>(grad2d + item * kGrad2dStride + 4);
+            g8 = grad2d[item * kGrad2dStride + 8];
+        }
+    };
+    load_view(0);
+    float s[3], sq[3], R[9];
+    {
+        float q[4];
+        rotation_of(p, q, R);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        s[k] = expf(p[3 + k]);
+        sq[k] = s[k] * s[k];
+    }
     for (int view = 0; view < n_views; ++view) {
-        size_t item = (size_t)view * n + gid;
-        if (tiles[item] == 0) continue;
+        if (view > 0) load_view(view);
+        if (!seen) continue;
         const DevCamera& cam = cams[view];
-        const float4 g0 = *reinterpret_cast<const float4*>(grad2d + item * kGrad2dStride);
-        const float4 g1 = *reinterpret_cast<const float4*>(grad2d + item * kGrad2dStride + 4);
-        const float g8 = grad2d[item * kGrad2dStride + 8];
         // the compositing adjoint leaves out the factor ln 2 of the first five values; with the
         // exp2 scaling of the conic (a' = -a log2(e) / 2, b' = -b log2(e)) it cancels there
         float gu = g0.x * kLn2, gv = g0.y * kLn2;
@@ -376,107 +425,104 @@ __global__ void __launch_bounds__(128, 6) k_preprocess_backward(
             gsum += sqrtf(nu * nu + nv * nv);
         }
         gcnt += 1.f;
-        project_one(p, g, cam, kc.dilation, o);
-        // conic (a, b, c) = inverse of [[A, B], [B, C]]
-        float id2 = 1.0f / (o.det * o.det);
-        float A = o.A, B = o.B, C = o.C;
-        float gA = id2 * (-C * C * ga + B * C * gb - B * B * gc);
-        float gB = id2 * (2.f * B * C * ga - (o.det + 2.f * B * B) * gb + 2.f * A * B * gc);
-        float gC = id2 * (-B * B * ga + A * B * gb - A * A * gc);
-        // dL/dSigma (symmetrised): 2 gA T0T0^T + gB (T0T1^T + T1T0^T) + 2 gC T1T1^T
-        const float* T0 = o.T0;
-        const float* T1 = o.T1;
-        dS[0] += 2.f * gA * T0[0] * T0[0] + 2.f * gB * T0[0] * T1[0] + 2.f * gC * T1[0] * T1[0];
-        dS[1] += 2.f * gA * T0[0] * T0[1] + gB * (T0[0] * T1[1] + T1[0] * T0[1]) + 2.f * gC * T1[0] * T1[1];
-        dS[2] += 2.f * gA * T0[0] * T0[2] + gB * (T0[0] * T1[2] + T1[0] * T0[2]) + 2.f * gC * T1[0] * T1[2];
-        dS[3] += 2.f * gA * T0[1] * T0[1] + 2.f * gB * T0[1] * T1[1] + 2.f * gC * T1[1] * T1[1];
-        dS[4] += 2.f * gA * T0[1] * T0[2] + gB * (T0[1] * T1[2] + T1[1] * T0[2]) + 2.f * gC * T1[1] * T1[2];
-        dS[5] += 2.f * gA * T0[2] * T0[2] + 2.f * gB * T0[2] * T1[2] + 2.f * gC * T1[2] * T1[2];
-        // dL/dT0 = 2 gA Sigma T0 + gB Sigma T1 ; dL/dT1 = gB Sigma T0 + 2 gC Sigma T1
-        float ST0[3], ST1[3];
-        ST0[0] = g.S[0] * T0[0] + g.S[1] * T0[1] + g.S[2] * T0[2];
-        ST0[1] = g.S[1] * T0[0] + g.S[3] * T0[1] + g.S[4] * T0[2];
-        ST0[2] = g.S[2] * T0[0] + g.S[4] * T0[1] + g.S[5] * T0[2];
-        ST1[0] = g.S[0] * T1[0] + g.S[1] * T1[1] + g.S[2] * T1[2];
-        ST1[1] = g.S[1] * T1[0] + g.S[3] * T1[1] + g.S[4] * T1[2];
-        ST1[2] = g.S[2] * T1[0] + g.S[4] * T1[1] + g.S[5] * T1[2];
-        float dT0[3], dT1[3];
+        const float d = kc.dilation;
+        const float tx = cam.R[0] * p[0] + cam.R[1] * p[1] + cam.R[2] * p[2] + cam.t[0];
+        const float ty = cam.R[3] * p[0] + cam.R[4] * p[1] + cam.R[5] * p[2] + cam.t[1];
+        const float tz = cam.R[6] * p[0] + cam.R[7] * p[1] + cam.R[8] * p[2] + cam.t[2];
+        const float iz = 1.0f / tz, iz2 = iz * iz, iz3 = iz2 * iz;
+        const float xr = tx * iz, yr = ty * iz;
+        const float xh = fminf(fmaxf(xr, -cam.lim_x), cam.lim_x), yh = fminf(fmaxf(yr, -cam.lim_y), cam.lim_y);
+        const float J00 = cam.fx * iz, J02 = -cam.fx * xh * iz, J11 = cam.fy * iz, J12 = -cam.fy * yh * iz;
+        float Vm[3][3], p0[3], p1[3], q0[3], q1[3];   // V = W R, P = J V, P S^2
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            dT0[k] = 2.f * gA * ST0[k] + gB * ST1[k];
-            dT1[k] = gB * ST0[k] + 2.f * gC * ST1[k];
+#pragma unroll
+            for (int r = 0; r < 3; ++r)
+                Vm[r][k] = cam.R[3 * r] * R[k] + cam.R[3 * r + 1] * R[3 + k] + cam.R[3 * r + 2] * R[6 + k];
+            p0[k] = J00 * Vm[0][k] + J02 * Vm[2][k];
+            p1[k] = J11 * Vm[1][k] + J12 * Vm[2][k];
+            q0[k] = sq[k] * p0[k];
+            q1[k] = sq[k] * p1[k];
         }
-        // T = J W with rows T0 = J00 W0 + J02 W2, T1 = J11 W1 + J12 W2
-        float dJ00 = dT0[0] * cam.R[0] + dT0[1] * cam.R[1] + dT0[2] * cam.R[2];
-        float dJ02 = dT0[0] * cam.R[6] + dT0[1] * cam.R[7] + dT0[2] * cam.R[8];
-        float dJ11 = dT1[0] * cam.R[3] + dT1[1] * cam.R[4] + dT1[2] * cam.R[5];
-        float dJ12 = dT1[0] * cam.R[6] + dT1[1] * cam.R[7] + dT1[2] * cam.R[8];
-        float iz = 1.0f / o.tz, iz2 = iz * iz, iz3 = iz2 * iz;
+        const float n0 = p0[1] * p1[2] - p0[2] * p1[1], n1 = p0[2] * p1[0] - p0[0] * p1[2],
+                    n2 = p0[0] * p1[1] - p0[1] * p1[0];
+        const float A0 = q0[0] * p0[0] + q0[1] * p0[1] + q0[2] * p0[2];   // A and C without the dilation
+        const float C0 = q1[0] * p1[0] + q1[1] * p1[1] + q1[2] * p1[2];
+        const float B = q0[0] * p1[0] + q0[1] * p1[1] + q0[2] * p1[2];
+        const float det = d * (d + A0 + C0) + sq[1] * sq[2] * n0 * n0 + sq[0] * sq[2] * n1 * n1 +
+                          sq[0] * sq[1] * n2 * n2;
+        const float idet = 1.0f / fmaxf(det, 1e-37f);   // (zero only where everything it scales is)
+        const float x0[3] = {(d * p0[0] + (q1[1] * n2 - q1[2] * n1)) * idet,
+                             (d * p0[1] + (q1[2] * n0 - q1[0] * n2)) * idet,
+                             (d * p0[2] + (q1[0] * n1 - q1[1] * n0)) * idet};
+        const float x1[3] = {(d * p1[0] - (q0[1] * n2 - q0[2] * n1)) * idet,
+                             (d * p1[1] - (q0[2] * n0 - q0[0] * n2)) * idet,
+                             (d * p1[2] - (q0[0] * n1 - q0[1] * n0)) * idet};
+        const float h = 0.5f * gb;
+        float z0[3], z1[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            z0[k] = -2.f * dot2(ga, x0[k], h, x1[k]);
+            z1[k] = -2.f * dot2(h, x0[k], gc, x1[k]);
+        }
+        K[0] += dot2(x0[0], z0[0], x1[0], z1[0]);
+        K[1] += dot2(x0[1], z0[1], x1[1], z1[1]);
+        K[2] += dot2(x0[2], z0[2], x1[2], z1[2]);
+        K[3] += dot2(x0[1], z0[2], x1[1], z1[2]);
+        K[4] += dot2(x0[0], z0[2], x1[0], z1[2]);
+        K[5] += dot2(x0[0], z0[1], x1[0], z1[1]);
+        // -2 Gc X S^2 (W R)^T, column by column of the camera's axes
+        float e0[3], e1[3];
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const float f0 = Vm[r][0] * (sq[0] * x0[0]) + Vm[r][1] * (sq[1] * x0[1]) + Vm[r][2] * (sq[2] * x0[2]);
+            const float f1 = Vm[r][0] * (sq[0] * x1[0]) + Vm[r][1] * (sq[1] * x1[1]) + Vm[r][2] * (sq[2] * x1[2]);
+            e0[r] = -2.f * (ga * f0 + h * f1);
+            e1[r] = -2.f * (h * f0 + gc * f1);
+        }
+        const float A = A0 + d, C = C0 + d;
+        const float dJ00 = (C * e0[0] - B * e1[0]) * idet, dJ02 = (C * e0[2] - B * e1[2]) * idet;
+        const float dJ11 = (A * e1[1] - B * e0[1]) * idet, dJ12 = (A * e1[2] - B * e0[2]) * idet;
         float dtx = 0.f, dty = 0.f, dtz = 0.f;
         dtz += -cam.fx * iz2 * dJ00 - cam.fy * iz2 * dJ11;
-        if (fabsf(o.xr) <= cam.lim_x) {
+        if (fabsf(xr) <= cam.lim_x) {
             dtx += -cam.fx * iz2 * dJ02;
-            dtz += 2.f * cam.fx * o.tx * iz3 * dJ02;
+            dtz += 2.f * cam.fx * tx * iz3 * dJ02;
         } else {
-            dtz += cam.fx * o.xh * iz2 * dJ02;
+            dtz += cam.fx * xh * iz2 * dJ02;
         }
-        if (fabsf(o.yr) <= cam.lim_y) {
+        if (fabsf(yr) <= cam.lim_y) {
             dty += -cam.fy * iz2 * dJ12;
-            dtz += 2.f * cam.fy * o.ty * iz3 * dJ12;
+            dtz += 2.f * cam.fy * ty * iz3 * dJ12;
         } else {
-            dtz += cam.fy * o.yh * iz2 * dJ12;
+            dtz += cam.fy * yh * iz2 * dJ12;
         }
         // screen mean u = fx tx/tz + cx, v = fy ty/tz + cy
         dtx += gu * cam.fx * iz;
         dty += gv * cam.fy * iz;
-        dtz += -(gu * cam.fx * o.tx + gv * cam.fy * o.ty) * iz2;
+        dtz += -(gu * cam.fx * tx + gv * cam.fy * ty) * iz2;
         // t = W mu + t_w
         dmu[0] += cam.R[0] * dtx + cam.R[3] * dty + cam.R[6] * dtz;
         dmu[1] += cam.R[1] * dtx + cam.R[4] * dty + cam.R[7] * dtz;
         dmu[2] += cam.R[2] * dtx + cam.R[5] * dty + cam.R[8] * dtz;
     }
-    // Sigma = M M^T with M = R S: dL/dM = dS M
-    float M[9];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) M[i * 3 + k] = g.R[i * 3 + k] * g.s[k];
-    const float Sf[9] = {dS[0], dS[1], dS[2], dS[1], dS[3], dS[4], dS[2], dS[4], dS[5]};
-    float dM[9];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-            dM[i * 3 + k] = Sf[i * 3 + 0] * M[0 * 3 + k] + Sf[i * 3 + 1] * M[1 * 3 + k] + Sf[i * 3 + 2] * M[2 * 3 + k];
-    float dls[3];
-    float dR[9];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        float ds = dM[0 * 3 + k] * g.R[0 * 3 + k] + dM[1 * 3 + k] * g.R[1 * 3 + k] + dM[2 * 3 + k] * g.R[2 * 3 + k];
-        dls[k] = ds * g.s[k];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) dR[i * 3 + k] = dM[i * 3 + k] * g.s[k];
-    }
+    float dls[3] = {K[0] * sq[0], K[1] * sq[1], K[2] * sq[2]};
     if (add_reg) {
         // Eq. 10 planar term: mean_i max(floor, min_k s_ik); gradient on the (first) smallest axis
         int km = 0;
-        float sm = g.s[0];
-        if (g.s[1] < sm) { sm = g.s[1]; km = 1; }
-        if (g.s[2] < sm) { sm = g.s[2]; km = 2; }
+        float sm = s[0];
+        if (s[1] < sm) { sm = s[1]; km = 1; }
+        if (s[2] < sm) { sm = s[2]; km = 2; }
         if (sm > kc.reg_floor) dls[km] += reg_scale * sm;
     }
-    // rotation of the normalised quaternion (w, x, y, z)
-    float w = g.qn[0], x = g.qn[1], y = g.qn[2], z = g.qn[3];
-    float dw = 2.f * (-z * dR[1] + y * dR[2] + z * dR[3] - x * dR[5] - y * dR[6] + x * dR[7]);
-    float dx = 2.f * (y * dR[1] + z * dR[2] + y * dR[3] - 2.f * x * dR[4] - w * dR[5] + z * dR[6] + w * dR[7] -
-                      2.f * x * dR[8]);
-    float dy = 2.f * (-2.f * y * dR[0] + x * dR[1] + w * dR[2] + x * dR[3] + z * dR[5] - w * dR[6] + z * dR[7] -
-                      2.f * y * dR[8]);
-    float dz = 2.f * (-2.f * z * dR[0] - w * dR[1] + x * dR[2] + w * dR[3] - 2.f * z * dR[4] + y * dR[5] +
-                      x * dR[6] + y * dR[7]);
-    // through the normalisation q / |q|
-    float dot = w * dw + x * dx + y * dy + z * dz;
-    float iq = 1.0f / g.qnorm;
+    // R exp([omega]x) is the quaternion q (1, omega / 2): dL/dq = 2 q (0, torque), tangent to the unit
+    // sphere, over |q| for the quaternion before its normalisation
+    float q[4];
+    const float qnorm = rotation_of(p, q, R);
+    const float w = q[0], x = q[1], y = q[2], z = q[3];
+    const float tw0 = K[3] * ((s[1] - s[2]) * (s[1] + s[2])), tw1 = K[4] * ((s[2] - s[0]) * (s[2] + s[0])),
+                tw2 = K[5] * ((s[0] - s[1]) * (s[0] + s[1]));
+    const float iq2 = 2.0f / qnorm;
     float oa = 1.0f / (1.0f + expf(-p[10]));
     size_t c = (size_t)cap;
     G[0 * c + gid] = dmu[0];
@@ -485,17 +531,17 @@ __global__ void __launch_bounds__(128, 6) k_preprocess_backward(
     G[3 * c + gid] = dls[0];
     G[4 * c + gid] = dls[1];
     G[5 * c + gid] = dls[2];
-    G[6 * c + gid] = (dw - w * dot) * iq;
-    G[7 * c + gid] = (dx - x * dot) * iq;
-    G[8 * c + gid] = (dy - y * dot) * iq;
-    G[9 * c + gid] = (dz - z * dot) * iq;
+    G[6 * c + gid] = -(x * tw0 + y * tw1 + z * tw2) * iq2;
+    G[7 * c + gid] = (w * tw0 + y * tw2 - z * tw1) * iq2;
+    G[8 * c + gid] = (w * tw1 + z * tw0 - x * tw2) * iq2;
+    G[9 * c + gid] = (w * tw2 + x * tw1 - y * tw0) * iq2;
     G[10 * c + gid] = dop * (1.f - oa);   // the records hold o dL/do, do/dlogit = o (1 - o)
     G[11 * c + gid] = dr;
     G[12 * c + gid] = dg;
     G[13 * c + gid] = db;
     if (dens_sum != nullptr && gcnt > 0.f) {
-        dens_sum[gid] += gsum;
-        dens_cnt[gid] += gcnt;
+        atomicAdd(dens_sum + gid, gsum);   // (one each: added in L2, nothing waits for it)
+        atomicAdd(dens_cnt + gid, gcnt);
     }
 }
 
