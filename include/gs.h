@@ -411,6 +411,9 @@ GS_API int gs_debug_grad2d(gs_ctx* ctx, float* out_host);
  * tests of the forward pass up to each pixel's stop, blended pairs, and the
  * pairs the backward pass walks (entries up to each pixel's last blend). */
 GS_API int gs_debug_work(gs_ctx* ctx, int64_t* out_host);
+/* Makes the nth next allocation of a pair buffer (two of keys, two of values; in the
+ * deterministic mode two more) fail on the host as if out of memory (0: none). */
+GS_API int gs_debug_fail_pair_alloc(gs_ctx* ctx, int nth);
 /* Number of kernels this context has launched since it was created. */
 GS_API int64_t gs_launch_count(const gs_ctx* ctx);
 /* Tile size the last render used. */

@@ -69,7 +69,12 @@ template <typename T>
 cudaError_t dalloc(T** p, size_t count) {
     *p = nullptr;
     if (count == 0) count = 1;
-    return cudaMalloc((void**)p, sizeof(T) * count);
+    const cudaError_t e = cudaMalloc((void**)p, sizeof(T) * count);
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        cudaGetLastError();   // the caller reports it; no later check sees it again
+    }
+    return e;
 }
 
 int ceil_log2(uint32_t x) {
@@ -118,20 +123,31 @@ void free_pairs(gs_ctx* c) {
     cudaFree(c->pairgrad);
     c->emit_item = nullptr;
     c->pairgrad = nullptr;
+    c->pair_cap = 0;
 }
 
+// New pair buffers. pair_cap is what the buffers hold at any time: zero while there are none, also after
+// a failure (a render then emits nothing, finds its bins empty and tries again to grow).
 cudaError_t alloc_pairs(gs_ctx* c, int64_t cap) {
     free_pairs(c);
+    auto get = [&](auto** p, size_t count) {
+        if (c->fail_pair_alloc > 0 && --c->fail_pair_alloc == 0) return cudaErrorMemoryAllocation;
+        return dalloc(p, count);
+    };
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
+        e = get(&c->pkey[i], (size_t)cap);
+        if (e == cudaSuccess) e = get(&c->pval[i], (size_t)cap);
+    }
+    if (c->cfg.deterministic && e == cudaSuccess) {
+        e = get(&c->emit_item, (size_t)cap);
+        if (e == cudaSuccess) e = get(&c->pairgrad, (size_t)cap * kPairGradStride);
+    }
+    if (e != cudaSuccess) {
+        free_pairs(c);
+        return e;
+    }
     c->pair_cap = cap;
-    cudaError_t e;
-    for (int i = 0; i < 2; ++i) {
-        if ((e = dalloc(&c->pkey[i], (size_t)cap)) != cudaSuccess) return e;
-        if ((e = dalloc(&c->pval[i], (size_t)cap)) != cudaSuccess) return e;
-    }
-    if (c->cfg.deterministic) {
-        if ((e = dalloc(&c->emit_item, (size_t)cap)) != cudaSuccess) return e;
-        if ((e = dalloc(&c->pairgrad, (size_t)cap * kPairGradStride)) != cudaSuccess) return e;
-    }
     return cudaSuccess;
 }
 
@@ -1145,7 +1161,7 @@ int gs_debug_pairs(gs_ctx* c, uint32_t* bins, uint32_t* vals, int64_t max, int64
     uint32_t P = 0;
     CK(cudaMemcpy(&P, c->dcount, sizeof(uint32_t), cudaMemcpyDeviceToHost));
     *count = P;
-    int64_t m = std::min<int64_t>(P, max);
+    int64_t m = std::min<int64_t>({(int64_t)P, max, c->pair_cap});
     if (m > 0 && bins) CK(cudaMemcpy(bins, c->pkey[c->pair_buf], sizeof(uint32_t) * m, cudaMemcpyDeviceToHost));
     if (m > 0 && vals) {
         CK(cudaMemcpy(vals, c->pval[c->pair_buf], sizeof(uint32_t) * m, cudaMemcpyDeviceToHost));
@@ -1156,6 +1172,12 @@ int gs_debug_pairs(gs_ctx* c, uint32_t* bins, uint32_t* vals, int64_t max, int64
             for (int64_t i = 0; i < m; ++i) vals[i] = vals[i] < items.size() ? items[vals[i]] : 0xFFFFFFFFu;
         }
     }
+    return GS_OK;
+}
+
+int gs_debug_fail_pair_alloc(gs_ctx* c, int nth) {
+    if (!c || nth < 0) return GS_ERR_ARG;
+    c->fail_pair_alloc = nth;
     return GS_OK;
 }
 

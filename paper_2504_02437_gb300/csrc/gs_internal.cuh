@@ -107,7 +107,8 @@ struct gs_ctx {
     uint32_t* dkey[2] = {nullptr, nullptr}; // depth-sort keys   [max_views * cap]
     uint32_t* dval[2] = {nullptr, nullptr}; // depth-sort values [max_views * cap]
     uint32_t* offsets = nullptr;            // deterministic mode: exclusive scan of tiles touched in depth order
-    int64_t pair_cap = 0;
+    int64_t pair_cap = 0;                   // pairs the buffers hold (zero while there are none)
+    int fail_pair_alloc = 0;                // tests: the n-th next allocation of a pair buffer fails
     uint32_t* pkey[2] = {nullptr, nullptr}; // bin of each pair
     uint32_t* pval[2] = {nullptr, nullptr}; // (view * cap + id) of each pair
     int pair_buf = 0;                       // which of the two buffers holds the sorted pairs
