@@ -167,7 +167,8 @@ GS_API int gs_render(gs_ctx* ctx, const gs_camera* cams_host, int n_views, float
 /* Loss of the last render (Eq. 10-11, Section 3.2 "Map Optimization"):
  * L = sum_views lambda_color mean_{3HW}|C - I| + lambda_reg mean_i max(reg_floor, min_k s_ik).
  * target_dev: [n_views][3][H][W]. loss_dev: optional float[3] = {L, photometric, planar}.
- * Stores dL/dC for gs_backward(ctx, NULL, ...). */
+ * Stores dL/dC for gs_backward(ctx, NULL, ...). Errors: GS_ERR_STATE as gs_backward, and
+ * after gs_count_dominant (whose render keeps no image). */
 GS_API int gs_loss(gs_ctx* ctx, const float* target_dev, float* loss_dev, void* stream);
 
 /* Adjoint of the last render: gradients of the loss with respect to all
@@ -176,7 +177,9 @@ GS_API int gs_loss(gs_ctx* ctx, const float* target_dev, float* loss_dev, void* 
  * upstream gradient of the rendered image, or NULL to use the L1 gradient
  * stored by gs_loss, in which case the planar-term gradient is added too.
  * Recomputes per-pixel transmittance back to front from the stored final T
- * (no per-Gaussian blend state is stored). Errors: GS_ERR_STATE if no render. */
+ * (no per-Gaussian blend state is stored). Errors: GS_ERR_STATE if no render,
+ * or none since the last gs_iterate, gs_insert or change of the map (an
+ * iteration keeps no per-pixel state). */
 GS_API int gs_backward(gs_ctx* ctx, const float* dL_drgb_dev, void* stream);
 
 /* One Adam step on every parameter with the gradient of the last gs_backward.

@@ -556,7 +556,7 @@ int gs_set_params(gs_ctx* c, const float* params_dev, int n, void* stream) {
     c->n = n;
     c->adam_t = 0;
     c->n_views = 0;
-    c->loss_ready = c->backward_ready = false;
+    c->render_ready = c->loss_ready = c->backward_ready = false;
     drop_graph(c);
     return GS_OK;
 }
@@ -593,7 +593,7 @@ int gs_render(gs_ctx* c, const gs_camera* cams, int n_views, float* rgb, float* 
     if (!rgb) return fail(c, GS_ERR_ARG, "rgb_dev is NULL");
     cudaStream_t s = (cudaStream_t)stream;
     CK(cudaSetDevice(c->device));
-    c->loss_ready = c->backward_ready = false;
+    c->render_ready = c->loss_ready = c->backward_ready = false;
     int code = setup_views(c, cams, n_views, s);
     if (code != GS_OK) {
         c->n_views = 0;
@@ -601,7 +601,11 @@ int gs_render(gs_ctx* c, const gs_camera* cams, int n_views, float* rgb, float* 
     }
     const DevConst k = dev_const(c->cfg);
     c->rendered_rgb = rgb;
-    if (c->n == 0) return render_empty(c, rgb, T, argmax, s);
+    if (c->n == 0) {
+        code = render_empty(c, rgb, T, argmax, s);
+        c->render_ready = code == GS_OK;
+        return code;
+    }
     if ((code = front_half(c, k, s)) != GS_OK) {
         c->n_views = 0;   // no image to take a loss of
         return code;
@@ -644,12 +648,13 @@ int gs_render(gs_ctx* c, const gs_camera* cams, int n_views, float* rgb, float* 
         }
     }
     CK(launch_copy_T(c, T, s));
+    c->render_ready = true;
     return GS_OK;
 }
 
 int gs_loss(gs_ctx* c, const float* target, float* loss_dev, void* stream) {
     if (!c) return GS_ERR_ARG;
-    if (c->n_views == 0 || !c->rendered_rgb) return fail(c, GS_ERR_STATE, "gs_loss before gs_render");
+    if (!c->render_ready || !c->rendered_rgb) return fail(c, GS_ERR_STATE, "gs_loss without a gs_render before it");
     if (!target) return fail(c, GS_ERR_ARG, "target_dev is NULL");
     cudaStream_t s = (cudaStream_t)stream;
     float* out = loss_dev ? loss_dev : c->partials + c->n_partials;
@@ -667,7 +672,7 @@ int gs_loss(gs_ctx* c, const float* target, float* loss_dev, void* stream) {
 
 int gs_backward(gs_ctx* c, const float* dL_drgb, void* stream) {
     if (!c) return GS_ERR_ARG;
-    if (c->n_views == 0) return fail(c, GS_ERR_STATE, "gs_backward before gs_render");
+    if (!c->render_ready) return fail(c, GS_ERR_STATE, "gs_backward without a gs_render before it");
     if (!dL_drgb && !c->loss_ready) return fail(c, GS_ERR_STATE, "gs_backward(NULL) before gs_loss");
     cudaStream_t s = (cudaStream_t)stream;
     const DevConst k = dev_const(c->cfg);
@@ -811,6 +816,7 @@ static int autotune(gs_ctx* c, const gs_camera* cams, int n_views, const float* 
         }
     }
     c->force_tile = c->force_ppt = 0;
+    c->render_ready = false;
     c->timing = timing;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -862,6 +868,9 @@ static int iterate_core(gs_ctx* c, const gs_camera* cams, int n_views, const flo
     CamBatch b;
     int code = prepare_views(c, cams, n_views, b);
     if (code != GS_OK) return code;
+    // an iteration leaves neither the transmittance and last entries that an adjoint reads nor, in a
+    // replay, a work list for them
+    c->render_ready = false;
     const bool same = c->graph && c->graph_views == n_views && c->graph_w == cams[0].width &&
                       c->graph_h == cams[0].height && c->graph_n == c->n && c->graph_tile == c->tile &&
                       c->graph_ppt == c->ppt && c->graph_pair_cap == c->pair_cap &&
@@ -1275,7 +1284,7 @@ struct Scratch {
 
 void invalidate_render(gs_ctx* c) {
     c->n_views = 0;
-    c->loss_ready = c->backward_ready = false;
+    c->render_ready = c->loss_ready = c->backward_ready = false;
     drop_graph(c);
 }
 
@@ -1362,6 +1371,7 @@ int gs_insert(gs_ctx* c, const gs_camera* cam, const float* image, const float* 
         if (code != GS_OK) return code;
     }
     c->n_views = 0;   // no whole image to take a loss of
+    c->render_ready = false;
     if (!gate) CK(launch_point_items(c, points, false, s));
     CK(launch_insert_test(c, points, image, part, keep, stage, s));
     if (c->init_mlp) CK(mlp_initialise(c->init_mlp, c->hcam[0], image, pts, n, stage, feat, s));
@@ -1389,6 +1399,7 @@ int gs_count_dominant(gs_ctx* c, const gs_camera* cams, int n_views, void* strea
     int32_t* am = t.take<int32_t>(pix);
     const int code = gs_render(c, cams, n_views, img, nullptr, am, stream);
     if (code != GS_OK) return code;
+    c->rendered_rgb = nullptr;   // the image is this call's scratch: nothing to take a loss of
     CK(launch_count_dominant(c, am, pix, s));
     CK(cudaStreamSynchronize(s));
     return GS_OK;
@@ -1572,7 +1583,7 @@ int gs_load(gs_ctx* c, const char* path, void* stream) {
     c->n = (int)n;
     c->adam_t = h.adam_steps_host;
     c->n_views = 0;
-    c->loss_ready = c->backward_ready = false;
+    c->render_ready = c->loss_ready = c->backward_ready = false;
     drop_graph(c);
     return GS_OK;
 }

@@ -127,6 +127,8 @@ struct gs_ctx {
     float* dLdC = nullptr;                  // [max_views * 3 * H * W]
     float* grad2d = nullptr;                // [max_views * cap * 12]
     const float* rendered_rgb = nullptr;    // caller buffer of the last render
+    bool render_ready = false;              // a whole gs_render is the last thing composited: its T_final,
+                                            // n_last, ranges, records and work list are there
     bool loss_ready = false;
     bool backward_ready = false;
 
