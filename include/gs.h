@@ -252,7 +252,13 @@ GS_API int gs_insert(gs_ctx* ctx, const gs_camera* cam_host, const float* image_
  * and a zero (80 floats). Output: log-scale (3), quaternion (4), opacity
  * logit (1), colour (3). Parameters are float32, one flat array of
  * gs_mlp_num_params() values: W1 [128][80], b1 [128], W2 [128][128], b2 [128],
- * W3 [16][128], b3 [16] (rows 11..15 of W3 and b3 stay zero). */
+ * W3 [16][128], b3 [16] (rows 11..15 of W3 and b3 stay zero).
+ * Every device-side wait is bounded. Where one gives up, that launch writes no
+ * results (a backward: the gradient is left as it was, the loss is NaN, a step
+ * enqueued after it leaves the weights), and from when its stream has passed
+ * it gs_mlp_forward, gs_mlp_backward, gs_mlp_step and a gs_insert with this
+ * MLP return GS_ERR_TIMEOUT; the gs_insert it happens in does so itself, with
+ * the map unchanged. */
 typedef struct gs_mlp gs_mlp;
 /* Create an MLP on `device` with uniform(+-1/sqrt(fan_in)) weights drawn from
  * SplitMix64(seed) and zero biases. */
@@ -417,6 +423,9 @@ GS_API int gs_debug_work(gs_ctx* ctx, int64_t* out_host);
 /* Makes the nth next allocation of a pair buffer (two of keys, two of values; in the
  * deterministic mode two more) fail on the host as if out of memory (0: none). */
 GS_API int gs_debug_fail_pair_alloc(gs_ctx* ctx, int nth);
+/* Makes the nth wait of each CTA of this MLP's launches (1: its weights, then its products) give up
+ * at once (0: none), to show what a wait that gives up leaves. */
+GS_API int gs_debug_mlp_give_up(gs_mlp* mlp, int nth);
 /* Number of kernels this context has launched since it was created. */
 GS_API int64_t gs_launch_count(const gs_ctx* ctx);
 /* Tile size the last render used. */

@@ -1339,6 +1339,8 @@ int gs_insert(gs_ctx* c, const gs_camera* cam, const float* image, const float* 
     CK(cudaSetDevice(c->device));
     const size_t HW = (size_t)cam->width * cam->height, np = (size_t)n;
     if (!camera_ok(*cam, c->cfg)) return fail(c, GS_ERR_ARG, "invalid camera");
+    static const char* const timed_out = "a bounded wait of the learned initialiser gave up";
+    if (c->init_mlp && mlp_timed_out(c->init_mlp)) return fail(c, GS_ERR_TIMEOUT, timed_out);
     const size_t n_part = knn_scratch(c, n, c->n), n_feat = c->init_mlp ? 80 * np : 0;
     const size_t bins = ((size_t)cam->width + 7) / 8 * (((size_t)cam->height + 7) / 8);   // of the smallest tiles
     Scratch t(c);
@@ -1377,6 +1379,8 @@ int gs_insert(gs_ctx* c, const gs_camera* cam, const float* image, const float* 
     if (c->init_mlp) CK(mlp_initialise(c->init_mlp, c->hcam[0], image, pts, n, stage, feat, s));
     CK(launch_append(c, stage, n, keep, inserted_dev, c->hcount + 5, s));
     CK(cudaStreamSynchronize(s));
+    // (what was appended lies past the map's Gaussians)
+    if (c->init_mlp && mlp_timed_out(c->init_mlp)) return fail(c, GS_ERR_TIMEOUT, timed_out);
     *n_ins = (int)c->hcount[5];
     c->n += *n_ins;
     invalidate_render(c);

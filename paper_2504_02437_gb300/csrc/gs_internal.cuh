@@ -325,7 +325,9 @@ __device__ __forceinline__ void adam_bias_end(uint32_t* st, double* pw, const fl
     }
 }
 cudaError_t launch_copy_T(gs_ctx* c, float* T_out, cudaStream_t s);
-// learned initialiser (k_mlp.cu): overwrite the staged plain parameters of the points
+// learned initialiser (k_mlp.cu): whether a wait of an earlier launch gave up; overwrite the staged plain
+// parameters of the points
+bool mlp_timed_out(const gs_mlp* M);
 cudaError_t mlp_initialise(gs_mlp* M, const DevCamera& cam, const float* image, const float* pts, int n, float* stage,
                            float* feat_tmp, cudaStream_t s);
 // map management (k_map.cu)

@@ -42,8 +42,8 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo, uint
 __host__ __device__ constexpr uint32_t umma_idesc_bf16(int m, int n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    for (uint32_t i = 0; i < kTcWaitLimit; ++i) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t limit = kTcWaitLimit) {
+    for (uint32_t i = 0; i < limit; ++i) {
         uint32_t done;
         asm volatile(
             "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
@@ -176,11 +176,20 @@ __device__ __forceinline__ void store_col(uint8_t* dst, int r0, int j, const bf1
 // them a read of TMEM, an erf (and, back, an exp) a value and a rewrite of the operands. One launch
 // takes the place of 20 (elementwise kernels and strided GEMMs that gathered their operands element by
 // element): gradients of 4,096 rows 400 -> 20 us, a prediction of 96 rows 58 -> 6 us.
+//
+// A wait that gives up ends the CTA's work: it writes nothing, sets both flags of `err`, and leaves once
+// its weight copy and its products have ended (a bounded wait again), so that neither runs on in shared
+// memory or TMEM that is no longer its own.
+struct NetErr {
+    uint32_t* device;     // read by the kernels that would use the results
+    uint32_t* host;       // pinned: read by the next calls
+    uint32_t give_up;     // tests: the wait of each CTA (counted from 1) that gives up at once; 0: none
+};
 template <bool TRAIN, int ROWS>
 __global__ void __launch_bounds__(kNetThreads, 1)
     k_mlp_net(const float* __restrict__ feat, const float* __restrict__ tgt, int n, const uint8_t* __restrict__ img,
               const float* __restrict__ par, float* __restrict__ out, float* __restrict__ part,
-              float* __restrict__ loss_part, uint32_t* __restrict__ err) {
+              float* __restrict__ loss_part, NetErr err) {
     typedef Smem<TRAIN, ROWS> S;
     constexpr int N = ROWS / 2;                  // rows of a thread
     extern __shared__ __align__(1024) uint8_t sm[];
@@ -218,8 +227,11 @@ __global__ void __launch_bounds__(kNetThreads, 1)
     const uint32_t tmem = tmem_slot;
     const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const float b1 = bias[j], b2 = bias[kHid + j];
-    uint32_t parity = 0;
-    bool ok = true;
+    uint32_t parity = 0, waits = 0;
+    bool ok = true, weights_in = false, products_in = true;
+    auto wait = [&](uint32_t b, uint32_t par) {
+        return __syncthreads_and(mbar_wait(b, par, ++waits == err.give_up ? 0u : kTcWaitLimit)) != 0;
+    };
     // the operands written so far become visible to the tensor cores, one thread issues, all wait
     auto products = [&](auto issue) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -231,7 +243,7 @@ __global__ void __launch_bounds__(kNetThreads, 1)
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                          : "memory");
         }
-        ok = __syncthreads_and(mbar_wait(bar, parity));
+        ok = products_in = wait(bar, parity);
         parity ^= 1u;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         return ok;
@@ -272,10 +284,7 @@ __global__ void __launch_bounds__(kNetThreads, 1)
             for (int e = threadIdx.x; e < ROWS * kOutPad; e += kNetThreads)
                 st[e] = row0 + e / kOutPad < n ? tgt[(size_t)row0 * kOutPad + e] : 0.f;
         }
-        if (first && !__syncthreads_and(mbar_wait(wbar, 0))) {   // the weights have arrived
-            ok = false;
-            break;
-        }
+        if (first && !(ok = weights_in = wait(wbar, 0))) break;   // the weights have arrived
         float z[N];
         __align__(16) bf16 h[N];
         if (!products([&] { umma<kIn, ROWS>(tmem + kTmZ1, base + kSmW + kImgW1, base + S::X, false); })) break;
@@ -374,7 +383,9 @@ __global__ void __launch_bounds__(kNetThreads, 1)
         first = false;
     }
     if (!ok) {
-        if (threadIdx.x == 0) *err = 1u;   // pinned host memory: the next call reports it
+        if (!weights_in) mbar_wait(wbar, 0);
+        if (!products_in) mbar_wait(bar, parity ^ 1u);
+        if (threadIdx.x == 0) *err.device = *err.host = 1u;
     } else if constexpr (TRAIN) {
         float* P = part + (size_t)blockIdx.x * kParams;
         const int half = warp >> 2;
@@ -442,8 +453,10 @@ __global__ void __launch_bounds__(kNetThreads, 1)
 // 32 groups of four parameters a CTA, eight threads a group. Bound by its one read of the partials
 // (113 KB a CTA of k_mlp_net, from L2).
 __global__ void __launch_bounds__(256) k_mlp_reduce(const float* __restrict__ part, const float* __restrict__ loss_part,
-                                                    int n_part, float* __restrict__ g, float* __restrict__ loss) {
+                                                    int n_part, float* __restrict__ g, float* __restrict__ loss,
+                                                    const uint32_t* __restrict__ err) {
     __shared__ float4 sh[8][32];
+    const bool failed = *err != 0u;   // some CTA left no partial sums: the gradient stays, the loss is NaN
     const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int i = blockIdx.x * 32 + c;
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -459,7 +472,7 @@ __global__ void __launch_bounds__(256) k_mlp_reduce(const float* __restrict__ pa
     }
     sh[w][c] = a;
     __syncthreads();
-    if (w == 0 && i < kParams / 4) {
+    if (w == 0 && i < kParams / 4 && !failed) {
 #pragma unroll
         for (int q = 1; q < 8; ++q) {
             const float4 v = sh[q][c];
@@ -475,7 +488,7 @@ __global__ void __launch_bounds__(256) k_mlp_reduce(const float* __restrict__ pa
         for (int p = c; p < n_part; p += 32) t += loss_part[p];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
-        if (c == 0) *loss = (float)t;
+        if (c == 0) *loss = failed ? NAN : (float)t;
     }
 }
 
@@ -498,11 +511,13 @@ __device__ __forceinline__ void store_weight(uint8_t* img, int i, float v) {
 
 __global__ void k_mlp_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                            float* __restrict__ v, int n, float lr, float b1, float b2, float eps, float bc1,
-                           float bc2, uint8_t* __restrict__ img) {
+                           float bc2, uint8_t* __restrict__ img, const uint32_t* __restrict__ err) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
+    const uint32_t failed = *err;
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi, vi = b2 * v[i] + (1.f - b2) * gi * gi;
+    if (failed != 0u) return;   // the gradient is not that of the last backward
     m[i] = mi;
     v[i] = vi;
     const float w = p[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
@@ -611,8 +626,16 @@ struct gs_mlp {
     int part_cap = 0;
     float* part = nullptr;        // [CTAs][kParams] partial gradients
     float* loss_part = nullptr;   // [CTAs]
-    uint32_t* herr = nullptr;  // pinned flag that a kernel sets when a wait of its gave up
+    // flags that a kernel sets when a wait of its gave up, pinned and on the device
+    uint32_t* herr = nullptr;
+    uint32_t* derr = nullptr;
+    uint32_t give_up = 0;     // tests: see NetErr
 };
+
+namespace gs {
+// whether a wait of an earlier launch gave up (once its stream has passed it)
+bool mlp_timed_out(const gs_mlp* M) { return *(volatile const uint32_t*)M->herr != 0u; }
+}  // namespace gs
 
 namespace {
 
@@ -661,7 +684,7 @@ int net_ctas(const gs_mlp* M, int rows) {
 template <bool TRAIN, int ROWS>
 void net_launch(gs_mlp* M, const float* feat, const float* tgt, int n, float* out, cudaStream_t s) {
     k_mlp_net<TRAIN, ROWS><<<net_ctas(M, n), kNetThreads, Smem<TRAIN, ROWS>::Bytes, s>>>(
-        feat, tgt, n, M->img, M->p, out, M->part, M->loss_part, M->herr);
+        feat, tgt, n, M->img, M->p, out, M->part, M->loss_part, NetErr{M->derr, M->herr, M->give_up});
 }
 
 template <bool TRAIN, int ROWS>
@@ -704,6 +727,8 @@ int gs_mlp_create(int device, uint64_t seed, gs_mlp** out) {
     ok = ok && cudaMalloc(&M->m, sizeof(float) * kParams) == cudaSuccess;
     ok = ok && cudaMalloc(&M->v, sizeof(float) * kParams) == cudaSuccess;
     ok = ok && cudaMalloc(&M->img, kImgBytes) == cudaSuccess;
+    ok = ok && cudaMalloc(&M->derr, sizeof(uint32_t)) == cudaSuccess;
+    ok = ok && cudaMemset(M->derr, 0, sizeof(uint32_t)) == cudaSuccess;
     ok = ok && cudaMallocHost((void**)&M->herr, sizeof(uint32_t)) == cudaSuccess;
     if (ok) *M->herr = 0u;
     if (!ok) {
@@ -746,7 +771,7 @@ int gs_mlp_create(int device, uint64_t seed, gs_mlp** out) {
 void gs_mlp_destroy(gs_mlp* M) {
     if (!M) return;
     cudaSetDevice(M->device);
-    void* ps[] = {M->p, M->g, M->m, M->v, M->img, M->y, M->part, M->loss_part};
+    void* ps[] = {M->p, M->g, M->m, M->v, M->img, M->y, M->part, M->loss_part, M->derr};
     for (void* q : ps) cudaFree(q);
     if (M->herr) cudaFreeHost(M->herr);
     delete M;
@@ -804,34 +829,42 @@ int gs_mlp_features(const gs_camera* cam, const float* image_dev, const float* p
 int gs_mlp_forward(gs_mlp* M, const float* feat_dev, int n, float* out_dev, void* stream) {
     if (!M || n < 0 || (n > 0 && (!feat_dev || !out_dev))) return GS_ERR_ARG;
     if (n == 0) return GS_OK;
-    if (*(volatile uint32_t*)M->herr != 0u) return GS_ERR_TIMEOUT;   // a wait of an earlier call gave up
+    if (mlp_timed_out(M)) return GS_ERR_TIMEOUT;   // a wait of an earlier call gave up
     return mlp_forward_rows(M, feat_dev, n, out_dev, (cudaStream_t)stream) == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
 int gs_mlp_backward(gs_mlp* M, const float* feat_dev, const float* target_dev, int n, float* loss_dev, void* stream) {
     if (!M || n <= 0 || !feat_dev || !target_dev) return GS_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    if (*(volatile uint32_t*)M->herr != 0u) return GS_ERR_TIMEOUT;   // a wait of an earlier call gave up
+    if (mlp_timed_out(M)) return GS_ERR_TIMEOUT;   // a wait of an earlier call gave up
     const int ctas = net_ctas(M, n);
     if (mlp_parts(M, ctas) != GS_OK) return GS_ERR_OOM;
     if (net_rows(M, n) == 32) net_launch<true, 32>(M, feat_dev, target_dev, n, nullptr, s);
     else net_launch<true, 64>(M, feat_dev, target_dev, n, nullptr, s);
-    k_mlp_reduce<<<(kParams / 4 + 31) / 32, 256, 0, s>>>(M->part, M->loss_part, ctas, M->g, loss_dev);
+    k_mlp_reduce<<<(kParams / 4 + 31) / 32, 256, 0, s>>>(M->part, M->loss_part, ctas, M->g, loss_dev,
+                                                             M->derr);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
 int gs_mlp_step(gs_mlp* M, float lr, void* stream) {
     if (!M || !(lr > 0.f)) return GS_ERR_ARG;
+    if (mlp_timed_out(M)) return GS_ERR_TIMEOUT;
     cudaStream_t s = (cudaStream_t)stream;
     M->t += 1;
     const double b1 = 0.9, b2 = 0.999;
     k_mlp_adam<<<(kParams + 255) / 256, 256, 0, s>>>(M->p, M->g, M->m, M->v, kParams, lr, (float)b1, (float)b2, 1e-8f,
                                                      (float)(1.0 - std::pow(b1, M->t)), (float)(1.0 - std::pow(b2, M->t)),
-                                                     M->img);
+                                                     M->img, M->derr);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
 
 int gs_mlp_num_params(void) { return kParams; }
+
+int gs_debug_mlp_give_up(gs_mlp* M, int nth) {
+    if (!M || nth < 0) return GS_ERR_ARG;
+    M->give_up = (uint32_t)nth;
+    return GS_OK;
+}
 
 }  // extern "C"
 
