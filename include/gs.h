@@ -157,8 +157,9 @@ GS_API int gs_init_map(gs_ctx* ctx, const float* points_dev, const float* rgb_de
  * argmax_dev: optional [n_views][H][W] int32 id of the Gaussian with the
  * largest blend weight (Eq. 8), -1 where nothing blends.
  * Keeps the per-pixel state that gs_backward needs. Synchronises the stream
- * once to size the pair buffers. Errors: GS_ERR_ARG, GS_ERR_CAPACITY (pair
- * buffer too small; the context grows it when possible), GS_ERR_CUDA,
+ * once to size the pair buffers. Errors: GS_ERR_ARG, GS_ERR_CAPACITY (the
+ * pair buffer grows as needed up to 2^32 - 16 pairs; more are refused, and
+ * nothing is rendered), GS_ERR_OOM (it could not grow), GS_ERR_CUDA,
  * GS_ERR_NONFINITE (an earlier loss or gradient was not finite; reported once,
  * the render is not made). */
 GS_API int gs_render(gs_ctx* ctx, const gs_camera* cams_host, int n_views, float* rgb_dev, float* T_dev,

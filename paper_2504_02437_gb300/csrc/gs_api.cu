@@ -113,6 +113,8 @@ void make_cam(const gs_camera& g, const gs_config& f, int tile, int view, DevCam
     d.pad = 0;
 }
 
+int64_t pair_count(const uint32_t* counts) { return (int64_t)((uint64_t)counts[1] << 32 | counts[0]); }
+
 void free_pairs(gs_ctx* c) {
     for (int i = 0; i < 2; ++i) {
         cudaFree(c->pkey[i]);
@@ -291,7 +293,7 @@ int check_nonfinite(gs_ctx* c, uint32_t flag, cudaStream_t s) {
 int side_begin(gs_ctx* c, cudaStream_t s) {
     CK(cudaEventRecord(c->side_ev[0], s));
     CK(cudaStreamWaitEvent(c->side, c->side_ev[0], 0));
-    CK(cudaMemsetAsync(c->dcount + 1, 0, sizeof(uint32_t), c->side));
+    CK(cudaMemsetAsync(c->dcount + 9, 0, sizeof(uint32_t), c->side));
     CK(cudaMemsetAsync(c->dcount + 6, 0, 2 * sizeof(uint32_t), c->side));   // the compositing work queues
     CK(cudaMemsetAsync(c->ranges, 0, sizeof(uint2) * (size_t)c->n_bins, c->side));
     CK(cudaEventRecord(c->side_ev[1], c->side));   // (waited for before the pair emission)
@@ -332,7 +334,7 @@ int back_half(gs_ctx* c, const DevConst& k, float* rgb, int32_t* argmax, cudaStr
         if (c->side_zeroed)
             CK(cudaStreamWaitEvent(s, c->side_ev[1], 0));   // overflow flag and ranges zeroed
         else
-            CK(cudaMemsetAsync(c->dcount + 1, 0, sizeof(uint32_t), s));
+            CK(cudaMemsetAsync(c->dcount + 9, 0, sizeof(uint32_t), s));
         CK(emit_pairs(c, items, c->dcount + 8, s));
         int bits = std::max(1, ceil_log2((uint32_t)c->n_bins));
         CK(radix_sort_pairs(c, c->pkey, c->pval, c->dcount, (uint32_t)std::min<int64_t>(c->pair_cap, 0xFFFFFFFFll),
@@ -354,7 +356,7 @@ int render_empty(gs_ctx* c, float* rgb, float* T, int32_t* argmax, cudaStream_t 
     CK(cudaMemsetAsync(c->n_last, 0, sizeof(uint32_t) * HW * c->n_views, s));
     if (argmax) CK(cudaMemsetAsync(argmax, 0xFF, sizeof(int32_t) * HW * c->n_views, s));
     CK(launch_copy_T(c, T, s));
-    CK(cudaMemsetAsync(c->dcount, 0, sizeof(uint32_t), s));
+    CK(cudaMemsetAsync(c->dcount, 0, 2 * sizeof(uint32_t), s));
     return GS_OK;
 }
 
@@ -628,19 +630,19 @@ int gs_render(gs_ctx* c, const gs_camera* cams, int n_views, float* rgb, float* 
         c->n_views = 0;
         return code;
     }
-    const int64_t P = c->hcount[0];
+    const int64_t P = pair_count(c->hcount);
     c->visible_hint = c->hcount[8];
     c->pairs_hint = (uint32_t)std::min<int64_t>(P, 0xFFFFFFFFll);
+    if (P > kMaxPairs) {
+        c->n_views = 0;
+        return fail(c, GS_ERR_CAPACITY, "pair count exceeds 2^32");
+    }
     if (P > c->pair_cap) {
         drop_graph(c);
         CK(cudaStreamSynchronize(s));
         if (alloc_pairs(c, std::min<int64_t>(P + P / 2 + 1024, kMaxPairs)) != cudaSuccess) {
             c->n_views = 0;
             return fail(c, GS_ERR_OOM, "growing the pair buffers failed");
-        }
-        if (P > c->pair_cap) {
-            c->n_views = 0;
-            return fail(c, GS_ERR_CAPACITY, "pair count exceeds 2^32");
         }
         if ((code = back_half(c, k, rgb, argmax, s)) != GS_OK) {
             c->n_views = 0;
@@ -854,16 +856,18 @@ static int iterate_core(gs_ctx* c, const gs_camera* cams, int n_views, const flo
     // The flags of an earlier replay: a pair-buffer overflow there skipped its Adam step.
     if (c->graph && c->graph_pending && cudaEventQuery(c->graph_done) == cudaSuccess) {
         c->graph_pending = false;
-        const uint32_t P = c->hflags[0];
+        const int64_t P = pair_count(c->hflags);
         if (c->hflags[10] != 0u) return check_nonfinite(c, c->hflags[10], s);
-        if (c->hflags[1] != 0u) {
+        if (c->hflags[9] != 0u) {
             drop_graph(c);
-            if (alloc_pairs(c, std::min<int64_t>((int64_t)P + P / 2 + 4096, kMaxPairs)) != cudaSuccess)
+            if (P > kMaxPairs)
+                return fail(c, GS_ERR_CAPACITY, "an earlier iteration's pair count exceeds 2^32; it skipped its update");
+            if (alloc_pairs(c, std::min<int64_t>(P + P / 2 + 4096, kMaxPairs)) != cudaSuccess)
                 return fail(c, GS_ERR_OOM, "growing the pair buffers failed");
             return fail(c, GS_ERR_CAPACITY, "an earlier iteration overflowed the pair buffer and skipped its update; "
                                             "the buffer has grown");
         }
-        c->pairs_hint = P;
+        c->pairs_hint = (uint32_t)P;
     }
     CamBatch b;
     int code = prepare_views(c, cams, n_views, b);
@@ -933,7 +937,7 @@ static int iterate_core(gs_ctx* c, const gs_camera* cams, int n_views, const flo
         CK(cudaMemcpyAsync(c->hcount, c->dcount, sizeof(uint32_t) * 11, cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         if ((cd = check_nonfinite(c, c->hcount[10], s)) != GS_OK) return cd;
-        const int64_t P = c->hcount[0];
+        const int64_t P = pair_count(c->hcount);
         c->visible_hint = c->hcount[8];
         c->pairs_hint = (uint32_t)std::min<int64_t>(P, 0xFFFFFFFFll);
         // headroom for the replays' changing cameras
@@ -1167,10 +1171,11 @@ int gs_debug_projection(gs_ctx* c, int view, double* out) {
 int gs_debug_pairs(gs_ctx* c, uint32_t* bins, uint32_t* vals, int64_t max, int64_t* count) {
     if (!c || !count) return GS_ERR_ARG;
     CK(cudaDeviceSynchronize());
-    uint32_t P = 0;
-    CK(cudaMemcpy(&P, c->dcount, sizeof(uint32_t), cudaMemcpyDeviceToHost));
+    uint32_t Pw[2] = {0, 0};
+    CK(cudaMemcpy(Pw, c->dcount, sizeof(Pw), cudaMemcpyDeviceToHost));
+    const int64_t P = pair_count(Pw);
     *count = P;
-    int64_t m = std::min<int64_t>({(int64_t)P, max, c->pair_cap});
+    int64_t m = std::min<int64_t>({P, max, c->pair_cap});
     if (m > 0 && bins) CK(cudaMemcpy(bins, c->pkey[c->pair_buf], sizeof(uint32_t) * m, cudaMemcpyDeviceToHost));
     if (m > 0 && vals) {
         CK(cudaMemcpy(vals, c->pval[c->pair_buf], sizeof(uint32_t) * m, cudaMemcpyDeviceToHost));
@@ -1199,11 +1204,11 @@ int gs_debug_work(gs_ctx* c, int64_t* out) {
     cudaError_t e = cudaMemset(d, 0, sizeof(h));
     if (e == cudaSuccess && c->n > 0) e = launch_count_work(c, dev_const(c->cfg), d, nullptr);
     if (e == cudaSuccess) e = cudaMemcpy(h, d, sizeof(h), cudaMemcpyDeviceToHost);
-    uint32_t P = 0;
-    if (e == cudaSuccess) e = cudaMemcpy(&P, c->dcount, sizeof(uint32_t), cudaMemcpyDeviceToHost);
+    uint32_t P[2] = {0, 0};
+    if (e == cudaSuccess) e = cudaMemcpy(P, c->dcount, sizeof(P), cudaMemcpyDeviceToHost);
     cudaFree(d);
     if (e != cudaSuccess) return fail(c, GS_ERR_CUDA, "work count", e);
-    out[0] = c->n > 0 ? (int64_t)P : 0;
+    out[0] = c->n > 0 ? pair_count(P) : 0;
     out[1] = (int64_t)h[0];
     out[2] = (int64_t)h[1];
     out[3] = (int64_t)h[2];

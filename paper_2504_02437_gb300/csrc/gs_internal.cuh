@@ -138,9 +138,10 @@ struct gs_ctx {
     float* ssim_maps = nullptr;             // [3][V][3][H][W] SSIM derivative maps (lambda_photo > 0)
     float* ssim_part = nullptr;             // [2 ssim_blocks] per-CTA photometric loss terms
     int sort_blocks = 0;
-    uint32_t* dcount = nullptr;             // device scalars [16]: [0] pairs, [1] overflow, [2] Adam
+    uint32_t* dcount = nullptr;             // device scalars [16]: [0], [1] pairs (64 bits), [2] Adam
                                             // ticket, [3] UINT32_MAX, [4] Adam steps, [5] totals,
                                             // [6], [7] work queues, [8] visible (view, Gaussian) items,
+                                            // [9] pair buffer overflow,
                                             // [10] a non-finite loss or gradient was seen (sticky until
                                             // a call reports it), [11], [12] smallest and largest visible
                                             // depth key, [13] the replay's cameras are not those of
@@ -300,7 +301,7 @@ __device__ __forceinline__ void adam_update(float& p, float g, float& m, float& 
 
 // Bias corrections of the next Adam step from device state (so that a graph
 // replays correctly): pw = {beta1^t, beta2^t} (float64 running products) after
-// t = st[4] completed steps; st[1] = pair-buffer overflow flag (step skipped).
+// t = st[4] completed steps; st[9] = pair-buffer overflow flag (step skipped).
 // Thread 0 of every CTA reads them before taking a ticket (st[2]); the last
 // CTA of the launch advances pw and t, so every CTA uses the same t + 1.
 // sbc = {1 / (1 - beta1^(t+1)), 1 / (1 - beta2^(t+1)), 1 if the step is skipped}.
@@ -311,7 +312,7 @@ __device__ __forceinline__ void adam_bias_begin(const AdamArgs& a, const uint32_
     spw[1] = p2;
     sbc[0] = (float)(1.0 / (1.0 - p1));
     sbc[1] = (float)(1.0 / (1.0 - p2));
-    sbc[2] = st[1] != 0u ? 1.f : 0.f;
+    sbc[2] = st[9] != 0u ? 1.f : 0.f;
 }
 __device__ __forceinline__ void adam_bias_end(uint32_t* st, double* pw, const float* sbc, const double* spw,
                                               uint32_t n_ctas) {

@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(256) k_compact_visible(const uint32_t* __restr
         if (threadIdx.x == 0) {
             uint2 r = wrange[0];
             for (int k = 1; k < 8; ++k) r = make_uint2(umin(r.x, wrange[k].x), umax(r.y, wrange[k].y));
-            counts[0] = 0u;
+            counts[0] = counts[1] = 0u;
             counts[8] = off;
             counts[11] = r.x;
             counts[12] = r.y;

@@ -369,7 +369,8 @@ struct SmallSmem {
     uint32_t key[kSmallItems], val[kSmallItems];
     uint16_t wcnt[32][1 << kSmallBits];
     uint32_t start[1 << kSmallBits];
-    uint32_t wsum[32], kmin, kmax, total;
+    uint32_t wsum[32], kmin, kmax;
+    unsigned long long total;
 };
 __global__ void __launch_bounds__(kSmallThreads, 1) k_small_depth(const uint32_t* __restrict__ kin, uint32_t n,
                                                                  const uint32_t* __restrict__ tiles,
@@ -506,24 +507,27 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_depth(const uint32_t
         if (lane == 0) sm.wsum[w] = c;
         __syncthreads();
         if (t < 4 && i0 + 256u * t < m) {
-            uint32_t b = 0;
+            unsigned long long b = 0;
             for (int q = 0; q < 8; ++q) b += sm.wsum[8 * t + q];
-            tile_blocks[i0 / 256 + t] = b;
+            tile_blocks[i0 / 256 + t] = (uint32_t)b;
             atomicAdd(&sm.total, b);
         }
         __syncthreads();
     }
     if (t == 0) {
-        counts[0] = sm.total;
+        counts[0] = (uint32_t)sm.total;
+        counts[1] = (uint32_t)(sm.total >> 32);
         counts[8] = m;
     }
 }
 
-// Tiles touched by each 256 items of the depth order (the emission's CTAs), and their total.
+// Tiles touched by each 256 items of the depth order (the emission's CTAs), and their total in 64 bits
+// (a map that fills the screen can have more than 2^32 pairs; nothing is emitted then).
 __global__ void __launch_bounds__(256) k_item_tiles(const uint32_t* __restrict__ order,
                                                     const uint32_t* __restrict__ tiles, uint32_t n_items,
                                                     const uint32_t* __restrict__ n_dev,
-                                                    uint32_t* __restrict__ tile_blocks, uint32_t* __restrict__ total) {
+                                                    uint32_t* __restrict__ tile_blocks,
+                                                    unsigned long long* __restrict__ total) {
     __shared__ uint32_t ws[8];
     const uint32_t nv = umin(n_items, *n_dev);
     for (uint32_t b = blockIdx.x; b * 256u < nv; b += gridDim.x) {
@@ -532,9 +536,9 @@ __global__ void __launch_bounds__(256) k_item_tiles(const uint32_t* __restrict__
         if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = c;
         __syncthreads();
         if (threadIdx.x == 0) {
-            uint32_t t = 0;
+            unsigned long long t = 0;
             for (int q = 0; q < 8; ++q) t += ws[q];
-            tile_blocks[b] = t;
+            tile_blocks[b] = (uint32_t)t;
             atomicAdd(total, t);   // (zeroed by the compaction)
         }
         __syncthreads();
@@ -620,7 +624,8 @@ __global__ void __launch_bounds__(256) k_scan(const uint32_t* __restrict__ in, u
 // pairs (a contiguous run of the output) 32 at a time: lane j writes pair t =
 // t0 + j of the run, owned by the last lane whose exclusive count is <= t, so
 // the stores are coalesced and a large Gaussian's pairs are spread over the
-// warp. An item whose pairs would pass pair_cap is skipped and sets *overflow.
+// warp. An item whose pairs would pass pair_cap is skipped and sets *overflow;
+// of more than 2^32 pairs (*total_hi) every item is, since o wraps.
 // In the deterministic mode (emit_item != NULL) a pair's value is its emission
 // index e instead of its item, emit_item[e] holds the item, and the pair's
 // gradient slot pairgrad[9 e ..] is cleared; off[k] = o for its reduction.
@@ -630,7 +635,8 @@ __global__ void __launch_bounds__(256) k_emit(const uint32_t* __restrict__ order
                                               const DevCamera* __restrict__ cams, int n, int tile, uint32_t n_items,
                                               const uint32_t* __restrict__ n_dev, uint64_t pair_cap,
                                               uint32_t* __restrict__ pkey, uint32_t* __restrict__ pval,
-                                              uint32_t* __restrict__ overflow, uint32_t* __restrict__ emit_item,
+                                              const uint32_t* __restrict__ total_hi, uint32_t* __restrict__ overflow,
+                                              uint32_t* __restrict__ emit_item,
                                               float* __restrict__ pairgrad) {
     __shared__ uint32_t sbef[8], stot[8];
     const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -668,7 +674,7 @@ __global__ void __launch_bounds__(256) k_emit(const uint32_t* __restrict__ order
     if (k < nv) {
         if (emit_item != nullptr) off[k] = o;
         if (cnt != 0) {
-            if ((uint64_t)o + cnt > pair_cap) {
+            if ((uint64_t)o + cnt > pair_cap || *total_hi != 0u) {
                 atomicMax(overflow, 1u);
                 cnt = 0;
             } else {
@@ -899,7 +905,8 @@ cudaError_t sort_depth(gs_ctx* c, uint32_t n_max, uint32_t n_hint, cudaStream_t 
     }
     ++c->launches;
     const int blocks = (int)std::max<uint32_t>(1u, std::min<uint32_t>((n_max + 255u) / 256u, (n_hint + 255u) / 256u));
-    k_item_tiles<<<blocks, 256, 0, s>>>(c->dval[0], c->tiles_touched, n_max, c->dcount + 8, c->tile_blocks, c->dcount);
+    k_item_tiles<<<blocks, 256, 0, s>>>(c->dval[0], c->tiles_touched, n_max, c->dcount + 8, c->tile_blocks,
+                                         reinterpret_cast<unsigned long long*>(c->dcount));
     return cudaGetLastError();
 }
 
@@ -945,7 +952,7 @@ cudaError_t emit_pairs(gs_ctx* c, uint32_t n_items, const uint32_t* n_dev, cudaS
     ++c->launches;
     k_emit<<<blocks, 256, 0, s>>>(c->dval[0], c->tiles_touched, tile_blocks, scanned, c->offsets, c->rec, c->dcam, c->n,
                                   c->tile, n_items, n_dev, (uint64_t)c->pair_cap, c->pkey[0], c->pval[0], c->dcount + 1,
-                                  c->emit_item, c->pairgrad);
+                                  c->dcount + 9, c->emit_item, c->pairgrad);
     return cudaGetLastError();
 }
 
@@ -1021,7 +1028,7 @@ cudaError_t compute_ranges(gs_ctx* c, cudaStream_t s) {
     if (!c->side_zeroed) cudaMemsetAsync(c->ranges, 0, sizeof(uint2) * (size_t)c->n_bins, s);
     ++c->launches;
     k_ranges<<<c->num_sms * 8, 256, 0, s>>>(c->pkey[c->pair_buf], c->dcount, (uint64_t)c->pair_cap,
-                                            (uint32_t)c->n_bins, c->dcount + 1, c->ranges,
+                                            (uint32_t)c->n_bins, c->dcount + 9, c->ranges,
                                             c->order_ahead ? c->dcount + 13 : nullptr, c->dcount + 14, order_spec(c),
                                             c->work_order);
     if (c->points != nullptr) return launch_point_items(c, *c->points, true, s);
