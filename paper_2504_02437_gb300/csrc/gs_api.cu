@@ -454,7 +454,8 @@ int gs_create(const gs_config* cfg, int device, gs_ctx** out) {
         ok = ok && dalloc(&c->n_last, V * maxpix) == cudaSuccess;
         ok = ok && dalloc(&c->dLdC, 3 * V * maxpix) == cudaSuccess;
         ok = ok && dalloc(&c->grad2d, kGrad2dStride * V * cap) == cudaSuccess;
-        ok = ok && dalloc(&c->hist, sort_hist_words(c->sort_blocks)) == cudaSuccess;
+        c->hist_words = sort_hist_words(c->sort_blocks, V * cap);
+        ok = ok && dalloc(&c->hist, c->hist_words) == cudaSuccess;
         ok = ok && dalloc(&c->dcount, 16) == cudaSuccess;
         ok = ok && dalloc(&c->vis_blocks, V * ((cap + 255) / 256) + 1) == cudaSuccess;
         ok = ok && dalloc(&c->vis_range, V * ((cap + 255) / 256) + 1) == cudaSuccess;

@@ -134,6 +134,7 @@ struct gs_ctx {
 
     // scratch
     uint32_t* hist = nullptr;               // radix / scan block counters
+    size_t hist_words = 0;
     const float** target_slot = nullptr;    // device: the target image of the current iteration
     float* ssim_maps = nullptr;             // [3][V][3][H][W] SSIM derivative maps (lambda_photo > 0)
     float* ssim_part = nullptr;             // [2 ssim_blocks] per-CTA photometric loss terms
@@ -249,7 +250,7 @@ cudaError_t radix_sort_pairs(gs_ctx* c, uint32_t** keys, uint32_t** vals, const 
 cudaError_t sort_depth(gs_ctx* c, uint32_t n_max, uint32_t n_hint, cudaStream_t s);
 bool depth_sort_small(const gs_ctx* c);    // the map is small enough for the one-CTA depth sort
 cudaError_t sort_kernels_init();           // once per context, on its device
-size_t sort_hist_words(int sort_blocks);
+size_t sort_hist_words(int sort_blocks, size_t max_items);   // of a context with so many (view, Gaussian) items
 int sort_max_blocks();
 cudaError_t emit_pairs(gs_ctx* c, uint32_t n_items, const uint32_t* n_dev, cudaStream_t s);
 // exclusive scan of n u32 values (in may equal out); the total goes to *total_dev

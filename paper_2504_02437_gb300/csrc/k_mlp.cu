@@ -619,7 +619,7 @@ struct gs_mlp {
     float* g = nullptr;      // gradient
     float* m = nullptr;
     float* v = nullptr;
-    uint8_t* img = nullptr;  // bf16 weights in the kernels' shared-memory layout [kImgBytes]
+    uint8_t* img = nullptr;  // bf16 weights in the kernels' shared-memory layout [kImgBytes], then derr
     int t = 0;
     int rows_cap = 0;
     float* y = nullptr;      // [rows][16] predictions for an insertion
@@ -726,8 +726,8 @@ int gs_mlp_create(int device, uint64_t seed, gs_mlp** out) {
     ok = ok && cudaMalloc(&M->g, sizeof(float) * kParams) == cudaSuccess;
     ok = ok && cudaMalloc(&M->m, sizeof(float) * kParams) == cudaSuccess;
     ok = ok && cudaMalloc(&M->v, sizeof(float) * kParams) == cudaSuccess;
-    ok = ok && cudaMalloc(&M->img, kImgBytes) == cudaSuccess;
-    ok = ok && cudaMalloc(&M->derr, sizeof(uint32_t)) == cudaSuccess;
+    ok = ok && cudaMalloc(&M->img, kImgBytes + sizeof(uint32_t)) == cudaSuccess;
+    if (ok) M->derr = reinterpret_cast<uint32_t*>(M->img + kImgBytes);
     ok = ok && cudaMemset(M->derr, 0, sizeof(uint32_t)) == cudaSuccess;
     ok = ok && cudaMallocHost((void**)&M->herr, sizeof(uint32_t)) == cudaSuccess;
     if (ok) *M->herr = 0u;
@@ -771,7 +771,7 @@ int gs_mlp_create(int device, uint64_t seed, gs_mlp** out) {
 void gs_mlp_destroy(gs_mlp* M) {
     if (!M) return;
     cudaSetDevice(M->device);
-    void* ps[] = {M->p, M->g, M->m, M->v, M->img, M->y, M->part, M->loss_part, M->derr};
+    void* ps[] = {M->p, M->g, M->m, M->v, M->img, M->y, M->part, M->loss_part};
     for (void* q : ps) cudaFree(q);
     if (M->herr) cudaFreeHost(M->herr);
     delete M;
