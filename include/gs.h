@@ -122,6 +122,15 @@ GS_API void gs_destroy(gs_ctx* ctx);
 /* Last error message of this context ("" if none); valid until the next call. */
 GS_API const char* gs_last_error(const gs_ctx* ctx);
 
+/* Give back the device memory that map management keeps from call to call
+ * until gs_destroy: a second set of parameters and moments, which the first
+ * gs_densify that splits allocates (168 bytes per Gaussian of capacity), and
+ * scratch as large as the largest gs_init_map, gs_insert, gs_densify or
+ * gs_count_dominant needed (the last: 16 bytes per pixel of all its views).
+ * The calls that need either allocate it again. Waits for the device.
+ * Errors: GS_ERR_CUDA. */
+GS_API int gs_trim(gs_ctx* ctx);
+
 /* Number of Gaussians currently in the map. */
 GS_API int gs_num_gaussians(const gs_ctx* ctx);
 

@@ -50,6 +50,7 @@ SIGNATURES = {
     "gs_default_config": (None, [C.POINTER(gs_config)]),
     "gs_create": (_I, [C.POINTER(gs_config), _I, C.POINTER(_P)]),
     "gs_destroy": (None, [_P]),
+    "gs_trim": (_I, [_P]),
     "gs_last_error": (C.c_char_p, [_P]),
     "gs_num_gaussians": (_I, [_P]),
     "gs_set_params": (_I, [_P, _P, _I, _P]),

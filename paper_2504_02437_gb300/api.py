@@ -142,6 +142,10 @@ class GaussianMap:
     def pixels_per_thread(self) -> int:
         return self.lib.gs_pixels_per_thread(self.ctx)
 
+    def trim(self):
+        """Give back the device memory that insertions and splits keep from call to call."""
+        self._check(self.lib.gs_trim(self.ctx))
+
     def set_params(self, params: torch.Tensor):
         p = params.detach().to(device=self._dev, dtype=torch.float32).contiguous()
         if p.dim() != 2 or p.shape[0] != 14:

@@ -1328,6 +1328,20 @@ int gs_init_map(gs_ctx* c, const float* pts, const float* rgb, int n, void* stre
     return GS_OK;
 }
 
+int gs_trim(gs_ctx* c) {
+    if (!c) return GS_ERR_ARG;
+    CK(cudaSetDevice(c->device));
+    CK(cudaDeviceSynchronize());
+    for (float*& q : c->spare) {
+        cudaFree(q);
+        q = nullptr;
+    }
+    cudaFree(c->scratch);
+    c->scratch = nullptr;
+    c->scratch_bytes = 0;
+    return GS_OK;
+}
+
 int gs_set_initializer(gs_ctx* c, gs_mlp* mlp) {
     if (!c) return GS_ERR_ARG;
     c->init_mlp = mlp;

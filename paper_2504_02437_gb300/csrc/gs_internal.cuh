@@ -231,7 +231,7 @@ struct gs_ctx {
     int force_tile = 0, force_ppt = 0;      // set while the autotuner times a candidate
     gs_mlp* init_mlp = nullptr;             // learned initialiser of gs_insert (NULL = plain)
     // what the map-management calls need while they run (each ends with a synchronisation): kept from
-    // call to call, grown when a call needs more, freed with the context
+    // call to call, grown when a call needs more, freed by gs_trim and with the context
     uint8_t* scratch = nullptr;
     size_t scratch_bytes = 0;
     float* spare[3] = {};                   // [14][cap] the other parameter and moment buffers of a split
