@@ -210,8 +210,10 @@ GS_API int gs_step(gs_ctx* ctx, void* stream);
  * thread) candidates without updating the map and keeps the fastest (not in
  * the deterministic mode, which has one layout and adds a fixed-order
  * per-Gaussian sum of the adjoint's per-pair gradients). An
- * overflow of the pair buffer during a replay skips that iteration's Adam
- * step; a later call then grows the buffer and returns GS_ERR_CAPACITY. A
+ * overflow of the pair buffer during a replay composites nothing: that
+ * iteration's image is black and its loss that of a black image, its Adam step
+ * is skipped and the densification statistics stay; a later call then grows
+ * the buffer and returns GS_ERR_CAPACITY. A
  * non-finite loss, or a non-finite gradient (its parameter and moments are
  * left unchanged by the Adam step), makes a later call return
  * GS_ERR_NONFINITE once, before it does any work. */

@@ -375,7 +375,8 @@ __device__ __forceinline__ float dot2(float a, float b, float c, float d) {
 __global__ void __launch_bounds__(128, 4) k_preprocess_backward(
     const float* __restrict__ P, int n, int cap, int n_views, const DevCamera* __restrict__ cams, DevConst kc,
     const float* __restrict__ grad2d, const uint32_t* __restrict__ tiles, float* __restrict__ G,
-    float* __restrict__ dens_sum, float* __restrict__ dens_cnt, int add_reg, float reg_scale) {
+    float* __restrict__ dens_sum, float* __restrict__ dens_cnt, const uint32_t* __restrict__ overflow, int add_reg,
+    float reg_scale) {
     int gid = blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= n) return;
     float p[kParamRows];
@@ -539,7 +540,7 @@ __global__ void __launch_bounds__(128, 4) k_preprocess_backward(
     G[11 * c + gid] = dr;
     G[12 * c + gid] = dg;
     G[13 * c + gid] = db;
-    if (dens_sum != nullptr && gcnt > 0.f) {
+    if (dens_sum != nullptr && gcnt > 0.f && *overflow == 0u) {   // (an overflow: nothing was composited)
         atomicAdd(dens_sum + gid, gsum);   // (one each: added in L2, nothing waits for it)
         atomicAdd(dens_cnt + gid, gcnt);
     }
@@ -572,7 +573,7 @@ cudaError_t launch_preprocess_backward(gs_ctx* c, const DevConst& k, bool add_re
     ++c->launches;
     k_preprocess_backward<<<(c->n + 127) / 128, 128, 0, s>>>(c->params, c->n, c->cap, c->n_views, c->dcam, k,
                                                               c->grad2d, c->tiles_touched, c->grads, c->dens_sum,
-                                                              c->dens_cnt, add_reg ? 1 : 0, reg_scale);
+                                                              c->dens_cnt, c->dcount + 9, add_reg ? 1 : 0, reg_scale);
     return cudaGetLastError();
 }
 
