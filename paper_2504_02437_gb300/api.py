@@ -21,9 +21,15 @@ from . import _native as N
 # Stream object, and a camera's rotation is written in one piece.
 
 
+# (not a public name: without it, the public call and the object it builds)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream() -> int:
     """The current stream of the current device."""
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
