@@ -189,9 +189,12 @@ void pick_layout(gs_ctx* c, int w, int h, int views, int& tile, int& ppt) {
     if (want == 1 || want == 2 || (want == 4 && tile == 16))
         ppt = want;
     else
-        // 16 x 2 (with halved long tiles) is the fastest 16-px layout at every size measured: iteration
-        // with 16 x 1 / 16 x 2 of a 160x120 keyframe with 2k Gaussians 112 / 104 us, 1200x680 with 300k
-        // 551 / 502 us, 8 x 640x480 with 150k 1,148 / 1,045 us
+        // 16 x 2 (with halved long tiles): iteration with 16 x 1 / 16 x 2 of a 160x120 keyframe with 2k
+        // Gaussians 112 / 104 us, 1200x680 with 300k 551 / 502, 8 x 640x480 with 150k 1,148 / 1,045, of
+        // rooms at 333x251 to 800x600 1.06 to 1.26 times as fast, of random Gaussians that overlap a lot
+        // 1.04 to 1.15 times. Of small random ones that leave most pixels of a box untouched 16 x 1 is up
+        // to 8 % the faster (two 640x480 views of 100k 243 / 263), which the host cannot tell; the
+        // autotuner (tile_size 0) times both.
         ppt = (t && t->tile == tile) ? t->ppt : (tile == 16 ? 2 : 1);
 }
 
