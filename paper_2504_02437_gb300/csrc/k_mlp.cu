@@ -5,7 +5,7 @@
 // a Gaussian inserted at a VO point from the keyframe's 5x5 patch around the
 // point, its depth and its camera-frame position.
 //
-// A CTA takes 64 rows through the whole network (and, in training, back through it) in one launch,
+// A CTA takes 32 or 64 rows through the whole network (and, in training, back through it) in one launch,
 // on tcgen05.mma with bf16 operands in shared memory and f32 accumulators in TMEM. Upstream
 // gradients dZ enter as bf16 hi + lo pairs (two products), so the backward
 // keeps ~16 mantissa bits where one bf16 rounding would keep 8.
@@ -171,11 +171,12 @@ __device__ __forceinline__ void store_col(uint8_t* dst, int r0, int j, const bf1
 // part[blockIdx.x][kParams], with its loss in loss_part.
 //
 // Every product has the 128 hidden units as its M dimension and rows (or units) as N, so a small
-// batch spreads over SMs and no accumulator lane is padding; a thread owns one hidden unit and 32
-// rows. What bounds it is latency: eight products, each a few hundred tensor cycles, and between
-// them a read of TMEM, an erf (and, back, an exp) a value and a rewrite of the operands. One launch
-// takes the place of 20 (elementwise kernels and strided GEMMs that gathered their operands element by
-// element): gradients of 4,096 rows 400 -> 20 us, a prediction of 96 rows 58 -> 6 us.
+// batch spreads over SMs and no accumulator lane is padding; a thread owns one hidden unit and half of
+// a pass's rows. What bounds it is latency: eight products, each a few hundred tensor cycles, and between
+// them a read of TMEM, an erf (and, back, an exp) a value and a rewrite of the operands. With k_mlp_reduce
+// it takes the place of 21 launches (elementwise kernels and strided GEMMs that gathered their operands
+// element by element; 7 of them for a prediction alone): gradients of 4,096 rows 400 -> 20 us, a
+// prediction of 96 rows 58 -> 6 us.
 //
 // A wait that gives up ends the CTA's work: it writes nothing, sets both flags of `err`, and leaves once
 // its weight copy and its products have ended (a bounded wait again), so that neither runs on in shared

@@ -885,8 +885,8 @@ __global__ void __launch_bounds__(1024) k_work_order(const uint2* __restrict__ r
 // The sorted pairs' (start, end) per bin. After an overflow of the pair buffer the sorted values hold
 // slots that no item wrote: every bin stays empty then, and nothing is composited. Where *fresh is set
 // (a replayed iteration whose cameras are not those of the one before, which left the work list for
-// them), the last CTA to finish writes the list of these ranges. Single views of a window in turn, with
-// the list of the view before: 522 us an iteration; with their own: 318.
+// them), the last CTA to finish writes the list of these ranges. Single 640x480 views of a window in
+// turn, with the list of the view before: 522 us an iteration; with their own: 318.
 __global__ void __launch_bounds__(256) k_ranges(const uint32_t* __restrict__ pkey, const uint32_t* __restrict__ P_dev,
                                                 uint64_t pair_cap, uint32_t n_bins, const uint32_t* __restrict__ overflow,
                                                 uint2* __restrict__ ranges, const uint32_t* __restrict__ fresh,
