@@ -8,7 +8,7 @@ import torch
 
 from synth import frustum_scene, random_target
 
-from gpu_helpers import cuda, new_map
+from gpu_helpers import cuda, new_map, rotated_cam
 
 pytestmark = pytest.mark.gpu
 
@@ -55,3 +55,22 @@ def test_even_lists(width, height, views):
     for a, b in zip(outs[0][1][:1], outs[1][1][:1]):
         # float32 sums of up to a few thousand pixel terms a Gaussian in another order
         assert float((a - b).norm()) <= 1e-5 * float(b.norm())
+
+
+def test_replays_of_other_cameras():
+    """A replay of other cameras writes the list of its own ranges (in another kernel, by 256 threads)."""
+    n, width, height = 40_000, 640, 480
+    p, cam = frustum_scene(n=n, width=width, height=height, fx=width * 0.9, fy=width * 0.9, cx=width / 2,
+                           cy=height / 2, seed=1, logscale_mean=-4.5)
+    cams = [cam, rotated_cam(cam, [0.01, -0.01, 0.02], [0.02, 0.0, 0.0]), rotated_cam(cam, [0, 0.01, 0], [0, 0, 0.1])]
+    tg = cuda(random_target(width, height, seed=2))
+    gm = new_map(n, W=width, H=height, tile_size=16, pixels_per_thread=2, lr=(0.0,) * 5)
+    ref = new_map(n, W=width, H=height, tile_size=16, pixels_per_thread=1)
+    for m in (gm, ref):
+        m.set_params(cuda(p))
+    rgb = torch.empty(1, 3, height, width, device="cuda")
+    for k in (0, 0, 1, 2, 2, 0, 1):
+        rgb.fill_(float("nan"))
+        gm.iterate(cams[k], tg, rgb_out=rgb)
+        assert torch.equal(rgb, ref.render(cams[k])), k
+    assert torch.equal(gm.params(), cuda(p))
