@@ -776,16 +776,16 @@ struct OrderSpec {
     uint32_t n_bins;
     int halves;
     uint32_t split_min, split_share;
-    uint32_t wave;   // 0: evenness is not looked at
+    uint32_t wave;   // CTAs that run at a time; 0: evenness is not looked at
     const uint32_t* n_pairs;
     const uint32_t* cancel;
 };
-template <int NT>
+template <int NT, bool EVEN>
 __device__ __forceinline__ void build_work_order(const uint2* ranges, const OrderSpec& o, uint32_t* __restrict__ order) {
     constexpr int E = 1024 / NT;   // buckets a thread
-    // lists a thread keeps in registers between the passes (of the one-CTA launch: its latency is a few
-    // round trips to L2)
-    constexpr int R = NT == 1024 ? 3 : 0;
+    // lists a thread keeps in registers between the passes (of a launch of its own, which is a few round
+    // trips to L2 long; with the evenness to look at they take one pass more)
+    constexpr int R = EVEN && NT == 1024 ? 3 : 0;
     __shared__ uint32_t cnt[1024];
     __shared__ uint32_t wsum[32];
     const int t = threadIdx.x, lane = t & 31;
@@ -811,7 +811,7 @@ __device__ __forceinline__ void build_work_order(const uint2* ranges, const Orde
     uint32_t longest = o.halves ? max(o.split_min, *o.n_pairs / o.split_share) : 0xFFFFFFFFu;
     uint32_t whole = 0xFFFFFFFFu;   // of even lists: the tiles before the halved ones
     for (int e = 0; e < E; ++e) cnt[t * E + e] = 0;
-    if (o.wave != 0u) {
+    if constexpr (EVEN) {
         __shared__ uint32_t most;
         if (t == 0) most = 0u;
         __syncthreads();
@@ -860,13 +860,13 @@ __device__ __forceinline__ void build_work_order(const uint2* ranges, const Orde
         cnt[t * E + e] = start;
         start += v[e];
     }
-    if (whole != 0xFFFFFFFFu) start = 2u * o.n_bins - whole;
+    if (EVEN && whole != 0xFFFFFFFFu) start = 2u * o.n_bins - whole;
     if (t == NT - 1) order[0] = o.cancel != nullptr && *o.cancel != 0u ? 0u : start;
     __syncthreads();
     each_bin([&](uint32_t b, uint32_t len) {
         const bool two = len > longest;
         const uint32_t p = atomicAdd(&cnt[order_slot(len)], two ? 2u : 1u);
-        if (p >= whole) {
+        if (EVEN && p >= whole) {
             order[1 + 2 * p - whole] = b | (1u << kItemShift);
             order[2 + 2 * p - whole] = b | (2u << kItemShift);
         } else if (two) {
@@ -877,9 +877,10 @@ __device__ __forceinline__ void build_work_order(const uint2* ranges, const Orde
         }
     });
 }
+template <bool EVEN>
 __global__ void __launch_bounds__(1024) k_work_order(const uint2* __restrict__ ranges, OrderSpec spec,
                                                       uint32_t* __restrict__ order) {
-    build_work_order<1024>(ranges, spec, order);
+    build_work_order<1024, EVEN>(ranges, spec, order);
 }
 
 // The sorted pairs' (start, end) per bin. After an overflow of the pair buffer the sorted values hold
@@ -887,6 +888,7 @@ __global__ void __launch_bounds__(1024) k_work_order(const uint2* __restrict__ r
 // (a replayed iteration whose cameras are not those of the one before, which left the work list for
 // them), the last CTA to finish writes the list of these ranges. Single 640x480 views of a window in
 // turn, with the list of the view before: 522 us an iteration; with their own: 318.
+template <bool EVEN>
 __global__ void __launch_bounds__(256) k_ranges(const uint32_t* __restrict__ pkey, const uint32_t* __restrict__ P_dev,
                                                 uint64_t pair_cap, uint32_t n_bins, const uint32_t* __restrict__ overflow,
                                                 uint2* __restrict__ ranges, const uint32_t* __restrict__ fresh,
@@ -909,7 +911,7 @@ __global__ void __launch_bounds__(256) k_ranges(const uint32_t* __restrict__ pke
     if (!last) return;
     __threadfence();
     if (threadIdx.x == 0) *ticket = 0u;
-    build_work_order<256>(ranges, spec, order);
+    build_work_order<256, EVEN>(ranges, spec, order);
 }
 
 }  // namespace
@@ -1086,17 +1088,20 @@ cudaError_t compute_ranges(gs_ctx* c, cudaStream_t s) {
     // (a mapping iteration zeroes the ranges on its side stream)
     if (!c->side_zeroed) cudaMemsetAsync(c->ranges, 0, sizeof(uint2) * (size_t)c->n_bins, s);
     ++c->launches;
-    k_ranges<<<c->num_sms * 8, 256, 0, s>>>(c->pkey[c->pair_buf], c->dcount, (uint64_t)c->pair_cap,
-                                            (uint32_t)c->n_bins, c->dcount + 9, c->ranges,
-                                            c->order_ahead ? c->dcount + 13 : nullptr, c->dcount + 14, order_spec(c),
-                                            c->work_order);
+    const OrderSpec spec = order_spec(c);
+    auto ranges = spec.wave != 0u ? k_ranges<true> : k_ranges<false>;
+    ranges<<<c->num_sms * 8, 256, 0, s>>>(c->pkey[c->pair_buf], c->dcount, (uint64_t)c->pair_cap, (uint32_t)c->n_bins,
+                                          c->dcount + 9, c->ranges, c->order_ahead ? c->dcount + 13 : nullptr,
+                                          c->dcount + 14, spec, c->work_order);
     if (c->points != nullptr) return launch_point_items(c, *c->points, true, s);
     return c->order_ahead ? cudaGetLastError() : launch_work_order(c, s);
 }
 
 cudaError_t launch_work_order(gs_ctx* c, cudaStream_t s) {
     ++c->launches;
-    k_work_order<<<1, 1024, 0, s>>>(c->ranges, order_spec(c), c->work_order);
+    const OrderSpec spec = order_spec(c);
+    auto work_order = spec.wave != 0u ? k_work_order<true> : k_work_order<false>;
+    work_order<<<1, 1024, 0, s>>>(c->ranges, spec, c->work_order);
     return cudaGetLastError();
 }
 
