@@ -370,7 +370,6 @@ struct SmallSmem {
     uint16_t wcnt[32][1 << kSmallBits];
     uint32_t start[1 << kSmallBits];
     uint32_t wsum[32], kmin, kmax;
-    unsigned long long total;
 };
 __global__ void __launch_bounds__(kSmallThreads, 1) k_small_depth(const uint32_t* __restrict__ kin, uint32_t n,
                                                                  const uint32_t* __restrict__ tiles,
@@ -492,8 +491,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_depth(const uint32_t
         }
         __syncthreads();
     }
-    if (t == 0) sm.total = 0;
-    __syncthreads();
+    unsigned long long total = 0;   // (threads 0 .. 3: their blocks')
     // tile counts per 256 ordered items (eight warps of 32 a block): sums for the emission
     for (uint32_t i0 = 0; i0 < m; i0 += kSmallThreads) {
         const uint32_t i = i0 + t;
@@ -510,13 +508,17 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small_depth(const uint32_t
             unsigned long long b = 0;
             for (int q = 0; q < 8; ++q) b += sm.wsum[8 * t + q];
             tile_blocks[i0 / 256 + t] = (uint32_t)b;
-            atomicAdd(&sm.total, b);
+            total += b;
         }
         __syncthreads();
     }
+    if (t < 4) {
+        total += __shfl_xor_sync(0xFu, total, 1);
+        total += __shfl_xor_sync(0xFu, total, 2);
+    }
     if (t == 0) {
-        counts[0] = (uint32_t)sm.total;
-        counts[1] = (uint32_t)(sm.total >> 32);
+        counts[0] = (uint32_t)total;
+        counts[1] = (uint32_t)(total >> 32);
         counts[8] = m;
     }
 }
@@ -642,6 +644,7 @@ __global__ void __launch_bounds__(256) k_emit(const uint32_t* __restrict__ order
     const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const uint32_t nv = umin(n_items, *n_dev);
+    const bool too_many = *total_hi != 0u;
     if (blockIdx.x * blockDim.x >= nv) return;   // the whole CTA is past the visible items
     uint32_t item = 0, cnt = 0, o = 0, bin0 = 0, tiles_x = 0;
     int tx0 = 0, ty0 = 0, wt = 1;
@@ -674,7 +677,7 @@ __global__ void __launch_bounds__(256) k_emit(const uint32_t* __restrict__ order
     if (k < nv) {
         if (emit_item != nullptr) off[k] = o;
         if (cnt != 0) {
-            if ((uint64_t)o + cnt > pair_cap || *total_hi != 0u) {
+            if (too_many || (uint64_t)o + cnt > pair_cap) {
                 atomicMax(overflow, 1u);
                 cnt = 0;
             } else {
